@@ -577,18 +577,15 @@ im_status im_policy_forward(im_policy *p, uint32_t step, int32_t n, const float 
     const float *in = obs;
     int ld_in = ld_obs;
     const int A = p->cfg.dims[p->nl];
-    for (int l = 0; l < p->nl; ++l) {
-        const bool last = l == p->nl - 1;
-        float *outp = last ? mean_out : p->d_act[l & 1];
-        const int ldc = last ? A : p->act_ld;
-        IM_CUDA(launch_linear_simt(in, ld_in, p->d_W[l], p->cfg.dtype == 1, p->d_b[l], outp, ldc, n,
-                                   p->cfg.dims[l + 1], p->cfg.dims[l], !last, p->stream));
-        in = outp;
-        ld_in = ldc;
+    for (int l = 0; l + 1 < p->nl; ++l) {
+        IM_CUDA(launch_linear_simt(in, ld_in, p->d_W[l], p->cfg.dtype == 1, p->d_b[l], p->d_act[l & 1], p->act_ld, n,
+                                   p->cfg.dims[l + 1], p->cfg.dims[l], p->stream));
+        in = p->d_act[l & 1];
+        ld_in = p->act_ld;
     }
-    if (action_out)
-        IM_CUDA(launch_sample(mean_out, action_out, logp_out, n, A, p->cfg.sigma, p->d_log_std, p->cfg.seed, step,
-                              p->cfg.env_id_base, p->stream));
+    const int last = p->nl - 1;
+    IM_CUDA(launch_head_simt(in, ld_in, p->d_W[last], p->cfg.dtype == 1, p->d_b[last], mean_out, action_out, logp_out, n, A,
+                             p->cfg.dims[last], p->cfg.sigma, p->d_log_std, p->cfg.seed, step, p->cfg.env_id_base, p->stream));
     return IM_OK;
 }
 

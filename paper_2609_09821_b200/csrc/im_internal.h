@@ -4,6 +4,7 @@
 #include <stdint.h>
 #include <atomic>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "../../include/im.h"
@@ -69,6 +70,22 @@ struct DeviceOnce {
         return e;
     }
 };
+// Launch with programmatic stream serialization: the kernel's prologue may overlap the tail of the kernel before it in
+// the stream.  The kernel executes griddepcontrol.wait before its first access to global memory.  cluster > 0: blocks per
+// cluster (along x) of a kernel that does not fix them itself.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = cluster > 0 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 // Number of SMs of the current device (cached per device).
 int device_sm_count();
 

@@ -20,10 +20,13 @@ struct im_policy {
 };
 
 namespace im {
+// Hidden layer: C = relu(A W^T + bias).
 cudaError_t launch_linear_simt(const float *A, int lda, const void *W, bool w_bf16, const float *bias, float *C,
-                               int ldc, int M, int N, int K, bool relu, cudaStream_t stream);
-cudaError_t launch_sample(const float *mean, float *action, float *logp, int n, int A, float sigma, const float *log_std,
-                          uint64_t seed, uint32_t step, uint32_t env_id_base, cudaStream_t stream);
+                               int ldc, int M, int N, int K, cudaStream_t stream);
+// Last layer with the Gaussian head: mean [M][N] and, unless action is null, action [M][N] (and logp [M] unless null).
+cudaError_t launch_head_simt(const float *A, int lda, const void *W, bool w_bf16, const float *bias, float *mean, float *action,
+                             float *logp, int M, int N, int K, float sigma, const float *log_std, uint64_t seed, uint32_t step,
+                             uint32_t env_id_base, cudaStream_t stream);
 
 // Tensor-core path (mlp_tc.cu).
 im_status tc_policy_create(im_policy *p, const void *const *W, const float *const *b);

@@ -14,7 +14,6 @@
 // through the common exit that frees its tensor memory.
 #include <cmath>
 #include <cstring>
-#include <utility>
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -1156,20 +1155,6 @@ namespace im {
 
 namespace {
 
-// Launch with programmatic stream serialization (see dep_wait): the kernel's prologue overlaps the tail of the
-// kernel before it in the stream.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args &&...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 template <int BLOCK_N, bool BWD = false>
 cudaError_t launch_hidden(const TcLayer &L, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
 {
@@ -1185,7 +1170,7 @@ cudaError_t launch_hidden(const TcLayer &L, const GemmParams &gp_in, int n_sm, c
     const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes(BWD));
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
     const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, dim3(grid), dim3(kThreads), smem, stream,
+    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, dim3(grid), dim3(kThreads), smem, stream, 0,
                                       L.map_a, L.map_b, L.map_c, L.map_m, gp);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -1208,7 +1193,7 @@ cudaError_t launch_hidden_mn(const TcLayer &L, const GemmParams &gp_in, int n_sm
     const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes());
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
     const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, true>, dim3(grid), dim3(kThreads), smem, stream,
+    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, true>, dim3(grid), dim3(kThreads), smem, stream, 0,
                                       L.map_a, L.map_b, L.map_c, L.map_c, gp);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -1225,7 +1210,7 @@ cudaError_t launch_hidden_pair(const TcLayer &L, const GemmParams &gp, int n_sm,
     }
     const int tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * (MN ? gp.n_batches : 1);
     const int pairs = tiles < n_sm / 2 ? tiles : n_sm / 2;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_pair_kernel<BWD, MN>, dim3(2 * pairs), dim3(pair_threads(BWD)), pair_smem_bytes(BWD), stream,
+    const cudaError_t le = launch_pdl(linear_tc_hidden_pair_kernel<BWD, MN>, dim3(2 * pairs), dim3(pair_threads(BWD)), pair_smem_bytes(BWD), stream, 0,
                                       L.map_a, MN ? L.map_b : L.map_b2, L.map_c, L.map_m, gp);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -1248,7 +1233,7 @@ cudaError_t launch_head(const TcLayer &L, const GemmParams &gp_in, int n_sm, cud
     const size_t smem = Plan::bytes(gp.stages, epi);
     const int tiles = (gp.M + BLOCK_M - 1) / BLOCK_M;
     const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_head_kernel<BLOCK_N>, dim3(grid), dim3(kHeadThreads), smem, stream, L.map_a, L.map_b, gp);
+    const cudaError_t le = launch_pdl(linear_tc_head_kernel<BLOCK_N>, dim3(grid), dim3(kHeadThreads), smem, stream, 0, L.map_a, L.map_b, gp);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
 }

@@ -70,17 +70,15 @@ extern "C" im_status im_policy_forward_noalloc(int32_t n_layers, const int32_t *
     const float *in = obs;
     int ld_in = ld_obs;
     const int A = dims[n_layers];
-    for (int l = 0; l < n_layers; ++l) {
-        const bool last = l == n_layers - 1;
-        float *outp = last ? mean_out : act[l & 1];
-        const int ldc = last ? A : IM_NOALLOC_MAX_WIDTH;
-        if (im::launch_linear_simt(in, ld_in, W[l], false, b[l], outp, ldc, n, dims[l + 1], dims[l], !last, stream) !=
-            cudaSuccess)
+    for (int l = 0; l + 1 < n_layers; ++l) {
+        if (im::launch_linear_simt(in, ld_in, W[l], false, b[l], act[l & 1], IM_NOALLOC_MAX_WIDTH, n, dims[l + 1], dims[l], stream) != cudaSuccess)
             return IM_ERR_CUDA;
-        in = outp;
-        ld_in = ldc;
+        in = act[l & 1];
+        ld_in = IM_NOALLOC_MAX_WIDTH;
     }
-    if (im::launch_sample(mean_out, action_out, logp_out, n, A, sigma, nullptr, seed, step, env_id_base, stream) != cudaSuccess)
+    const int last = n_layers - 1;
+    if (im::launch_head_simt(in, ld_in, W[last], false, b[last], mean_out, action_out, logp_out, n, A, dims[last], sigma, nullptr, seed,
+                             step, env_id_base, stream) != cudaSuccess)
         return IM_ERR_CUDA;
     return IM_OK;
 }

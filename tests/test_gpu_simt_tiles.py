@@ -1,0 +1,36 @@
+"""fp32 policy layers at the edges of their tiles: row counts around 16 / 32 / 64, widths and depths that are no
+multiples of a tile or of four, every choice of tile, action widths of one and of several 32-column groups."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2609_09821_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,dims", [
+    (1, (5, 3, 2)), (15, (361, 17, 28)), (17, (360, 1024, 512, 28)), (64, (361, 1024, 512, 33)), (65, (259, 130, 69)),
+    (300, (577, 1024, 512, 69)), (1025, (362, 1021, 64, 300)),
+])
+def test_forward_matches_oracle(n, dims):
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    w = W.make_policy_weights(dims, "f32", seed=3)
+    pol = B.Policy(dims, w["W"], w["b"], "f32", 0.2, 7, n)
+    ld = B.padded_ld(dims[0], 4)
+    obs = torch.randn(n, ld, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    mean, action = torch.empty(n, dims[-1], device="cuda"), torch.empty(n, dims[-1], device="cuda")
+    logp = torch.empty(n, device="cuda")
+    pol.forward(5, obs, mean, action, logp)
+    m2 = torch.empty_like(mean)
+    pol.forward(5, obs, m2, None)
+    torch.cuda.synchronize()
+    ref = O.policy_forward(dims, w["W"], w["b"], 0.2, 7, 5, obs[:, :dims[0]].cpu().numpy())
+    for got, want, tol in ((mean, ref["mean"], 1e-4), (action, ref["action"], 1e-4)):
+        got, want = got.cpu().numpy().astype(np.float64), np.asarray(want, np.float64)
+        assert np.all(np.abs(got - want) <= tol * (np.abs(want) + np.sqrt(np.mean(want ** 2))))
+    # fp32 sums of A squared normals, each with relative error 2^-23 and the noise's own 1e-6
+    lp = np.asarray(ref["logp"], np.float64)
+    assert np.all(np.abs(logp.cpu().numpy() - lp) <= 1e-3 + 1e-5 * np.abs(lp))
+    assert torch.equal(mean, m2)
