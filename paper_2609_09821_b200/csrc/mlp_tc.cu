@@ -192,6 +192,9 @@ struct GemmParams {
     // with rows [b b_batch_rows, +N) of B into rows [b a_batch_rows, +M) of C.  n_batches = 1: plain GEMM.
     int n_batches, a_batch_rows, b_batch_rows;
     int c_batch_rows;  // rows of C between two batches
+    // M/N-major products: the contraction's kb_total k-blocks are shared out over the batches ("slices") as evenly as
+    // whole k-blocks allow, slice b taking [b kb_total / n_batches, (b + 1) kb_total / n_batches)
+    int kb_total;
     // Backward-pass epilogue (BWD instantiations): output (r, c) is zeroed where mask[r][c] <= 0 (the ReLU of the
     // forward pass), and the column sums of the masked fp32 values over each 32-row block r / 32 go to
     // colsum_partial[(r / 32) * ld_partial + c] (M a multiple of 32).  Either may be null.
@@ -239,6 +242,15 @@ struct SmemPlan {
     }
     __host__ __device__ static constexpr size_t bytes(int stages, int epi_bytes) { return 1024 + (size_t)stages * kStageBytes + epi_bytes + kBarBytes; }
 };
+
+// k-blocks of a tile of batch b: first and count.
+template <bool MN>
+__device__ __forceinline__ void slice_k_blocks(const GemmParams &P, int b, int &kb0, int &n_kb)
+{
+    if (!MN) { kb0 = 0; n_kb = P.K_blocks; return; }
+    kb0 = (int)((long long)b * P.kb_total / P.n_batches);
+    n_kb = (int)((long long)(b + 1) * P.kb_total / P.n_batches) - kb0;
+}
 
 struct Pipe {
     int stages;
@@ -315,9 +327,11 @@ __device__ __forceinline__ void producer_role(const Pipe &p, const CUtensorMap *
         const int b = tile / tiles_per_batch, t = tile - b * tiles_per_batch;
         if (MN) {
             // operands are [contraction rows][M or N columns]: a K block is 64 rows, fetched as boxes of 64 columns;
-            // batch b is the row range starting at b * a_batch_rows of both operands
-            const int mm = (t / P.n_tiles_n) * BLOCK_M, nn = (t % P.n_tiles_n) * BLOCK_N, r0 = b * P.a_batch_rows;
-            for (int kb = 0; kb < P.K_blocks; ++kb) {
+            // batch b is a range of the k-blocks of both operands
+            int kb0, n_kb;
+            slice_k_blocks<true>(P, b, kb0, n_kb);
+            const int mm = (t / P.n_tiles_n) * BLOCK_M, nn = (t % P.n_tiles_n) * BLOCK_N, r0 = kb0 * BLOCK_K;
+            for (int kb = 0; kb < n_kb; ++kb) {
                 if (!mbar_wait(&p.empty[stage], phase ^ 1u, p.abort_flag)) return;
                 uint8_t *sa = p.tiles + (size_t)stage * Plan::kStageBytes;
                 mbar_arrive_expect_tx(&p.full[stage], Plan::kABytes + Plan::kBBytes);
@@ -354,7 +368,9 @@ __device__ __forceinline__ void mma_role(const Pipe &p, uint32_t tmem_base, cons
         if (!mbar_wait(&p.acc_empty[acc], acc_phase ^ 1u, p.abort_flag)) return;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * Plan::kAccStride);
-        for (int kb = 0; kb < P.K_blocks; ++kb) {
+        int kb0, n_kb;
+        slice_k_blocks<MN>(P, MN ? tile / (n_tiles / P.n_batches) : 0, kb0, n_kb);
+        for (int kb = 0; kb < n_kb; ++kb) {
             if (!mbar_wait(&p.full[stage], phase, p.abort_flag)) return;
             tc_fence_after();
             const uint32_t sa = smem_u32(p.tiles + (size_t)stage * Plan::kStageBytes);
@@ -722,14 +738,16 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                 const int m0 = (tt / P.n_tiles_n) * 2 * BLOCK_M + (int)rank * BLOCK_M;
                 const int n0 = (tt % P.n_tiles_n) * 256 + (int)rank * 128;
                 bool ok = true;
-                for (int kb = 0; kb < P.K_blocks; ++kb) {
+                int kb0, n_kb;
+                slice_k_blocks<MN>(P, bt, kb0, n_kb);
+                for (int kb = 0; kb < n_kb; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t *sa = tiles + (size_t)stage * kPairStageBytes;
                     const uint32_t leader_full = map_to_rank(smem_u32(&full[stage]), 0);
                     if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * kPairStageBytes);
                     if (MN) {
                         // a K block is 64 rows of the slice; this CTA's 128 M columns and its 128 N columns as 64-column boxes
-                        const int r = bt * P.a_batch_rows + kb * BLOCK_K;
+                        const int r = (kb0 + kb) * BLOCK_K;
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
                             tma_load_2d_pair(sa + i * 8192, &map_a, leader_full, m0 + 64 * i, r);
@@ -755,7 +773,9 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                 if (!mbar_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 256);
-                for (int kb = 0; kb < P.K_blocks; ++kb) {
+                int kb0, n_kb;
+                slice_k_blocks<MN>(P, MN ? tile / tiles_per_batch : 0, kb0, n_kb);
+                for (int kb = 0; kb < n_kb; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t sa = smem_u32(tiles + (size_t)stage * kPairStageBytes);
@@ -1452,8 +1472,33 @@ im_status tc_gemm(const void *A, int64_t lda, const void *B, int64_t ldb, void *
 }
 
 
+// CTA pairs (256 x 256 tiles, half of the N operand per SM) when the output splits into whole 256-row tiles, the
+// slices' pitch keeps those tiles apart and there are tiles for most pairs.
+static bool tn_takes_pairs(int Mo, int No, int R, int slices, int c_pitch, int n_sm)
+{
+    const int tiles = (Mo / 256) * ((No + 255) / 256) * slices;
+    return (No > 256 || No % 256 == 0) && Mo % 256 == 0 && c_pitch % 256 == 0 && tiles >= n_sm / 3 && R / BLOCK_K / slices >= 8;
+}
+
+// Row slices of a transposed product (see tc_gemm_tn) on R rows: the count with the least modelled time.  A wave of
+// tiles takes 0.32 us per k-block (128 x 256 per SM: 5 ns a row, measured at 1024 x 1024 on 262144 rows) plus 4 us to
+// fill, empty and write; every slice writes and the sum over slices reads the output once more in bf16 (1 ps an element).
+int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm)
+{
+    const int kb = R / BLOCK_K, tiles_n = (No + 255) / 256;
+    int best = 1;
+    double best_cost = -1.0;
+    for (int S = 1; S <= max_slices && S <= kb; ++S) {
+        const bool pairs = tn_takes_pairs(Mo, No, R, S, c_pitch, n_sm);
+        const long long tiles = (long long)(pairs ? Mo / 256 : (Mo + 127) / 128) * tiles_n * S, slots = pairs ? n_sm / 2 : n_sm;
+        const double cost = (double)((tiles + slots - 1) / slots) * (0.32e-6 * (double)((kb + S - 1) / S) + 4e-6) + 1e-12 * (double)S * c_pitch * No;
+        if (best_cost < 0.0 || cost < best_cost * (1.0 - 1e-9)) { best = S; best_cost = cost; }
+    }
+    return best;
+}
+
 // C_s[Mo][No] = sum over the rows r of slice s of A[r][0..Mo) (x) B[r][0..No)  (bf16, fp32 accumulation):
-// the transposed product A^T B of two row-major matrices over `slices` equal row ranges, the partial
+// the transposed product A^T B of two row-major matrices over `slices` row ranges of whole 64-row blocks, the partial
 // results stacked with a pitch of `c_pitch` rows.  Operands are read M/N-major, so no transposed copy
 // of either matrix is needed.
 im_status tc_gemm_tn(const void *A, int64_t lda, const void *B, int64_t ldb, void *C, int64_t ldc, int R, int Mo, int No,
@@ -1462,7 +1507,7 @@ im_status tc_gemm_tn(const void *A, int64_t lda, const void *B, int64_t ldb, voi
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
     TcLayer L;
-    L.N = No; L.K = R / slices; L.Kpad = L.K;
+    L.N = No; L.K = R; L.Kpad = R;
     // wide outputs take 256-column tiles even when that leaves a ragged last tile (640 columns: three tiles,
     // a sixth of the MMAs wasted, against five 128-column tiles at little more than half the tensor-pipe rate);
     // TMA fills the operand columns past No with zeros and clips the stores
@@ -1475,15 +1520,12 @@ im_status tc_gemm_tn(const void *A, int64_t lda, const void *B, int64_t ldb, voi
         return IM_ERR_CUDA;
     GemmParams gp;
     std::memset(&gp, 0, sizeof(gp));
-    gp.M = Mo; gp.N = No; gp.K_blocks = (R / slices) / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = nullptr;    // no bias in this product
+    gp.M = Mo; gp.N = No; gp.kb_total = R / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = nullptr;    // no bias in this product
     gp.act_floor = -INFINITY;
-    gp.n_batches = slices; gp.a_batch_rows = R / slices; gp.b_batch_rows = 0; gp.c_batch_rows = c_pitch;
+    gp.n_batches = slices; gp.c_batch_rows = c_pitch;
     gp.status = status;
     cudaError_t e;
-    // CTA pairs (256 x 256 tiles, half of the N operand per SM) when the output splits into whole 256-row tiles,
-    // the slices' pitch keeps those tiles apart and there are tiles for most pairs
-    const int pair_tiles = ((Mo + 255) / 256) * L.n_tiles_n * slices;
-    if (L.block_n == 256 && Mo % 256 == 0 && c_pitch % 256 == 0 && pair_tiles >= n_sm / 3 && gp.K_blocks >= 8) {
+    if (tn_takes_pairs(Mo, No, R, slices, c_pitch, n_sm)) {
         L.map_m = L.map_c;
         return launch_hidden_pair<false, true>(L, gp, n_sm, stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
     }

@@ -23,6 +23,18 @@ template <typename T> bool dev_alloc(T **p, size_t n, cudaStream_t st, bool zero
     return !zero || cudaMemsetAsync(*p, 0, n * sizeof(T), st) == cudaSuccess;
 }
 
+// The most slices tc_tn_slices takes for a layer on up to max_rows rows.
+int max_slices(int Np, int Kp, int max_rows, int max_split)
+{
+    int most = 1;
+    for (int M = 64; M <= max_rows; M += 64) {
+        const int S = im::tc_tn_slices(Np, Kp, pad128(Np), M, max_split, im::device_sm_count());
+        most = S > most ? S : most;
+        if (most == max_split) break;
+    }
+    return most;
+}
+
 }  // namespace
 
 struct im_trainer {
@@ -54,8 +66,8 @@ struct im_ppo_updater {
 
 extern "C" {
 
-/* Row slices of the dW product of a layer with Np (padded) outputs and Kp (padded) inputs on M rows.  dW contracts
- * over the batch -- a long sum feeding few output tiles -- so the rows are cut into S slices that run as one launch.
+/* Equal row slices for the dW product of a layer with Np (padded) outputs and Kp (padded) inputs on M rows through
+ * im_gemm_bf16_tn (the trainer itself slices by whole 64-row blocks: tc_tn_slices).  dW contracts over the batch -- a long sum feeding few output tiles -- so the rows are cut into S slices that run as one launch.
  * S is the power of two (slices of whole 128-row blocks) with the least modelled time: waves of tiles on 148 SMs
  * times rows per slice (5 ns per row and wave, measured on a 1024 x 1024 layer), plus the pass that adds the S
  * partial products (1 ps per element).  any_rows: ignore the divisibility rule (an upper bound for sizing). */
@@ -116,8 +128,8 @@ im_status im_trainer_create(int32_t n_layers, const int32_t *dims, const float *
              dev_alloc(&tr->dW[l], wn, st) && dev_alloc(&tr->db[l], (size_t)N, st) && dev_alloc(&tr->Wb[l], (size_t)Np * Kp, st) &&
              dev_alloc(&tr->WbT[l], (size_t)Kp * Np, st) && dev_alloc(&tr->H[l], (size_t)max_rows * Kp, st) &&
              dev_alloc(&tr->dZ[l], (size_t)max_rows * Np, st);
-        // partial dW products: room for the most slices the model can choose (more rows never favour fewer slices)
-        const size_t s_max = (size_t)im_trainer_dw_slices(Np, Kp, max_rows, tr->max_split, 1);
+        // partial dW products: room for the most slices the model can choose for any number of rows
+        const size_t s_max = (size_t)max_slices(Np, Kp, max_rows, tr->max_split);
         const size_t n = s_max * pad128(Np) * Kp;
         need = n > need ? n : need;
     }
@@ -204,8 +216,8 @@ im_status im_trainer_backward(im_trainer *tr, const float *d_out, int32_t M)
         // dW = dZ^T H over S row slices in one launch (both operands read as they lie, M/N-major tensor-core
         // operands: no transposed copies); the S partial products are added afterwards
         const int Npb = pad128(Np);
-        const int S = im_trainer_dw_slices(Np, Kp, M, tr->max_split, 0);
-        s = im_gemm_bf16_tn(tr->dZ[l], Np, tr->H[l], Kp, tr->dWs, Kp, M, Np, Kp, S, Npb, tr->status, tr->stream);
+        const int S = im::tc_tn_slices(Np, Kp, Npb, M, tr->max_split, im::device_sm_count());
+        s = im::tc_gemm_tn(tr->dZ[l], Np, tr->H[l], Kp, tr->dWs, Kp, M, Np, Kp, S, Npb, tr->status, tr->stream);
         if (s == IM_OK) s = im_sum_slices_bf16_to_f32(tr->dWs, (int64_t)Npb * Kp, Kp, S, N, K, tr->dW[l], tr->stream);
         if (l > 0 && s == IM_OK) {
             // dH = (H > 0) * (dZ W); the product's epilogue applies the ReLU mask and leaves the column sums of every
