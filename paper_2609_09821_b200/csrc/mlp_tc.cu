@@ -1140,22 +1140,31 @@ bool make_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int pick_block_n(int N, bool last)
+// Columns of a tile: the whole action row for the last layer; else the narrowest of 64, 128, 256 whose tiles still fit
+// the SMs in one wave (a lone tile's time is its operand loads and its epilogue, both shorter when it is narrow:
+// 1024 x 1024 x 384 in a chain of launches 4.96 us with 64 columns, 5.68 with 128, 7.22 with 256; 2048 rows 6.96 / 5.79 /
+// 7.37), and the widest that divides N once there are several waves (8192 rows 17.1 / 12.1 / 10.4).
+int pick_block_n(int M, int N, bool last, int n_sm)
 {
-    if (last) return (N + 15) / 16 * 16;            // one tile holds the whole action row
-    if (N % 256 == 0) return 256;
-    if (N % 128 == 0) return 128;
-    return 64;
+    if (last) return (N + 15) / 16 * 16;
+    const int rows = (M + BLOCK_M - 1) / BLOCK_M;
+    int widest = 64;
+    for (int bn = 64; bn <= 256 && N % bn == 0; bn *= 2) {
+        if (rows * (N / bn) <= n_sm) return bn;
+        widest = bn;
+    }
+    return widest;
 }
 
 }  // namespace
 
 struct TcLayer {
-    int N, K, Kpad, block_n, n_tiles_n;
+    int N, K, Kpad, block_n, n_tiles_n;      // block_n: the widest tile the layer may take
     __nv_bfloat16 *d_W;      // [n_tiles_n * block_n][Kpad], zero padded
     float *d_bias;           // [n_tiles_n * block_n]
     CUtensorMap map_a, map_b, map_c;    // map_c: the hidden-activation buffer this layer stores to
-    CUtensorMap map_b2;                 // W in 128-row boxes: one CTA's half of a 256-column tile
+    CUtensorMap map_b2;                 // W in 128-row boxes: one CTA's half of a 256-column tile, or a 128-column tile
+    CUtensorMap map_b1;                 // W in 64-row boxes: a 64-column tile
     CUtensorMap map_m;                  // backward epilogue: the forward activations behind the ReLU mask (boxes like map_c)
 };
 
@@ -1329,7 +1338,7 @@ im_status tc_policy_create(im_policy *p, const void *const *W, const float *cons
         L.N = cfg.dims[l + 1];
         L.K = cfg.dims[l];
         L.Kpad = (L.K + BLOCK_K - 1) / BLOCK_K * BLOCK_K;
-        L.block_n = pick_block_n(L.N, last);
+        L.block_n = pick_block_n(cfg.max_batch, L.N, last, 0);          // (no SMs: the widest)
         L.n_tiles_n = (L.N + L.block_n - 1) / L.block_n;
         const size_t rows = (size_t)L.n_tiles_n * L.block_n;
         std::vector<uint16_t> hw(rows * L.Kpad, 0);
@@ -1349,7 +1358,8 @@ im_status tc_policy_create(im_policy *p, const void *const *W, const float *cons
         if (!make_map(&L.map_a, a_base, mb, (uint64_t)L.Kpad, (uint64_t)a_ld, BLOCK_M) ||
             !make_map(&L.map_b, L.d_W, rows, (uint64_t)L.Kpad, (uint64_t)L.Kpad, (uint32_t)L.block_n))
             return IM_ERR_CUDA;
-        if (!last && L.block_n == 256 && !make_map(&L.map_b2, L.d_W, rows, (uint64_t)L.Kpad, (uint64_t)L.Kpad, 128))
+        if (!last && (!make_map(&L.map_b1, L.d_W, rows, (uint64_t)L.Kpad, (uint64_t)L.Kpad, 64) ||
+                      !make_map(&L.map_b2, L.d_W, rows, (uint64_t)L.Kpad, (uint64_t)L.Kpad, L.block_n >= 128 ? 128 : 64)))
             return IM_ERR_CUDA;
         // hidden layers store 32-row x 64-column slabs of their output buffer
         if (!last && !make_map(&L.map_c, tc->d_hidden[l & 1], mb, rows, (uint64_t)tc->ld_hidden, 32))
@@ -1417,6 +1427,12 @@ im_status tc_policy_forward(im_policy *p, uint32_t step, int32_t n, const float 
         TcLayer L = tc->layers[l];
         if (l == 0 && external) L.map_a = tc->map_a_ext;
         const bool last = l == p->nl - 1;
+        const int bn = pick_block_n(n, L.N, last, tc->n_sm);
+        if (bn < L.block_n && cfg.impl != 2) {
+            L.map_b = bn == 128 ? L.map_b2 : L.map_b1;
+            L.block_n = bn;
+            L.n_tiles_n = L.N / bn;
+        }
         GemmParams gp;
         std::memset(&gp, 0, sizeof(gp));
         gp.M = n; gp.N = L.N; gp.K_blocks = L.Kpad / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = L.d_bias;
@@ -1448,7 +1464,7 @@ im_status tc_gemm(const void *A, int64_t lda, const void *B, int64_t ldb, void *
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
     TcLayer L;
     L.N = N; L.K = K; L.Kpad = K;
-    L.block_n = pick_block_n(N, false);
+    L.block_n = pick_block_n(M, N, false, n_sm);
     L.n_tiles_n = N / L.block_n;
     L.d_W = nullptr; L.d_bias = nullptr;
     const uint64_t nb = (uint64_t)batches;
@@ -1511,7 +1527,7 @@ im_status tc_gemm_tn(const void *A, int64_t lda, const void *B, int64_t ldb, voi
     // wide outputs take 256-column tiles even when that leaves a ragged last tile (640 columns: three tiles,
     // a sixth of the MMAs wasted, against five 128-column tiles at little more than half the tensor-pipe rate);
     // TMA fills the operand columns past No with zeros and clips the stores
-    L.block_n = No > 256 ? 256 : pick_block_n(No, false);
+    L.block_n = No > 256 ? 256 : pick_block_n(Mo, No, false, 0);
     L.n_tiles_n = (No + L.block_n - 1) / L.block_n;
     L.d_W = nullptr; L.d_bias = nullptr;
     if (!make_map(&L.map_a, A, (uint64_t)R, (uint64_t)Mo, (uint64_t)lda, 64) ||
@@ -1546,7 +1562,7 @@ im_status tc_gemm_head(const void *A, int64_t lda, const void *B, int64_t ldb, i
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
     TcLayer L;
     L.N = N; L.K = K; L.Kpad = K;
-    L.block_n = pick_block_n(N, true);
+    L.block_n = pick_block_n(M, N, true, n_sm);
     L.n_tiles_n = 1;
     L.d_W = nullptr; L.d_bias = nullptr;
     if (!make_map(&L.map_a, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BLOCK_M) ||
