@@ -931,9 +931,34 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
 // ------------------------------------------------------------------ Gaussian head (last layer)
 // mean = A W^T + b; action = mean + sigma z with z from Philox counter (env, step, 1, block)
 // and Box-Muller; logp = -0.5 sum z^2 - A ln sigma - (A/2) ln 2 pi.  The GEMM is tiny, the
-// noise is not: sixteen epilogue warps share the tile, four per group of 16 columns.
+// noise is not: sixteen epilogue warps share the tile, four per group of 16 columns, and draw a
+// tile's noise while its operands are on their way (the first tile's even before the previous
+// kernel has finished: it depends on nothing in memory).  A finished 32-row band leaves as one
+// bulk copy per output.  Against noise drawn after the accumulator and a warp copying the band: a rollout
+// step (policy and env) of 4096 envs x 28 actions 46.6 -> 45.2 us, of 16384 envs 74.2 -> 73.1 us.
 constexpr int kHeadEpiWarps = 16;
 constexpr int kHeadThreads = 64 + 32 * kHeadEpiWarps;
+
+// Standard normals of one row for the columns [c0, c0 + 16) and [c0 + 64, c0 + 80) below A.
+template <int CHUNKS>
+__device__ __forceinline__ float head_noise(const GemmParams &P, int row, int c0, int A, float (&z)[16 * CHUNKS])
+{
+    float zz = 0.0f;
+#pragma unroll
+    for (int g = 0; g < 4 * CHUNKS; ++g) {
+        const int col = c0 + (g >> 2) * 64 + 4 * (g & 3);
+        if (col < A) {
+            const uint4 x = philox4x32_10(make_uint4(P.env_id_base + (uint32_t)row, P.step, IM_STREAM_ACTION, (uint32_t)(col >> 2)),
+                                          make_uint2(P.seed_lo, P.seed_hi));
+            box_muller(x.x, x.y, z[4 * g], z[4 * g + 1]);
+            box_muller(x.z, x.w, z[4 * g + 2], z[4 * g + 3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (col + i < A) zz += z[4 * g + i] * z[4 * g + i];
+        }
+    }
+    return zz;
+}
 
 template <int BLOCK_N>
 __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const __grid_constant__ CUtensorMap map_a,
@@ -958,25 +983,33 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
     pipe_init<Plan>(p, kHeadEpiWarps);
     const uint32_t tmem_base = *p.tmem_slot;
     dep_release();
-    dep_wait();                       // nothing before this line touches global memory
-    // the epilogue reads bias and sigma from shared memory as 16-byte words instead of one global load per output
-    if (threadIdx.x < BLOCK_N) {
-        const int cidx = threadIdx.x;
-        s_bias[cidx] = __ldg(P.bias + cidx);
-        s_sigma[cidx] = cidx < A ? (P.log_std ? expf(__ldg(P.log_std + cidx)) : P.sigma) : 0.0f;
-    }
-    __syncthreads();
 
     if (warp == 0) {
+        dep_wait();                   // nothing before this line touches global memory
         if (lane == 0) producer_role<Plan, BLOCK_N>(p, &map_a, &map_b, P, n_tiles);
     } else if (warp == 1) {
+        dep_wait();
         if (lane == 0) mma_role<Plan, BLOCK_N>(p, tmem_base, P, n_tiles);
     } else {
         const int quad = warp & 3;                                  // 32-row band of the tile (TMEM lane quadrant)
         const int group = (warp - 2) >> 2;                          // 16-column groups group, group+4, ...
         const int row_in_tile = quad * 32 + lane;
         constexpr int kGroups = (BLOCK_N / 16) < 4 ? (BLOCK_N / 16) : 4;
+        constexpr int kChunks = (BLOCK_N + 63) / 64;
         const bool sample = P.action != nullptr;                     // a value head reads only the mean
+        float z[16 * kChunks], zz = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 16 * kChunks; ++i) z[i] = 0.0f;
+        if (sample && group < kGroups)
+            zz = head_noise<kChunks>(P, (int)blockIdx.x * BLOCK_M + row_in_tile, 16 * group, A, z);
+        dep_wait();
+        // the epilogue reads bias and sigma from shared memory as 16-byte words instead of one global load per output
+        if ((int)threadIdx.x - 64 < BLOCK_N) {
+            const int cidx = (int)threadIdx.x - 64;
+            s_bias[cidx] = __ldg(P.bias + cidx);
+            s_sigma[cidx] = cidx < A ? (P.log_std ? expf(__ldg(P.log_std + cidx)) : P.sigma) : 0.0f;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kHeadEpiWarps) : "memory");
         float logp_const = 0.0f;
         if (sample) {
             float sum_log = (float)A * logf(P.sigma);
@@ -996,36 +1029,26 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
             const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * Plan::kAccStride);
             float *s_mean = out_tiles + (size_t)acc * 2 * out_floats;
             float *s_act = s_mean + out_floats;
-            float zz = 0.0f;
             if (group < kGroups) {
-#pragma unroll 1
-                for (int c0 = 16 * group; c0 < BLOCK_N; c0 += 64) {
+#pragma unroll
+                for (int ch = 0; ch < kChunks; ++ch) {
+                    const int c0 = 16 * group + 64 * ch;
+                    if (c0 >= A) break;
                     float v[16];
                     tmem_ld16(t_row + (uint32_t)c0, v);
-                    if (c0 < A) {
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) {
-                            const int col = c0 + 4 * g;
-                            if (col >= A) break;
-                            float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-                            if (sample) {
-                                const uint4 x = philox4x32_10(make_uint4(P.env_id_base + (uint32_t)row, P.step,
-                                                                         IM_STREAM_ACTION, (uint32_t)(col >> 2)),
-                                                              make_uint2(P.seed_lo, P.seed_hi));
-                                box_muller(x.x, x.y, z[0], z[1]);
-                                box_muller(x.z, x.w, z[2], z[3]);
-                            }
-                            const float4 b4 = *reinterpret_cast<const float4 *>(s_bias + col);
-                            const float4 s4 = *reinterpret_cast<const float4 *>(s_sigma + col);
-                            const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, ss[4] = {s4.x, s4.y, s4.z, s4.w};
+                    for (int g = 0; g < 4; ++g) {
+                        const int col = c0 + 4 * g;
+                        if (col >= A) break;
+                        const float4 b4 = *reinterpret_cast<const float4 *>(s_bias + col);
+                        const float4 s4 = *reinterpret_cast<const float4 *>(s_sigma + col);
+                        const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, ss[4] = {s4.x, s4.y, s4.z, s4.w};
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                if (col + i < A) {
-                                    const float mu = v[4 * g + i] + bb[i];
-                                    s_mean[row_in_tile * A + col + i] = mu;
-                                    if (sample) s_act[row_in_tile * A + col + i] = mu + ss[i] * z[i];
-                                    zz += z[i] * z[i];
-                                }
+                        for (int i = 0; i < 4; ++i) {
+                            if (col + i < A) {
+                                const float mu = v[4 * g + i] + bb[i];
+                                s_mean[row_in_tile * A + col + i] = mu;
+                                if (sample) s_act[row_in_tile * A + col + i] = mu + ss[i] * z[16 * ch + 4 * g + i];
                             }
                         }
                     }
@@ -1034,10 +1057,11 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
             }
             tc_fence_before();
             // The last of the column-group warps to finish a 32-row band sums that band's partial z^2
-            // in group order (so the result does not depend on which warp that is) and copies the
-            // band's mean and action rows out as contiguous 16-byte stores.  The accumulator buffer,
-            // and with it this staging buffer, is released only afterwards.
+            // in group order (so the result does not depend on which warp that is) and sends the
+            // band's mean and action rows out.  The accumulator buffer, and with it this staging buffer,
+            // is released only when they have been read.
             if (group < kGroups) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the copy engine reads what was written above
                 __threadfence_block();
                 __syncwarp();
                 int prev = 0;
@@ -1050,33 +1074,41 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
                     int rows_valid = P.M - band_row0;
                     rows_valid = rows_valid > 32 ? 32 : rows_valid;
                     if (rows_valid > 0) {
+                        const int count = rows_valid * A;                       // floats, contiguous in global
+                        const float *src_m = s_mean + quad * 32 * A, *src_a = s_act + quad * 32 * A;
+                        float *dst_m = P.mean + (size_t)band_row0 * A;
+                        float *dst_a = sample ? P.action + (size_t)band_row0 * A : nullptr;
+                        // both sides start on a 16-byte boundary: band offsets are multiples of 32 rows
+                        const int bulk = count & ~3;
+                        if (lane == 0 && bulk > 0) {
+                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst_m), "r"(smem_u32(src_m)), "r"(4 * bulk) : "memory");
+                            if (sample)
+                                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst_a), "r"(smem_u32(src_a)), "r"(4 * bulk) : "memory");
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
+                        for (int i = bulk + lane; i < count; i += 32) {         // ragged last band: at most three floats
+                            dst_m[i] = src_m[i];
+                            if (sample) dst_a[i] = src_a[i];
+                        }
                         if (P.logp && lane < rows_valid) {
                             float sum = 0.0f;
 #pragma unroll
                             for (int g = 0; g < kGroups; ++g) sum += zz_part[(acc * 4 + g) * 128 + row_in_tile];
                             P.logp[row] = -0.5f * sum + logp_const;
                         }
-                        const int count = rows_valid * A;                       // floats, contiguous in global
-                        const float *src_m = s_mean + quad * 32 * A, *src_a = s_act + quad * 32 * A;
-                        float *dst_m = P.mean + (size_t)band_row0 * A;
-                        float *dst_a = sample ? P.action + (size_t)band_row0 * A : nullptr;
-                        // both sides start on a 16-byte boundary: band offsets are multiples of 32 rows
-                        const int n4 = count >> 2;
-                        for (int i = lane; i < n4; i += 32) {
-                            reinterpret_cast<float4 *>(dst_m)[i] = reinterpret_cast<const float4 *>(src_m)[i];
-                            if (sample) reinterpret_cast<float4 *>(dst_a)[i] = reinterpret_cast<const float4 *>(src_a)[i];
-                        }
-                        for (int i = 4 * n4 + lane; i < count; i += 32) {
-                            dst_m[i] = src_m[i];
-                            if (sample) dst_a[i] = src_a[i];
-                        }
                     }
                 }
+                // the next tile's noise, while this band leaves and the tile's operands arrive
+                if (sample && tile + (int)gridDim.x < n_tiles)
+                    zz = head_noise<kChunks>(P, (tile + (int)gridDim.x) * BLOCK_M + row_in_tile, 16 * group, A, z);
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&p.acc_empty[acc]);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     pipe_exit<Plan>(p, tmem_base, P.status);
 }
@@ -1087,6 +1119,8 @@ __global__ void obs_to_bf16_kernel(const float *__restrict__ obs, int ld_obs, in
 {
     const int chunks = ld_out / 8;
     const long long total = (long long)n * chunks;
+    dep_release();
+    dep_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const int r = (int)(i / chunks), c = (int)(i % chunks) * 8;
         float v[8];
@@ -1419,7 +1453,7 @@ im_status tc_policy_forward(im_policy *p, uint32_t step, int32_t n, const float 
         const int block = 256;
         long long grid = (chunks + block - 1) / block;
         if (grid > 148 * 16) grid = 148 * 16;
-        obs_to_bf16_kernel<<<(int)grid, block, 0, p->stream>>>(obs, ld_obs, cfg.dims[0], tc->d_in, tc->ld_in, n);
+        launch_pdl(obs_to_bf16_kernel, dim3((unsigned)grid), dim3(block), 0, p->stream, 0, obs, ld_obs, cfg.dims[0], tc->d_in, tc->ld_in, n);
         g_launches.fetch_add(1, std::memory_order_relaxed);
         if (cudaGetLastError() != cudaSuccess) return IM_ERR_CUDA;
     }
