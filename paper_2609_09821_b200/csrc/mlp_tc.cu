@@ -982,7 +982,6 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
     if (threadIdx.x < 8) band_count[threadIdx.x] = 0;
     pipe_init<Plan>(p, kHeadEpiWarps);
     const uint32_t tmem_base = *p.tmem_slot;
-    dep_release();
 
     if (warp == 0) {
         dep_wait();                   // nothing before this line touches global memory
@@ -1111,6 +1110,9 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     pipe_exit<Plan>(p, tmem_base, P.status);
+    // Released late: the env step usually comes next, several CTAs to an SM, and an earlier start would pack them onto
+    // the SMs that this grid leaves idle
+    dep_release();
 }
 
 // fp32 observations -> bf16 rows of a padded buffer; columns beyond `cols` are written as zero.
@@ -1119,8 +1121,6 @@ __global__ void obs_to_bf16_kernel(const float *__restrict__ obs, int ld_obs, in
 {
     const int chunks = ld_out / 8;
     const long long total = (long long)n * chunks;
-    dep_release();
-    dep_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const int r = (int)(i / chunks), c = (int)(i % chunks) * 8;
         float v[8];
@@ -1453,7 +1453,7 @@ im_status tc_policy_forward(im_policy *p, uint32_t step, int32_t n, const float 
         const int block = 256;
         long long grid = (chunks + block - 1) / block;
         if (grid > 148 * 16) grid = 148 * 16;
-        launch_pdl(obs_to_bf16_kernel, dim3((unsigned)grid), dim3(block), 0, p->stream, 0, obs, ld_obs, cfg.dims[0], tc->d_in, tc->ld_in, n);
+        obs_to_bf16_kernel<<<(int)grid, block, 0, p->stream>>>(obs, ld_obs, cfg.dims[0], tc->d_in, tc->ld_in, n);
         g_launches.fetch_add(1, std::memory_order_relaxed);
         if (cudaGetLastError() != cudaSuccess) return IM_ERR_CUDA;
     }
