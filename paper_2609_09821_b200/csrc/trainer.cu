@@ -10,6 +10,7 @@
 
 #include "im_internal.h"
 #include "mlp.h"
+#include "update.h"
 
 namespace {
 
@@ -35,6 +36,11 @@ int max_slices(int Np, int Kp, int max_rows, int max_split)
     return most;
 }
 
+bool adam_ok(const im_adam_config *c)
+{
+    return c->beta1 >= 0.0f && c->beta1 < 1.0f && c->beta2 >= 0.0f && c->beta2 < 1.0f && c->eps > 0.0f;
+}
+
 }  // namespace
 
 struct im_trainer {
@@ -47,12 +53,71 @@ struct im_trainer {
     uint16_t *H[IM_MAX_LAYERS];                            // H[0]: input rows [Mb][Kp0]; H[l]: activations [Mb][Np[l-1]]
     uint16_t *dZ[IM_MAX_LAYERS];                           // gradient at layer l's pre-activation [Mb][Np[l]]
     float *out;                                            // [Mb][dims[nl]]
-    uint16_t *dWs;                                         // partial dW products of one layer, all row slices
-    float *colsum_ws, *col_partial;
-    size_t colsum_ws_bytes;
-    int ld_partial;
+    uint16_t *dWs[IM_MAX_LAYERS];                          // partial dW products, all row slices
+    float *db_partial[IM_MAX_LAYERS];                      // partial column sums of dZ: per 32 rows, last layer per 128 rows; [.][Np]
     uint32_t *status;
 };
+
+namespace {
+
+// The net on M input rows x (its own, or those of another trainer of the same input width).
+im_status forward_on(im_trainer *tr, uint16_t *x, int M)
+{
+    const int L = tr->nl - 1;
+    for (int l = 0; l < L; ++l) {
+        const im_status s = im_gemm_bf16(l == 0 ? x : tr->H[l], tr->Kp[l], tr->Wb[l], tr->Kp[l], tr->H[l + 1], tr->Np[l], M, tr->Np[l],
+                                         tr->Kp[l], tr->b[l], 1, tr->status, tr->stream);
+        if (s != IM_OK) return s;
+    }
+    return im_gemm_bf16_f32out(tr->H[L], tr->Kp[L], tr->Wb[L], tr->Kp[L], tr->out, M, tr->dims[tr->nl], tr->Kp[L], tr->b[L],
+                               tr->status, tr->stream);
+}
+
+im::OutGrad out_grad(im_trainer *tr, const float *d_out)
+{
+    const int L = tr->nl - 1;
+    return {d_out, tr->dZ[L], tr->db_partial[L], tr->dims[tr->nl], tr->Np[L]};
+}
+
+// The tensor-core products of the backward pass.  dW = dZ^T H over slices[l] row slices in one launch (both operands
+// read as they lie, M/N-major tensor-core operands: no transposed copies).  dH = (H > 0) * (dZ W); the product's
+// epilogue applies the ReLU mask and leaves the column sums of every 32-row block, which add up to the bias gradient of
+// the layer below.
+im_status backward_products(im_trainer *tr, uint16_t *x, int M, int *slices)
+{
+    im_status s = IM_OK;
+    for (int l = tr->nl - 1; l >= 0 && s == IM_OK; --l) {
+        const int Np = tr->Np[l], Kp = tr->Kp[l], Npb = pad128(Np);
+        slices[l] = im::tc_tn_slices(Np, Kp, Npb, M, tr->max_split, im::device_sm_count());
+        s = im::tc_gemm_tn(tr->dZ[l], Np, l == 0 ? x : tr->H[l], Kp, tr->dWs[l], Kp, M, Np, Kp, slices[l], Npb, tr->status, tr->stream);
+        if (l > 0 && s == IM_OK)
+            s = im_gemm_bf16_dgrad(tr->dZ[l], Np, tr->WbT[l], Np, tr->dZ[l - 1], Kp, M, Kp, Np, tr->H[l], Kp, tr->db_partial[l - 1], Kp,
+                                   tr->status, tr->stream);
+    }
+    return s;
+}
+
+void add_weight_grads(im::GradReduceArgs &ga, im_trainer *tr, const int *slices)
+{
+    for (int l = 0; l < tr->nl; ++l)
+        im::grad_reduce_add(ga, tr->dWs[l], (long long)pad128(tr->Np[l]) * tr->Kp[l], tr->Kp[l], slices[l], tr->dims[l + 1], tr->dims[l], tr->dW[l]);
+}
+void add_bias_grads(im::GradReduceArgs &ga, im_trainer *tr, int M)
+{
+    for (int l = 0; l < tr->nl; ++l)
+        im::grad_reduce_add(ga, tr->db_partial[l], l == tr->nl - 1 ? (M + 127) / 128 : M / 32, tr->Np[l], tr->dims[l + 1], tr->db[l]);
+}
+
+void add_adam(im::AdamMultiArgs &aa, im_trainer *tr)
+{
+    for (int l = 0; l < tr->nl; ++l) {
+        const int N = tr->dims[l + 1], K = tr->dims[l];
+        im::adam_multi_add(aa, tr->W[l], tr->dW[l], tr->mW[l], tr->vW[l], N, K, tr->Wb[l], tr->Kp[l], tr->WbT[l], tr->Np[l], tr->t);
+        im::adam_multi_add(aa, tr->b[l], tr->db[l], tr->mb[l], tr->vb[l], 1, N, nullptr, 0, nullptr, 0, tr->t);
+    }
+}
+
+}  // namespace
 
 struct im_ppo_updater {
     im_trainer *actor, *critic;
@@ -60,9 +125,60 @@ struct im_ppo_updater {
     int A, Mb, t;
     float *log_std, *log_std_old, *m_ls, *v_ls, *d_log_std, *lr, *scale, *moments, *summary, *d_mean, *d_value;
     void *ws;
+    double *norm_partial;          // one sum of squares per block of the gradient reduction
+    int *done;                     // [2] block counters: gradient norm, Adam
     float *g_action, *g_mean_old, *g_logp_old, *g_advantage, *g_value_old, *g_returns;   // gathered minibatch (shuffled updates)
     int g_rows;
 };
+
+// One minibatch update; the critic's input rows are critic_x (its own, or the actor's).
+static im_status update_on(im_ppo_updater *u, int M, const im_ppo_minibatch *mb, uint16_t *critic_x)
+{
+    if (!mb || M < 64 || (M & 63) || M > u->Mb) return IM_ERR_INVALID_ARG;
+    if (!mb->action || !mb->mean_old || !mb->logp_old || !mb->advantage || !mb->returns) return IM_ERR_INVALID_ARG;
+    if (u->cfg.clip_value_loss && !mb->value_old) return IM_ERR_INVALID_ARG;
+    if (!adam_ok(&u->cfg.adam) || !(u->cfg.kl_target > 0.0f) || !(u->cfg.lr_min > 0.0f)) return IM_ERR_INVALID_ARG;
+    im_trainer *a = u->actor, *c = u->critic;
+    cudaStream_t st = a->stream;
+    im_status s = forward_on(a, a->H[0], M);
+    if (s == IM_OK) s = forward_on(c, critic_x, M);
+    if (s != IM_OK) return s;
+    const float *mom = nullptr;
+    if (u->cfg.normalize_advantage) {
+        s = im_moments(mb->advantage, M, u->moments, u->ws, st);
+        if (s != IM_OK) return s;
+        mom = u->moments;
+    }
+    const im_ppo_config pc = {u->cfg.clip, u->cfg.value_coef, u->cfg.entropy_coef, u->cfg.clip_value_loss};
+    const im_ppo_batch pb = {a->out, u->log_std, mb->action, mb->logp_old, mb->mean_old,
+                             mb->log_std_old ? mb->log_std_old : u->log_std_old, mb->advantage, mom, c->out, mb->value_old, mb->returns};
+    s = im_ppo_loss(&pc, M, u->A, &pb, u->d_mean, u->d_log_std, u->d_value, u->summary, u->ws, st);
+    if (s != IM_OK) return s;
+    im::OutGradArgs og = {};
+    og.n_nets = 2; og.M = M; og.net[0] = out_grad(a, u->d_mean); og.net[1] = out_grad(c, u->d_value);
+    if (im::launch_out_grads(og, st) != cudaSuccess) return IM_ERR_CUDA;
+    int slices_a[IM_MAX_LAYERS], slices_c[IM_MAX_LAYERS];
+    s = backward_products(a, a->H[0], M, slices_a);
+    if (s == IM_OK) s = backward_products(c, critic_x, M, slices_c);
+    if (s != IM_OK) return s;
+    // every gradient tensor of both nets, and the global-norm clip factor over them and the log-std's
+    im::GradReduceArgs ga = {};
+    add_weight_grads(ga, a, slices_a);
+    add_weight_grads(ga, c, slices_c);
+    add_bias_grads(ga, a, M);
+    add_bias_grads(ga, c, M);
+    ga.extra = u->d_log_std; ga.n_extra = u->A;
+    ga.partial = u->norm_partial; ga.done = u->done; ga.max_norm = u->cfg.max_grad_norm; ga.scale_out = u->scale;
+    if (im::launch_grad_reduce(ga, st) != cudaSuccess) return IM_ERR_CUDA;
+    im::AdamMultiArgs aa = {};
+    aa.cfg = u->cfg.adam; aa.lr = u->lr; aa.grad_scale = u->scale;
+    aa.kl = u->summary + 4; aa.kl_target = u->cfg.kl_target; aa.lr_min = u->cfg.lr_min; aa.lr_max = u->cfg.lr_max; aa.done = u->done + 1;
+    a->t += 1; c->t += 1; u->t += 1;
+    add_adam(aa, a);
+    add_adam(aa, c);
+    im::adam_multi_add(aa, u->log_std, u->d_log_std, u->m_ls, u->v_ls, 1, u->A, nullptr, 0, nullptr, 0, u->t);
+    return im::launch_adam_multi(aa, st) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+}
 
 extern "C" {
 
@@ -91,8 +207,9 @@ void im_trainer_destroy(im_trainer *tr)
     for (int l = 0; l < IM_MAX_LAYERS; ++l) {
         cudaFree(tr->W[l]); cudaFree(tr->b[l]); cudaFree(tr->mW[l]); cudaFree(tr->vW[l]); cudaFree(tr->mb[l]); cudaFree(tr->vb[l]);
         cudaFree(tr->dW[l]); cudaFree(tr->db[l]); cudaFree(tr->Wb[l]); cudaFree(tr->WbT[l]); cudaFree(tr->H[l]); cudaFree(tr->dZ[l]);
+        cudaFree(tr->dWs[l]); cudaFree(tr->db_partial[l]);
     }
-    cudaFree(tr->out); cudaFree(tr->dWs); cudaFree(tr->colsum_ws); cudaFree(tr->col_partial); cudaFree(tr->status);
+    cudaFree(tr->out); cudaFree(tr->status);
     delete tr;
 }
 
@@ -115,13 +232,10 @@ im_status im_trainer_create(int32_t n_layers, const int32_t *dims, const float *
     tr->nl = n_layers; tr->Mb = max_rows; tr->max_split = 64; tr->stream = (cudaStream_t)cuda_stream;
     cudaStream_t st = tr->stream;
     for (int l = 0; l <= n_layers; ++l) tr->dims[l] = dims[l];
-    int maxNp = 0;
-    size_t need = 0;
     bool ok = true;
     for (int l = 0; l < n_layers && ok; ++l) {
         const int N = dims[l + 1], K = dims[l], Np = pad64(N), Kp = pad64(K);
         tr->Np[l] = Np; tr->Kp[l] = Kp;
-        maxNp = Np > maxNp ? Np : maxNp;
         const size_t wn = (size_t)N * K;
         ok = dev_alloc(&tr->W[l], wn, st, false) && dev_alloc(&tr->b[l], (size_t)Np, st) && dev_alloc(&tr->mW[l], wn, st) &&
              dev_alloc(&tr->vW[l], wn, st) && dev_alloc(&tr->mb[l], (size_t)N, st) && dev_alloc(&tr->vb[l], (size_t)N, st) &&
@@ -130,15 +244,10 @@ im_status im_trainer_create(int32_t n_layers, const int32_t *dims, const float *
              dev_alloc(&tr->dZ[l], (size_t)max_rows * Np, st);
         // partial dW products: room for the most slices the model can choose for any number of rows
         const size_t s_max = (size_t)max_slices(Np, Kp, max_rows, tr->max_split);
-        const size_t n = s_max * pad128(Np) * Kp;
-        need = n > need ? n : need;
+        ok = ok && dev_alloc(&tr->dWs[l], s_max * pad128(Np) * Kp, st, false) &&
+             dev_alloc(&tr->db_partial[l], (size_t)(l == n_layers - 1 ? (max_rows + 127) / 128 : max_rows / 32) * Np, st, false);
     }
-    const size_t slices256 = ((size_t)max_rows + 255) / 256;
-    tr->colsum_ws_bytes = slices256 * (size_t)(maxNp > 80 ? maxNp : 80) * sizeof(float);
-    tr->ld_partial = maxNp;
-    ok = ok && dev_alloc(&tr->out, (size_t)max_rows * dims[n_layers], st) && dev_alloc(&tr->dWs, need, st) &&
-         dev_alloc(&tr->colsum_ws, tr->colsum_ws_bytes / sizeof(float), st, false) &&
-         dev_alloc(&tr->col_partial, (size_t)(max_rows / 32) * maxNp, st, false) && dev_alloc(&tr->status, 1, st);
+    ok = ok && dev_alloc(&tr->out, (size_t)max_rows * dims[n_layers], st) && dev_alloc(&tr->status, 1, st);
     if (!ok) { im_trainer_destroy(tr); return IM_ERR_ALLOC; }
     // weights: fp32 masters as given; bf16 working copies (rounded on the device, zero padded) and their transposes
     for (int l = 0; l < n_layers; ++l) {
@@ -195,56 +304,32 @@ im_status im_trainer_set_step_count(im_trainer *tr, int32_t t)
 im_status im_trainer_forward(im_trainer *tr, int32_t M)
 {
     if (!tr || M < 1 || M > tr->Mb) return IM_ERR_INVALID_ARG;
-    const int L = tr->nl - 1;
-    for (int l = 0; l < L; ++l) {
-        const im_status s = im_gemm_bf16(tr->H[l], tr->Kp[l], tr->Wb[l], tr->Kp[l], tr->H[l + 1], tr->Np[l], M, tr->Np[l],
-                                         tr->Kp[l], tr->b[l], 1, tr->status, tr->stream);
-        if (s != IM_OK) return s;
-    }
-    return im_gemm_bf16_f32out(tr->H[L], tr->Kp[L], tr->Wb[L], tr->Kp[L], tr->out, M, tr->dims[tr->nl], tr->Kp[L], tr->b[L],
-                               tr->status, tr->stream);
+    return forward_on(tr, tr->H[0], M);
 }
 
 im_status im_trainer_backward(im_trainer *tr, const float *d_out, int32_t M)
 {
     if (!tr || !d_out || M < 64 || (M & 63) || M > tr->Mb) return IM_ERR_INVALID_ARG;
-    const int L = tr->nl - 1, A = tr->dims[tr->nl];
-    im_status s = im_f32_to_bf16_padded(d_out, A, M, A, tr->dZ[L], tr->Np[L], tr->stream);
-    if (s == IM_OK) s = im_colsum_f32(d_out, A, M, A, tr->db[L], tr->colsum_ws, tr->colsum_ws_bytes, tr->stream);
-    for (int l = L; l >= 0 && s == IM_OK; --l) {
-        const int N = tr->dims[l + 1], K = tr->dims[l], Np = tr->Np[l], Kp = tr->Kp[l];
-        // dW = dZ^T H over S row slices in one launch (both operands read as they lie, M/N-major tensor-core
-        // operands: no transposed copies); the S partial products are added afterwards
-        const int Npb = pad128(Np);
-        const int S = im::tc_tn_slices(Np, Kp, Npb, M, tr->max_split, im::device_sm_count());
-        s = im::tc_gemm_tn(tr->dZ[l], Np, tr->H[l], Kp, tr->dWs, Kp, M, Np, Kp, S, Npb, tr->status, tr->stream);
-        if (s == IM_OK) s = im_sum_slices_bf16_to_f32(tr->dWs, (int64_t)Npb * Kp, Kp, S, N, K, tr->dW[l], tr->stream);
-        if (l > 0 && s == IM_OK) {
-            // dH = (H > 0) * (dZ W); the product's epilogue applies the ReLU mask and leaves the column sums of every
-            // 32-row block, which add up to the bias gradient of the layer below
-            s = im_gemm_bf16_dgrad(tr->dZ[l], Np, tr->WbT[l], Np, tr->dZ[l - 1], Kp, M, Kp, Np, tr->H[l], Kp, tr->col_partial,
-                                   tr->ld_partial, tr->status, tr->stream);
-            if (s == IM_OK)
-                s = im_colsum_f32(tr->col_partial, tr->ld_partial, M / 32, K, tr->db[l - 1], tr->colsum_ws, tr->colsum_ws_bytes,
-                                  tr->stream);
-        }
-    }
-    return s;
+    im::OutGradArgs og = {};
+    og.n_nets = 1; og.M = M; og.net[0] = out_grad(tr, d_out);
+    if (im::launch_out_grads(og, tr->stream) != cudaSuccess) return IM_ERR_CUDA;
+    int slices[IM_MAX_LAYERS];
+    const im_status s = backward_products(tr, tr->H[0], M, slices);
+    if (s != IM_OK) return s;
+    im::GradReduceArgs ga = {};
+    add_weight_grads(ga, tr, slices);
+    add_bias_grads(ga, tr, M);
+    return im::launch_grad_reduce(ga, tr->stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
 
 im_status im_trainer_step(im_trainer *tr, const im_adam_config *adam, const float *lr, const float *grad_scale)
 {
-    if (!tr || !adam || !lr) return IM_ERR_INVALID_ARG;
+    if (!tr || !adam || !lr || !adam_ok(adam)) return IM_ERR_INVALID_ARG;
+    im::AdamMultiArgs aa = {};
+    aa.cfg = *adam; aa.lr = const_cast<float *>(lr); aa.grad_scale = grad_scale;      // (lr is only written with kl)
     tr->t += 1;
-    for (int l = 0; l < tr->nl; ++l) {
-        const int N = tr->dims[l + 1], K = tr->dims[l];
-        im_status s = im_adam_step(adam, tr->t, (int64_t)N * K, tr->W[l], tr->dW[l], tr->mW[l], tr->vW[l], lr, grad_scale,
-                                   tr->Wb[l], K, tr->Kp[l], tr->stream);
-        if (s == IM_OK) s = im_adam_step(adam, tr->t, N, tr->b[l], tr->db[l], tr->mb[l], tr->vb[l], lr, grad_scale, nullptr, 0, 0, tr->stream);
-        if (s == IM_OK) s = im_transpose_bf16(tr->Wb[l], tr->Kp[l], tr->Np[l], tr->Kp[l], tr->WbT[l], tr->Np[l], tr->stream);
-        if (s != IM_OK) return s;
-    }
-    return IM_OK;
+    add_adam(aa, tr);
+    return im::launch_adam_multi(aa, tr->stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
 
 im_status im_trainer_push_to_policy(im_trainer *tr, im_policy *p)
@@ -277,8 +362,8 @@ void im_ppo_updater_destroy(im_ppo_updater *u)
     if (!u) return;
     cudaFree(u->log_std); cudaFree(u->log_std_old); cudaFree(u->m_ls); cudaFree(u->v_ls); cudaFree(u->d_log_std); cudaFree(u->lr);
     cudaFree(u->scale); cudaFree(u->moments); cudaFree(u->summary); cudaFree(u->d_mean); cudaFree(u->d_value); cudaFree(u->ws);
-    cudaFree(u->g_action); cudaFree(u->g_mean_old); cudaFree(u->g_logp_old); cudaFree(u->g_advantage); cudaFree(u->g_value_old);
-    cudaFree(u->g_returns);
+    cudaFree(u->norm_partial); cudaFree(u->done);
+    cudaFree(u->g_action);
     delete u;
 }
 
@@ -294,7 +379,10 @@ im_status im_ppo_updater_create(im_trainer *actor, im_trainer *critic, const flo
     u->actor = actor; u->critic = critic; u->cfg = *cfg; u->A = actor->dims[actor->nl]; u->Mb = actor->Mb;
     const size_t A = (size_t)u->A;
     cudaStream_t st = actor->stream;
-    bool ok = dev_alloc(&u->log_std, A, st) && dev_alloc(&u->log_std_old, A, st) && dev_alloc(&u->m_ls, A, st) && dev_alloc(&u->v_ls, A, st) &&
+    size_t n_blocks = 1;
+    for (im_trainer *t : {actor, critic})
+        for (int l = 0; l < t->nl; ++l) n_blocks += im::grad_matrix_blocks(t->dims[l + 1], t->dims[l]) + im::grad_vector_blocks(t->dims[l + 1]);
+    bool ok = dev_alloc(&u->norm_partial, n_blocks, st, false) && dev_alloc(&u->done, 2, st) && dev_alloc(&u->log_std, A, st) && dev_alloc(&u->log_std_old, A, st) && dev_alloc(&u->m_ls, A, st) && dev_alloc(&u->v_ls, A, st) &&
               dev_alloc(&u->d_log_std, A, st) && dev_alloc(&u->lr, 1, st) && dev_alloc(&u->scale, 2, st) && dev_alloc(&u->moments, 2, st) &&
               dev_alloc(&u->summary, 6, st) && dev_alloc(&u->d_mean, (size_t)u->Mb * A, st) && dev_alloc(&u->d_value, (size_t)u->Mb, st) &&
               cudaMalloc(&u->ws, im_ppo_workspace_bytes()) == cudaSuccess;
@@ -334,43 +422,8 @@ im_status im_ppo_updater_set_step_count(im_ppo_updater *u, int32_t t)
 
 im_status im_ppo_update(im_ppo_updater *u, int32_t M, const im_ppo_minibatch *mb)
 {
-    if (!u || !mb || M < 64 || (M & 63) || M > u->Mb) return IM_ERR_INVALID_ARG;
-    if (!mb->action || !mb->mean_old || !mb->logp_old || !mb->advantage || !mb->returns) return IM_ERR_INVALID_ARG;
-    if (u->cfg.clip_value_loss && !mb->value_old) return IM_ERR_INVALID_ARG;
-    im_trainer *a = u->actor, *c = u->critic;
-    cudaStream_t st = a->stream;
-    im_status s = im_trainer_forward(a, M);
-    if (s == IM_OK) s = im_trainer_forward(c, M);
-    if (s != IM_OK) return s;
-    const float *mom = nullptr;
-    if (u->cfg.normalize_advantage) {
-        s = im_moments(mb->advantage, M, u->moments, u->ws, st);
-        if (s != IM_OK) return s;
-        mom = u->moments;
-    }
-    const im_ppo_config pc = {u->cfg.clip, u->cfg.value_coef, u->cfg.entropy_coef, u->cfg.clip_value_loss};
-    const im_ppo_batch pb = {a->out, u->log_std, mb->action, mb->logp_old, mb->mean_old,
-                             mb->log_std_old ? mb->log_std_old : u->log_std_old, mb->advantage, mom, c->out, mb->value_old, mb->returns};
-    s = im_ppo_loss(&pc, M, u->A, &pb, u->d_mean, u->d_log_std, u->d_value, u->summary, u->ws, st);
-    if (s == IM_OK) s = im_trainer_backward(a, u->d_mean, M);
-    if (s == IM_OK) s = im_trainer_backward(c, u->d_value, M);
-    if (s != IM_OK) return s;
-    // global-norm clip over every gradient tensor of both nets and the log-std
-    const float *grads[4 * IM_MAX_LAYERS + 1];
-    int64_t sizes[4 * IM_MAX_LAYERS + 1];
-    int n = 0;
-    for (im_trainer *t : {a, c}) {
-        for (int l = 0; l < t->nl; ++l) { grads[n] = t->dW[l]; sizes[n++] = (int64_t)t->dims[l + 1] * t->dims[l]; }
-        for (int l = 0; l < t->nl; ++l) { grads[n] = t->db[l]; sizes[n++] = t->dims[l + 1]; }
-    }
-    grads[n] = u->d_log_std; sizes[n++] = u->A;
-    s = im_grad_scale(n, grads, sizes, u->cfg.max_grad_norm, u->scale, u->ws, st);
-    if (s == IM_OK) s = im_trainer_step(a, &u->cfg.adam, u->lr, u->scale);
-    if (s == IM_OK) s = im_trainer_step(c, &u->cfg.adam, u->lr, u->scale);
-    u->t += 1;
-    if (s == IM_OK) s = im_adam_step(&u->cfg.adam, u->t, u->A, u->log_std, u->d_log_std, u->m_ls, u->v_ls, u->lr, u->scale, nullptr, 0, 0, st);
-    if (s == IM_OK) s = im_adaptive_lr(u->lr, u->summary + 4, u->cfg.kl_target, u->cfg.lr_min, u->cfg.lr_max, st);
-    return s;
+    if (!u) return IM_ERR_INVALID_ARG;
+    return update_on(u, M, mb, u->critic->H[0]);
 }
 
 im_status im_ppo_update_rollout(im_ppo_updater *u, const im_rollout_view *v, int32_t epochs, int32_t n_minibatches,
@@ -387,13 +440,12 @@ im_status im_ppo_update_rollout(im_ppo_updater *u, const im_rollout_view *v, int
     cudaStream_t st = u->actor->stream;
     if (perm && u->g_rows < M) {
         // (first shuffled update of this size: buffers for the gathered minibatch)
-        cudaFree(u->g_action); cudaFree(u->g_mean_old); cudaFree(u->g_logp_old); cudaFree(u->g_advantage); cudaFree(u->g_value_old);
-        cudaFree(u->g_returns);
+        cudaFree(u->g_action);
         u->g_rows = 0;
-        if (!dev_alloc(&u->g_action, (size_t)M * A, st, false) || !dev_alloc(&u->g_mean_old, (size_t)M * A, st, false) ||
-            !dev_alloc(&u->g_logp_old, (size_t)M, st, false) || !dev_alloc(&u->g_advantage, (size_t)M, st, false) ||
-            !dev_alloc(&u->g_value_old, (size_t)M, st, false) || !dev_alloc(&u->g_returns, (size_t)M, st, false))
-            return IM_ERR_ALLOC;
+        if (!dev_alloc(&u->g_action, (size_t)M * (2 * A + 4), st, false)) return IM_ERR_ALLOC;
+        u->g_mean_old = u->g_action + (size_t)M * A;                  // (M is a multiple of 64: every part is 16-byte aligned)
+        u->g_logp_old = u->g_mean_old + (size_t)M * A;
+        u->g_advantage = u->g_logp_old + M; u->g_value_old = u->g_advantage + M; u->g_returns = u->g_value_old + M;
         u->g_rows = M;
     }
     for (int ep = 0; ep < epochs; ++ep) {
@@ -401,23 +453,20 @@ im_status im_ppo_update_rollout(im_ppo_updater *u, const im_rollout_view *v, int
             const int64_t r0 = (int64_t)k * M;
             im_ppo_minibatch mb;
             im_status s = IM_OK;
+            // (one copy of the observations as bf16 rows, in the actor's input buffer, serves both nets)
+            im_trainer *t = u->actor;
             if (!perm) {
-                // contiguous block: the observations are converted into both nets' input rows, the rest is read in place
-                for (im_trainer *t : {u->actor, u->critic})
-                    if (s == IM_OK) s = im_f32_to_bf16_padded(v->obs + r0 * v->ld_obs, v->ld_obs, M, D, t->H[0], t->Kp[0], st);
+                // contiguous block: the observations are converted, the rest is read in place
+                s = im_f32_to_bf16_padded(v->obs + r0 * v->ld_obs, v->ld_obs, M, D, t->H[0], t->Kp[0], st);
                 mb = {v->action + r0 * A, v->mean + r0 * A, nullptr, v->logp + r0, v->advantage + r0, v->value + r0, v->returns + r0};
             } else {
-                const int32_t *idx = perm + (int64_t)ep * total + r0;
-                for (im_trainer *t : {u->actor, u->critic})
-                    if (s == IM_OK) s = im_gather_rows_f32(v->obs, v->ld_obs, idx, total, M, D, t->H[0], t->Kp[0], 1, u->actor->status, st);
-                const struct { const float *src; int cols; float *dst; } g[6] = {
-                    {v->action, A, u->g_action}, {v->mean, A, u->g_mean_old}, {v->logp, 1, u->g_logp_old},
-                    {v->advantage, 1, u->g_advantage}, {v->value, 1, u->g_value_old}, {v->returns, 1, u->g_returns}};
-                for (const auto &x : g)
-                    if (s == IM_OK) s = im_gather_rows_f32(x.src, x.cols, idx, total, M, x.cols, x.dst, x.cols, 0, u->actor->status, st);
+                const im::GatherArgs ga = {v->obs, v->action, v->mean, v->logp, v->advantage, v->value, v->returns, perm + (int64_t)ep * total + r0,
+                                           v->ld_obs, total, M, D, A, t->Kp[0], t->H[0], u->g_action, u->g_mean_old, u->g_logp_old,
+                                           u->g_advantage, u->g_value_old, u->g_returns, t->status};
+                if (im::launch_gather_minibatch(ga, st) != cudaSuccess) s = IM_ERR_CUDA;
                 mb = {u->g_action, u->g_mean_old, nullptr, u->g_logp_old, u->g_advantage, u->g_value_old, u->g_returns};
             }
-            if (s == IM_OK) s = im_ppo_update(u, M, &mb);
+            if (s == IM_OK) s = update_on(u, M, &mb, t->H[0]);
             if (s != IM_OK) return s;
         }
     }

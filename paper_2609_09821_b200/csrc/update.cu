@@ -1,0 +1,353 @@
+// Multi-tensor kernels of the update phase (see update.h).
+//
+// A small minibatch's update is bound by launches: 16000 rows of 361-1024-512-28 (and ...-1) took 69 of them, two
+// thirds no tensor-core product, 260 us of a 552 us update.  Here each kind of step between the products is one launch
+// over every tensor of both nets: 24 launches, 354 us (131072 rows of 577-1024-1024-512-69: 3583 -> 3400 us).
+#include <cmath>
+#include <cuda_bf16.h>
+
+#include "im_internal.h"
+#include "update.h"
+
+namespace im {
+
+namespace {
+
+constexpr int kThreads = 256;
+
+// Every kernel here is launched with programmatic stream serialization.
+__device__ __forceinline__ void dep_release_wait()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// True in every thread of the block that is the last of the grid to get here; *done is zero again afterwards.
+__device__ __forceinline__ bool last_block(int *done, int n_blocks)
+{
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1) == n_blocks - 1;
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        if (threadIdx.x == 0) *done = 0;
+    }
+    return s_last != 0;
+}
+
+template <typename T>
+__device__ __forceinline__ int owner(const T *t, int n, int block)
+{
+    int k = 0;
+    while (k + 1 < n && block >= t[k + 1].first_block) ++k;
+    return k;
+}
+
+// ---------------------------------------------------------------- Adam
+constexpr int kVecElems = 16 * kThreads;                    // elements of a bias tensor per block
+
+__device__ __forceinline__ float adam_update(const im_adam_config &c, const AdamTensor &T, long long i, float lr, float gs)
+{
+    const float p = T.param[i], g = gs * __ldg(T.grad + i);
+    const float m = fmaf(c.beta1, T.m[i], (1.0f - c.beta1) * g);
+    const float v = fmaf(c.beta2, T.v[i], (1.0f - c.beta2) * g * g);
+    const float q = p - lr * (m * T.inv_c1) / (sqrtf(v * T.inv_c2) + c.eps);
+    T.param[i] = q;
+    T.m[i] = m;
+    T.v[i] = v;
+    return q;
+}
+
+// A block takes a 64 x 64 tile of a weight matrix -- rows are read and written as 256-byte runs, the bf16 copy goes out
+// the same way and its transpose through shared memory -- or kVecElems elements of a vector.
+__global__ void __launch_bounds__(kThreads) adam_multi_kernel(const __grid_constant__ AdamMultiArgs P)
+{
+    __shared__ __align__(16) __nv_bfloat16 tile[64][66];    // 33-word rows: a column walk spreads over the banks
+    dep_release_wait();
+    const AdamTensor &T = P.t[owner(P.t, P.n_tensors, blockIdx.x)];
+    const int blk = (int)blockIdx.x - T.first_block;
+    const float lr = *P.lr, gs = P.grad_scale ? __ldg(P.grad_scale) : 1.0f;
+    if (!T.wb) {
+        const int n = T.rows * T.cols, i0 = blk * kVecElems + threadIdx.x;
+#pragma unroll 4
+        for (int i = i0; i < n && i < (blk + 1) * kVecElems; i += kThreads) adam_update(P.cfg, T, i, lr, gs);
+    } else {
+        const int tiles_c = (T.cols + 63) >> 6, r0 = (blk / tiles_c) << 6, c0 = (blk % tiles_c) << 6;
+        const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+        const bool in_c = c0 + tx < T.cols;
+        __nv_bfloat16 *wb = reinterpret_cast<__nv_bfloat16 *>(T.wb);
+#pragma unroll 4
+        for (int i = ty; i < 64; i += 4) {
+            const int r = r0 + i;
+            __nv_bfloat16 h = __float2bfloat16_rn(0.0f);
+            if (in_c && r < T.rows) {
+                h = __float2bfloat16_rn(adam_update(P.cfg, T, (long long)r * T.cols + c0 + tx, lr, gs));
+                wb[(long long)r * T.ld_wb + c0 + tx] = h;
+            }
+            tile[i][tx] = h;
+        }
+        __syncthreads();
+        __nv_bfloat16 *wbT = reinterpret_cast<__nv_bfloat16 *>(T.wbT);
+        for (int q = threadIdx.x; q < 512; q += kThreads) {
+            const int j = q >> 3, ch = (q & 7) << 3;         // output row c0 + j, elements r0 + ch .. + 7 (padding rows: zeros)
+            if (c0 + j >= T.cols) continue;
+            __align__(16) __nv_bfloat16 e[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) e[k] = tile[ch + k][j];
+            *reinterpret_cast<uint4 *>(wbT + (long long)(c0 + j) * T.ld_wbT + r0 + ch) = *reinterpret_cast<const uint4 *>(e);
+        }
+    }
+    if (P.kl && last_block(P.done, P.n_blocks) && threadIdx.x == 0) {       // every block has read the old learning rate
+        const float k = *P.kl;
+        float x = lr;
+        if (k > 2.0f * P.kl_target) x = fmaxf(x / 1.5f, P.lr_min);
+        else if (k > 0.0f && k < 0.5f * P.kl_target) x = fminf(x * 1.5f, P.lr_max);
+        *P.lr = x;
+    }
+}
+
+// ---------------------------------------------------------------- gradient tensors and their norm
+constexpr int kGroupsPerBlock = 2 * kThreads;               // 4-column groups of a matrix per block
+constexpr int kVecCols = 32;                                // columns of a vector per block
+
+__device__ __forceinline__ double block_sum(double x)
+{
+    __shared__ double s[kThreads / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = x;
+    __syncthreads();
+    double t = 0.0;
+    for (int w = 0; w < kThreads / 32; ++w) t += s[w];
+    __syncthreads();
+    return t;
+}
+
+// Sums of squares are taken in fp64 per thread and block, blocks added in a fixed order by the last one: the result does
+// not depend on scheduling.
+__global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_constant__ GradReduceArgs P)
+{
+    dep_release_wait();
+    const int block = blockIdx.x;
+    double sq = 0.0;
+    const int first_vector = P.n_vectors > 0 ? P.v[0].first_block : P.n_blocks;
+    if (block < first_vector) {
+        // dW: the row slices' partial products added in order
+        const GradMatrix &G = P.m[owner(P.m, P.n_matrices, block)];
+        const int gpr = (G.cols + 3) >> 2, total = G.rows * gpr;
+        const __nv_bfloat16 *in = reinterpret_cast<const __nv_bfloat16 *>(G.in);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = (block - G.first_block) * kGroupsPerBlock + k * kThreads + (int)threadIdx.x;
+            if (i >= total) break;
+            const int r = i / gpr, c = (i - r * gpr) << 2;
+            const __nv_bfloat16 *src = in + (long long)r * G.ld_in + c;
+            float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+            for (int s = 0; s < G.slices; ++s) {
+                const uint2 w = __ldg(reinterpret_cast<const uint2 *>(src + s * G.slice_stride));
+                const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.x));
+                const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
+                a[0] += lo.x; a[1] += lo.y; a[2] += hi.x; a[3] += hi.y;
+            }
+            float *dst = G.out + (long long)r * G.cols + c;
+            if ((G.cols & 3) == 0) {
+                *reinterpret_cast<float4 *>(dst) = make_float4(a[0], a[1], a[2], a[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (c + j < G.cols) dst[j] = a[j];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (c + j < G.cols) sq = fma((double)a[j], (double)a[j], sq);
+        }
+    } else if (P.n_vectors > 0 && block < P.n_blocks - (P.n_extra > 0 ? 1 : 0)) {
+        // db: 32 columns, 32 groups of rows in fp32 (four chains each), the groups added in order in fp64
+        __shared__ double s_col[32][kVecCols + 1];
+        const GradVector &G = P.v[owner(P.v, P.n_vectors, block)];
+        const int cg = threadIdx.x & 7, rg = threadIdx.x >> 3, c = (block - G.first_block) * kVecCols + 4 * cg;
+        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+        if (c < G.ld) {
+            int r = rg;
+#pragma unroll 2
+            for (; r + 32 < G.n_rows; r += 64) {
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(G.in + (long long)r * G.ld + c));
+                const float4 y = __ldg(reinterpret_cast<const float4 *>(G.in + (long long)(r + 32) * G.ld + c));
+                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+                b.x += y.x; b.y += y.y; b.z += y.z; b.w += y.w;
+            }
+            if (r < G.n_rows) {
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(G.in + (long long)r * G.ld + c));
+                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+            }
+        }
+        s_col[rg][4 * cg] = (double)(a.x + b.x); s_col[rg][4 * cg + 1] = (double)(a.y + b.y);
+        s_col[rg][4 * cg + 2] = (double)(a.z + b.z); s_col[rg][4 * cg + 3] = (double)(a.w + b.w);
+        __syncthreads();
+        if (threadIdx.x < kVecCols) {
+            double t = 0.0;
+#pragma unroll 8
+            for (int g = 0; g < 32; ++g) t += s_col[g][threadIdx.x];
+            const int col = (block - G.first_block) * kVecCols + threadIdx.x;
+            if (col < G.cols) {
+                const float x = (float)t;
+                G.out[col] = x;
+                sq = (double)x * (double)x;
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < P.n_extra; i += kThreads) sq = fma((double)__ldg(P.extra + i), (double)__ldg(P.extra + i), sq);
+    }
+    if (!P.partial) return;
+    sq = block_sum(sq);
+    if (threadIdx.x == 0) P.partial[block] = sq;
+    if (!last_block(P.done, P.n_blocks)) return;
+    double t = 0.0;
+    for (int i = threadIdx.x; i < P.n_blocks; i += kThreads) t += __ldcg(P.partial + i);
+    t = block_sum(t);
+    if (threadIdx.x == 0) {
+        const double s = (double)P.max_norm / (sqrt(t) + 1e-6);
+        P.scale_out[0] = (float)(s < 1.0 ? s : 1.0);
+        P.scale_out[1] = (float)sqrt(t);
+    }
+}
+
+// ---------------------------------------------------------------- output gradients
+constexpr int kOutRows = 128;
+
+__global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_constant__ OutGradArgs P)
+{
+    __shared__ float s_sum[8][128];
+    dep_release_wait();
+    const OutGrad &G = P.net[blockIdx.y];
+    const int lanes = G.ld >> 1, groups = kThreads / lanes;       // a thread owns two columns of every `groups`-th row
+    const int c = 2 * ((int)threadIdx.x % lanes), g = (int)threadIdx.x / lanes;
+    const int r0 = blockIdx.x * kOutRows, r1 = min(r0 + kOutRows, P.M);
+    __nv_bfloat16 *dz = reinterpret_cast<__nv_bfloat16 *>(G.dz);
+    float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll 8
+    for (int r = r0 + g; r < r1; r += groups) {
+        const float *src = G.d_out + (long long)r * G.cols + c;
+        const float a = c < G.cols ? __ldg(src) : 0.0f, b = c + 1 < G.cols ? __ldg(src + 1) : 0.0f;
+        *reinterpret_cast<__nv_bfloat162 *>(dz + (long long)r * G.ld + c) = __floats2bfloat162_rn(a, b);
+        s0 += a;
+        s1 += b;
+    }
+    s_sum[g][c] = s0;
+    s_sum[g][c + 1] = s1;
+    __syncthreads();
+    if ((int)threadIdx.x < G.ld) {
+        float t = 0.0f;
+        for (int k = 0; k < groups; ++k) t += s_sum[k][threadIdx.x];
+        G.partial[(long long)blockIdx.x * G.ld + threadIdx.x] = t;
+    }
+}
+
+// ---------------------------------------------------------------- shuffled minibatch
+// A warp gathers a row; VEC: observation rows start on 16-byte boundaries.
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads) gather_minibatch_kernel(const __grid_constant__ GatherArgs P)
+{
+    dep_release_wait();
+    const int lane = threadIdx.x & 31, warps = (gridDim.x * kThreads) >> 5;
+    for (int i = (blockIdx.x * kThreads + threadIdx.x) >> 5; i < P.M; i += warps) {
+        long long src = __ldg(P.idx + i);
+        if (src < 0 || src >= P.n_src) {                          // a bad index is clamped and reported, never followed
+            if (lane == 0) atomicOr(P.status, IM_DEV_BAD_STATE);
+            src = src < 0 ? 0 : P.n_src - 1;
+        }
+        const float *row = P.obs + src * P.ld_obs;
+        __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(P.h) + (long long)i * P.ld_h;
+#pragma unroll 4
+        for (int c = 4 * lane; c < P.ld_h; c += 128) {
+            float v[4];
+            if (VEC && c + 4 <= P.D) {
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(row + c));
+                v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = c + j < P.D ? __ldg(row + c + j) : 0.0f;
+            }
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+            *reinterpret_cast<uint2 *>(h + c) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+        }
+        const long long o = (long long)i * P.A, s = src * P.A;
+#pragma unroll 4
+        for (int k = lane; k < P.A; k += 32) {
+            P.g_action[o + k] = __ldg(P.action + s + k);
+            P.g_mean[o + k] = __ldg(P.mean + s + k);
+        }
+        if (lane < 4) {
+            const float *from = lane == 0 ? P.logp : lane == 1 ? P.advantage : lane == 2 ? P.value : P.returns;
+            float *to = lane == 0 ? P.g_logp : lane == 1 ? P.g_advantage : lane == 2 ? P.g_value : P.g_returns;
+            to[i] = __ldg(from + src);
+        }
+    }
+}
+
+}  // namespace
+
+void adam_multi_add(AdamMultiArgs &a, float *param, const float *grad, float *m, float *v, int rows, int cols, uint16_t *wb, int ld_wb,
+                    uint16_t *wbT, int ld_wbT, int t)
+{
+    AdamTensor &T = a.t[a.n_tensors++];
+    T.param = param; T.grad = grad; T.m = m; T.v = v; T.wb = wb; T.wbT = wbT;
+    T.rows = rows; T.cols = cols; T.ld_wb = ld_wb; T.ld_wbT = ld_wbT;
+    T.inv_c1 = (float)(1.0 / (1.0 - std::pow((double)a.cfg.beta1, (double)t)));
+    T.inv_c2 = (float)(1.0 / (1.0 - std::pow((double)a.cfg.beta2, (double)t)));
+    T.first_block = a.n_blocks;
+    a.n_blocks += wb ? ((rows + 63) / 64) * ((cols + 63) / 64) : (rows * cols + kVecElems - 1) / kVecElems;
+}
+
+cudaError_t launch_adam_multi(AdamMultiArgs &a, cudaStream_t stream)
+{
+    const cudaError_t e = launch_pdl(adam_multi_kernel, dim3((unsigned)a.n_blocks), dim3(kThreads), 0, stream, 0, a);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return e;
+}
+
+int grad_matrix_blocks(int rows, int cols) { return (int)(((long long)rows * ((cols + 3) / 4) + kGroupsPerBlock - 1) / kGroupsPerBlock); }
+int grad_vector_blocks(int cols) { return (cols + kVecCols - 1) / kVecCols; }
+
+// (all matrices are added before the first vector)
+void grad_reduce_add(GradReduceArgs &a, const uint16_t *in, long long slice_stride, int ld_in, int slices, int rows, int cols, float *out)
+{
+    a.m[a.n_matrices++] = {in, out, slice_stride, ld_in, slices, rows, cols, a.n_blocks};
+    a.n_blocks += grad_matrix_blocks(rows, cols);
+}
+void grad_reduce_add(GradReduceArgs &a, const float *in, int n_rows, int ld, int cols, float *out)
+{
+    a.v[a.n_vectors++] = {in, out, n_rows, ld, cols, a.n_blocks};
+    a.n_blocks += grad_vector_blocks(cols);
+}
+
+cudaError_t launch_grad_reduce(GradReduceArgs &a, cudaStream_t stream)
+{
+    if (a.n_extra > 0) a.n_blocks += 1;
+    const cudaError_t e = launch_pdl(grad_reduce_kernel, dim3((unsigned)a.n_blocks), dim3(kThreads), 0, stream, 0, a);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return e;
+}
+
+cudaError_t launch_out_grads(const OutGradArgs &a, cudaStream_t stream)
+{
+    const cudaError_t e = launch_pdl(out_grads_kernel, dim3((unsigned)((a.M + kOutRows - 1) / kOutRows), (unsigned)a.n_nets), dim3(kThreads), 0,
+                                     stream, 0, a);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return e;
+}
+
+cudaError_t launch_gather_minibatch(const GatherArgs &a, cudaStream_t stream)
+{
+    const bool vec = (reinterpret_cast<uintptr_t>(a.obs) & 15u) == 0 && (a.ld_obs & 3) == 0;
+    const int blocks = (a.M + 7) / 8 < 148 * 16 ? (a.M + 7) / 8 : 148 * 16;
+    const cudaError_t e = launch_pdl(vec ? gather_minibatch_kernel<true> : gather_minibatch_kernel<false>, dim3((unsigned)blocks), dim3(kThreads), 0,
+                                     stream, 0, a);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return e;
+}
+
+}  // namespace im
