@@ -3,16 +3,23 @@
 // observation (the post-physics phase of the paper's Figure 2 as one kernel).
 //
 // Mapping: one CTA handles 32 consecutive envs; lane e handles env e of the
-// tile and warp c handles kinematic chain c of the skeleton, a root-to-leaf
-// path.  A thread walks its path once per pass, carrying the world transform
-// (and velocities) in registers, so forward kinematics needs no exchange
-// between threads; bodies shared by several paths are recomputed (pose only)
-// and "owned" by one path, which alone loads their simulated state, scores them
-// and writes their observation entries.  Every global load of the
-// structure-of-arrays body state is one fully used 128-byte line per warp.
-// The observation rows of the 32 envs are assembled in shared memory in two
-// halves that reuse the same space (row stride 4 x odd: conflict-free 16-byte
-// column writes, 16-byte aligned rows) and written out as whole lines.
+// tile.  A warp walks a kinematic chain of the skeleton, a root-to-leaf path,
+// with the world transform (and velocities) in registers, so forward
+// kinematics needs no exchange between threads; bodies shared by several paths
+// are recomputed (pose only) and "owned" by one path, which alone loads their
+// simulated state, scores them and writes their observation entries.  Every
+// global load of the structure-of-arrays body state is one fully used 128-byte
+// line per warp.  Observation rows are assembled in shared memory (row stride
+// 4 x odd: conflict-free 16-byte column writes, 16-byte aligned rows) and
+// written out as whole lines.
+//
+// Two kernels.  While the tiles fit the SMs at once, a CTA's own latency is what
+// counts: the role kernel gives every chain two warps whose work is independent
+// and about equally long -- one scores the simulated bodies against the reference,
+// the other builds the observation -- and stages whole rows.  With more tiles than
+// that the issue slots count: the chain kernel does both in one warp per chain,
+// which loads every body once, and stages half rows, so that four CTAs share an SM.
+// Figures at launch_env_kernel.
 #include <cuda_bf16.h>
 
 #include "im_internal.h"
@@ -55,7 +62,7 @@ __host__ __device__ inline int tile_stride(int D)
     return 4 * s4;
 }
 
-// The observation row is staged in two halves; the split is the end of the body blocks rounded
+// The chain kernel stages the observation row in two halves; the split is the end of the body blocks rounded
 // up to a multiple of four columns so that both halves start on a 16-byte boundary.
 __host__ __device__ inline int split_col(int J) { return (15 * J + 3) / 4 * 4; }
 
@@ -65,6 +72,19 @@ __host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, 
     const int D = 24 * J + 1 + extra_cols, c1 = split_col(J);
     const int s1 = tile_stride(c1), s2 = tile_stride(D - c1);
     return (size_t)kTile * (s1 > s2 ? s1 : s2) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links;
+}
+
+// The role kernel: the staged rows, the chains' partial sums, their link records.  Staged columns: all, or, where an extended observation is too wide for that, the first
+// 24 J (the rest is then written column by column).
+__host__ __device__ inline size_t role_smem_floats(int cols, int n_chains, int n_links)
+{
+    return (size_t)kTile * tile_stride(cols) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links;
+}
+constexpr size_t kMaxSmemFloats = 232448 / 4;       // opt-in shared memory per block on this architecture (227 KB)
+__host__ __device__ inline int staged_cols(int J, int n_chains, int n_links, int extra_cols)
+{
+    const int cols = 24 * J + 1 + extra_cols;
+    return extra_cols == 0 || role_smem_floats(cols, n_chains, n_links) <= kMaxSmemFloats ? cols : 24 * J;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -386,14 +406,19 @@ struct SimBody {
     Vec3 p, v, w;
 };
 
-// A simulated quaternion of zero or non-finite norm is replaced by the identity and reported.
-__device__ __forceinline__ Quat sanitize(Quat q, uint32_t *status)
+// A simulated quaternion of zero or non-finite norm is replaced by the identity; `bad` collects whether one was.
+__device__ __forceinline__ Quat sanitize(Quat q, bool &bad)
 {
     const float n2 = fmaf(q.z, q.z, fmaf(q.y, q.y, fmaf(q.x, q.x, q.w * q.w)));
-    if (!(n2 > 1e-12f && n2 < 1e12f)) {
-        atomicOr(status, IM_DEV_BAD_SIM_QUAT);
-        return {1, 0, 0, 0};
-    }
+    const bool ok = n2 > 1e-12f && n2 < 1e12f;
+    bad = bad || !ok;
+    return {ok ? q.w : 1.0f, ok ? q.x : 0.0f, ok ? q.y : 0.0f, ok ? q.z : 0.0f};
+}
+__device__ __forceinline__ Quat sanitize(Quat q, uint32_t *status)
+{
+    bool bad = false;
+    q = sanitize(q, bad);
+    if (bad) atomicOr(status, IM_DEV_BAD_SIM_QUAT);
     return q;
 }
 
@@ -437,6 +462,7 @@ struct SimView {
         const uint32_t o = 3 * (uint32_t)b * st + e;
         return {__ldcs(base + o), __ldcs(base + o + st), __ldcs(base + o + 2 * st)};
     }
+    __device__ __forceinline__ SimBody ld_body(int b) const { return {ld_quat(b), ld_pos(b), ld_lin(b), ld_ang(b)}; }
     __device__ __forceinline__ Vec3 ld_pos(int b) const { return ld_vec(pos, bs_pos, b); }
     __device__ __forceinline__ Vec3 ld_lin(int b) const { return ld_vec(lin, bs_lin, b); }
     __device__ __forceinline__ Vec3 ld_ang(int b) const { return ld_vec(ang, bs_ang, b); }
@@ -500,13 +526,446 @@ __device__ __forceinline__ void copy_out_any(const EnvKernelParams &P, const flo
     else copy_out<false, true>(P, tile, S, rows, quads, first, last, warp, n_warps, lane);
 }
 
-// Kernel body.  The observation row is assembled in two halves that reuse the same shared
+// Per-env values of the step that every thread of the env holds.
+struct EnvState {
+    int clip, cyc;                 // before a reset
+    float t;
+    ClipMeta cm;
+    ClipLoop loop;
+    int flags;
+    bool reset;
+    int clip_new, cyc_new;         // after it (unchanged for an env that is not reset)
+    float t_new;
+    ClipMeta cm_new;
+};
+
+// Flags (step a4) given the reward.
+template <bool OPT>
+__device__ __forceinline__ int flags_of(const EnvKernelParams &P, int env, float root_z, float r, const EnvState &E)
+{
+    bool terminated = (root_z < P.reward.h_min) || (r < P.reward.r_min);
+    if (OPT && P.ep_len[env] < P.grace_steps) terminated = false;
+    const bool truncated = !(OPT && E.loop.on) && __fadd_rn(E.t, P.dt) > E.cm.dur;    // a looped clip has no end
+    return (terminated ? 1 : 0) | (truncated ? 2 : 0);
+}
+
+// Flags and masked reset (step a5) given the reward; a function of (env, step) that every thread of the env repeats.
+// count: this thread keeps the adaptive-initialisation statistics of its env.
+template <bool RESET_ALL, bool OPT>
+__device__ __forceinline__ void decide(const EnvKernelParams &P, int env, float root_z, float r, bool count, EnvState &E)
+{
+    E.flags = 0;
+    if (!RESET_ALL) {
+        E.flags = flags_of<OPT>(P, env, root_z, r, E);
+        if (OPT && P.n_bins > 0 && (E.flags & 1) && count) {
+            // the (clip, phase bin) the episode failed in
+            const float span = fmaxf(__fsub_rn(E.cm.dur, P.dt), 0.0f);
+            atomicAdd(P.stat_failures + E.clip * P.n_bins + phase_bin(E.t, span, P.n_bins), 1u);
+        }
+    }
+    E.reset = RESET_ALL || E.flags != 0;
+    E.clip_new = E.clip; E.cyc_new = E.cyc; E.t_new = E.t; E.cm_new = E.cm;
+    if (!E.reset) return;
+    const uint4 x = philox4x32_10(make_uint4(P.env_id_base + (uint32_t)env, P.step, IM_STREAM_RESET, 0u),
+                                  make_uint2(P.seed_lo, P.seed_hi));
+    const float u = (float)(x.y >> 8) * 5.9604644775390625e-08f;
+    if (OPT && P.n_bins > 0) {
+        // weighted (clip, phase bin) from the cumulative table: smallest i with x < T_i
+        const int B = P.n_bins;
+        int lo = 0, hi = P.C * B - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if ((unsigned long long)x.x < __ldg(P.reset_cdf + mid)) hi = mid;
+            else lo = mid + 1;
+        }
+        E.clip_new = lo / B;
+        E.cm_new = P.meta[E.clip_new];
+        const float span = fmaxf(__fsub_rn(E.cm_new.dur, P.dt), 0.0f);
+        const float width = __fdiv_rn(span, (float)B);
+        E.t_new = fminf(__fmul_rn(__fadd_rn((float)(lo - E.clip_new * B), u), width), span);
+        if (count) atomicAdd(P.stat_starts + lo, 1u);
+    } else {
+        E.clip_new = (int)__umulhi(x.x, (uint32_t)P.C);
+        E.cm_new = P.meta[E.clip_new];
+        E.t_new = __fmul_rn(u, fmaxf(__fsub_rn(E.cm_new.dur, P.dt), 0.0f));
+    }
+    E.cyc_new = 0;
+    if (OPT && P.loops) E.loop = P.loops[E.clip_new];
+}
+
+// The seven error terms of an env from the chains' partial sums, added in chain order, and the reward.
+__device__ __forceinline__ float reward_of(const EnvKernelParams &P, const float *part, int C, int lane, float (&term)[IM_N_TERMS])
+{
+    float e[kPartials];
+#pragma unroll
+    for (int i = 0; i < kPartials; ++i) {
+        float a = 0.0f;
+        for (int cc = 0; cc < C; ++cc) a += part[(i * C + cc) * kTile + lane];
+        e[i] = a;
+    }
+    // term order of the configuration: pose, vel, ee_pos, ee_rot, com, body_pos, body_vel
+    term[0] = e[0]; term[1] = e[1]; term[2] = e[2]; term[3] = e[3];
+    term[4] = e[6] * e[6] + e[7] * e[7] + e[8] * e[8];
+    term[5] = e[4]; term[6] = e[5];
+    float r = 0.0f;
+    if (P.reward.mode == 0) {
+        float sum = 0.0f;
+#pragma unroll
+        for (int k = 0; k < IM_N_TERMS; ++k) sum += P.reward.w[k] * term[k];
+        r = expf(-sum);
+    } else {
+#pragma unroll
+        for (int k = 0; k < IM_N_TERMS; ++k) r += P.reward.a[k] * expf(-P.reward.w[k] * term[k]);
+    }
+    return r;
+}
+
+// The env's new state; returns the steps of the episode that ended (0: none did).
+template <bool OPT>
+__device__ __forceinline__ int store_env_state(const EnvKernelParams &P, int env, const EnvState &E)
+{
+    const int len_now = P.ep_len[env] + 1;
+    P.clip_id[env] = E.clip_new;
+    P.t[env] = E.t_new;
+    if (OPT && P.loops) P.cycle[env] = E.cyc_new;
+    P.ep_len[env] = E.reset ? 0 : len_now;
+    return E.reset ? len_now : 0;
+}
+
+// Training summaries: integer sums over the tile (one warp), then one atomic per quantity.
+__device__ __forceinline__ void add_summary(const EnvKernelParams &P, bool valid, float r, int flags, int ep_done, int lane)
+{
+    unsigned long long v[4] = {valid ? (unsigned long long)__float2ll_rn(r * 1099511627776.0f) : 0ull,
+                               (unsigned long long)(valid ? (flags & 1) : 0), (unsigned long long)(valid ? (flags >> 1) & 1 : 0),
+                               (unsigned long long)ep_done};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+        if (lane == 0 && v[i]) atomicAdd(P.summary + i, v[i]);
+    }
+}
+
+// One observation entry past the staged columns, straight to the row of env `env` (extended observations too wide to stage).
+__device__ __forceinline__ void st_direct(const EnvKernelParams &P, int env, int col, float v)
+{
+    const size_t o = (size_t)env * P.ld_obs + col;
+    if (P.obs) P.obs[o] = v;
+    if (P.obs_bf16) {
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        P.obs_bf16[o] = *reinterpret_cast<const uint16_t *>(&h);
+    }
+}
+
+// The role kernel.  OPT compiles in the optional semantics (grace steps, motion randomisation, adaptive initialisation,
+// extended observation, looped clips, summaries); envs that use none run the instantiation without them.  WIDE: more
+// (chain, role) pairs than warps (trees with more than eight leaves).
+template <bool RESET_ALL, bool OPT, bool AOS, bool WIDE>
+__device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *smem_raw)
+{
+    // a successor launched with programmatic stream serialization (the policy's first GEMM) may be scheduled
+    // onto SMs as this grid drains; it waits for this grid's completion before it reads anything
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const SkelDev &sk = P.sk;
+    const int J = sk.J, C = sk.n_chains, D = 24 * J + 1, RS = 2 + 2 * J;
+    // extended observation: end-effector targets of further future frames, then the previous action
+    const int n_ee = OPT ? __popc(sk.ee_mask) : 0;
+    const int ext_future = (OPT && P.n_future > 1) ? (P.n_future - 1) * 9 * n_ee : 0;
+    const int D_ext = D + ext_future + (OPT ? P.act_dim : 0);
+    const int cols = OPT ? staged_cols(J, C, sk.n_links, D_ext - D) : D;
+    const bool direct = OPT && cols < D;
+    const int S = tile_stride(cols);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    const int env = blockIdx.x * kTile + lane;
+    const bool valid = env < P.N;
+    const int envc = valid ? env : P.N - 1;
+    float *row = smem_raw + (size_t)lane * S;
+    float *part = smem_raw + (size_t)kTile * S;
+    float4 *all_links = reinterpret_cast<float4 *>(part + (size_t)kPartials * C * kTile);
+
+    for (int i = threadIdx.x; i < 2 * sk.n_links; i += blockDim.x) all_links[i] = __ldg(P.links + i);
+    __syncthreads();
+    // this kernel is launched the same way: everything above reads only what the env's creation left in memory
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    EnvState E;
+    E.clip = 0; E.cyc = 0; E.t = 0.0f;
+    E.cm = {2, 1.0f, 1.0f, 0};
+    E.loop = {0.0f, 0.0f, 0.0f, 0};
+    Heading H = {0.0f, 0.0f, 1.0f, 0.0f};
+    float root_z = 0.0f, r = INFINITY;
+    bool bad = false;
+    const SimView<AOS> sv(P, envc);
+    if (!RESET_ALL) {
+        const Quat q_root = sv.ld_quat(0);
+        const Vec3 p_root = sv.ld_pos(0);
+        E.clip = P.clip_id[envc];
+        if (E.clip < 0 || E.clip >= P.C) {
+            E.clip = min(max(E.clip, 0), P.C - 1);
+            if (warp == 0) atomicOr(P.status, IM_DEV_BAD_STATE);
+        }
+        E.t = __fadd_rn(P.t[envc], P.dt);
+        E.cm = P.meta[E.clip];
+        if (OPT && P.loops) {
+            // a clip played in a loop: the time wraps at the clip's end and the env's cycle count goes up
+            E.loop = P.loops[E.clip];
+            E.cyc = P.cycle[envc];
+            if (E.loop.on && E.t >= E.cm.dur) { E.t = __fsub_rn(E.t, E.cm.dur); ++E.cyc; }
+        }
+        H = make_heading(sanitize(q_root, bad), p_root);
+        root_z = p_root.z;
+    }
+    const ClipLoop loop = E.loop;              // of the clip before a reset
+    // whether the reward can end an episode; if not, the root height and the clip end decide, which are known already
+    const bool need_r = !RESET_ALL && P.reward.r_min > -INFINITY;
+    const bool known_reset = !RESET_ALL && !need_r && flags_of<OPT>(P, envc, root_z, r, E) != 0;
+
+    if (!RESET_ALL) {
+#pragma unroll 1
+        for (int task = warp; task < 2 * C; task += n_warps) {
+            const int c = task < C ? task : task - C;
+            const int len = sk.chain_len[c], first_own = sk.chain_first_own[c];
+            const float4 *links = all_links + 2 * sk.link_start[c];
+            if (task < C) {
+                // ---- reference at the advanced time, errors against the simulated state
+                int frame;
+                float alpha;
+                lookup(E.cm, E.t, frame, alpha);
+                const float4 *r0 = P.frames + (size_t)IM_CHECKED(frame, P.n_rows) * RS;
+                LinkRec L = ld_link(links, 0);
+                KeyPair keys = ld_keys(r0, L.b);
+                float acc[kPartials];
+#pragma unroll
+                for (int i = 0; i < kPartials; ++i) acc[i] = 0.0f;
+                Walk s;
+                Quat qa = {1, 0, 0, 0};                      // simulated state of the previous body of the chain
+                Vec3 wa = {0, 0, 0};
+                if (first_own > 0) {
+                    const int a = ld_link(links, first_own - 1).b;
+                    qa = sanitize(sv.ld_quat(a), bad);
+                    wa = sv.ld_ang(a);
+                }
+                for (int k = 0; k < len; ++k) {
+                    const LinkRec Lc = L;
+                    const int b = Lc.b;
+                    const bool own = Lc.flags & LINK_OWN;
+                    SimBody sim;
+                    if (own) {                                // issue the loads before the interpolation math
+                        if (!AOS) (void)IM_CHECKED((4 * (uint32_t)b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
+                        sim.q = sv.ld_quat(b);
+                        sim.p = sv.ld_pos(b);
+                        sim.v = sv.ld_lin(b);
+                        sim.w = sv.ld_ang(b);
+                    }
+                    const KeyPair cur = keys;
+                    if (k + 1 < len) {                        // next joint's link and keyframe words in flight
+                        L = ld_link(links, k + 1);
+                        keys = ld_keys(r0, L.b);
+                    }
+                    Quat ql;
+                    Vec3 wl;
+                    joint_step<true>(r0, cur, alpha, E.cm.fps, Lc, k, s, ql, wl);
+                    if (OPT && k == 0) s.p = s.p + loop_shift(loop, E.cyc);    // completed cycles of a looped clip move the root
+                    if (own) {
+                        sim.q = sanitize(sim.q, bad);
+                        // the root's "parent" is the identity: qa = (1, 0, 0, 0), wa = 0 on the chain that owns it
+                        const Quat ql_sim = qmul_conj(qa, sim.q);
+                        const Vec3 wl_sim = qrot_inv(sim.q, sim.w - wa);
+                        const float th_sq = angle_sq(qmul_conj(ql, ql_sim));
+                        const Vec3 dwl = wl_sim - wl;
+                        const Vec3 dp = sim.p - s.p;
+                        const Vec3 dv = sim.v - s.v;
+                        const float dp2 = dot(dp, dp);
+                        acc[0] += th_sq;
+                        acc[1] += dot(dwl, dwl);
+                        if (Lc.flags & LINK_EE) {
+                            acc[2] += dp2;
+                            acc[3] += angle_sq(qmul_conj(s.q, sim.q));
+                        }
+                        acc[4] += dp2;
+                        acc[5] += dot(dv, dv);
+                        acc[6] = fmaf(Lc.mass_frac, dp.x, acc[6]);
+                        acc[7] = fmaf(Lc.mass_frac, dp.y, acc[7]);
+                        acc[8] = fmaf(Lc.mass_frac, dp.z, acc[8]);
+                        qa = sim.q;
+                        wa = sim.w;
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < kPartials; ++i) part[(i * C + c) * kTile + lane] = acc[i];
+            } else {
+                // ---- observation entries of the simulated bodies (an env known to be reset gets the reference's instead)
+                bool ignore = false;
+                SimBody next = sv.ld_body(ld_link(links, first_own).b);
+                for (int k = first_own; k < len; ++k) {
+                    const int b = ld_link(links, k).b;
+                    const SimBody sim = next;
+                    if (k + 1 < len) next = sv.ld_body(ld_link(links, k + 1).b);
+                    (void)IM_CHECKED(15 * b + 14, S);
+                    if (!known_reset) body_obs(H, sanitize(sim.q, ignore), sim.p, sim.v, sim.w, row, b);
+                }
+            }
+            if (!WIDE) break;
+        }
+        if (bad) atomicOr(P.status, IM_DEV_BAD_SIM_QUAT);
+        if (need_r) {
+            __syncthreads();
+            float term[IM_N_TERMS];
+            r = reward_of(P, part, C, lane, term);
+        }
+    }
+    decide<RESET_ALL, OPT>(P, envc, root_z, r, warp == 0 && valid, E);
+
+    // ---- reference state of reset envs, and the targets
+    int frame_n;
+    float alpha_n;
+    lookup(E.cm_new, E.t_new, frame_n, alpha_n);
+    const float4 *rn0 = P.frames + (size_t)IM_CHECKED(frame_n, P.n_rows) * RS;
+    const bool any_reset = __any_sync(0xffffffffu, E.reset);
+    const bool noisy = OPT && P.reset_noise_std > 0.0f;
+#pragma unroll 1
+    for (int task = warp; task < 2 * C; task += n_warps) {
+        const int c = task < C ? task : task - C;
+        const int len = sk.chain_len[c];
+        const float4 *links = all_links + 2 * sk.link_start[c];
+        if (task < C) {
+            if (any_reset) {
+                // the new reference state replaces the simulated one in the observation, and optionally in the caller's arrays
+                LinkRec L = ld_link(links, 0);
+                KeyPair keys = ld_keys(rn0, L.b);
+                Walk s;
+                Heading Hn = H;
+                for (int k = 0; k < len; ++k) {
+                    const LinkRec Lc = L;
+                    const int b = Lc.b;
+                    const KeyPair cur = keys;
+                    if (k + 1 < len) {
+                        L = ld_link(links, k + 1);
+                        keys = ld_keys(rn0, L.b);
+                    }
+                    Quat ql;
+                    Vec3 wl;
+                    if (noisy) {
+                        // motion randomisation: the joint turns by a small random rotation in its own frame and
+                        // the root is shifted; every chain that walks a shared body draws the same numbers
+                        slerp_joint<true>(cur, alpha_n, E.cm_new.fps + E.cm_new.fps, ql, wl);
+                        ql = qmul(ql, reset_noise_quat(P, envc, b));
+                        joint_compose<true>(rn0, alpha_n, E.cm_new.fps, Lc, k, s, ql, wl);
+                        if (k == 0) s.p = s.p + reset_noise_vec(P, envc, sk.J);
+                    } else {
+                        joint_step<true>(rn0, cur, alpha_n, E.cm_new.fps, Lc, k, s, ql, wl);
+                    }
+                    if (k == 0) Hn = make_heading(s.q, s.p);
+                    if ((Lc.flags & LINK_OWN) && E.reset) {
+                        body_obs(Hn, s.q, s.p, s.v, s.w, row, b);
+                        if (!RESET_ALL && P.write_back && valid) sv.st_body(b, s.q, s.p, s.v, s.w);
+                    }
+                }
+            }
+        }
+        if (any_reset && (OPT || task >= C)) {
+            // heading of the observed root where it is a reset env's new one
+            Quat ql;
+            Vec3 wl;
+            slerp_joint<false>(ld_keys(rn0, 0), alpha_n, 0.0f, ql, wl);
+            if (noisy) ql = qmul(ql, reset_noise_quat(P, envc, 0));
+            const KeyPair root = ld_pair(rn0);
+            Vec3 pr = {fmaf(alpha_n, root.b.x, root.a.x), fmaf(alpha_n, root.b.y, root.a.y), fmaf(alpha_n, root.b.z, root.a.z)};
+            if (noisy) pr = pr + reset_noise_vec(P, envc, sk.J);
+            const Heading Hn = make_heading(ql, pr);
+            if (E.reset) H = Hn;
+        }
+        // the reference one control interval ahead (frame 1), seen from the observed root's heading frame; frames
+        // f = 2 .. n_future of an extended observation, t + f dt (two fp32 operations, clamped to the clip's end), go to the
+        // warps of the other role, which are the less loaded ones
+        const int f0 = task < C ? 2 : 1, f1 = task < C ? (OPT ? P.n_future : 1) : 1;
+        for (int f = f0; f <= f1; ++f) {
+            int cyc_f = E.cyc_new, frame_f;
+            float alpha_f;
+            const float t_f = time_ahead<OPT>(E.loop, E.cm_new.dur, E.t_new, f == 1 ? P.dt : __fmul_rn((float)f, P.dt), cyc_f);
+            lookup(E.cm_new, t_f, frame_f, alpha_f);
+            const float4 *rf0 = P.frames + (size_t)IM_CHECKED(frame_f, P.n_rows) * RS;
+            LinkRec L = ld_link(links, 0);
+            KeyPair keys = ld_keys(rf0, L.b);
+            Walk s;
+            for (int k = 0; k < len; ++k) {
+                const LinkRec Lc = L;
+                const int b = Lc.b;
+                const KeyPair cur = keys;
+                if (k + 1 < len) {
+                    L = ld_link(links, k + 1);
+                    keys = ld_keys(rf0, L.b);
+                }
+                Quat ql;
+                Vec3 wl;
+                joint_step<false>(rf0, cur, alpha_f, E.cm_new.fps, Lc, k, s, ql, wl);
+                if (OPT && k == 0) s.p = s.p + loop_shift(E.loop, cyc_f);
+                if (!(Lc.flags & LINK_OWN) || (OPT && f > 1 && !(Lc.flags & LINK_EE))) continue;
+                float o[9];
+                target_obs(H, s.q, s.p, o);
+                const int col = !OPT || f == 1 ? 15 * J + 1 + 9 * b : D + ((f - 2) * n_ee + __popc(sk.ee_mask & ((1u << b) - 1u))) * 9;
+                if (!OPT || col + 9 <= cols) {
+                    (void)IM_CHECKED(col + 8, S);
+                    store_run<9>(row, col, o);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        if (col + i < cols) row[col + i] = o[i];
+                        else if (valid) st_direct(P, env, col + i, o[i]);
+                    }
+                }
+            }
+        }
+        if (task == C) {
+            row[15 * J] = E.t_new / E.cm_new.dur;                                  // phase
+            if (!direct) {
+                for (int i = D_ext; i < S; ++i) row[i] = 0.0f;
+            } else if (valid) {
+                for (int i = D_ext; i < P.ld_obs; ++i) st_direct(P, env, i, 0.0f);
+            }
+        }
+        if (!WIDE) break;
+    }
+    if (OPT && P.act_dim > 0) {
+        // the action the policy took before this step; an env that was just reset has none
+        for (int j = warp; j < P.act_dim; j += n_warps) {
+            const float a = (E.reset || !valid) ? 0.0f : __ldg(P.prev_action + (size_t)env * P.ld_action + j);
+            const int col = D + ext_future + j;
+            if (!direct) row[col] = a;
+            else if (valid) st_direct(P, env, col, a);
+        }
+    }
+    __syncthreads();
+
+    // ---- the first warp forms reward, flags and the new per-env state, the others send the rows out
+    if (warp > 0) {
+        copy_out_any(P, smem_raw, S, direct ? cols >> 2 : S >> 2, 0, direct ? cols >> 2 : P.ld_obs >> 2, warp - 1, n_warps - 1, lane);
+        return;
+    }
+    int ep_done = 0;                            // steps of the episode this step ended (0 where none ended)
+    if (!RESET_ALL) {
+        float term[IM_N_TERMS];
+        r = reward_of(P, part, C, lane, term);
+        if (valid) {
+            P.reward_out[env] = r;
+            P.flags_out[env] = (uint8_t)E.flags;
+            if (P.terms_out) {
+#pragma unroll
+                for (int k = 0; k < IM_N_TERMS; ++k) P.terms_out[(size_t)k * P.N + env] = term[k];
+            }
+        }
+    }
+    if (valid) ep_done = store_env_state<OPT>(P, env, E);
+    if (OPT && !RESET_ALL && P.summary) add_summary(P, valid, r, E.flags, ep_done, lane);
+}
+
+// The chain kernel.  The observation row is assembled in two halves that reuse the same shared
 // memory: columns [0, c1) -- the body blocks and, if 15 J is not a multiple of 4, the phase and
 // the first target floats -- and columns [c1, D) -- the targets.
 // OPT compiles in the optional semantics (grace steps, motion randomisation, adaptive initialisation, extended
 // observation); envs that use none run the instantiation without them.
-template <bool RESET_ALL, bool OPT, bool AOS>
-__device__ __forceinline__ void env_step_body(const EnvKernelParams &P, float *smem_raw)
+template <bool OPT, bool AOS>
+__device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
     // a successor launched with programmatic stream serialization (the policy's first GEMM) may be scheduled
     // onto SMs as this grid drains; it waits for this grid's completion before it reads anything
@@ -554,7 +1013,7 @@ __device__ __forceinline__ void env_step_body(const EnvKernelParams &P, float *s
 
     // ---- pass A: reference at the advanced time, errors against the simulated state,
     //      observation entries of the simulated bodies
-    if (!RESET_ALL) {
+    {
         clip = P.clip_id[envc];
         if (clip < 0 || clip >= P.C) {
             clip = min(max(clip, 0), P.C - 1);
@@ -648,103 +1107,31 @@ __device__ __forceinline__ void env_step_body(const EnvKernelParams &P, float *s
     //      flags and the new per-env state.  Every other thread of the env needs the flags as well: it repeats the
     //      reward only if the reward can terminate an episode (r_min above -inf), else the root height and the
     //      clip end decide alone.  The reset draw is a function of (env, step) and is repeated by every thread.
-    int flags = 0;
-    float t_cur = t1;
-    int clip_cur = clip;
-    float reward_val = 0.0f;
-    if (!RESET_ALL) {
-        float r = 0.0f;
-        const bool need_r = c == 0 || P.reward.r_min > -INFINITY;
-        if (need_r) {
-            float e[kPartials];
-#pragma unroll
-            for (int i = 0; i < kPartials; ++i) {
-                float a = 0.0f;
-                for (int cc = 0; cc < C; ++cc) a += part[(i * C + cc) * kTile + lane];
-                e[i] = a;
-            }
-            // term order of the configuration: pose, vel, ee_pos, ee_rot, com, body_pos, body_vel
-            const float term[IM_N_TERMS] = {e[0], e[1], e[2], e[3], e[6] * e[6] + e[7] * e[7] + e[8] * e[8], e[4], e[5]};
-            if (P.reward.mode == 0) {
-                float sum = 0.0f;
-#pragma unroll
-                for (int k = 0; k < IM_N_TERMS; ++k) sum += P.reward.w[k] * term[k];
-                r = expf(-sum);
-            } else {
-#pragma unroll
-                for (int k = 0; k < IM_N_TERMS; ++k) r += P.reward.a[k] * expf(-P.reward.w[k] * term[k]);
-            }
-            if (c == 0 && valid) {
+    EnvState E;
+    E.clip = clip; E.cyc = cyc; E.t = t1; E.cm = cm; E.loop = loop;
+    {
+        float term[IM_N_TERMS], r = INFINITY;
+        if (c == 0 || P.reward.r_min > -INFINITY) r = reward_of(P, part, C, lane, term);
+        decide<false, OPT>(P, envc, root_z, r, c == 0 && valid, E);
+        if (c == 0) {
+            int ep_done = 0;                    // steps of the episode this step ended (0 where none ended)
+            if (valid) {
                 P.reward_out[env] = r;
                 if (P.terms_out) {
 #pragma unroll
                     for (int k = 0; k < IM_N_TERMS; ++k) P.terms_out[(size_t)k * P.N + env] = term[k];
                 }
+                P.flags_out[env] = (uint8_t)E.flags;
+                ep_done = store_env_state<OPT>(P, env, E);
             }
-        }
-        bool terminated = (root_z < P.reward.h_min) || (r < P.reward.r_min);
-        if (OPT && P.ep_len[envc] < P.grace_steps) terminated = false;
-        if (OPT && P.n_bins > 0 && terminated && c == 0 && valid) {
-            // adaptive initialisation statistics: the (clip, phase bin) the episode failed in
-            const float span = fmaxf(__fsub_rn(cm.dur, P.dt), 0.0f);
-            atomicAdd(P.stat_failures + clip * P.n_bins + phase_bin(t1, span, P.n_bins), 1u);
-        }
-        const bool truncated = !(OPT && loop.on) && __fadd_rn(t1, P.dt) > cm.dur;    // a looped clip has no end
-        flags = (terminated ? 1 : 0) | (truncated ? 2 : 0);
-        reward_val = r;
-        if (c == 0 && valid) P.flags_out[env] = (uint8_t)flags;
-    }
-    const bool reset = RESET_ALL || flags != 0;
-    if (reset) {
-        const uint4 x = philox4x32_10(make_uint4(P.env_id_base + (uint32_t)envc, P.step, IM_STREAM_RESET, 0u),
-                                      make_uint2(P.seed_lo, P.seed_hi));
-        const float u = (float)(x.y >> 8) * 5.9604644775390625e-08f;
-        if (OPT && P.n_bins > 0) {
-            // weighted (clip, phase bin) from the cumulative table: smallest i with x < T_i
-            const int B = P.n_bins;
-            int lo = 0, hi = P.C * B - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if ((unsigned long long)x.x < __ldg(P.reset_cdf + mid)) hi = mid;
-                else lo = mid + 1;
-            }
-            clip_cur = lo / B;
-            const float span = fmaxf(__fsub_rn(P.meta[clip_cur].dur, P.dt), 0.0f);
-            const float width = __fdiv_rn(span, (float)B);
-            t_cur = fminf(__fmul_rn(__fadd_rn((float)(lo - clip_cur * B), u), width), span);
-            if (c == 0 && valid) atomicAdd(P.stat_starts + lo, 1u);
-        } else {
-            clip_cur = (int)__umulhi(x.x, (uint32_t)P.C);
-            const float span = fmaxf(__fsub_rn(P.meta[clip_cur].dur, P.dt), 0.0f);
-            t_cur = __fmul_rn(u, span);
+            if (OPT && P.summary) add_summary(P, valid, r, E.flags, ep_done, lane);
         }
     }
+    const bool reset = E.reset;
+    const float t_cur = E.t_new;
+    const ClipMeta cmc = E.cm_new;
     if (reset) cyc = 0;
-    if (c == 0) {
-        int ep_done = 0;                    // steps of the episode this step ended (0 where none ended)
-        if (valid) {
-            const int len_now = P.ep_len[env] + 1;
-            P.clip_id[env] = clip_cur;
-            P.t[env] = t_cur;
-            if (OPT && P.loops) P.cycle[env] = cyc;
-            P.ep_len[env] = reset ? 0 : len_now;
-            ep_done = reset ? len_now : 0;
-        }
-        if (OPT && !RESET_ALL && P.summary) {
-            // training summaries: integer sums over the tile (one warp), then one atomic per quantity
-            unsigned long long v[4] = {valid ? (unsigned long long)__float2ll_rn(reward_val * 1099511627776.0f) : 0ull,
-                                       (unsigned long long)(valid ? (flags & 1) : 0), (unsigned long long)(valid ? (flags >> 1) & 1 : 0),
-                                       (unsigned long long)ep_done};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-                if (lane == 0 && v[i]) atomicAdd(P.summary + i, v[i]);
-            }
-        }
-    }
-    const ClipMeta cmc = reset ? P.meta[clip_cur] : cm;
-    if (OPT && P.loops && reset) loop = P.loops[clip_cur];
+    loop = E.loop;
 
     // ---- pass C (only where an env of this warp was reset): reference state at the new phase
     //      replaces the simulated one in the observation, and optionally in the caller's arrays
@@ -780,7 +1167,7 @@ __device__ __forceinline__ void env_step_body(const EnvKernelParams &P, float *s
             if (k == 0) Hn = make_heading(s.q, s.p);
             if ((Lc.flags & LINK_OWN) && reset) {
                 body_obs(Hn, s.q, s.p, s.v, s.w, row1, b);
-                if (!RESET_ALL && P.write_back && valid) {
+                if (P.write_back && valid) {
                     sv.st_body(b, s.q, s.p, s.v, s.w);
                 }
             }
@@ -909,42 +1296,77 @@ __global__ void debug_math_kernel(int op, int n, const float *__restrict__ in, f
     }
 }
 
-// Two instantiations per mode: skeletons with at most 8 leaves (blocks of up to 256 threads) get a
-// register budget that lets four blocks share an SM; wider trees fall back to 64 registers.
-#ifndef IM_ENV_MAXNREG
-#define IM_ENV_MAXNREG 96
-#endif
-template <bool RESET_ALL, bool OPT, bool AOS>
-__global__ void __maxnreg__(IM_ENV_MAXNREG) env_step_kernel_small(const __grid_constant__ EnvKernelParams P)
+// Registers: the chain kernel has 96, so that four CTAs of five chains share an SM (64 for trees with more than eight
+// leaves, whose CTAs have up to 1024 threads); the role kernel 168 where every CTA has an SM of its own, else 96 (two).
+template <bool OPT, bool AOS>
+__global__ void __maxnreg__(96) env_chain_kernel(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_step_body<RESET_ALL, OPT, AOS>(P, smem_raw);
+    env_chain_body<OPT, AOS>(P, smem_raw);
 }
-
-template <bool RESET_ALL, bool OPT, bool AOS>
-__global__ void __launch_bounds__(1024, 1) env_step_kernel_wide(const __grid_constant__ EnvKernelParams P)
+template <bool OPT, bool AOS>
+__global__ void __launch_bounds__(1024, 1) env_chain_kernel_wide(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_step_body<RESET_ALL, OPT, AOS>(P, smem_raw);
+    env_chain_body<OPT, AOS>(P, smem_raw);
+}
+template <bool RESET_ALL, bool OPT, bool AOS>
+__global__ void __maxnreg__(168) env_role_kernel_1(const __grid_constant__ EnvKernelParams P)
+{
+    extern __shared__ __align__(16) float smem_raw[];
+    env_role_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
+}
+template <bool RESET_ALL, bool OPT, bool AOS>
+__global__ void __maxnreg__(96) env_role_kernel_2(const __grid_constant__ EnvKernelParams P)
+{
+    extern __shared__ __align__(16) float smem_raw[];
+    env_role_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
+}
+template <bool RESET_ALL, bool OPT, bool AOS>
+__global__ void __launch_bounds__(1024, 1) env_role_kernel_wide(const __grid_constant__ EnvKernelParams P)
+{
+    extern __shared__ __align__(16) float smem_raw[];
+    env_role_body<RESET_ALL, OPT, AOS, true>(P, smem_raw);
 }
 
-template <bool RESET_ALL, bool OPT, bool AOS>
-cudaError_t prepare_one(size_t smem)
+template <typename K>
+cudaError_t allow_smem(K kernel)
 {
-    const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(env_step_kernel_small<RESET_ALL, OPT, AOS>, attr, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(env_step_kernel_wide<RESET_ALL, OPT, AOS>, attr, (int)smem);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmemFloats * sizeof(float)));
+}
+template <bool RESET_ALL, bool OPT, bool AOS>
+cudaError_t prepare_one()
+{
+    cudaError_t e = allow_smem(env_role_kernel_1<RESET_ALL, OPT, AOS>);
+    if (e == cudaSuccess) e = allow_smem(env_role_kernel_2<RESET_ALL, OPT, AOS>);
+    if (e == cudaSuccess) e = allow_smem(env_role_kernel_wide<RESET_ALL, OPT, AOS>);
+    if (e == cudaSuccess && !RESET_ALL) e = allow_smem(env_chain_kernel<OPT, AOS>);
+    if (e == cudaSuccess && !RESET_ALL) e = allow_smem(env_chain_kernel_wide<OPT, AOS>);
     return e;
 }
 
+// (The kernels with options start plainly: started early their CTAs, several to an SM, crowd onto the SMs that drain
+// first; 9001 envs x 24 bodies 392 us per four steps plain, 408 early.  Without options 4096 envs x 8 steps 342 against 361.)
 template <bool RESET_ALL, bool OPT, bool AOS>
-void launch_one(const EnvKernelParams &p, dim3 grid, dim3 block, size_t smem, cudaStream_t stream)
+void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream)
 {
-    // (the kernels with options start plainly: started early their CTAs, three to an SM, crowd onto the SMs that drain
-    // first; 9001 envs x 24 bodies 392 us per four steps plain, 408 early.  Without options 4096 envs x 8 steps 342 against 361.)
-    const auto kernel = block.x <= 256 ? env_step_kernel_small<RESET_ALL, OPT, AOS> : env_step_kernel_wide<RESET_ALL, OPT, AOS>;
-    if (OPT) kernel<<<grid, block, smem, stream>>>(p);
-    else launch_pdl(kernel, grid, block, smem, stream, 0, p);
+    const int C = p.sk.n_chains, n_sm = device_sm_count();
+    const unsigned tiles = (unsigned)((p.N + kTile - 1) / kTile);
+    const int extra = (p.n_future - 1) * 9 * __builtin_popcount(p.sk.ee_mask) + p.act_dim;
+    const size_t role_smem = role_smem_floats(staged_cols(p.sk.J, C, p.sk.n_links, extra), C, p.sk.n_links) * sizeof(float);
+    const int role_per_sm = C <= 8 && role_smem <= 112 * 1024 && C * 64 * 96 * 2 <= 65536 ? 2 : 1;
+    void (*kernel)(EnvKernelParams);
+    if (RESET_ALL || tiles <= (unsigned)(role_per_sm * n_sm)) {
+        kernel = C > 8 ? env_role_kernel_wide<RESET_ALL, OPT, AOS>
+                 : tiles <= (unsigned)n_sm && C * 64 * 168 <= 65536 ? env_role_kernel_1<RESET_ALL, OPT, AOS> : env_role_kernel_2<RESET_ALL, OPT, AOS>;
+        const dim3 block(32 * (C <= 16 ? 2 * C : 32));
+        if (OPT) kernel<<<tiles, block, role_smem, stream>>>(p);
+        else launch_pdl(kernel, dim3(tiles), block, role_smem, stream, 0, p);
+    } else if constexpr (!RESET_ALL) {
+        kernel = C > 8 ? env_chain_kernel_wide<OPT, AOS> : env_chain_kernel<OPT, AOS>;
+        if (OPT) kernel<<<tiles, 32 * C, chain_smem, stream>>>(p);
+        else launch_pdl(kernel, dim3(tiles), dim3(32 * C), chain_smem, stream, 0, p);
+    }
 }
 
 }  // namespace
@@ -954,16 +1376,16 @@ size_t env_kernel_smem_bytes(int J, int n_chains, int n_links, int extra_cols)
     return smem_floats(J, n_chains, n_links, extra_cols) * sizeof(float);
 }
 
-cudaError_t env_kernel_prepare(size_t smem)
+cudaError_t env_kernel_prepare()
 {
     static DeviceOnce once;
-    return once.run([&] {
-        cudaError_t e = prepare_one<false, false, false>(smem);
-        if (e == cudaSuccess) e = prepare_one<true, false, false>(smem);
-        if (e == cudaSuccess) e = prepare_one<false, true, false>(smem);
-        if (e == cudaSuccess) e = prepare_one<true, true, false>(smem);
-        if (e == cudaSuccess) e = prepare_one<false, false, true>(smem);
-        if (e == cudaSuccess) e = prepare_one<false, true, true>(smem);
+    return once.run([] {
+        cudaError_t e = prepare_one<false, false, false>();
+        if (e == cudaSuccess) e = prepare_one<true, false, false>();
+        if (e == cudaSuccess) e = prepare_one<false, true, false>();
+        if (e == cudaSuccess) e = prepare_one<true, true, false>();
+        if (e == cudaSuccess) e = prepare_one<false, false, true>();
+        if (e == cudaSuccess) e = prepare_one<false, true, true>();
         return e;
     });
 }
@@ -984,20 +1406,24 @@ cudaError_t launch_debug_math(int op, int n, const float *in, float *out, cudaSt
     return cudaGetLastError();
 }
 
+// Which kernel: the role kernel while its tiles fit the SMs at once, the chain kernel beyond (us per launch in a chain of
+// them, 15 bodies / 24 bodies, role against chain: 64 envs 7.8 / 12.4 against 15.0 / 22.5; 4096 envs 9.7 / 14.1 against
+// 17.6 / 23.6; 9472 envs, two CTAs per SM, 14.2 / 20.9 against 19.4 / 26.2; 12000 envs 24.2 / 34.9 against 23.5 / 32.0;
+// 65536 envs 89.5 / 142 against 88 / 125).  A reset of all envs has no simulated state to load twice: always the role
+// kernel (65536 envs x 24 bodies 77 against 85 us).
 cudaError_t launch_env_kernel(const EnvKernelParams &p, bool reset_all, size_t smem, cudaStream_t stream)
 {
-    const dim3 grid((p.N + kTile - 1) / kTile), block(32 * p.sk.n_chains);
     const bool opt = p.grace_steps > 0 || p.reset_noise_std > 0.0f || p.n_bins > 0 || p.n_future > 1 || p.act_dim > 0 ||
                      p.summary != nullptr || p.loops != nullptr;
     if (p.aos && !reset_all) {               // simulator records read in place (the reset-all launch reads no body states)
-        if (opt) launch_one<false, true, true>(p, grid, block, smem, stream);
-        else launch_one<false, false, true>(p, grid, block, smem, stream);
+        if (opt) launch_one<false, true, true>(p, smem, stream);
+        else launch_one<false, false, true>(p, smem, stream);
     } else if (opt) {
-        if (reset_all) launch_one<true, true, false>(p, grid, block, smem, stream);
-        else launch_one<false, true, false>(p, grid, block, smem, stream);
+        if (reset_all) launch_one<true, true, false>(p, smem, stream);
+        else launch_one<false, true, false>(p, smem, stream);
     } else {
-        if (reset_all) launch_one<true, false, false>(p, grid, block, smem, stream);
-        else launch_one<false, false, false>(p, grid, block, smem, stream);
+        if (reset_all) launch_one<true, false, false>(p, smem, stream);
+        else launch_one<false, false, false>(p, smem, stream);
     }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError();

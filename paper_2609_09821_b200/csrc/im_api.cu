@@ -244,8 +244,7 @@ im_status im_env_create(const im_skeleton *skel, const im_clips *clips, const im
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if ((int)e->smem_bytes > max_smem) { delete e; return IM_ERR_UNSUPPORTED; }
-    // opt in to the device maximum once: environments of different sizes share the kernels
-    if (env_kernel_prepare((size_t)max_smem) != cudaSuccess) { delete e; return IM_ERR_CUDA; }
+    if (env_kernel_prepare() != cudaSuccess) { delete e; return IM_ERR_CUDA; }
     const size_t n = (size_t)cfg->n_envs;
     if (cudaMalloc(&e->d_clip_id, n * 4) != cudaSuccess || cudaMalloc(&e->d_t, n * 4) != cudaSuccess ||
         cudaMalloc(&e->d_ep_len, n * 4) != cudaSuccess || cudaMalloc(&e->d_status, 4) != cudaSuccess ||

@@ -196,7 +196,7 @@ size_t env_kernel_smem_bytes(int J, int n_chains, int n_links, int extra_cols);
 cudaError_t launch_clip_table(const float *root_pos, const float *local_quat, const uint8_t *last, int64_t rows, int J,
                               float4 *frames, cudaStream_t stream);
 inline int clip_row_stride(int J) { return 2 + 2 * J; }
-cudaError_t env_kernel_prepare(size_t smem);
+cudaError_t env_kernel_prepare();
 cudaError_t launch_env_kernel(const EnvKernelParams &p, bool reset_all, size_t smem, cudaStream_t stream);
 cudaError_t launch_debug_math(int op, int n, const float *in, float *out, cudaStream_t stream);
 // simulator-native (array of structures) body states <-> component rows [13 J][stride]

@@ -1,0 +1,95 @@
+"""The env step has two kernels, chosen by the number of 32-env tiles.  A batch large enough for the chain kernel must
+equal the same envs run in shards small enough for the role kernel (env_id_base), which the oracle tests cover: flags
+and per-env state bit for bit, floats within the oracle's tolerance.  Options, records, wide trees, reward termination,
+an extended observation too wide to stage."""
+import numpy as np
+import pytest
+
+from paper_2609_09821_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+N = 9728            # 304 tiles: more than two per SM; shards of 4864 envs have one or two
+
+
+def _tree(leaves):
+    """Root with `leaves` two-body branches."""
+    parents = [-1] + [0] * leaves + list(range(1, leaves + 1))
+    g = np.random.default_rng(leaves)
+    return dict(parents=np.asarray(parents, np.int32), offsets=g.uniform(-0.3, 0.3, (len(parents), 3)).astype(np.float32),
+                masses=None, J=len(parents))
+
+
+CASES = {
+    "plain": dict(),
+    "reward": dict(reward=W.REWARD_FIG5, r_min=0.3, write_back=True),
+    "aos": dict(aos=True, write_back=True, h_min=0.8),
+    "options": dict(options=True, r_min=0.1, reward=W.REWARD_ADD4),
+    "aos_options": dict(options=True, aos=True, h_min=0.8),
+    "wide_extension": dict(options=True, n_future=8, act_dim=900),
+    "many_leaves": dict(leaves=12, options=True, h_min=0.8),
+    "too_many_leaves_for_a_warp_each": dict(leaves=15, h_min=0.8),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+@pytest.mark.parametrize("skeleton", ["humanoid15", "smpl24"])
+def test_large_batch_equals_its_shards(name, skeleton):
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    c = CASES[name]
+    if c.get("leaves") and skeleton == "smpl24":
+        pytest.skip("the tree is the case's own")
+    skel = _tree(c["leaves"]) if c.get("leaves") else W.make_skeleton(skeleton, 1)
+    J = skel["J"]
+    lib = W.make_clip_library(J, 4, (20, 40), 30.0, 1)
+    sk = B.Skeleton(skel["parents"], skel["offsets"], skel["masses"])
+    clips = B.Clips(sk, lib["n_frames"], lib["fps"], lib["root_pos"], lib["local_quat"])
+    options = c.get("options", False)
+    if options:
+        clips.set_cyclic([1, 0, 0, 1])
+    n_future, act_dim = c.get("n_future", 2), c.get("act_dim", 7)
+    extra = (n_future - 1) * 9 * sk.n_ee + act_dim if options else 0
+    g = torch.Generator("cuda").manual_seed(3)
+    sim = torch.randn(13 * J, N, device="cuda", generator=g) * 0.3
+    sim[2] += 0.9
+    prev = torch.randn(N, act_dim, device="cuda", generator=g)
+
+    def run(base, n):
+        cfg = B.make_env_config(n, 1 / 30, 5, c.get("reward", W.REWARD_MULT), c.get("h_min", 0.3), B.padded_ld(24 * J + 1 + extra),
+                                r_min=c.get("r_min", -np.inf), env_id_base=base, write_back_reset=c.get("write_back", False),
+                                **(dict(grace_steps=2, reset_noise_std=0.05) if options else {}))
+        env = B.Env(sk, clips, cfg)
+        acc = torch.zeros(4, dtype=torch.int64, device="cuda")
+        if options:
+            env.set_obs_extension(n_future, prev[base:base + n])
+            env.set_reset_bins(3, np.arange(12, dtype=np.float32).reshape(4, 3))
+            env.set_summary(acc)
+        obs, rew, fl, terms = env.new_obs(), torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda"), torch.empty(7, n, device="cuda")
+        env.reset_all(obs, 0)
+        out = [obs.clone()]
+        mine = sim[:, base:base + n].clone()
+        for s in range(1, 4):
+            if c.get("aos"):
+                rec = [mine[a * J:b * J].view(J, b - a, n).permute(2, 0, 1).contiguous() for a, b in ((0, 3), (3, 7), (7, 10), (10, 13))]
+                env.step_aos(s, *rec, obs, rew, fl, terms)
+                mine = torch.cat([r.permute(1, 2, 0).reshape(-1, n) for r in rec])
+            else:
+                env.step(s, mine, obs, rew, fl, terms)
+            out += [obs.clone(), rew.clone(), fl.clone(), terms.T.clone(), mine.T.clone()]
+        out += list(env.get_state()) + [env.get_cycles()]
+        assert env.device_status() == 0
+        return out, acc
+
+    whole, acc = run(0, N)
+    (a, acc_a), (b, acc_b) = run(0, N // 2), run(N // 2, N // 2)
+    assert bool((whole[3] != 0).any())
+    for x, p, q in zip(whole, a, b):
+        y = torch.cat([p, q])
+        if x.dtype == torch.float32 and x.dim() == 2 or x.dtype == torch.float32 and x is not whole[-3]:
+            # one fp32 program compiled twice: at most the oracle tests' 1e-5 + 1e-4 |x| apart
+            assert bool(((x - y).abs() <= 1e-5 + 1e-4 * y.abs()).all())
+        else:
+            assert torch.equal(x, y)
+    if options:
+        d = acc - acc_a - acc_b
+        assert bool((d[1:] == 0).all()) and abs(int(d[0])) <= 3 * N * 1e-5 * 2 ** 40
