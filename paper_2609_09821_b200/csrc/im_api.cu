@@ -1,5 +1,6 @@
 // C-ABI entry points: validation, uploads, handle management, kernel launches.
 #include <cmath>
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -743,6 +744,19 @@ static im_status ensure_staging(im_env *e, int A)
     return IM_OK;
 }
 
+// The device address of `bytes` of pinned host memory, or null where the memory is not pinned (asked anew on each call).
+static void *device_view(void *host, size_t bytes)
+{
+    cudaPointerAttributes a, z;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&z, static_cast<char *>(host) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const bool pinned = a.type == cudaMemoryTypeHost && z.type == cudaMemoryTypeHost && a.devicePointer &&
+                        static_cast<char *>(z.devicePointer) - static_cast<char *>(a.devicePointer) == (ptrdiff_t)(bytes - 1);
+    return pinned ? a.devicePointer : nullptr;
+}
+
 im_status im_env_reset_all_host(im_env *e, uint32_t step)
 {
     if (!e) return IM_ERR_INVALID_ARG;
@@ -772,8 +786,11 @@ im_status im_step_host(im_env *e, im_policy *p, uint32_t step, const float *sim_
     const int chunks = (n >= 49152 && n % (4 * 32) == 0) ? kHostChunks : 1;
     const size_t nc = n / chunks;
     for (int c = 0; c < chunks; ++c) {
-        IM_CUDA(cudaMemcpy2DAsync(e->d_sim + c * nc, n * 4, sim_host + c * nc, n * 4, nc * 4, 13 * J, cudaMemcpyHostToDevice,
-                                  e->h2d_stream));
+        // One range is one contiguous copy: as 13 J rows of 4 KB the step takes 15 us longer at 1000 envs x 15 bodies (at 4096
+        // envs the two are alike).  A few KB of pageable memory go faster by rows (64 envs: 82 us a step against 89-107).
+        if (chunks == 1 && (13 * J * n * 4 >= 65536 || device_view(const_cast<float *>(sim_host), 13 * J * n * 4))) IM_CUDA(cudaMemcpyAsync(e->d_sim, sim_host, 13 * J * n * 4, cudaMemcpyHostToDevice, e->h2d_stream));
+        else IM_CUDA(cudaMemcpy2DAsync(e->d_sim + c * nc, n * 4, sim_host + c * nc, n * 4, nc * 4, 13 * J, cudaMemcpyHostToDevice,
+                                       e->h2d_stream));
         IM_CUDA(cudaEventRecord(e->ev_h2d[c], e->h2d_stream));
     }
     int32_t ld_in = 0;
@@ -786,13 +803,18 @@ im_status im_step_host(im_env *e, im_policy *p, uint32_t step, const float *sim_
     IM_CUDA(cudaStreamWaitEvent(e->d2h_stream, e->ev_policy, 0));
     IM_CUDA(cudaMemcpyAsync(action_host, e->d_action, n * (size_t)A * 4, cudaMemcpyDeviceToHost, e->d2h_stream));
     im_body_state sim = {e->d_sim, e->d_sim + 3 * J * n, e->d_sim + 7 * J * n, e->d_sim + 10 * J * n, (int64_t)n};
+    // Five bytes per env: where the caller's arrays are pinned the env kernel writes them there itself, which saves two
+    // copies after the kernel (a step of 64 envs 55 -> 48 us, of 1000 envs 82 -> 73, of 4096 envs 106 -> 95)
+    float *reward_direct = static_cast<float *>(device_view(reward_host, n * 4));
+    uint8_t *flags_direct = static_cast<uint8_t *>(device_view(flags_host, n));
     for (int c = 0; c < chunks; ++c) {
         IM_CUDA(cudaStreamWaitEvent(e->stream, e->ev_h2d[c], 0));
-        s = env_step_range(e, step, &sim, e->d_obs, e->d_reward, e->d_flags, (int)(c * nc), (int)nc);
+        s = env_step_range(e, step, &sim, e->d_obs, reward_direct ? reward_direct : e->d_reward, flags_direct ? flags_direct : e->d_flags,
+                           (int)(c * nc), (int)nc);
         if (s != IM_OK) return s;
     }
-    IM_CUDA(cudaMemcpyAsync(reward_host, e->d_reward, n * 4, cudaMemcpyDeviceToHost, e->stream));
-    IM_CUDA(cudaMemcpyAsync(flags_host, e->d_flags, n, cudaMemcpyDeviceToHost, e->stream));
+    if (!reward_direct) IM_CUDA(cudaMemcpyAsync(reward_host, e->d_reward, n * 4, cudaMemcpyDeviceToHost, e->stream));
+    if (!flags_direct) IM_CUDA(cudaMemcpyAsync(flags_host, e->d_flags, n, cudaMemcpyDeviceToHost, e->stream));
     IM_CUDA(cudaStreamSynchronize(e->stream));
     IM_CUDA(cudaStreamSynchronize(e->d2h_stream));
     return IM_OK;
