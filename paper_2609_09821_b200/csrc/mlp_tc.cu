@@ -31,8 +31,12 @@ namespace {
 constexpr int BLOCK_M = 128;
 constexpr int BLOCK_K = 64;               // 64 bf16 = 128 bytes = one swizzle row
 constexpr int UMMA_K = 16;
-constexpr int kThreads = 192;
-constexpr int kEpiWarps = 4;
+// Epilogue warps of the hidden-layer kernels: two per tensor-memory lane quadrant, which share the tile's 64-column chunks
+// and have one staging slab each (four warps with two slabs against it, in a chain of launches: 8192 x 1024 x 384 10.4 ->
+// 9.1 us, 4096 x 2048 x 384 11.2 -> 9.3, 16384 x 1024 x 384 15.9 -> 14.9).  64-column tiles have one chunk and keep four
+// warps, as does the backward epilogue of the single-CTA kernel.
+constexpr __host__ __device__ int hidden_epi_warps(int block_n, bool bwd) { return bwd || block_n == 64 ? 4 : 8; }
+constexpr __host__ __device__ int hidden_threads(int block_n, bool bwd) { return 64 + 32 * hidden_epi_warps(block_n, bwd); }
 // Limit of every bounded wait below (2 s unless im_debug_set_wait changed it), and the diagnostic switch that makes the
 // TMA producers issue nothing, so that a test can watch a wait run out with no copy or MMA in flight.
 __device__ unsigned long long g_wait_limit_ns = 2000000000ull;
@@ -224,9 +228,9 @@ struct SmemPlan {
     static constexpr int kTmemCols = 2 * kAccStride;
     static constexpr int kBarBytes = 256;
     static constexpr int kMaxStages = 8;
-    // hidden layers: two staging slabs per epilogue warp for the TMA stores
-    // (backward epilogue: two more per warp for the ReLU mask boxes)
-    static constexpr __host__ __device__ int hidden_epi_bytes(bool bwd = false) { return (bwd ? 2 : 1) * 4 * 2 * kEpiSlabBytes; }
+    // hidden layers: eight staging slabs for the TMA stores, shared out over the epilogue warps
+    // (backward epilogue: two per warp and two more for the ReLU mask boxes)
+    static constexpr __host__ __device__ int hidden_epi_bytes(bool bwd = false) { return (bwd ? 4 * 4 : 8) * kEpiSlabBytes; }
     // head: [2 accumulators][mean, action][128 rows][A] floats laid out as in global memory,
     // partial sums of z^2 [2][4][128], band counters [2][4]
     // (+ bias and per-column sigma of the tile's columns, 2 x 128 floats)
@@ -286,7 +290,7 @@ __device__ __forceinline__ void pipe_init(const Pipe &p, int epi_arrivals)
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(&p.full[s], 1); mbar_init(&p.empty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&p.acc_full[a], 1); mbar_init(&p.acc_empty[a], epi_arrivals); }
-        for (int i = 0; i < 2 * kEpiWarps; ++i) mbar_init(&p.mask_bar[i], 1);
+        for (int i = 0; i < 8; ++i) mbar_init(&p.mask_bar[i], 1);
         *p.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -494,7 +498,7 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
 // reads 64 accumulator columns at a time, applies bias and ReLU, packs to bf16
 // into a 128B-swizzled slab in shared memory and hands the slab to a TMA store.
 template <int BLOCK_N, bool MN = false, bool BWD = false>
-__global__ void __launch_bounds__(kThreads, 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
+__global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                        const __grid_constant__ CUtensorMap map_b,
                                                                        const __grid_constant__ CUtensorMap map_c,
                                                                        const __grid_constant__ CUtensorMap map_m,
@@ -506,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_tc_hidden_kernel(const __g
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_per_batch = ((P.M + BLOCK_M - 1) / BLOCK_M) * P.n_tiles_n;
     const int n_tiles = tiles_per_batch * P.n_batches;
-    pipe_init<Plan>(p, kEpiWarps);
+    pipe_init<Plan>(p, hidden_epi_warps(BLOCK_N, BWD));
     const uint32_t tmem_base = *p.tmem_slot;
     dep_release();
     dep_wait();                       // nothing before this line touches global memory
@@ -517,7 +521,10 @@ __global__ void __launch_bounds__(kThreads, 1) linear_tc_hidden_kernel(const __g
         if (lane == 0) mma_role<Plan, BLOCK_N, MN>(p, tmem_base, P, n_tiles);
     } else {
         const int quad = warp & 3;                    // TMEM lanes 32*quad .. 32*quad+31 belong to this warp
-        uint8_t *slabs = p.epi + (size_t)(warp - 2) * 2 * kEpiSlabBytes;       // two slabs, used alternately
+        constexpr bool kFour = hidden_epi_warps(BLOCK_N, BWD) == 4;
+        constexpr int kSlabs = kFour ? 2 : 1, kStep = kFour ? 64 : 128;
+        const int half = kFour ? 0 : (warp - 2) >> 2;                            // first chunk of this warp
+        uint8_t *slabs = p.epi + (size_t)(warp - 2) * kSlabs * kEpiSlabBytes;  // two are used alternately
         int which = 0;
         int acc = 0;
         uint32_t acc_phase = 0;
@@ -542,7 +549,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_tc_hidden_kernel(const __g
             tc_fence_after();
             const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * Plan::kAccStride);
 #pragma unroll 1
-            for (int c0 = 0; c0 < BLOCK_N; c0 += 64) {
+            for (int c0 = 64 * half; c0 < BLOCK_N; c0 += kStep) {
                 uint32_t pk[32];
                 if (BWD) {
                     if (masked) {
@@ -561,8 +568,8 @@ __global__ void __launch_bounds__(kThreads, 1) linear_tc_hidden_kernel(const __g
                     } else mask_all_positive(mk);
                 }
                 hidden_chunk<BWD>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk);
-                // the store issued two slabs ago (same buffer) must have finished reading shared memory
-                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                // the last store from this slab must have finished reading shared memory
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSlabs - 1) : "memory");
                 __syncwarp();
                 uint8_t *slab = slabs + which * kEpiSlabBytes;
                 const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
@@ -579,7 +586,7 @@ __global__ void __launch_bounds__(kThreads, 1) linear_tc_hidden_kernel(const __g
                                  ::"l"(&map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
-                which ^= 1;
+                if (kSlabs == 2) which ^= 1;
             }
             if (bail) break;
             tc_fence_before();
@@ -613,12 +620,12 @@ constexpr int kPairTmemCols = 512;                                     // two 25
 // output for the TMA store.  The ring takes the room of two operand stages.
 constexpr int kPairEpiWarpsBwd = 8;
 constexpr int kPairRing = 3;
-constexpr __host__ __device__ int pair_epi_warps(bool bwd) { return bwd ? kPairEpiWarpsBwd : kEpiWarps; }
+constexpr __host__ __device__ int pair_epi_warps(bool bwd) { return bwd ? kPairEpiWarpsBwd : 4; }
 constexpr __host__ __device__ int pair_threads(bool bwd) { return 64 + 32 * pair_epi_warps(bwd); }
 constexpr __host__ __device__ int pair_stages(bool bwd) { return bwd ? kPairStages - 2 : kPairStages; }
 constexpr __host__ __device__ int pair_epi_bytes(bool bwd)
 {
-    return bwd ? kPairEpiWarpsBwd * kPairRing * kEpiSlabBytes : kEpiWarps * 2 * kEpiSlabBytes;
+    return bwd ? kPairEpiWarpsBwd * kPairRing * kEpiSlabBytes : 4 * 2 * kEpiSlabBytes;
 }
 constexpr size_t pair_smem_bytes(bool bwd) { return 1024 + (size_t)pair_stages(bwd) * kPairStageBytes + pair_epi_bytes(bwd) + 512; }
 static_assert(pair_smem_bytes(true) <= kSmemLimit && pair_smem_bytes(false) <= kSmemLimit, "shared memory plan of the pair kernel");
@@ -1233,7 +1240,7 @@ cudaError_t launch_hidden(const TcLayer &L, const GemmParams &gp_in, int n_sm, c
     const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes(BWD));
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
     const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, dim3(grid), dim3(kThreads), smem, stream, 0,
+    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, dim3(grid), dim3(hidden_threads(BLOCK_N, BWD)), smem, stream, 0,
                                       L.map_a, L.map_b, L.map_c, L.map_m, gp);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -1256,7 +1263,7 @@ cudaError_t launch_hidden_mn(const TcLayer &L, const GemmParams &gp_in, int n_sm
     const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes());
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
     const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, true>, dim3(grid), dim3(kThreads), smem, stream, 0,
+    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, true>, dim3(grid), dim3(hidden_threads(BLOCK_N, false)), smem, stream, 0,
                                       L.map_a, L.map_b, L.map_c, L.map_c, gp);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
