@@ -190,6 +190,7 @@ struct GemmParams {
     int K_blocks;      // K / 64 (K is padded with zeros)
     int n_tiles_n;     // N tiles of BLOCK_N
     int stages;        // depth of the operand ring in shared memory
+    int bufs;          // head: staging buffers
     const float *bias; // [n_tiles_n * BLOCK_N], zero padded
     float act_floor;   // hidden-layer epilogue: out = max(acc + bias, act_floor); 0 is ReLU, -inf no activation
     // Batched products on the single-CTA hidden kernel: batch b multiplies rows [b a_batch_rows, +M) of A
@@ -218,12 +219,18 @@ constexpr int kEpiSlabBytes = 32 * 128;    // one epilogue warp's 32 rows x 64 b
 
 constexpr size_t kSmemLimit = 232448;       // opt-in shared memory per block on this architecture (227 KB)
 
-template <int BLOCK_N>
+// KD: k-blocks per stage.  One trip of the producer and of the MMA issuer round the ring costs about 290 cycles besides the
+// MMAs (barrier waits, commit; measured without loads and with one MMA per trip), which narrow tiles do not cover with one
+// k-block (four 128 x 64 x 16 MMAs: 260 cycles).  Two per stage, in a chain of launches: 1024 x 512 x 1024 7.9 -> 6.8 us,
+// 1024 x 1024 x 384 5.1 -> 4.7; a forward of 361-1024-512-28 on 64 rows 17.7 -> 15.6, on 4096 rows 22.3 -> 20.7.
+template <int BLOCK_N, int KD = 1>
 struct SmemPlan {
-    static constexpr int kABytes = BLOCK_M * BLOCK_K * 2;
+    static constexpr int kDepth = KD;
+    static constexpr int kABytes = BLOCK_M * BLOCK_K * 2;                    // one k-block
     static constexpr int kBBytes = BLOCK_N * BLOCK_K * 2;
     static constexpr int kBBytesPadded = (kBBytes + 1023) / 1024 * 1024;     // keep every tile 1024-byte aligned
-    static constexpr int kStageBytes = kABytes + kBBytesPadded;
+    static constexpr int kStageBytes = KD * (kABytes + kBBytesPadded);      // KD blocks of A, then KD of W
+    static constexpr int kBOffset = KD * kABytes;
     static constexpr int kAccStride = BLOCK_N <= 128 ? 128 : 256;           // TMEM columns between the two accumulators
     static constexpr int kTmemCols = 2 * kAccStride;
     static constexpr int kBarBytes = 256;
@@ -234,9 +241,10 @@ struct SmemPlan {
     // head: [2 accumulators][mean, action][128 rows][A] floats laid out as in global memory,
     // partial sums of z^2 [2][4][128], band counters [2][4]
     // (+ bias and per-column sigma of the tile's columns, 2 x 128 floats)
-    __host__ __device__ static constexpr int head_epi_bytes(int A)
+    // (one buffer where no CTA has a second tile)
+    __host__ __device__ static constexpr int head_epi_bytes(int A, int bufs)
     {
-        return (2 * 2 * 128 * A * 4 + 2 * 4 * 128 * 4 + 64 + 2 * 128 * 4 + 1023) / 1024 * 1024;
+        return (bufs * 2 * 128 * A * 4 + 2 * 4 * 128 * 4 + 64 + 2 * 128 * 4 + 1023) / 1024 * 1024;
     }
     __host__ __device__ static constexpr int stages_for(int epi_bytes)
     {
@@ -350,12 +358,15 @@ __device__ __forceinline__ void producer_role(const Pipe &p, const CUtensorMap *
             continue;
         }
         const int m0 = b * P.a_batch_rows + (t / P.n_tiles_n) * BLOCK_M, n0 = b * P.b_batch_rows + (t % P.n_tiles_n) * BLOCK_N;
-        for (int kb = 0; kb < P.K_blocks; ++kb) {
+        for (int kb = 0; kb < P.K_blocks; kb += Plan::kDepth) {
             if (!mbar_wait(&p.empty[stage], phase ^ 1u, p.abort_flag)) return;
             uint8_t *sa = p.tiles + (size_t)stage * Plan::kStageBytes;
-            mbar_arrive_expect_tx(&p.full[stage], Plan::kABytes + Plan::kBBytes);
-            tma_load_2d(sa, map_a, &p.full[stage], kb * BLOCK_K, m0);
-            tma_load_2d(sa + Plan::kABytes, map_b, &p.full[stage], kb * BLOCK_K, n0);
+            mbar_arrive_expect_tx(&p.full[stage], Plan::kDepth * (Plan::kABytes + Plan::kBBytes));
+#pragma unroll
+            for (int d = 0; d < Plan::kDepth; ++d) {                // (a block past K arrives as zeros)
+                tma_load_2d(sa + d * Plan::kABytes, map_a, &p.full[stage], (kb + d) * BLOCK_K, m0);
+                tma_load_2d(sa + Plan::kBOffset + d * Plan::kBBytesPadded, map_b, &p.full[stage], (kb + d) * BLOCK_K, n0);
+            }
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
     }
@@ -374,7 +385,7 @@ __device__ __forceinline__ void mma_role(const Pipe &p, uint32_t tmem_base, cons
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * Plan::kAccStride);
         int kb0, n_kb;
         slice_k_blocks<MN>(P, MN ? tile / (n_tiles / P.n_batches) : 0, kb0, n_kb);
-        for (int kb = 0; kb < n_kb; ++kb) {
+        for (int kb = 0; kb < n_kb; kb += Plan::kDepth) {
             if (!mbar_wait(&p.full[stage], phase, p.abort_flag)) return;
             tc_fence_after();
             const uint32_t sa = smem_u32(p.tiles + (size_t)stage * Plan::kStageBytes);
@@ -386,11 +397,15 @@ __device__ __forceinline__ void mma_role(const Pipe &p, uint32_t tmem_base, cons
                     umma_bf16(d_tmem, da + (uint64_t)(128 * k), db + (uint64_t)(128 * k), idesc, (kb | k) != 0 ? 1u : 0u);
                 }
             } else {
-                const uint64_t da = smem_desc_k_major_sw128(sa), db = smem_desc_k_major_sw128(sa + Plan::kABytes);
 #pragma unroll
-                for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
-                    // advancing K by 16 bf16 = 32 bytes inside the swizzled row: +2 in 16-byte units
-                    umma_bf16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (kb | k) != 0 ? 1u : 0u);
+                for (int d = 0; d < Plan::kDepth; ++d) {
+                    const uint64_t da = smem_desc_k_major_sw128(sa + d * Plan::kABytes);
+                    const uint64_t db = smem_desc_k_major_sw128(sa + Plan::kBOffset + d * Plan::kBBytesPadded);
+#pragma unroll
+                    for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
+                        // advancing K by 16 bf16 = 32 bytes inside the swizzled row: +2 in 16-byte units
+                        umma_bf16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (kb | d | k) != 0 ? 1u : 0u);
+                    }
                 }
             }
             umma_commit(&p.empty[stage]);            // smem stage is free once these MMAs have read it
@@ -497,6 +512,8 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
 // C = relu(A W^T + b) as bf16.  Each epilogue warp owns 32 rows of the tile: it
 // reads 64 accumulator columns at a time, applies bias and ReLU, packs to bf16
 // into a 128B-swizzled slab in shared memory and hands the slab to a TMA store.
+constexpr __host__ __device__ int hidden_depth(int block_n, bool mn, bool bwd) { return block_n < 256 && !mn && !bwd ? 2 : 1; }
+
 template <int BLOCK_N, bool MN = false, bool BWD = false>
 __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                        const __grid_constant__ CUtensorMap map_b,
@@ -504,7 +521,7 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
                                                                        const __grid_constant__ CUtensorMap map_m,
                                                                        const GemmParams P)
 {
-    using Plan = SmemPlan<BLOCK_N>;
+    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, MN, BWD)>;
     extern __shared__ uint8_t smem_raw[];
     const Pipe p = carve_pipe<Plan>(smem_raw, P.stages, Plan::hidden_epi_bytes(BWD));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -945,6 +962,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
 // step (policy and env) of 4096 envs x 28 actions 46.6 -> 45.2 us, of 16384 envs 74.2 -> 73.1 us.
 constexpr int kHeadEpiWarps = 16;
 constexpr int kHeadThreads = 64 + 32 * kHeadEpiWarps;
+constexpr __host__ __device__ int head_depth(int block_n) { return block_n <= 32 ? 2 : 1; }      // (wider: too few stages beside the staging)
 
 // Standard normals of one row for the columns [c0, c0 + 16) and [c0 + 64, c0 + 80) below A.
 template <int CHUNKS>
@@ -972,17 +990,17 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
                                                                          const __grid_constant__ CUtensorMap map_b,
                                                                          const GemmParams P)
 {
-    using Plan = SmemPlan<BLOCK_N>;
+    using Plan = SmemPlan<BLOCK_N, head_depth(BLOCK_N)>;
     extern __shared__ uint8_t smem_raw[];
-    const int A = P.N;
-    const Pipe p = carve_pipe<Plan>(smem_raw, P.stages, Plan::head_epi_bytes(A));
+    const int A = P.N, bufs = P.bufs;
+    const Pipe p = carve_pipe<Plan>(smem_raw, P.stages, Plan::head_epi_bytes(A, bufs));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles = (P.M + BLOCK_M - 1) / BLOCK_M;             // one N tile holds the whole action row
     const int out_floats = 128 * A;
     // staging: per accumulator buffer the tile's mean and action rows laid out exactly as in global
     // memory ([128][A], dense), so a 32-row band leaves as one contiguous copy
-    float *out_tiles = reinterpret_cast<float *>(p.epi);                            // [2][2][128 * A]
-    float *zz_part = out_tiles + 2 * 2 * out_floats;                                // [2][4][128]
+    float *out_tiles = reinterpret_cast<float *>(p.epi);                            // [bufs][2][128 * A]
+    float *zz_part = out_tiles + bufs * 2 * out_floats;                                // [2][4][128]
     int *band_count = reinterpret_cast<int *>(zz_part + 2 * 4 * 128);               // [2][4]
     float *s_bias = reinterpret_cast<float *>(band_count + 16);                     // [128]: bias of the tile's columns
     float *s_sigma = s_bias + 128;                                                  // [128]: standard deviation per column
@@ -1228,7 +1246,7 @@ namespace {
 template <int BLOCK_N, bool BWD = false>
 cudaError_t launch_hidden(const TcLayer &L, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
 {
-    using Plan = SmemPlan<BLOCK_N>;
+    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, false, BWD)>;
     static DeviceOnce once;                      // the attribute is per device
     {
         const cudaError_t e = once.run([] { return cudaFuncSetAttribute(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1289,7 +1307,7 @@ cudaError_t launch_hidden_pair(const TcLayer &L, const GemmParams &gp, int n_sm,
 template <int BLOCK_N>
 cudaError_t launch_head(const TcLayer &L, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
 {
-    using Plan = SmemPlan<BLOCK_N>;
+    using Plan = SmemPlan<BLOCK_N, head_depth(BLOCK_N)>;
     static DeviceOnce once;                      // the attribute is per device
     {
         const cudaError_t e = once.run([] { return cudaFuncSetAttribute(linear_tc_head_kernel<BLOCK_N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1297,11 +1315,12 @@ cudaError_t launch_head(const TcLayer &L, const GemmParams &gp_in, int n_sm, cud
         if (e != cudaSuccess) return e;
     }
     GemmParams gp = gp_in;
-    const int epi = Plan::head_epi_bytes(gp.N);
+    const int tiles = (gp.M + BLOCK_M - 1) / BLOCK_M;
+    gp.bufs = tiles <= n_sm ? 1 : 2;
+    const int epi = Plan::head_epi_bytes(gp.N, gp.bufs);
     gp.stages = Plan::stages_for(epi);
     if (gp.stages < 2) return cudaErrorInvalidValue;
     const size_t smem = Plan::bytes(gp.stages, epi);
-    const int tiles = (gp.M + BLOCK_M - 1) / BLOCK_M;
     const int grid = tiles < n_sm ? tiles : n_sm;
     const cudaError_t le = launch_pdl(linear_tc_head_kernel<BLOCK_N>, dim3(grid), dim3(kHeadThreads), smem, stream, 0, L.map_a, L.map_b, gp);
     g_launches.fetch_add(1, std::memory_order_relaxed);

@@ -78,7 +78,7 @@ __device__ __forceinline__ float group_sum(float v)
 // Per-lane constants of the action dimensions k = sl + LPR i a lane owns, and per-batch scalars.
 template <int NI>
 struct RowConsts {
-    float inv_sg[NI], so2[NI], dls[NI];
+    float inv_sg[NI], kl0[NI];             // 1 / sigma_k; the part of KL(old || new) that does not depend on the means
     float logp_const, adv_mean, adv_rstd, eps, cv, inv_M;
     int clip_value;
 };
@@ -101,8 +101,9 @@ __device__ __forceinline__ void setup_lane(const PpoParams &P, int sl, RowConsts
         const float ls = ok ? __ldg(P.b.log_std + k) : 0.0f;
         const float lo = ok ? __ldg(P.b.log_std_old + k) : 0.0f;
         C.inv_sg[i] = expf(-ls);
-        C.so2[i] = expf(2.0f * lo);
-        C.dls[i] = ls - lo;
+        // d + (sigma_old^2 / sigma^2 - 1) / 2 with d = ln(sigma / sigma_old): not below zero by more than its own rounding,
+        // and zero where the standard deviations are the same
+        C.kl0[i] = (ls - lo) + 0.5f * expm1f(-2.0f * (ls - lo));
         acc.ls[i] = 0.0f;
         sum_log += ls;
     }
@@ -134,7 +135,8 @@ __device__ __forceinline__ float process_row(const RowConsts<NI> &C, int A, int 
             const float dm = mean_old[k] - mu;
             z[i] = (action[k] - mu) * C.inv_sg[i];
             zz = fmaf(z[i], z[i], zz);
-            kl += C.dls[i] + 0.5f * (C.so2[i] + dm * dm) * C.inv_sg[i] * C.inv_sg[i] - 0.5f;
+            const float zm = dm * C.inv_sg[i];
+            kl += fmaf(0.5f * zm, zm, C.kl0[i]);
         }
     }
     zz = group_sum<LPR>(zz);
