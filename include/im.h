@@ -389,6 +389,11 @@ im_status im_policy_forward_staged(im_policy *p, uint32_t step, int32_t n,
  * created on the same stream; src->max_batch >= n. */
 im_status im_value_forward(im_policy *critic, int32_t n, const float *obs, int32_t ld_obs, float *value_out);
 im_status im_value_forward_staged(im_policy *critic, im_policy *src, int32_t n, float *value_out);
+/* What a rollout step asks of both nets: im_policy_forward on the actor, then im_value_forward on the critic, on the
+ * same observations (obs == NULL: the bf16 rows staged in the actor's buffer, as for the *_staged calls).  Tensor-core
+ * nets on one stream with equal widths but for the last run layer by layer in common launches. */
+im_status im_policy_value_forward(im_policy *actor, im_policy *critic, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
+                                  float *mean_out, float *action_out, float *logp_out, float *value_out);
 
 /* Generalised advantage estimation (Schulman et al. 2016) over T control steps of N envs:
  *   done_t  = flags_t != 0        (the flag bytes im_env_step writes)

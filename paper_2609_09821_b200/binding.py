@@ -35,7 +35,7 @@ EXPORTS = [
     "im_ppo_updater_create", "im_ppo_updater_destroy", "im_ppo_update", "im_ppo_update_rollout", "im_ppo_updater_tensor",
     "im_ppo_updater_set_step_count",
     "im_copy_f32", "im_gemm_bf16_tn", "im_gather_rows_f32", "im_gemm_bf16_dgrad", "im_env_set_obs_extension", "im_env_adapt_reset_bins", "im_debug_math", "im_debug_set_wait", "im_env_set_summary", "im_clips_set_cyclic",
-    "im_env_get_cycles", "im_env_set_cycles", "im_env_set_aos_staging",
+    "im_env_get_cycles", "im_env_set_cycles", "im_env_set_aos_staging", "im_policy_value_forward",
 ]
 
 
@@ -193,6 +193,7 @@ def load():
         L.im_colsum_f32.argtypes = [vp, i64, i64, i32, vp, vp, C.c_size_t, vp]
         L.im_value_forward.argtypes = [vp, i32, vp, i32, vp]
         L.im_value_forward_staged.argtypes = [vp, vp, i32, vp]
+        L.im_policy_value_forward.argtypes = [vp, vp, u32, i32, vp, i32, vp, vp, vp, vp]
         L.im_gae.argtypes = [C.POINTER(GaeConfig), i32, i32, C.c_int64, vp, vp, vp, vp, vp, vp]
         for name in EXPORTS:
             if name not in ("im_status_string", "im_launch_count", "im_ppo_workspace_bytes") \
@@ -482,6 +483,14 @@ class Policy:
         """Critic forward on the bf16 rows an env attached to `src` (default: this policy) has staged."""
         _check(load().im_value_forward_staged(self.h, src.h if src is not None else None, n, _ptr(value_out)),
                "im_value_forward_staged")
+
+    def forward_with_value(self, step: int, critic: "Policy", obs, mean_out, action_out, logp_out, value_out, n: Optional[int] = None):
+        """forward() and critic.value_forward() on the same observations (obs None: the rows staged in this policy's
+        input buffer); nets of equal hidden widths share their launches."""
+        n = obs.shape[0] if n is None else n
+        _check(load().im_policy_value_forward(self.h, critic.h, step, n, _ptr(obs), obs.stride(0) if obs is not None else 0,
+                                              _ptr(mean_out), _ptr(action_out), _ptr(logp_out), _ptr(value_out)),
+               "im_policy_value_forward")
 
     def device_status(self) -> int:
         out = C.c_uint32(0)

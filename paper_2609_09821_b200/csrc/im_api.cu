@@ -717,6 +717,24 @@ im_status im_value_forward_staged(im_policy *critic, im_policy *src, int32_t n, 
     return tc_policy_forward(critic, 0u, n, nullptr, 0, value_out, nullptr, nullptr, src);
 }
 
+im_status im_policy_value_forward(im_policy *actor, im_policy *critic, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
+                                  float *mean_out, float *action_out, float *logp_out, float *value_out)
+{
+    if (!actor || !critic || actor == critic || !mean_out || !action_out || !value_out) return IM_ERR_INVALID_ARG;
+    if (!obs && (!actor->tensor_path || !critic->tensor_path)) return IM_ERR_UNSUPPORTED;
+    if (n < 1 || n > actor->cfg.max_batch || n > critic->cfg.max_batch) return IM_ERR_INVALID_ARG;
+    if (obs && (ld_obs < actor->cfg.dims[0] || ld_obs < critic->cfg.dims[0] || (ld_obs & 3) || !aligned16(obs))) return IM_ERR_INVALID_ARG;
+    if ((actor->tensor_path && (!aligned16(mean_out) || !aligned16(action_out))) || (critic->tensor_path && !aligned16(value_out)))
+        return IM_ERR_INVALID_ARG;
+    if (!obs && (actor->stream != critic->stream || actor->cfg.dims[0] != critic->cfg.dims[0])) return IM_ERR_INVALID_ARG;
+    if (tc_can_pair_nets(actor, critic, n))
+        return tc_policy_value_forward(actor, critic, step, n, obs, ld_obs, mean_out, action_out, logp_out, value_out);
+    const im_status s = obs ? im_policy_forward(actor, step, n, obs, ld_obs, mean_out, action_out, logp_out)
+                            : im_policy_forward_staged(actor, step, n, mean_out, action_out, logp_out);
+    if (s != IM_OK) return s;
+    return obs ? im_value_forward(critic, n, obs, ld_obs, value_out) : im_value_forward_staged(critic, actor, n, value_out);
+}
+
 /* ------------------------------------------------------------------ host-buffer step */
 static im_status ensure_staging(im_env *e, int A)
 {

@@ -35,6 +35,10 @@ void tc_policy_layer(im_policy *p, int layer, void **W, int32_t *ld, float **bia
 void *tc_policy_input(im_policy *p, int32_t *ld);     // bf16 [max_batch][ld] staging buffer of the first layer
 im_status tc_policy_forward(im_policy *p, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
                             float *mean_out, float *action_out, float *logp_out, im_policy *src = nullptr);
+// Whether an actor's and a critic's forward can run layer by layer in common launches (equal widths but for the last).
+bool tc_can_pair_nets(const im_policy *a, const im_policy *c, int n);
+im_status tc_policy_value_forward(im_policy *a, im_policy *c, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
+                                  float *mean_out, float *action_out, float *logp_out, float *value_out);
 im_status tc_gemm(const void *A, int64_t lda, const void *B, int64_t ldb, void *C, int64_t ldc, int M, int N, int K,
                   const float *bias, bool relu, uint32_t *status, cudaStream_t stream, int batches = 1,
                   const void *mask = nullptr, int64_t ld_mask = 0, float *colsum_partial = nullptr, int ld_partial = 0);

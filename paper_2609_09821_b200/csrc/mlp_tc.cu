@@ -14,6 +14,7 @@
 // through the common exit that frees its tensor memory.
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -207,6 +208,11 @@ struct GemmParams {
     long long ld_mask;
     float *colsum_partial;
     int ld_partial;
+    // Two nets of equal hidden widths in one launch (DUAL instantiations): tiles [0, n) are the first net's, the rest the
+    // second's, which has operand and output maps of its own; its head is a value head (no sampling).
+    const float *bias2;
+    int N2;
+    float *mean2;
     // Gaussian head
     float *mean, *action, *logp;
     float sigma;
@@ -240,11 +246,11 @@ struct SmemPlan {
     static constexpr __host__ __device__ int hidden_epi_bytes(bool bwd = false) { return (bwd ? 4 * 4 : 8) * kEpiSlabBytes; }
     // head: [2 accumulators][mean, action][128 rows][A] floats laid out as in global memory,
     // partial sums of z^2 [2][4][128], band counters [2][4]
-    // (+ bias and per-column sigma of the tile's columns, 2 x 128 floats)
+    // (+ bias, per-column sigma and the second net's bias of the tile's columns, 3 x 128 floats)
     // (one buffer where no CTA has a second tile)
     __host__ __device__ static constexpr int head_epi_bytes(int A, int bufs)
     {
-        return (bufs * 2 * 128 * A * 4 + 2 * 4 * 128 * 4 + 64 + 2 * 128 * 4 + 1023) / 1024 * 1024;
+        return (bufs * 2 * 128 * A * 4 + 2 * 4 * 128 * 4 + 64 + 3 * 128 * 4 + 1023) / 1024 * 1024;
     }
     __host__ __device__ static constexpr int stages_for(int epi_bytes)
     {
@@ -327,9 +333,10 @@ __device__ __forceinline__ void pipe_exit(const Pipe &p, uint32_t tmem_base, uin
 }
 
 // TMA producer (one thread): A and W tiles of every k-block of every tile of this CTA.
-template <class Plan, int BLOCK_N, bool MN = false>
+template <class Plan, int BLOCK_N, bool MN = false, bool DUAL = false>
 __device__ __forceinline__ void producer_role(const Pipe &p, const CUtensorMap *map_a, const CUtensorMap *map_b,
-                                              const GemmParams &P, int n_tiles)
+                                              const GemmParams &P, int n_tiles, const CUtensorMap *map_a2 = nullptr,
+                                              const CUtensorMap *map_b2 = nullptr)
 {
     int stage = 0;
     uint32_t phase = 0;
@@ -358,14 +365,15 @@ __device__ __forceinline__ void producer_role(const Pipe &p, const CUtensorMap *
             continue;
         }
         const int m0 = b * P.a_batch_rows + (t / P.n_tiles_n) * BLOCK_M, n0 = b * P.b_batch_rows + (t % P.n_tiles_n) * BLOCK_N;
+        const CUtensorMap *ma = DUAL && b ? map_a2 : map_a, *mb = DUAL && b ? map_b2 : map_b;
         for (int kb = 0; kb < P.K_blocks; kb += Plan::kDepth) {
             if (!mbar_wait(&p.empty[stage], phase ^ 1u, p.abort_flag)) return;
             uint8_t *sa = p.tiles + (size_t)stage * Plan::kStageBytes;
             mbar_arrive_expect_tx(&p.full[stage], Plan::kDepth * (Plan::kABytes + Plan::kBBytes));
 #pragma unroll
             for (int d = 0; d < Plan::kDepth; ++d) {                // (a block past K arrives as zeros)
-                tma_load_2d(sa + d * Plan::kABytes, map_a, &p.full[stage], (kb + d) * BLOCK_K, m0);
-                tma_load_2d(sa + Plan::kBOffset + d * Plan::kBBytesPadded, map_b, &p.full[stage], (kb + d) * BLOCK_K, n0);
+                tma_load_2d(sa + d * Plan::kABytes, ma, &p.full[stage], (kb + d) * BLOCK_K, m0);
+                tma_load_2d(sa + Plan::kBOffset + d * Plan::kBBytesPadded, mb, &p.full[stage], (kb + d) * BLOCK_K, n0);
             }
             if (++stage == p.stages) { stage = 0; phase ^= 1u; }
         }
@@ -455,15 +463,15 @@ __device__ __forceinline__ void mask_all_positive(uint4 (&mk)[8])
 
 template <bool BWD>
 __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_addr, int row, int col0, int lane,
-                                             const uint4 (&mk)[8], uint32_t (&pk)[32])
+                                             const uint4 (&mk)[8], uint32_t (&pk)[32], const float *bias)
 {
     float v[64];
     tmem_ld32_issue(t_addr, v);
     tmem_ld32_issue(t_addr + 32u, v + 32);
     tmem_ld_wait();
     const float fl = P.act_floor;          // 0: ReLU; -inf: linear output
-    if (P.bias) {
-        const float4 *b4 = reinterpret_cast<const float4 *>(P.bias + col0);
+    if (bias) {
+        const float4 *b4 = reinterpret_cast<const float4 *>(bias + col0);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const float4 b = __ldg(b4 + i);
@@ -514,12 +522,21 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
 // into a 128B-swizzled slab in shared memory and hands the slab to a TMA store.
 constexpr __host__ __device__ int hidden_depth(int block_n, bool mn, bool bwd) { return block_n < 256 && !mn && !bwd ? 2 : 1; }
 
-template <int BLOCK_N, bool MN = false, bool BWD = false>
+// Kernel parameters of the second net of a DUAL launch.
+struct NoMaps {};
+struct DualMaps {
+    CUtensorMap a, b, c;
+};
+template <bool DUAL>
+using SecondNet = std::conditional_t<DUAL, DualMaps, NoMaps>;
+
+template <int BLOCK_N, bool MN = false, bool BWD = false, bool DUAL = false>
 __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                        const __grid_constant__ CUtensorMap map_b,
                                                                        const __grid_constant__ CUtensorMap map_c,
                                                                        const __grid_constant__ CUtensorMap map_m,
-                                                                       const GemmParams P)
+                                                                       const GemmParams P,
+                                                                       const __grid_constant__ SecondNet<DUAL> second)
 {
     using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, MN, BWD)>;
     extern __shared__ uint8_t smem_raw[];
@@ -533,7 +550,10 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
     dep_wait();                       // nothing before this line touches global memory
 
     if (warp == 0) {
-        if (lane == 0) producer_role<Plan, BLOCK_N, MN>(p, &map_a, &map_b, P, n_tiles);
+        if (lane == 0) {
+            if constexpr (DUAL) producer_role<Plan, BLOCK_N, MN, true>(p, &map_a, &map_b, P, n_tiles, &second.a, &second.b);
+            else producer_role<Plan, BLOCK_N, MN>(p, &map_a, &map_b, P, n_tiles);
+        }
     } else if (warp == 1) {
         if (lane == 0) mma_role<Plan, BLOCK_N, MN>(p, tmem_base, P, n_tiles);
     } else {
@@ -584,7 +604,7 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
                         ++ci;
                     } else mask_all_positive(mk);
                 }
-                hidden_chunk<BWD>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk);
+                hidden_chunk<BWD>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, DUAL && bt ? P.bias2 : P.bias);
                 // the last store from this slab must have finished reading shared memory
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSlabs - 1) : "memory");
                 __syncwarp();
@@ -599,8 +619,10 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
+                    const CUtensorMap *mc = &map_c;
+                    if constexpr (DUAL) mc = bt ? &second.c : &map_c;
                     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                 ::"l"(&map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
+                                 ::"l"(mc), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
                 if (kSlabs == 2) which ^= 1;
@@ -842,7 +864,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
 #pragma unroll 1
                 for (int c0 = 0; c0 < 256; c0 += 64) {
                     uint32_t pk[32];
-                    hidden_chunk<false>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk);
+                    hidden_chunk<false>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, P.bias);
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                     __syncwarp();
                     uint8_t *slab = slabs + which * kEpiSlabBytes;
@@ -908,7 +930,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                         mask_read(slab, lane, mk);
                     } else mask_all_positive(mk);
                     uint32_t pk[32];
-                    hidden_chunk<true>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk);
+                    hidden_chunk<true>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, P.bias);
                     // each lane overwrites the 128 bytes it read its own mask words from
                     const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
 #pragma unroll
@@ -985,18 +1007,20 @@ __device__ __forceinline__ float head_noise(const GemmParams &P, int row, int c0
     return zz;
 }
 
-template <int BLOCK_N>
+template <int BLOCK_N, bool DUAL = false>
 __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                          const __grid_constant__ CUtensorMap map_b,
-                                                                         const GemmParams P)
+                                                                         const GemmParams P,
+                                                                         const __grid_constant__ SecondNet<DUAL> second)
 {
     using Plan = SmemPlan<BLOCK_N, head_depth(BLOCK_N)>;
     extern __shared__ uint8_t smem_raw[];
     const int A = P.N, bufs = P.bufs;
     const Pipe p = carve_pipe<Plan>(smem_raw, P.stages, Plan::head_epi_bytes(A, bufs));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = (P.M + BLOCK_M - 1) / BLOCK_M;             // one N tile holds the whole action row
-    const int out_floats = 128 * A;
+    const int net_tiles = (P.M + BLOCK_M - 1) / BLOCK_M;           // one N tile holds the whole action row
+    const int n_tiles = DUAL ? 2 * net_tiles : net_tiles;
+    const int out_floats = 128 * A;                                // (A is the wider of two nets)
     // staging: per accumulator buffer the tile's mean and action rows laid out exactly as in global
     // memory ([128][A], dense), so a 32-row band leaves as one contiguous copy
     float *out_tiles = reinterpret_cast<float *>(p.epi);                            // [bufs][2][128 * A]
@@ -1004,13 +1028,17 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
     int *band_count = reinterpret_cast<int *>(zz_part + 2 * 4 * 128);               // [2][4]
     float *s_bias = reinterpret_cast<float *>(band_count + 16);                     // [128]: bias of the tile's columns
     float *s_sigma = s_bias + 128;                                                  // [128]: standard deviation per column
+    float *s_bias2 = s_sigma + 128;                                                 // [128]: bias of the second net
     if (threadIdx.x < 8) band_count[threadIdx.x] = 0;
     pipe_init<Plan>(p, kHeadEpiWarps);
     const uint32_t tmem_base = *p.tmem_slot;
 
     if (warp == 0) {
         dep_wait();                   // nothing before this line touches global memory
-        if (lane == 0) producer_role<Plan, BLOCK_N>(p, &map_a, &map_b, P, n_tiles);
+        if (lane == 0) {
+            if constexpr (DUAL) producer_role<Plan, BLOCK_N, false, true>(p, &map_a, &map_b, P, n_tiles, &second.a, &second.b);
+            else producer_role<Plan, BLOCK_N>(p, &map_a, &map_b, P, n_tiles);
+        }
     } else if (warp == 1) {
         dep_wait();
         if (lane == 0) mma_role<Plan, BLOCK_N>(p, tmem_base, P, n_tiles);
@@ -1020,22 +1048,23 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
         const int row_in_tile = quad * 32 + lane;
         constexpr int kGroups = (BLOCK_N / 16) < 4 ? (BLOCK_N / 16) : 4;
         constexpr int kChunks = (BLOCK_N + 63) / 64;
-        const bool sample = P.action != nullptr;                     // a value head reads only the mean
+        const bool sample_1 = P.action != nullptr;                   // a value head reads only the mean
         float z[16 * kChunks], zz = 0.0f;
 #pragma unroll
         for (int i = 0; i < 16 * kChunks; ++i) z[i] = 0.0f;
-        if (sample && group < kGroups)
+        if (sample_1 && group < kGroups && (!DUAL || (int)blockIdx.x < net_tiles))
             zz = head_noise<kChunks>(P, (int)blockIdx.x * BLOCK_M + row_in_tile, 16 * group, A, z);
         dep_wait();
         // the epilogue reads bias and sigma from shared memory as 16-byte words instead of one global load per output
         if ((int)threadIdx.x - 64 < BLOCK_N) {
             const int cidx = (int)threadIdx.x - 64;
             s_bias[cidx] = __ldg(P.bias + cidx);
+            if (DUAL) s_bias2[cidx] = cidx < P.N2 ? __ldg(P.bias2 + cidx) : 0.0f;
             s_sigma[cidx] = cidx < A ? (P.log_std ? expf(__ldg(P.log_std + cidx)) : P.sigma) : 0.0f;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * kHeadEpiWarps) : "memory");
         float logp_const = 0.0f;
-        if (sample) {
+        if (sample_1) {
             float sum_log = (float)A * logf(P.sigma);
             if (P.log_std) {                                         // same order in every thread
                 sum_log = 0.0f;
@@ -1046,7 +1075,10 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
         int acc = 0;
         uint32_t acc_phase = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            const int m0 = tile * BLOCK_M;
+            const bool net2 = DUAL && tile >= net_tiles;
+            const int m0 = (net2 ? tile - net_tiles : tile) * BLOCK_M, A = net2 ? P.N2 : P.N;
+            const bool sample = sample_1 && !net2;
+            const float *bias = net2 ? s_bias2 : s_bias;
             if (!mbar_wait(&p.acc_full[acc], acc_phase, p.abort_flag)) break;
             tc_fence_after();
             const int row = m0 + row_in_tile;
@@ -1064,7 +1096,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
                     for (int g = 0; g < 4; ++g) {
                         const int col = c0 + 4 * g;
                         if (col >= A) break;
-                        const float4 b4 = *reinterpret_cast<const float4 *>(s_bias + col);
+                        const float4 b4 = *reinterpret_cast<const float4 *>(bias + col);
                         const float4 s4 = *reinterpret_cast<const float4 *>(s_sigma + col);
                         const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, ss[4] = {s4.x, s4.y, s4.z, s4.w};
 #pragma unroll
@@ -1100,7 +1132,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
                     if (rows_valid > 0) {
                         const int count = rows_valid * A;                       // floats, contiguous in global
                         const float *src_m = s_mean + quad * 32 * A, *src_a = s_act + quad * 32 * A;
-                        float *dst_m = P.mean + (size_t)band_row0 * A;
+                        float *dst_m = (net2 ? P.mean2 : P.mean) + (size_t)band_row0 * A;
                         float *dst_a = sample ? P.action + (size_t)band_row0 * A : nullptr;
                         // both sides start on a 16-byte boundary: band offsets are multiples of 32 rows
                         const int bulk = count & ~3;
@@ -1115,7 +1147,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
                             dst_m[i] = src_m[i];
                             if (sample) dst_a[i] = src_a[i];
                         }
-                        if (P.logp && lane < rows_valid) {
+                        if (P.logp && !net2 && lane < rows_valid) {
                             float sum = 0.0f;
 #pragma unroll
                             for (int g = 0; g < kGroups; ++g) sum += zz_part[(acc * 4 + g) * 128 + row_in_tile];
@@ -1124,7 +1156,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
                     }
                 }
                 // the next tile's noise, while this band leaves and the tile's operands arrive
-                if (sample && tile + (int)gridDim.x < n_tiles)
+                if (sample && tile + (int)gridDim.x < net_tiles)
                     zz = head_noise<kChunks>(P, (tile + (int)gridDim.x) * BLOCK_M + row_in_tile, 16 * group, A, z);
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             }
@@ -1203,10 +1235,9 @@ bool make_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, 
 // the SMs in one wave (a lone tile's time is its operand loads and its epilogue, both shorter when it is narrow:
 // 1024 x 1024 x 384 in a chain of launches 4.96 us with 64 columns, 5.68 with 128, 7.22 with 256; 2048 rows 6.96 / 5.79 /
 // 7.37), and the widest that divides N once there are several waves (8192 rows 17.1 / 12.1 / 10.4).
-int pick_block_n(int M, int N, bool last, int n_sm)
+int pick_block_n(int rows, int N, bool last, int n_sm)       // rows: 128-row tiles
 {
     if (last) return (N + 15) / 16 * 16;
-    const int rows = (M + BLOCK_M - 1) / BLOCK_M;
     int widest = 64;
     for (int bn = 64; bn <= 256 && N % bn == 0; bn *= 2) {
         if (rows * (N / bn) <= n_sm) return bn;
@@ -1224,6 +1255,8 @@ struct TcLayer {
     CUtensorMap map_a, map_b, map_c;    // map_c: the hidden-activation buffer this layer stores to
     CUtensorMap map_b2;                 // W in 128-row boxes: one CTA's half of a 256-column tile, or a 128-column tile
     CUtensorMap map_b1;                 // W in 64-row boxes: a 64-column tile
+    CUtensorMap map_head[5];            // last layer: W in boxes of 16, 32, .. 80 rows (rows past the layer's read as zeros)
+    const CUtensorMap &map_b_head(int block_n) const { return map_head[block_n / 16 - 1]; }
     CUtensorMap map_m;                  // backward epilogue: the forward activations behind the ReLU mask (boxes like map_c)
 };
 
@@ -1235,8 +1268,6 @@ struct im_policy_tc {
     __nv_bfloat16 *d_hidden[2];   // [max_batch][max hidden]
     int ld_in, ld_hidden;
     int n_sm;
-    const __nv_bfloat16 *ext_in;  // another policy's input buffer the first layer last read from (or null)
-    CUtensorMap map_a_ext;        // first-layer operand map over ext_in
 };
 
 namespace im {
@@ -1259,7 +1290,7 @@ cudaError_t launch_hidden(const TcLayer &L, const GemmParams &gp_in, int n_sm, c
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
     const int grid = tiles < n_sm ? tiles : n_sm;
     const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, dim3(grid), dim3(hidden_threads(BLOCK_N, BWD)), smem, stream, 0,
-                                      L.map_a, L.map_b, L.map_c, L.map_m, gp);
+                                      L.map_a, L.map_b, L.map_c, L.map_m, gp, NoMaps());
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
 }
@@ -1282,7 +1313,7 @@ cudaError_t launch_hidden_mn(const TcLayer &L, const GemmParams &gp_in, int n_sm
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
     const int grid = tiles < n_sm ? tiles : n_sm;
     const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, true>, dim3(grid), dim3(hidden_threads(BLOCK_N, false)), smem, stream, 0,
-                                      L.map_a, L.map_b, L.map_c, L.map_c, gp);
+                                      L.map_a, L.map_b, L.map_c, L.map_c, gp, NoMaps());
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
 }
@@ -1304,42 +1335,80 @@ cudaError_t launch_hidden_pair(const TcLayer &L, const GemmParams &gp, int n_sm,
     return le != cudaSuccess ? le : cudaGetLastError();
 }
 
+// The forward products of one layer of two nets (equal widths) in one launch.
 template <int BLOCK_N>
-cudaError_t launch_head(const TcLayer &L, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
+cudaError_t launch_hidden_dual(const TcLayer &L, const TcLayer &L2, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
+{
+    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, false, false)>;
+    const auto kernel = linear_tc_hidden_kernel<BLOCK_N, false, false, true>;
+    static DeviceOnce once;                      // the attribute is per device
+    const cudaError_t e = once.run([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit); });
+    if (e != cudaSuccess) return e;
+    GemmParams gp = gp_in;
+    gp.n_batches = 2;
+    gp.stages = Plan::stages_for(Plan::hidden_epi_bytes());
+    const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes());
+    const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * 2;
+    const int grid = tiles < n_sm ? tiles : n_sm;
+    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, false)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
+                                      L.map_c, gp, DualMaps{L2.map_a, L2.map_b, L2.map_c});
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return le;
+}
+
+template <int BLOCK_N, bool DUAL>
+cudaError_t launch_head(const TcLayer &L, const GemmParams &gp_in, int n_sm, const SecondNet<DUAL> &second, cudaStream_t stream)
 {
     using Plan = SmemPlan<BLOCK_N, head_depth(BLOCK_N)>;
+    const auto kernel = linear_tc_head_kernel<BLOCK_N, DUAL>;
     static DeviceOnce once;                      // the attribute is per device
-    {
-        const cudaError_t e = once.run([] { return cudaFuncSetAttribute(linear_tc_head_kernel<BLOCK_N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kSmemLimit); });
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = once.run([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit); });
+    if (e != cudaSuccess) return e;
     GemmParams gp = gp_in;
-    const int tiles = (gp.M + BLOCK_M - 1) / BLOCK_M;
+    const int tiles = (gp.M + BLOCK_M - 1) / BLOCK_M * (DUAL ? 2 : 1);
     gp.bufs = tiles <= n_sm ? 1 : 2;
+    gp.n_batches = DUAL ? 2 : 1;
     const int epi = Plan::head_epi_bytes(gp.N, gp.bufs);
     gp.stages = Plan::stages_for(epi);
     if (gp.stages < 2) return cudaErrorInvalidValue;
     const size_t smem = Plan::bytes(gp.stages, epi);
     const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_head_kernel<BLOCK_N>, dim3(grid), dim3(kHeadThreads), smem, stream, 0, L.map_a, L.map_b, gp);
+    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(kHeadThreads), smem, stream, 0, L.map_a, L.map_b, gp, second);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
+}
+
+template <bool DUAL>
+cudaError_t dispatch_head(const TcLayer &L, const GemmParams &gp, int n_sm, const SecondNet<DUAL> &second, cudaStream_t stream)
+{
+    switch (L.block_n) {
+    case 16: return launch_head<16, DUAL>(L, gp, n_sm, second, stream);
+    case 32: return launch_head<32, DUAL>(L, gp, n_sm, second, stream);
+    case 48: return launch_head<48, DUAL>(L, gp, n_sm, second, stream);
+    case 64: return launch_head<64, DUAL>(L, gp, n_sm, second, stream);
+    case 80: return launch_head<80, DUAL>(L, gp, n_sm, second, stream);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+// Whether a hidden layer's product runs on CTA pairs.  They pay off when the main loop is long enough to amortise the
+// cluster set-up and there are at least two waves of 256 x 256 tiles; otherwise the single-CTA kernel's finer tiles
+// balance the machine better (measured: 16384 x 1024 x 384 is 8 % faster single, 16384 x 1024 x 2048 7 % faster paired).
+// The backward epilogue is the longer part of a tile when K is short, and the pair kernel runs it on eight warps: it
+// takes those products whenever its tiles fill the machine.
+bool takes_pairs(const TcLayer &L, const GemmParams &gp, int n_sm, bool force_pairs)
+{
+    const int pair_tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n;
+    const bool bwd = gp.mask || gp.colsum_partial;
+    return L.block_n == 256 && gp.n_batches == 1 &&
+           (force_pairs || (pair_tiles >= n_sm && gp.K_blocks >= 8) || (bwd && pair_tiles >= n_sm / 2));
 }
 
 cudaError_t dispatch_tc(const TcLayer &L, const GemmParams &gp, bool last, int n_sm, bool force_pairs, cudaStream_t stream)
 {
     if (!last) {
-        // CTA pairs pay off when the main loop is long enough to amortise the cluster set-up and there
-        // are at least two waves of 256 x 256 tiles; otherwise the single-CTA kernel's finer tiles
-        // balance the machine better (measured: 16384 x 1024 x 384 is 8 % faster single, 16384 x 1024 x 2048
-        // 7 % faster paired)
-        const int pair_tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n;
         const bool bwd = gp.mask || gp.colsum_partial;
-        // (the backward epilogue is the longer part of a tile when K is short, and the pair kernel runs it on
-        // eight warps: it takes those products whenever its tiles fill the machine)
-        if (L.block_n == 256 && gp.n_batches == 1 &&
-            (force_pairs || (pair_tiles >= n_sm && gp.K_blocks >= 8) || (bwd && pair_tiles >= n_sm / 2)))
+        if (takes_pairs(L, gp, n_sm, force_pairs))
             return bwd ? launch_hidden_pair<true>(L, gp, n_sm, stream) : launch_hidden_pair<false>(L, gp, n_sm, stream);
         switch (L.block_n) {
         case 256: return bwd ? launch_hidden<256, true>(L, gp, n_sm, stream) : launch_hidden<256>(L, gp, n_sm, stream);
@@ -1347,14 +1416,7 @@ cudaError_t dispatch_tc(const TcLayer &L, const GemmParams &gp, bool last, int n
         default: return bwd ? launch_hidden<64, true>(L, gp, n_sm, stream) : launch_hidden<64>(L, gp, n_sm, stream);
         }
     }
-    switch (L.block_n) {
-    case 16: return launch_head<16>(L, gp, n_sm, stream);
-    case 32: return launch_head<32>(L, gp, n_sm, stream);
-    case 48: return launch_head<48>(L, gp, n_sm, stream);
-    case 64: return launch_head<64>(L, gp, n_sm, stream);
-    case 80: return launch_head<80>(L, gp, n_sm, stream);
-    default: return cudaErrorInvalidValue;
-    }
+    return dispatch_head<false>(L, gp, n_sm, NoMaps(), stream);
 }
 
 }  // namespace
@@ -1378,7 +1440,6 @@ im_status tc_policy_create(im_policy *p, const void *const *W, const float *cons
     p->tc = tc;
     tc->n_sm = n_sm;
     tc->d_in = nullptr;
-    tc->ext_in = nullptr;
     tc->d_hidden[0] = tc->d_hidden[1] = nullptr;
     tc->layers.resize(nl);
     for (auto &L : tc->layers) { L.d_W = nullptr; L.d_bias = nullptr; }
@@ -1398,7 +1459,7 @@ im_status tc_policy_create(im_policy *p, const void *const *W, const float *cons
         L.N = cfg.dims[l + 1];
         L.K = cfg.dims[l];
         L.Kpad = (L.K + BLOCK_K - 1) / BLOCK_K * BLOCK_K;
-        L.block_n = pick_block_n(cfg.max_batch, L.N, last, 0);          // (no SMs: the widest)
+        L.block_n = pick_block_n(1, L.N, last, 0);          // (no SMs: the widest)
         L.n_tiles_n = (L.N + L.block_n - 1) / L.block_n;
         const size_t rows = (size_t)L.n_tiles_n * L.block_n;
         std::vector<uint16_t> hw(rows * L.Kpad, 0);
@@ -1424,6 +1485,8 @@ im_status tc_policy_create(im_policy *p, const void *const *W, const float *cons
         // hidden layers store 32-row x 64-column slabs of their output buffer
         if (!last && !make_map(&L.map_c, tc->d_hidden[l & 1], mb, rows, (uint64_t)tc->ld_hidden, 32))
             return IM_ERR_CUDA;
+        for (int i = 0; last && i < 5; ++i)
+            if (!make_map(&L.map_head[i], L.d_W, rows, (uint64_t)L.Kpad, (uint64_t)L.Kpad, 16 * (i + 1))) return IM_ERR_CUDA;
         L.map_m = L.map_c;               // the forward pass has no mask: a valid placeholder
     }
     return IM_OK;
@@ -1453,55 +1516,121 @@ void *tc_policy_input(im_policy *p, int32_t *ld)
     return p->tc->d_in;
 }
 
+namespace {
+
+GemmParams head_params(const im_policy *p, uint32_t step, int n, float *mean, float *action, float *logp)
+{
+    const im_policy_config &cfg = p->cfg;
+    GemmParams gp;
+    std::memset(&gp, 0, sizeof(gp));
+    gp.M = n; gp.act_floor = 0.0f; gp.n_batches = 1;
+    gp.mean = mean; gp.action = action; gp.logp = logp;
+    gp.sigma = cfg.sigma; gp.log_std = p->d_log_std; gp.seed_lo = (uint32_t)cfg.seed; gp.seed_hi = (uint32_t)(cfg.seed >> 32);
+    gp.step = step; gp.env_id_base = cfg.env_id_base; gp.status = p->d_status;
+    return gp;
+}
+void set_layer(GemmParams &gp, const TcLayer &L)
+{
+    gp.N = L.N; gp.K_blocks = L.Kpad / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = L.d_bias;
+}
+// The layer with the tile width for `rows` row tiles.
+TcLayer with_width(const TcLayer &Y, int rows, bool last, int n_sm)
+{
+    TcLayer L = Y;
+    const int bn = pick_block_n(rows, L.N, last, n_sm);
+    if (bn < L.block_n) {
+        L.map_b = bn == 128 ? L.map_b2 : L.map_b1;
+        L.block_n = bn;
+        L.n_tiles_n = L.N / bn;
+    }
+    return L;
+}
+
+im_status convert_obs(im_policy *p, int n, const float *obs, int ld_obs)
+{
+    im_policy_tc *tc = p->tc;
+    const long long chunks = (long long)n * (tc->ld_in / 8);
+    const int block = 256;
+    long long grid = (chunks + block - 1) / block;
+    if (grid > 148 * 16) grid = 148 * 16;
+    obs_to_bf16_kernel<<<(int)grid, block, 0, p->stream>>>(obs, ld_obs, p->cfg.dims[0], tc->d_in, tc->ld_in, n);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+}
+
+}  // namespace
+
 // obs == nullptr: the bf16 input buffer has already been filled (by an attached environment); it is
-// this policy's own buffer, or that of `src` (same input width), whose rows the first layer then reads
-// through a tensor map built on first use.  action_out == nullptr: no sampling, only the mean is written.
+// this policy's own buffer, or that of `src` (same input width), whose rows the first layer then reads.
+// action_out == nullptr: no sampling, only the mean is written.
 im_status tc_policy_forward(im_policy *p, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
                             float *mean_out, float *action_out, float *logp_out, im_policy *src)
 {
     im_policy_tc *tc = p->tc;
     const im_policy_config &cfg = p->cfg;
     const bool external = !obs && src && src != p;
-    if (external) {
-        im_policy_tc *st = src->tc;
-        if (!st || st->ld_in != tc->ld_in || src->cfg.dims[0] != cfg.dims[0] || src->cfg.max_batch < n)
-            return IM_ERR_INVALID_ARG;
-        if (tc->ext_in != st->d_in) {
-            const TcLayer &L0 = tc->layers[0];
-            if (!make_map(&tc->map_a_ext, st->d_in, (uint64_t)src->cfg.max_batch, (uint64_t)L0.Kpad, (uint64_t)st->ld_in,
-                          BLOCK_M))
-                return IM_ERR_CUDA;
-            tc->ext_in = st->d_in;
-        }
-    }
+    if (external && (!src->tc || src->tc->ld_in != tc->ld_in || src->cfg.dims[0] != cfg.dims[0] || src->cfg.max_batch < n))
+        return IM_ERR_INVALID_ARG;
     if (obs) {
-        const long long chunks = (long long)n * (tc->ld_in / 8);
-        const int block = 256;
-        long long grid = (chunks + block - 1) / block;
-        if (grid > 148 * 16) grid = 148 * 16;
-        obs_to_bf16_kernel<<<(int)grid, block, 0, p->stream>>>(obs, ld_obs, cfg.dims[0], tc->d_in, tc->ld_in, n);
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        if (cudaGetLastError() != cudaSuccess) return IM_ERR_CUDA;
+        const im_status s = convert_obs(p, n, obs, ld_obs);
+        if (s != IM_OK) return s;
     }
+    GemmParams gp = head_params(p, step, n, mean_out, action_out, logp_out);
     for (int l = 0; l < p->nl; ++l) {
-        TcLayer L = tc->layers[l];
-        if (l == 0 && external) L.map_a = tc->map_a_ext;
         const bool last = l == p->nl - 1;
-        const int bn = pick_block_n(n, L.N, last, tc->n_sm);
-        if (bn < L.block_n && cfg.impl != 2) {
-            L.map_b = bn == 128 ? L.map_b2 : L.map_b1;
-            L.block_n = bn;
-            L.n_tiles_n = L.N / bn;
-        }
-        GemmParams gp;
-        std::memset(&gp, 0, sizeof(gp));
-        gp.M = n; gp.N = L.N; gp.K_blocks = L.Kpad / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = L.d_bias;
-        gp.act_floor = 0.0f;
-        gp.n_batches = 1; gp.a_batch_rows = 0; gp.b_batch_rows = 0; gp.c_batch_rows = 0;
-        gp.mean = mean_out; gp.action = action_out; gp.logp = logp_out;
-        gp.sigma = cfg.sigma; gp.log_std = p->d_log_std; gp.seed_lo = (uint32_t)cfg.seed; gp.seed_hi = (uint32_t)(cfg.seed >> 32);
-        gp.step = step; gp.env_id_base = cfg.env_id_base; gp.status = p->d_status;
+        TcLayer L = cfg.impl == 2 ? tc->layers[l] : with_width(tc->layers[l], (n + BLOCK_M - 1) / BLOCK_M, last, tc->n_sm);
+        if (l == 0 && external) L.map_a = src->tc->layers[0].map_a;
+        set_layer(gp, L);
         if (dispatch_tc(L, gp, last, tc->n_sm, cfg.impl == 2, p->stream) != cudaSuccess) return IM_ERR_CUDA;
+    }
+    return IM_OK;
+}
+
+bool tc_can_pair_nets(const im_policy *a, const im_policy *c, int n)
+{
+    bool same = a->tensor_path && c->tensor_path && a != c && a->stream == c->stream && a->nl == c->nl && a->cfg.impl == 0 && c->cfg.impl == 0 &&
+                a->cfg.max_batch >= n && c->cfg.max_batch >= n && a->cfg.dims[a->nl] >= c->cfg.dims[c->nl];
+    for (int l = 0; same && l < a->nl; ++l) same = a->cfg.dims[l] == c->cfg.dims[l];
+    return same;
+}
+
+// Policy and value head on the same observations: the layers of both nets, which have equal widths (tc_can_pair_nets), two by
+// two in one launch.  A layer that runs on CTA pairs fills the machine by itself and keeps a launch per net.  Below some
+// 16,000 rows a layer costs its fixed chain of barriers, loads and stores (about 5 us) rather than its arithmetic, and one
+// net's tiles leave SMs idle: both nets in one launch cost hardly more than one.  Actor (361, 1024, 512, 28) and its
+// critic, us for n = 64 / 1000 / 4096 / 9001 / 16384: one after the other 30.8 / 32.7 / 40.0 / 51.6 / 81.0, together
+// 16.4 / 18.4 / 25.7 / 39.5 / 67.4; (577, 1024, 1024, 512, 69) 33.6 / 36.0 / 44.8 / 61.1 / 94.1 and 18.5 / 20.8 / 30.3 /
+// 47.9 / 90.9.
+im_status tc_policy_value_forward(im_policy *a, im_policy *c, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
+                                  float *mean_out, float *action_out, float *logp_out, float *value_out)
+{
+    const int n_sm = a->tc->n_sm, rows = (n + BLOCK_M - 1) / BLOCK_M;
+    if (obs) {
+        const im_status s = convert_obs(a, n, obs, ld_obs);
+        if (s != IM_OK) return s;
+    }
+    GemmParams gp = head_params(a, step, n, mean_out, action_out, logp_out), gc = head_params(c, 0u, n, value_out, nullptr, nullptr);
+    for (int l = 0; l < a->nl; ++l) {
+        const bool last = l == a->nl - 1;
+        TcLayer L = with_width(a->tc->layers[l], 2 * rows, last, n_sm), L2 = with_width(c->tc->layers[l], 2 * rows, last, n_sm);
+        if (l == 0) L2.map_a = L.map_a;                          // one copy of the observations serves both
+        set_layer(gp, L);
+        set_layer(gc, L2);
+        gp.bias2 = L2.d_bias; gp.N2 = L2.N; gp.mean2 = value_out;
+        cudaError_t e;
+        if (last) {
+            e = dispatch_head<true>(L, gp, n_sm, DualMaps{L2.map_a, L2.map_b_head(L.block_n), L2.map_a}, a->stream);
+        } else if (takes_pairs(L, gp, n_sm, false)) {
+            e = launch_hidden_pair<false>(L, gp, n_sm, a->stream);
+            if (e == cudaSuccess) e = launch_hidden_pair<false>(L2, gc, n_sm, a->stream);
+        } else {
+            switch (L.block_n) {
+            case 256: e = launch_hidden_dual<256>(L, L2, gp, n_sm, a->stream); break;
+            case 128: e = launch_hidden_dual<128>(L, L2, gp, n_sm, a->stream); break;
+            default: e = launch_hidden_dual<64>(L, L2, gp, n_sm, a->stream); break;
+            }
+        }
+        if (e != cudaSuccess) return IM_ERR_CUDA;
     }
     return IM_OK;
 }
@@ -1524,7 +1653,7 @@ im_status tc_gemm(const void *A, int64_t lda, const void *B, int64_t ldb, void *
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
     TcLayer L;
     L.N = N; L.K = K; L.Kpad = K;
-    L.block_n = pick_block_n(M, N, false, n_sm);
+    L.block_n = pick_block_n((M + BLOCK_M - 1) / BLOCK_M, N, false, n_sm);
     L.n_tiles_n = N / L.block_n;
     L.d_W = nullptr; L.d_bias = nullptr;
     const uint64_t nb = (uint64_t)batches;
@@ -1587,7 +1716,7 @@ im_status tc_gemm_tn(const void *A, int64_t lda, const void *B, int64_t ldb, voi
     // wide outputs take 256-column tiles even when that leaves a ragged last tile (640 columns: three tiles,
     // a sixth of the MMAs wasted, against five 128-column tiles at little more than half the tensor-pipe rate);
     // TMA fills the operand columns past No with zeros and clips the stores
-    L.block_n = No > 256 ? 256 : pick_block_n(Mo, No, false, 0);
+    L.block_n = No > 256 ? 256 : pick_block_n(1, No, false, 0);
     L.n_tiles_n = (No + L.block_n - 1) / L.block_n;
     L.d_W = nullptr; L.d_bias = nullptr;
     if (!make_map(&L.map_a, A, (uint64_t)R, (uint64_t)Mo, (uint64_t)lda, 64) ||
@@ -1622,7 +1751,7 @@ im_status tc_gemm_head(const void *A, int64_t lda, const void *B, int64_t ldb, i
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
     TcLayer L;
     L.N = N; L.K = K; L.Kpad = K;
-    L.block_n = pick_block_n(M, N, true, n_sm);
+    L.block_n = pick_block_n(1, N, true, n_sm);
     L.n_tiles_n = 1;
     L.d_W = nullptr; L.d_bias = nullptr;
     if (!make_map(&L.map_a, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BLOCK_M) ||

@@ -60,14 +60,13 @@ def collect(env: B.Env, actor: B.Policy, critic: Optional[B.Policy], storage: Ro
     for t in range(T):
         s = step0 + t
         obs = st.obs_row(t)
-        if staged:
+        if critic is not None:
+            actor.forward_with_value(s, critic, None if staged else obs, st.mean[t], st.action[t], st.logp[t],
+                                     st.value[t].unsqueeze(1), n=N)
+        elif staged:
             actor.forward_staged(s, N, st.mean[t], st.action[t], st.logp[t])
-            if critic is not None:
-                critic.value_forward_staged(N, st.value[t].unsqueeze(1), src=actor)
         else:
             actor.forward(s, obs, st.mean[t], st.action[t], st.logp[t])
-            if critic is not None:
-                critic.value_forward(obs, st.value[t].unsqueeze(1))
         if getattr(env, "_prev_action", None) is not None:
             # extended observation: the next row's previous-action entries are this step's actions (host state
             # only; the pointer travels with the launch, so a captured graph keeps one per step)

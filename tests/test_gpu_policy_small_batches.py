@@ -59,3 +59,52 @@ def test_forward_reads_another_policys_rows():
     actor.forward(1, obs, mean, act)
     critic.value_forward_staged(n, v1, src=actor)
     assert torch.equal(v0, v1)
+
+
+@pytest.mark.parametrize("dims,dv", [((361, 1024, 512, 28), 1), ((577, 1024, 1024, 512, 69), 3), ((70, 64, 17), 1), ((361, 2048, 1024, 80), 33)])
+@pytest.mark.parametrize("n", [1, 128, 129, 1000, 4096, 9600, 20000])
+@pytest.mark.parametrize("staged", [False, True])
+def test_joint_forward_matches_the_separate_calls(n, dims, dv, staged):
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    wa, wc = W.make_policy_weights(dims, "bf16", 1), W.make_policy_weights(dims[:-1] + (dv,), "bf16", 2)
+    A = dims[-1]
+    actor = B.Policy(dims, wa["W_bf16"], wa["b"], "bf16", 0.3, 9, n, env_id_base=5)
+    critic = B.Policy(dims[:-1] + (dv,), wc["W_bf16"], wc["b"], "bf16", 0.3, 9, n)
+    actor.set_log_std(torch.linspace(-2, 0, A, device="cuda"))
+    obs = torch.randn(n, B.padded_ld(dims[0]), device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+
+    def outputs():                                   # one guard row behind each
+        return [torch.full((n + 1, k), 7.0, device="cuda") for k in (A, A, 1, dv)]
+    sep, joint = outputs(), outputs()
+    actor.forward(3, obs, *sep[:3], n=n)             # leaves the rows staged
+    critic.value_forward(obs, sep[3], n=n)
+    for _ in range(2):
+        actor.forward_with_value(3, critic, None if staged else obs, *joint, n=n)
+    torch.cuda.synchronize()
+    assert all(bool((t[n] == 7.0).all()) for t in joint)
+    assert actor.device_status() == 0 and critic.device_status() == 0
+    for i, (a, b) in enumerate(zip(joint, sep)):
+        a, b = a[:n], b[:n]
+        if i == 2:
+            assert float((a - b).abs().max()) <= 1e-5 * A + 1e-6 * float(b.abs().max())
+        else:
+            # a tile of another width may add the same products along k in another order: the bounds of the test above
+            rms = float(b.square().mean().sqrt())
+            assert float((a - b).abs().max()) <= 2e-2 * (float(b.abs().max()) + rms) and float((a - b).norm() / b.norm()) <= 2e-3
+
+
+def test_joint_forward_runs_nets_of_other_widths_one_after_the_other():
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    n, dims, cdims = 300, (361, 512, 256, 28), (361, 256, 128, 1)
+    for dtype in ("bf16", "f32"):
+        wa, wc = W.make_policy_weights(dims, dtype, 1), W.make_policy_weights(cdims, dtype, 2)
+        key = "W_bf16" if dtype == "bf16" else "W"
+        actor, critic = B.Policy(dims, wa[key], wa["b"], dtype, 0.3, 9, n), B.Policy(cdims, wc[key], wc["b"], dtype, 0.3, 9, n)
+        obs = torch.randn(n, 384, device="cuda")
+        sep, joint = [[torch.empty(n, k, device="cuda") for k in (28, 28, 1, 1)] for _ in range(2)]
+        actor.forward(3, obs, *sep[:3])
+        critic.value_forward(obs, sep[3])
+        actor.forward_with_value(3, critic, obs, *joint)
+        assert all(torch.equal(a, b) for a, b in zip(joint, sep))
