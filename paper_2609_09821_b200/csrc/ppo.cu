@@ -17,8 +17,11 @@
 // kept per lane, folded per CTA in a fixed order and finished by a second one-CTA launch, so the
 // result does not depend on scheduling.  No value is read on the host.
 #include <cmath>
+#include <cooperative_groups.h>
 
 #include "im_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace im {
 
@@ -26,7 +29,16 @@ namespace {
 
 constexpr int kWarps = 4;                 // per CTA
 constexpr int kMaxGrid = 888;              // six CTAs per SM: bounds the partial rows the finishing launch walks
-constexpr int kFinishGroups = 4;
+// Every kernel of the update's loss is launched with programmatic stream serialization.
+__device__ __forceinline__ void dep_release_wait()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+constexpr int kFinishThreads = 1024;
+constexpr int kFinishGroups = 32;
+constexpr int kFinishBatch = 16;            // partial rows of a group whose loads are in flight together
 constexpr int kMaxA = 128;
 constexpr int kScalars = 4;               // surrogate, value loss, kl, clip count
 constexpr int kPartial = kMaxA + kScalars;
@@ -219,6 +231,7 @@ __global__ void __launch_bounds__(32 * kWarps) ppo_loss_kernel(const PpoParams P
     const int A = P.A;
     RowConsts<NI> C;
     Acc<NI> acc;
+    dep_release_wait();
     setup_lane<LPR, NI>(P, sl, C, acc);
 
     // A lane reads back only what it copied itself (element k of the three arrays); the five per-row
@@ -353,6 +366,7 @@ __global__ void __launch_bounds__(32 * bulk_warps(LPR)) ppo_loss_bulk_kernel(con
     const int TA = kTileRows * A, SF = stage_floats(A, kTileRows);
     RowConsts<NI> C;
     Acc<NI> acc;
+    dep_release_wait();
     setup_lane<LPR, NI>(P, sl, C, acc);
     if (threadIdx.x == 0) {
         mbar_init(&s_bar[0], 1);
@@ -424,28 +438,47 @@ __global__ void __launch_bounds__(32 * bulk_warps(LPR)) ppo_loss_bulk_kernel(con
     fold_and_write<LPR, NI, kBulkWarps>(acc, s_acc, P.partial + (size_t)(P.partial_begin + blockIdx.x) * kPartial);
 }
 
-// Sums the CTAs' partial rows (fp64, four interleaved groups, each in order, then the groups in order)
-// and writes d_log_std and the summary.
-__global__ void __launch_bounds__(kFinishGroups * kPartial) ppo_finish_kernel(const PpoParams P, int grid)
+// Sums the CTAs' partial rows (fp64: as many interleaved groups of rows as the block has threads for the A + kScalars
+// columns in use, each in order, then the groups in order) and writes d_log_std and the summary.  One block's time is its
+// chain of loads: 500 rows of A = 28 took 9 to 12 us in four groups
+// of one load at a time, 4.8 us now.
+__global__ void __launch_bounds__(kFinishThreads) ppo_finish_kernel(const PpoParams P, int grid)
 {
-    __shared__ double s_grp[kFinishGroups][kPartial];
+    __shared__ double s_grp[kFinishThreads];               // [groups][columns]
     __shared__ double s_tot[kPartial];
-    const int j = threadIdx.x % kPartial, q = threadIdx.x / kPartial;
-    double t = 0.0;
-    for (int g = q; g < grid; g += kFinishGroups) t += (double)P.partial[(size_t)g * kPartial + j];
-    s_grp[q][j] = t;
+    __shared__ double s_H;
+    __shared__ float s_ls[kMaxA];
+    const int cols = P.A + kScalars, groups = min(kFinishThreads / cols, kFinishGroups);
+    const int jj = (int)threadIdx.x % cols, q = (int)threadIdx.x / cols, j = jj < P.A ? jj : kMaxA + jj - P.A;
+    dep_release_wait();
+    if (q < groups) {
+        const float *col = P.partial + j;
+        double t = 0.0;
+        for (int g = q; g < grid; g += kFinishBatch * groups) {
+            float x[kFinishBatch];                          // loads in flight together, added in order
+#pragma unroll
+            for (int k = 0; k < kFinishBatch; ++k) x[k] = g + k * groups < grid ? __ldcg(col + (size_t)(g + k * groups) * kPartial) : 0.0f;
+#pragma unroll
+            for (int k = 0; k < kFinishBatch; ++k) t += (double)x[k];
+        }
+        s_grp[threadIdx.x] = t;
+        if (q == groups - 1 && jj < P.A) s_ls[jj] = __ldg(P.b.log_std + jj);
+    }
     __syncthreads();
     if (q == 0) {
-        t = 0.0;
-        for (int k = 0; k < kFinishGroups; ++k) t += s_grp[k][j];
+        double t = 0.0;
+        for (int k = 0; k < groups; ++k) t += s_grp[k * cols + jj];
         s_tot[j] = t;
-        if (j < P.A) P.d_log_std[j] = (float)(t - (double)P.cfg.entropy_coef);   // the row terms already carry 1/M
+        if (jj < P.A) P.d_log_std[jj] = (float)(t - (double)P.cfg.entropy_coef);   // the row terms already carry 1/M
+    } else if (threadIdx.x == kFinishThreads - 1) {
+        double H = 0.0;
+        for (int k = 0; k < P.A; ++k) H += (double)s_ls[k] + 0.5 * 2.8378770664093453;   // 1/2 ln(2 pi e)
+        s_H = H;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         const double M = (double)P.M;
-        double H = 0.0;
-        for (int k = 0; k < P.A; ++k) H += (double)P.b.log_std[k] + 0.5 * 2.8378770664093453;   // 1/2 ln(2 pi e)
+        const double H = s_H;
         const double surr = s_tot[kMaxA + 0] / M, vl = s_tot[kMaxA + 1] / M;
         P.summary[0] = (float)(surr + (double)P.cfg.value_coef * vl - (double)P.cfg.entropy_coef * H);
         P.summary[1] = (float)surr;
@@ -458,16 +491,21 @@ __global__ void __launch_bounds__(kFinishGroups * kPartial) ppo_finish_kernel(co
 
 // ---- moments: mean and 1 / (std + 1e-8), n - 1 divisor
 constexpr int kMomThreads = 256;
+constexpr int kMomCluster = 8;
+constexpr long long kMomClusterMax = 1 << 17;               // (64 values a thread; more than that wants more SMs)
 
-__global__ void __launch_bounds__(kMomThreads) moments_partial_kernel(const float *__restrict__ x, long long n,
-                                                                      double *__restrict__ partial)
+// This block's sums of x and x^2 over its grid stride, in thread 0.
+__device__ __forceinline__ double2 moments_of_block(const float *__restrict__ x, long long n)
 {
     __shared__ double s_sum[kMomThreads], s_sq[kMomThreads];
     double s = 0.0, q = 0.0;
-    for (long long i = (long long)blockIdx.x * kMomThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kMomThreads) {
-        const double v = (double)__ldg(x + i);
-        s += v;
-        q = fma(v, v, q);
+    const long long stride = (long long)gridDim.x * kMomThreads;
+    for (long long i = (long long)blockIdx.x * kMomThreads + threadIdx.x; i < n; i += 8 * stride) {
+        float v[8];                                         // loads in flight together
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = i + k * stride < n ? __ldg(x + i + k * stride) : 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { s += (double)v[k]; q = fma((double)v[k], (double)v[k], q); }
     }
     s_sum[threadIdx.x] = s;
     s_sq[threadIdx.x] = q;
@@ -476,26 +514,54 @@ __global__ void __launch_bounds__(kMomThreads) moments_partial_kernel(const floa
         if (threadIdx.x < o) { s_sum[threadIdx.x] += s_sum[threadIdx.x + o]; s_sq[threadIdx.x] += s_sq[threadIdx.x + o]; }
         __syncthreads();
     }
-    if (threadIdx.x == 0) { partial[2 * blockIdx.x] = s_sum[0]; partial[2 * blockIdx.x + 1] = s_sq[0]; }
+    return make_double2(s_sum[0], s_sq[0]);
 }
-
-// One warp: lane l adds partials l, l + 32, ... in order, then a butterfly in a fixed order.
-__global__ void __launch_bounds__(32) moments_finish_kernel(const double *__restrict__ partial, int grid, long long n,
-                                                            float *__restrict__ out)
+__device__ __forceinline__ void moments_write(double s, double q, long long n, float *__restrict__ out)
 {
-    double s = 0.0, q = 0.0;
-    for (int g = threadIdx.x; g < grid; g += 32) { s += partial[2 * g]; q += partial[2 * g + 1]; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        q += __shfl_xor_sync(0xffffffffu, q, o);
-    }
-    if (threadIdx.x != 0) return;
     const double mean = s / (double)n;
     double var = n > 1 ? (q - s * mean) / (double)(n - 1) : 0.0;
     var = var > 0.0 ? var : 0.0;
     out[0] = (float)mean;
     out[1] = (float)(1.0 / (sqrt(var) + 1e-8));
+}
+__global__ void __launch_bounds__(kMomThreads) moments_partial_kernel(const float *__restrict__ x, long long n,
+                                                                      double *__restrict__ partial)
+{
+    dep_release_wait();
+    const double2 t = moments_of_block(x, n);
+    if (threadIdx.x == 0) { partial[2 * blockIdx.x] = t.x; partial[2 * blockIdx.x + 1] = t.y; }
+}
+__global__ void __launch_bounds__(32) moments_finish_kernel(const double *__restrict__ partial, int grid, long long n,
+                                                            float *__restrict__ out)
+{
+    dep_release_wait();
+    double s = 0.0, q = 0.0;
+    for (int g = threadIdx.x; g < grid; g += 32) { s += __ldcg(partial + 2 * g); q += __ldcg(partial + 2 * g + 1); }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        q += __shfl_xor_sync(0xffffffffu, q, o);
+    }
+    if (threadIdx.x == 0) moments_write(s, q, n, out);
+}
+// Up to kMomClusterMax values in one launch: the blocks of one cluster, whose first reads the others' sums from their
+// shared memory.  16000 values: 7.7 us in
+// two launches whose last loads of a thread came one by one, 5.5 us.
+__global__ void __cluster_dims__(kMomCluster, 1, 1) __launch_bounds__(kMomThreads) moments_cluster_kernel(const float *__restrict__ x, long long n,
+                                                                                                          float *__restrict__ out)
+{
+    __shared__ double2 s_all[kMomCluster];                  // (the first block's is used)
+    dep_release_wait();
+    const double2 t = moments_of_block(x, n);
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();                                         // every block of the cluster has started
+    if (threadIdx.x == 0) *cluster.map_shared_rank(&s_all[blockIdx.x], 0) = t;
+    cluster.sync();
+    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    double s = 0.0, q = 0.0;
+#pragma unroll
+    for (int g = 0; g < kMomCluster; ++g) { s += s_all[g].x; q += s_all[g].y; }
+    moments_write(s, q, n, out);
 }
 
 }  // namespace
@@ -521,8 +587,14 @@ im_status im_moments(const float *x, int64_t n, float *out2, void *workspace, vo
     long long g = (n + kMomThreads * 8 - 1) / (kMomThreads * 8);
     const int grid = (int)(g < 1 ? 1 : (g > kMaxGrid ? kMaxGrid : g));
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    moments_partial_kernel<<<grid, kMomThreads, 0, st>>>(x, n, static_cast<double *>(workspace));
-    moments_finish_kernel<<<1, 32, 0, st>>>(static_cast<const double *>(workspace), grid, n, out2);
+    if (n <= kMomClusterMax) {
+        if (launch_pdl(moments_cluster_kernel, dim3(kMomCluster), dim3(kMomThreads), 0, st, 0, x, (long long)n, out2) != cudaSuccess) return IM_ERR_CUDA;
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+    }
+    if (launch_pdl(moments_partial_kernel, dim3(grid), dim3(kMomThreads), 0, st, 0, x, (long long)n, static_cast<double *>(workspace)) != cudaSuccess ||
+        launch_pdl(moments_finish_kernel, dim3(1), dim3(32), 0, st, 0, static_cast<const double *>(workspace), grid, (long long)n, out2) != cudaSuccess)
+        return IM_ERR_CUDA;
     g_launches.fetch_add(2, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
@@ -595,7 +667,9 @@ im_status im_ppo_loss(const im_ppo_config *cfg, int64_t M, int32_t A, const im_p
             const long long gb = (long long)n_sm * per_sm;                                                          \
             grid_bulk = (int)(gb > n_tiles ? n_tiles : gb);                                                         \
             if (grid_bulk > kMaxGrid) grid_bulk = kMaxGrid;                                                         \
-            ppo_loss_bulk_kernel<LPR, NI><<<grid_bulk, 32 * bulk_warps(LPR), smem, st>>>(p, n_tiles, T);            \
+            if (launch_pdl(ppo_loss_bulk_kernel<LPR, NI>, dim3(grid_bulk), dim3(32 * bulk_warps(LPR)), smem, st, 0, \
+                           p, n_tiles, T) != cudaSuccess)                                                           \
+                return IM_ERR_CUDA;                                                                                 \
         } while (0)
         IM_PPO_DISPATCH(IM_PPO_BULK)
 #undef IM_PPO_BULK
@@ -608,14 +682,18 @@ im_status im_ppo_loss(const im_ppo_config *cfg, int64_t M, int32_t A, const im_p
         long long g = (rest + kWarps * 16 - 1) / (kWarps * 16);  // a few trips per warp
         grid = (int)(g < 1 ? 1 : (g > kMaxGrid ? kMaxGrid : g));
         p.row_begin = n_tiles * T; p.partial_begin = grid_bulk;
-#define IM_PPO_LAUNCH(LPR, NI) ppo_loss_kernel<LPR, NI><<<grid, 32 * kWarps, 0, st>>>(p)
+#define IM_PPO_LAUNCH(LPR, NI)                                                                                      \
+        do {                                                                                                        \
+            if (launch_pdl(ppo_loss_kernel<LPR, NI>, dim3(grid), dim3(32 * kWarps), 0, st, 0, p) != cudaSuccess)    \
+                return IM_ERR_CUDA;                                                                                 \
+        } while (0)
         IM_PPO_DISPATCH(IM_PPO_LAUNCH)
 #undef IM_PPO_LAUNCH
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
 #undef IM_PPO_DISPATCH
     grid += grid_bulk;
-    ppo_finish_kernel<<<1, kFinishGroups * kPartial, 0, st>>>(p, grid);
+    if (launch_pdl(ppo_finish_kernel, dim3(1), dim3(kFinishThreads), 0, st, 0, p, grid) != cudaSuccess) return IM_ERR_CUDA;
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }

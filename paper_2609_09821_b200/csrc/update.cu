@@ -2,7 +2,8 @@
 //
 // A small minibatch's update is bound by launches: 16000 rows of 361-1024-512-28 (and ...-1) took 69 of them, two
 // thirds no tensor-core product, 260 us of a 552 us update.  Here each kind of step between the products is one launch
-// over every tensor of both nets: 24 launches, 354 us (131072 rows of 577-1024-1024-512-69: 3583 -> 3400 us).
+// over every tensor of both nets: 24 launches, 354 us, and 314 us with every thread's
+// loads issued in batches before anything is done with them (131072 rows of 577-1024-1024-512-69: 3583 -> 3400 us).
 #include <cmath>
 #include <cuda_bf16.h>
 
@@ -37,27 +38,42 @@ __device__ __forceinline__ bool last_block(int *done, int n_blocks)
     return s_last != 0;
 }
 
-template <typename T>
-__device__ __forceinline__ int owner(const T *t, int n, int block)
+// The tensor whose blocks include `block`.  The first blocks lie together: one by one out of the tensors' records they
+// cost a constant-cache miss each.
+__device__ __forceinline__ int owner(const int *first_block, int n, int block)
 {
     int k = 0;
-    while (k + 1 < n && block >= t[k + 1].first_block) ++k;
+    while (k + 1 < n && block >= first_block[k + 1]) ++k;
     return k;
 }
 
 // ---------------------------------------------------------------- Adam
 constexpr int kVecElems = 16 * kThreads;                    // elements of a bias tensor per block
+constexpr int kAdamBatch = 8;                               // elements of a thread whose loads are in flight together
 
-__device__ __forceinline__ float adam_update(const im_adam_config &c, const AdamTensor &T, long long i, float lr, float gs)
+// N elements `step` apart: all their loads are issued before the first store (the compiler cannot move them there).
+template <int N>
+__device__ __forceinline__ void adam_update(const im_adam_config &c, const AdamTensor &T, long long i, long long step, const bool (&on)[N],
+                                            float lr, float gs, float (&q)[N])
 {
-    const float p = T.param[i], g = gs * __ldg(T.grad + i);
-    const float m = fmaf(c.beta1, T.m[i], (1.0f - c.beta1) * g);
-    const float v = fmaf(c.beta2, T.v[i], (1.0f - c.beta2) * g * g);
-    const float q = p - lr * (m * T.inv_c1) / (sqrtf(v * T.inv_c2) + c.eps);
-    T.param[i] = q;
-    T.m[i] = m;
-    T.v[i] = v;
-    return q;
+    float p[N], g[N], m[N], v[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const long long e = on[k] ? i + k * step : 0;
+        p[k] = T.param[e]; g[k] = __ldg(T.grad + e); m[k] = T.m[e]; v[k] = T.v[e];
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const float gk = gs * g[k];
+        m[k] = fmaf(c.beta1, m[k], (1.0f - c.beta1) * gk);
+        v[k] = fmaf(c.beta2, v[k], (1.0f - c.beta2) * gk * gk);
+        q[k] = p[k] - lr * (m[k] * T.inv_c1) / (sqrtf(v[k] * T.inv_c2) + c.eps);
+        if (on[k]) {
+            T.param[i + k * step] = q[k];
+            T.m[i + k * step] = m[k];
+            T.v[i + k * step] = v[k];
+        }
+    }
 }
 
 // A block takes a 64 x 64 tile of a weight matrix -- rows are read and written as 256-byte runs, the bf16 copy goes out
@@ -66,27 +82,36 @@ __global__ void __launch_bounds__(kThreads) adam_multi_kernel(const __grid_const
 {
     __shared__ __align__(16) __nv_bfloat16 tile[64][66];    // 33-word rows: a column walk spreads over the banks
     dep_release_wait();
-    const AdamTensor &T = P.t[owner(P.t, P.n_tensors, blockIdx.x)];
+    const AdamTensor T = P.t[owner(P.first_block, P.n_tensors, blockIdx.x)];
     const int blk = (int)blockIdx.x - T.first_block;
     const float lr = *P.lr, gs = P.grad_scale ? __ldg(P.grad_scale) : 1.0f;
     if (!T.wb) {
         const int n = T.rows * T.cols, i0 = blk * kVecElems + threadIdx.x;
-#pragma unroll 4
-        for (int i = i0; i < n && i < (blk + 1) * kVecElems; i += kThreads) adam_update(P.cfg, T, i, lr, gs);
+        for (int k0 = 0; k0 < kVecElems / kThreads && i0 + k0 * kThreads < n; k0 += kAdamBatch) {
+            bool on[kAdamBatch];
+            float q[kAdamBatch];
+#pragma unroll
+            for (int k = 0; k < kAdamBatch; ++k) on[k] = i0 + (k0 + k) * kThreads < n;
+            adam_update<kAdamBatch>(P.cfg, T, i0 + k0 * kThreads, kThreads, on, lr, gs, q);
+        }
     } else {
         const int tiles_c = (T.cols + 63) >> 6, r0 = (blk / tiles_c) << 6, c0 = (blk % tiles_c) << 6;
         const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
         const bool in_c = c0 + tx < T.cols;
         __nv_bfloat16 *wb = reinterpret_cast<__nv_bfloat16 *>(T.wb);
-#pragma unroll 4
-        for (int i = ty; i < 64; i += 4) {
-            const int r = r0 + i;
-            __nv_bfloat16 h = __float2bfloat16_rn(0.0f);
-            if (in_c && r < T.rows) {
-                h = __float2bfloat16_rn(adam_update(P.cfg, T, (long long)r * T.cols + c0 + tx, lr, gs));
-                wb[(long long)r * T.ld_wb + c0 + tx] = h;
+#pragma unroll 1
+        for (int i = ty; i < 64; i += 4 * kAdamBatch) {
+            bool on[kAdamBatch];
+            float q[kAdamBatch];
+#pragma unroll
+            for (int k = 0; k < kAdamBatch; ++k) on[k] = in_c && r0 + i + 4 * k < T.rows;
+            adam_update<kAdamBatch>(P.cfg, T, (long long)(r0 + i) * T.cols + c0 + tx, 4ll * T.cols, on, lr, gs, q);
+#pragma unroll
+            for (int k = 0; k < kAdamBatch; ++k) {
+                const __nv_bfloat16 h = __float2bfloat16_rn(on[k] ? q[k] : 0.0f);
+                if (on[k]) wb[(long long)(r0 + i + 4 * k) * T.ld_wb + c0 + tx] = h;
+                tile[i + 4 * k][tx] = h;
             }
-            tile[i][tx] = h;
         }
         __syncthreads();
         __nv_bfloat16 *wbT = reinterpret_cast<__nv_bfloat16 *>(T.wbT);
@@ -109,7 +134,7 @@ __global__ void __launch_bounds__(kThreads) adam_multi_kernel(const __grid_const
 }
 
 // ---------------------------------------------------------------- gradient tensors and their norm
-constexpr int kGroupsPerBlock = 2 * kThreads;               // 4-column groups of a matrix per block
+constexpr int kBatch = 8;                                   // slices whose loads are in flight together
 constexpr int kVecCols = 32;                                // columns of a vector per block
 
 __device__ __forceinline__ double block_sum(double x)
@@ -125,63 +150,85 @@ __device__ __forceinline__ double block_sum(double x)
     return t;
 }
 
+// Bound by the latency of its loads: 16-byte words, eight slices in flight (scalar 8-byte words, at most four in flight and
+// less at the ends took 42.8 us for the 47 MB of partial products of 361-1024-512-28 and ...-1; now 16.0).
 // Sums of squares are taken in fp64 per thread and block, blocks added in a fixed order by the last one: the result does
 // not depend on scheduling.
 __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_constant__ GradReduceArgs P)
 {
     dep_release_wait();
-    const int block = blockIdx.x;
+    const int block = P.n_blocks - 1 - (int)blockIdx.x;      // (the vectors' long columns first: they would be the tail)
     double sq = 0.0;
-    const int first_vector = P.n_vectors > 0 ? P.v[0].first_block : P.n_blocks;
+    const int first_vector = P.n_vectors > 0 ? P.v_first[0] : P.n_blocks;
     if (block < first_vector) {
-        // dW: the row slices' partial products added in order
-        const GradMatrix &G = P.m[owner(P.m, P.n_matrices, block)];
-        const int gpr = (G.cols + 3) >> 2, total = G.rows * gpr;
-        const __nv_bfloat16 *in = reinterpret_cast<const __nv_bfloat16 *>(G.in);
+        // dW: the row slices' partial products added in order, eight columns a thread
+        __shared__ __align__(16) float s_out[kThreads][8];
+        const GradMatrix G = P.m[owner(P.m_first, P.n_matrices, block)];
+        const int gpr = (G.cols + 7) >> 3, i = (block - G.first_block) * kThreads + (int)threadIdx.x;
+        const bool on = i < G.rows * gpr;
+        const int r = on ? i / gpr : 0, c = on ? (i - r * gpr) << 3 : 0;
+        const uint4 *src = reinterpret_cast<const uint4 *>(G.in + (long long)r * G.ld_in + c);
+        const long long stride = G.slice_stride >> 3;
+        float a[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+        for (int s = 0; s < G.slices; s += kBatch) {
+            uint4 w[kBatch];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int i = (block - G.first_block) * kGroupsPerBlock + k * kThreads + (int)threadIdx.x;
-            if (i >= total) break;
-            const int r = i / gpr, c = (i - r * gpr) << 2;
-            const __nv_bfloat16 *src = in + (long long)r * G.ld_in + c;
-            float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 4
-            for (int s = 0; s < G.slices; ++s) {
-                const uint2 w = __ldg(reinterpret_cast<const uint2 *>(src + s * G.slice_stride));
-                const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.x));
-                const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
-                a[0] += lo.x; a[1] += lo.y; a[2] += hi.x; a[3] += hi.y;
+            for (int k = 0; k < kBatch; ++k) w[k] = s + k < G.slices ? __ldg(src + (s + k) * stride) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) {
+                const uint32_t x[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x[j]));
+                    a[2 * j] += f.x;
+                    a[2 * j + 1] += f.y;
+                }
             }
-            float *dst = G.out + (long long)r * G.cols + c;
-            if ((G.cols & 3) == 0) {
-                *reinterpret_cast<float4 *>(dst) = make_float4(a[0], a[1], a[2], a[3]);
-            } else {
+        }
+        const int n = on ? min(G.cols - c, 8) : 0;            // columns of this thread
+        const long long o = (long long)r * G.cols + c;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (c + j < G.cols) dst[j] = a[j];
+        for (int j = 0; j < 8; ++j)
+            if (j < n) sq = fma((double)a[j], (double)a[j], sq);
+        if ((G.cols & 7) == 0) {
+            if (on) {
+                *reinterpret_cast<float4 *>(G.out + o) = make_float4(a[0], a[1], a[2], a[3]);
+                *reinterpret_cast<float4 *>(G.out + o + 4) = make_float4(a[4], a[5], a[6], a[7]);
             }
+        } else {
+            // rows that do not start on 32-byte boundaries: the warp's 32 x 8 values leave in the order of memory
+            const int lane = threadIdx.x & 31, w0 = threadIdx.x & ~31;
+            *reinterpret_cast<float4 *>(s_out[threadIdx.x]) = make_float4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<float4 *>(s_out[threadIdx.x] + 4) = make_float4(a[4], a[5], a[6], a[7]);
+            __syncwarp();
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (c + j < G.cols) sq = fma((double)a[j], (double)a[j], sq);
+            for (int k = 0; k < 8; ++k) {
+                const int from = 4 * k + (lane >> 3);
+                const long long of = __shfl_sync(0xffffffffu, o, from);
+                const int nf = __shfl_sync(0xffffffffu, n, from);
+                if ((lane & 7) < nf) G.out[of + (lane & 7)] = s_out[w0 + from][lane & 7];
+            }
         }
     } else if (P.n_vectors > 0 && block < P.n_blocks - (P.n_extra > 0 ? 1 : 0)) {
-        // db: 32 columns, 32 groups of rows in fp32 (four chains each), the groups added in order in fp64
+        // db: 32 columns, 32 groups of rows in fp32 (two chains each), the groups added in order in fp64
         __shared__ double s_col[32][kVecCols + 1];
-        const GradVector &G = P.v[owner(P.v, P.n_vectors, block)];
+        const GradVector G = P.v[owner(P.v_first, P.n_vectors, block)];
         const int cg = threadIdx.x & 7, rg = threadIdx.x >> 3, c = (block - G.first_block) * kVecCols + 4 * cg;
         float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
         if (c < G.ld) {
-            int r = rg;
-#pragma unroll 2
-            for (; r + 32 < G.n_rows; r += 64) {
-                const float4 x = __ldg(reinterpret_cast<const float4 *>(G.in + (long long)r * G.ld + c));
-                const float4 y = __ldg(reinterpret_cast<const float4 *>(G.in + (long long)(r + 32) * G.ld + c));
-                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
-                b.x += y.x; b.y += y.y; b.z += y.z; b.w += y.w;
-            }
-            if (r < G.n_rows) {
-                const float4 x = __ldg(reinterpret_cast<const float4 *>(G.in + (long long)r * G.ld + c));
-                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+#pragma unroll 1
+            for (int r = rg; r < G.n_rows; r += 8 * 32) {
+                float4 x[8];                                  // loads in flight together
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    x[k] = r + 32 * k < G.n_rows ? __ldg(reinterpret_cast<const float4 *>(G.in + (long long)(r + 32 * k) * G.ld + c))
+                                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+                for (int k = 0; k < 8; k += 2) {
+                    a.x += x[k].x; a.y += x[k].y; a.z += x[k].z; a.w += x[k].w;
+                    b.x += x[k + 1].x; b.y += x[k + 1].y; b.z += x[k + 1].z; b.w += x[k + 1].w;
+                }
             }
         }
         s_col[rg][4 * cg] = (double)(a.x + b.x); s_col[rg][4 * cg + 1] = (double)(a.y + b.y);
@@ -228,7 +275,7 @@ __global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_consta
     const int r0 = blockIdx.x * kOutRows, r1 = min(r0 + kOutRows, P.M);
     __nv_bfloat16 *dz = reinterpret_cast<__nv_bfloat16 *>(G.dz);
     float s0 = 0.0f, s1 = 0.0f;
-#pragma unroll 8
+#pragma unroll 16
     for (int r = r0 + g; r < r1; r += groups) {
         const float *src = G.d_out + (long long)r * G.cols + c;
         const float a = c < G.cols ? __ldg(src) : 0.0f, b = c + 1 < G.cols ? __ldg(src + 1) : 0.0f;
@@ -293,6 +340,7 @@ __global__ void __launch_bounds__(kThreads) gather_minibatch_kernel(const __grid
 void adam_multi_add(AdamMultiArgs &a, float *param, const float *grad, float *m, float *v, int rows, int cols, uint16_t *wb, int ld_wb,
                     uint16_t *wbT, int ld_wbT, int t)
 {
+    a.first_block[a.n_tensors] = a.n_blocks;
     AdamTensor &T = a.t[a.n_tensors++];
     T.param = param; T.grad = grad; T.m = m; T.v = v; T.wb = wb; T.wbT = wbT;
     T.rows = rows; T.cols = cols; T.ld_wb = ld_wb; T.ld_wbT = ld_wbT;
@@ -309,17 +357,19 @@ cudaError_t launch_adam_multi(AdamMultiArgs &a, cudaStream_t stream)
     return e;
 }
 
-int grad_matrix_blocks(int rows, int cols) { return (int)(((long long)rows * ((cols + 3) / 4) + kGroupsPerBlock - 1) / kGroupsPerBlock); }
+int grad_matrix_blocks(int rows, int cols) { return (int)(((long long)rows * ((cols + 7) / 8) + kThreads - 1) / kThreads); }
 int grad_vector_blocks(int cols) { return (cols + kVecCols - 1) / kVecCols; }
 
 // (all matrices are added before the first vector)
 void grad_reduce_add(GradReduceArgs &a, const uint16_t *in, long long slice_stride, int ld_in, int slices, int rows, int cols, float *out)
 {
+    a.m_first[a.n_matrices] = a.n_blocks;
     a.m[a.n_matrices++] = {in, out, slice_stride, ld_in, slices, rows, cols, a.n_blocks};
     a.n_blocks += grad_matrix_blocks(rows, cols);
 }
 void grad_reduce_add(GradReduceArgs &a, const float *in, int n_rows, int ld, int cols, float *out)
 {
+    a.v_first[a.n_vectors] = a.n_blocks;
     a.v[a.n_vectors++] = {in, out, n_rows, ld, cols, a.n_blocks};
     a.n_blocks += grad_vector_blocks(cols);
 }

@@ -20,6 +20,7 @@ struct AdamTensor {
 };
 struct AdamMultiArgs {
     AdamTensor t[2 * kMaxNetTensors + 1];
+    int first_block[2 * kMaxNetTensors + 1];               // (of t, together)
     int n_tensors, n_blocks;
     im_adam_config cfg;
     float *lr;
@@ -48,6 +49,7 @@ struct GradVector {
 struct GradReduceArgs {
     GradMatrix m[kMaxNetTensors];
     GradVector v[kMaxNetTensors];
+    int m_first[kMaxNetTensors], v_first[kMaxNetTensors];  // first blocks of m and v, together
     int n_matrices, n_vectors, n_blocks;
     const float *extra;
     int n_extra;

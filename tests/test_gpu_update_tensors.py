@@ -73,3 +73,17 @@ def test_rollout_update_clip_factor_and_summary(T_, N, mb, shuffled):
     assert norm * 0.9 <= norm2 ** 0.5 <= norm * (1 + 1e-6) and bool(torch.isfinite(upd.summary).all())
     assert abs(float(upd.scale[0]) - min(1.0, 1.0 / (norm + 1e-6))) <= 1e-6
     assert a.device_status() == 0 and c.device_status() == 0
+
+
+@pytest.mark.parametrize("n", [1, 2, 255, 2049, 16000, 2 ** 17, 2 ** 17 + 1, 300001])
+def test_moments_of_any_length(n):
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    x = 3.0 + 2.0 * torch.randn(n + 8, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    out, ws = torch.empty(2, device="cuda"), B.ppo_workspace()
+    B.moments(x[:n], out, ws)
+    got = out.cpu().numpy().astype(np.float64)
+    ref = x[:n].cpu().numpy().astype(np.float64)
+    std = ref.std(ddof=1) if n > 1 else 0.0
+    want = np.array([ref.mean(), 1.0 / (std + 1e-8)])
+    assert np.all(np.abs(got - want) <= 2e-7 * np.abs(want))         # fp64 sums, one rounding to fp32
