@@ -39,14 +39,25 @@ im_status tc_policy_forward(im_policy *p, uint32_t step, int32_t n, const float 
 bool tc_can_pair_nets(const im_policy *a, const im_policy *c, int n);
 im_status tc_policy_value_forward(im_policy *a, im_policy *c, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
                                   float *mean_out, float *action_out, float *logp_out, float *value_out);
-im_status tc_gemm(const void *A, int64_t lda, const void *B, int64_t ldb, void *C, int64_t ldc, int M, int N, int K,
-                  const float *bias, bool relu, uint32_t *status, cudaStream_t stream, int batches = 1,
-                  const void *mask = nullptr, int64_t ld_mask = 0, float *colsum_partial = nullptr, int ld_partial = 0);
-int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm);
-im_status tc_gemm_tn(const void *A, int64_t lda, const void *B, int64_t ldb, void *C, int64_t ldc, int R, int Mo, int No,
-                     int slices, int c_pitch, uint32_t *status, cudaStream_t stream);
-im_status tc_gemm_head(const void *A, int64_t lda, const void *B, int64_t ldb, int M, int N, int K, const float *bias,
-                       float *mean_out, uint32_t *status, cudaStream_t stream);
+// Operands of a tensor-core product; colsum_partial, mask: its backward epilogue (see GemmParams).
+struct GemmOperands {
+    const void *A;
+    int64_t lda;
+    const void *B;
+    int64_t ldb;
+    void *C;
+    int64_t ldc;
+    const float *bias;
+    const void *mask;
+    int64_t ld_mask;
+    float *colsum_partial;
+};
+im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status,
+                  cudaStream_t stream);
+int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm, int nets);
+im_status tc_gemm_tn(const GemmOperands &x, const GemmOperands *y, int R, int Mo, int No, int slices, int c_pitch, uint32_t *status,
+                     cudaStream_t stream);
+im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int N, int N2, int K, uint32_t *status, cudaStream_t stream);
 // bounded-wait diagnostics of the tensor-core GEMM kernels and of the bulk-copy PPO loss kernel (current device)
 cudaError_t tc_set_wait_debug(unsigned long long limit_ns, int skip_loads);
 cudaError_t ppo_set_wait_debug(unsigned long long limit_ns, int skip_loads);

@@ -194,10 +194,8 @@ struct GemmParams {
     int bufs;          // head: staging buffers
     const float *bias; // [n_tiles_n * BLOCK_N], zero padded
     float act_floor;   // hidden-layer epilogue: out = max(acc + bias, act_floor); 0 is ReLU, -inf no activation
-    // Batched products on the single-CTA hidden kernel: batch b multiplies rows [b a_batch_rows, +M) of A
-    // with rows [b b_batch_rows, +N) of B into rows [b a_batch_rows, +M) of C.  n_batches = 1: plain GEMM.
-    int n_batches, a_batch_rows, b_batch_rows;
-    int c_batch_rows;  // rows of C between two batches
+    int n_batches;     // M/N-major products: slices of the contraction, each with its own output; else 1
+    int c_batch_rows;  // rows of C between two slices
     // M/N-major products: the contraction's kb_total k-blocks are shared out over the batches ("slices") as evenly as
     // whole k-blocks allow, slice b taking [b kb_total / n_batches, (b + 1) kb_total / n_batches)
     int kb_total;
@@ -208,9 +206,11 @@ struct GemmParams {
     long long ld_mask;
     float *colsum_partial;
     int ld_partial;
-    // Two nets of equal hidden widths in one launch (DUAL instantiations): tiles [0, n) are the first net's, the rest the
-    // second's, which has operand and output maps of its own; its head is a value head (no sampling).
+    // Two nets' products of equal sizes in one launch (DUAL instantiations): the first half of the tiles is the first net's,
+    // the second half the second's, which has operand, output and mask maps of its own; its head is a value head (no
+    // sampling) and may have fewer columns.
     const float *bias2;
+    float *colsum_partial2;
     int N2;
     float *mean2;
     // Gaussian head
@@ -268,6 +268,21 @@ __device__ __forceinline__ void slice_k_blocks(const GemmParams &P, int b, int &
     if (!MN) { kb0 = 0; n_kb = P.K_blocks; return; }
     kb0 = (int)((long long)b * P.kb_total / P.n_batches);
     n_kb = (int)((long long)(b + 1) * P.kb_total / P.n_batches) - kb0;
+}
+
+// Which output tile the number `tile` stands for: net, slice, row and column of tiles.
+struct TileAt {
+    bool second;
+    int slice, m, n;
+};
+template <bool MN, bool DUAL>
+__device__ __forceinline__ TileAt tile_at(const GemmParams &P, int tile, int tiles_per_slice)
+{
+    const int net_tiles = MN ? tiles_per_slice * P.n_batches : tiles_per_slice;
+    const bool second = DUAL && tile >= net_tiles;
+    if (second) tile -= net_tiles;
+    const int slice = MN ? tile / tiles_per_slice : 0, t = tile - slice * tiles_per_slice, m = t / P.n_tiles_n;
+    return {second, slice, m, t - m * P.n_tiles_n};
 }
 
 struct Pipe {
@@ -335,37 +350,36 @@ __device__ __forceinline__ void pipe_exit(const Pipe &p, uint32_t tmem_base, uin
 // TMA producer (one thread): A and W tiles of every k-block of every tile of this CTA.
 template <class Plan, int BLOCK_N, bool MN = false, bool DUAL = false>
 __device__ __forceinline__ void producer_role(const Pipe &p, const CUtensorMap *map_a, const CUtensorMap *map_b,
-                                              const GemmParams &P, int n_tiles, const CUtensorMap *map_a2 = nullptr,
-                                              const CUtensorMap *map_b2 = nullptr)
+                                              const GemmParams &P, int n_tiles, int tiles_per_slice,
+                                              const CUtensorMap *map_a2 = nullptr, const CUtensorMap *map_b2 = nullptr)
 {
     int stage = 0;
     uint32_t phase = 0;
-    const int tiles_per_batch = n_tiles / P.n_batches;
     if (g_skip_loads) return;                        // diagnostic: the consumers' first wait runs out
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int b = tile / tiles_per_batch, t = tile - b * tiles_per_batch;
+        const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
+        const CUtensorMap *ma = at.second ? map_a2 : map_a, *mb = at.second ? map_b2 : map_b;
         if (MN) {
             // operands are [contraction rows][M or N columns]: a K block is 64 rows, fetched as boxes of 64 columns;
             // batch b is a range of the k-blocks of both operands
             int kb0, n_kb;
-            slice_k_blocks<true>(P, b, kb0, n_kb);
-            const int mm = (t / P.n_tiles_n) * BLOCK_M, nn = (t % P.n_tiles_n) * BLOCK_N, r0 = kb0 * BLOCK_K;
+            slice_k_blocks<true>(P, at.slice, kb0, n_kb);
+            const int mm = at.m * BLOCK_M, nn = at.n * BLOCK_N, r0 = kb0 * BLOCK_K;
             for (int kb = 0; kb < n_kb; ++kb) {
                 if (!mbar_wait(&p.empty[stage], phase ^ 1u, p.abort_flag)) return;
                 uint8_t *sa = p.tiles + (size_t)stage * Plan::kStageBytes;
                 mbar_arrive_expect_tx(&p.full[stage], Plan::kABytes + Plan::kBBytes);
 #pragma unroll
                 for (int i = 0; i < BLOCK_M / 64; ++i)
-                    tma_load_2d(sa + i * 8192, map_a, &p.full[stage], mm + 64 * i, r0 + kb * BLOCK_K);
+                    tma_load_2d(sa + i * 8192, ma, &p.full[stage], mm + 64 * i, r0 + kb * BLOCK_K);
 #pragma unroll
                 for (int i = 0; i < BLOCK_N / 64; ++i)
-                    tma_load_2d(sa + Plan::kABytes + i * 8192, map_b, &p.full[stage], nn + 64 * i, r0 + kb * BLOCK_K);
+                    tma_load_2d(sa + Plan::kABytes + i * 8192, mb, &p.full[stage], nn + 64 * i, r0 + kb * BLOCK_K);
                 if (++stage == p.stages) { stage = 0; phase ^= 1u; }
             }
             continue;
         }
-        const int m0 = b * P.a_batch_rows + (t / P.n_tiles_n) * BLOCK_M, n0 = b * P.b_batch_rows + (t % P.n_tiles_n) * BLOCK_N;
-        const CUtensorMap *ma = DUAL && b ? map_a2 : map_a, *mb = DUAL && b ? map_b2 : map_b;
+        const int m0 = at.m * BLOCK_M, n0 = at.n * BLOCK_N;
         for (int kb = 0; kb < P.K_blocks; kb += Plan::kDepth) {
             if (!mbar_wait(&p.empty[stage], phase ^ 1u, p.abort_flag)) return;
             uint8_t *sa = p.tiles + (size_t)stage * Plan::kStageBytes;
@@ -381,8 +395,8 @@ __device__ __forceinline__ void producer_role(const Pipe &p, const CUtensorMap *
 }
 
 // MMA issuer (one thread).
-template <class Plan, int BLOCK_N, bool MN = false>
-__device__ __forceinline__ void mma_role(const Pipe &p, uint32_t tmem_base, const GemmParams &P, int n_tiles)
+template <class Plan, int BLOCK_N, bool MN = false, bool DUAL = false>
+__device__ __forceinline__ void mma_role(const Pipe &p, uint32_t tmem_base, const GemmParams &P, int n_tiles, int tiles_per_slice)
 {
     constexpr uint32_t idesc = MN ? instr_desc_bf16_mn(BLOCK_M, BLOCK_N) : instr_desc_bf16(BLOCK_M, BLOCK_N);
     int stage = 0, acc = 0;
@@ -392,7 +406,7 @@ __device__ __forceinline__ void mma_role(const Pipe &p, uint32_t tmem_base, cons
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * Plan::kAccStride);
         int kb0, n_kb;
-        slice_k_blocks<MN>(P, MN ? tile / (n_tiles / P.n_batches) : 0, kb0, n_kb);
+        slice_k_blocks<MN>(P, MN ? tile_at<MN, DUAL>(P, tile, tiles_per_slice).slice : 0, kb0, n_kb);
         for (int kb = 0; kb < n_kb; kb += Plan::kDepth) {
             if (!mbar_wait(&p.full[stage], phase, p.abort_flag)) return;
             tc_fence_after();
@@ -463,7 +477,7 @@ __device__ __forceinline__ void mask_all_positive(uint4 (&mk)[8])
 
 template <bool BWD>
 __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_addr, int row, int col0, int lane,
-                                             const uint4 (&mk)[8], uint32_t (&pk)[32], const float *bias)
+                                             const uint4 (&mk)[8], uint32_t (&pk)[32], const float *bias, float *colsum)
 {
     float v[64];
     tmem_ld32_issue(t_addr, v);
@@ -502,7 +516,7 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
         pk[i] = *reinterpret_cast<const uint32_t *>(&h);
     }
     if (BWD) {
-        if (P.colsum_partial) {
+        if (colsum) {
             reduce_scatter_step<32>(v, lane, 16);
             reduce_scatter_step<16>(v, lane, 8);
             reduce_scatter_step<8>(v, lane, 4);
@@ -510,7 +524,7 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
             reduce_scatter_step<2>(v, lane, 1);
             const int row0 = row - lane;                 // lane now holds columns 2 lane, 2 lane + 1 of the 64
             if (row0 < P.M)
-                *reinterpret_cast<float2 *>(P.colsum_partial + (long long)(row0 >> 5) * P.ld_partial + col0 + 2 * lane) =
+                *reinterpret_cast<float2 *>(colsum + (long long)(row0 >> 5) * P.ld_partial + col0 + 2 * lane) =
                     make_float2(v[0], v[1]);
         }
     }
@@ -522,10 +536,10 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
 // into a 128B-swizzled slab in shared memory and hands the slab to a TMA store.
 constexpr __host__ __device__ int hidden_depth(int block_n, bool mn, bool bwd) { return block_n < 256 && !mn && !bwd ? 2 : 1; }
 
-// Kernel parameters of the second net of a DUAL launch.
+// Kernel parameters of the second net of a DUAL launch (m: mask, as map_m).
 struct NoMaps {};
 struct DualMaps {
-    CUtensorMap a, b, c;
+    CUtensorMap a, b, c, m;
 };
 template <bool DUAL>
 using SecondNet = std::conditional_t<DUAL, DualMaps, NoMaps>;
@@ -542,8 +556,10 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
     extern __shared__ uint8_t smem_raw[];
     const Pipe p = carve_pipe<Plan>(smem_raw, P.stages, Plan::hidden_epi_bytes(BWD));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles_per_batch = ((P.M + BLOCK_M - 1) / BLOCK_M) * P.n_tiles_n;
-    const int n_tiles = tiles_per_batch * P.n_batches;
+    const int tiles_per_slice = ((P.M + BLOCK_M - 1) / BLOCK_M) * P.n_tiles_n;
+    const int n_tiles = tiles_per_slice * (MN ? P.n_batches : 1) * (DUAL ? 2 : 1);
+    const CUtensorMap *map_c2 = &map_c, *map_m2 = &map_m;
+    if constexpr (DUAL) { map_c2 = &second.c; map_m2 = &second.m; }
     pipe_init<Plan>(p, hidden_epi_warps(BLOCK_N, BWD));
     const uint32_t tmem_base = *p.tmem_slot;
     dep_release();
@@ -551,11 +567,11 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
 
     if (warp == 0) {
         if (lane == 0) {
-            if constexpr (DUAL) producer_role<Plan, BLOCK_N, MN, true>(p, &map_a, &map_b, P, n_tiles, &second.a, &second.b);
-            else producer_role<Plan, BLOCK_N, MN>(p, &map_a, &map_b, P, n_tiles);
+            if constexpr (DUAL) producer_role<Plan, BLOCK_N, MN, true>(p, &map_a, &map_b, P, n_tiles, tiles_per_slice, &second.a, &second.b);
+            else producer_role<Plan, BLOCK_N, MN>(p, &map_a, &map_b, P, n_tiles, tiles_per_slice);
         }
     } else if (warp == 1) {
-        if (lane == 0) mma_role<Plan, BLOCK_N, MN>(p, tmem_base, P, n_tiles);
+        if (lane == 0) mma_role<Plan, BLOCK_N, MN, DUAL>(p, tmem_base, P, n_tiles, tiles_per_slice);
     } else {
         const int quad = warp & 3;                    // TMEM lanes 32*quad .. 32*quad+31 belong to this warp
         constexpr bool kFour = hidden_epi_warps(BLOCK_N, BWD) == 4;
@@ -574,12 +590,12 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
         bool bail = false;
         uint4 mk[8];
         if (masked && (int)blockIdx.x < n_tiles && lane == 0) {
-            const int bt = (int)blockIdx.x / tiles_per_batch, tt = (int)blockIdx.x - bt * tiles_per_batch;
-            mask_issue(&map_m, mslabs, &mbar[0], (tt % P.n_tiles_n) * BLOCK_N, bt * P.c_batch_rows + (tt / P.n_tiles_n) * BLOCK_M + quad * 32);
+            const TileAt at = tile_at<MN, DUAL>(P, blockIdx.x, tiles_per_slice);
+            mask_issue(at.second ? map_m2 : &map_m, mslabs, &mbar[0], at.n * BLOCK_N, at.m * BLOCK_M + quad * 32);
         }
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-            const int bt = tile / tiles_per_batch, tt = tile - bt * tiles_per_batch;
-            const int m0 = bt * P.c_batch_rows + (tt / P.n_tiles_n) * BLOCK_M, n0 = (tt % P.n_tiles_n) * BLOCK_N;
+            const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
+            const int m0 = at.slice * P.c_batch_rows + at.m * BLOCK_M, n0 = at.n * BLOCK_N;
             bool ready = mbar_wait(&p.acc_full[acc], acc_phase, p.abort_flag);
             if (BWD) ready = __all_sync(0xffffffffu, ready);           // the column sums shuffle across the whole warp
             if (!ready) break;
@@ -592,11 +608,11 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
                     if (masked) {
                         if (lane == 0) {
                             uint8_t *nslab = mslabs + ((ci + 1u) & 1u) * kEpiSlabBytes;
-                            if (c0 + 64 < BLOCK_N) mask_issue(&map_m, nslab, &mbar[(ci + 1u) & 1u], n0 + c0 + 64, m0 + quad * 32);
+                            if (c0 + 64 < BLOCK_N) mask_issue(at.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], n0 + c0 + 64, m0 + quad * 32);
                             else if (tile + (int)gridDim.x < n_tiles) {
-                                const int t2 = tile + (int)gridDim.x, bt2 = t2 / tiles_per_batch, tt2 = t2 - bt2 * tiles_per_batch;
-                                mask_issue(&map_m, nslab, &mbar[(ci + 1u) & 1u], (tt2 % P.n_tiles_n) * BLOCK_N,
-                                           bt2 * P.c_batch_rows + (tt2 / P.n_tiles_n) * BLOCK_M + quad * 32);
+                                const TileAt next = tile_at<MN, DUAL>(P, tile + (int)gridDim.x, tiles_per_slice);
+                                mask_issue(next.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], next.n * BLOCK_N,
+                                           next.m * BLOCK_M + quad * 32);
                             }
                         }
                         if (!__all_sync(0xffffffffu, mbar_wait(&mbar[ci & 1u], (ci >> 1) & 1u, p.abort_flag))) { bail = true; break; }
@@ -604,7 +620,8 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
                         ++ci;
                     } else mask_all_positive(mk);
                 }
-                hidden_chunk<BWD>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, DUAL && bt ? P.bias2 : P.bias);
+                hidden_chunk<BWD>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, at.second ? P.bias2 : P.bias,
+                                  at.second ? P.colsum_partial2 : P.colsum_partial);
                 // the last store from this slab must have finished reading shared memory
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSlabs - 1) : "memory");
                 __syncwarp();
@@ -619,10 +636,8 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) {
-                    const CUtensorMap *mc = &map_c;
-                    if constexpr (DUAL) mc = bt ? &second.c : &map_c;
                     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                 ::"l"(mc), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
+                                 ::"l"(at.second ? map_c2 : &map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
                     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                 }
                 if (kSlabs == 2) which ^= 1;
@@ -725,11 +740,11 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t *bar)
 
 // MN: both operands are stored [contraction rows][M or N columns] (the transposed product of two row-major
 // matrices, as in the single-CTA kernel's MN instantiation), possibly over several row slices ("batches").
-template <bool BWD = false, bool MN = false>
+template <bool BWD = false, bool MN = false, bool DUAL = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads(BWD), 1)
 linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                              const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_m,
-                             const GemmParams P)
+                             const GemmParams P, const __grid_constant__ SecondNet<DUAL> second)
 {
     constexpr int kStages = pair_stages(BWD);
     constexpr int kEpi = pair_epi_warps(BWD);
@@ -747,8 +762,10 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
     const uint32_t rank = cluster_rank();
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
     const int tiles_m = (P.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M);
-    const int tiles_per_batch = tiles_m * P.n_tiles_n;               // 256 x 256 tiles
-    const int n_tiles = tiles_per_batch * (MN ? P.n_batches : 1);
+    const int tiles_per_slice = tiles_m * P.n_tiles_n;               // 256 x 256 tiles
+    const int n_tiles = tiles_per_slice * (MN ? P.n_batches : 1) * (DUAL ? 2 : 1);
+    const CUtensorMap *map_a2 = &map_a, *map_b2 = &map_b, *map_c2 = &map_c, *map_m2 = &map_m;
+    if constexpr (DUAL) { map_a2 = &second.a; map_b2 = &second.b; map_c2 = &second.c; map_m2 = &second.m; }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -780,12 +797,13 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
             int stage = 0;
             uint32_t phase = 0;
             for (int tile = pair; tile < n_tiles; tile += n_pairs) {
-                const int bt = MN ? tile / tiles_per_batch : 0, tt = tile - bt * tiles_per_batch;
-                const int m0 = (tt / P.n_tiles_n) * 2 * BLOCK_M + (int)rank * BLOCK_M;
-                const int n0 = (tt % P.n_tiles_n) * 256 + (int)rank * 128;
+                const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
+                const CUtensorMap *ma = at.second ? map_a2 : &map_a, *mb = at.second ? map_b2 : &map_b;
+                const int m0 = at.m * 2 * BLOCK_M + (int)rank * BLOCK_M;
+                const int n0 = at.n * 256 + (int)rank * 128;
                 bool ok = true;
                 int kb0, n_kb;
-                slice_k_blocks<MN>(P, bt, kb0, n_kb);
+                slice_k_blocks<MN>(P, at.slice, kb0, n_kb);
                 for (int kb = 0; kb < n_kb; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t *sa = tiles + (size_t)stage * kPairStageBytes;
@@ -796,12 +814,12 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                         const int r = (kb0 + kb) * BLOCK_K;
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
-                            tma_load_2d_pair(sa + i * 8192, &map_a, leader_full, m0 + 64 * i, r);
-                            tma_load_2d_pair(sa + BLOCK_M * BLOCK_K * 2 + i * 8192, &map_b, leader_full, n0 + 64 * i, r);
+                            tma_load_2d_pair(sa + i * 8192, ma, leader_full, m0 + 64 * i, r);
+                            tma_load_2d_pair(sa + BLOCK_M * BLOCK_K * 2 + i * 8192, mb, leader_full, n0 + 64 * i, r);
                         }
                     } else {
-                        tma_load_2d_pair(sa, &map_a, leader_full, kb * BLOCK_K, m0);
-                        tma_load_2d_pair(sa + BLOCK_M * BLOCK_K * 2, &map_b, leader_full, kb * BLOCK_K, n0);
+                        tma_load_2d_pair(sa, ma, leader_full, kb * BLOCK_K, m0);
+                        tma_load_2d_pair(sa + BLOCK_M * BLOCK_K * 2, mb, leader_full, kb * BLOCK_K, n0);
                     }
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
@@ -820,7 +838,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 256);
                 int kb0, n_kb;
-                slice_k_blocks<MN>(P, MN ? tile / tiles_per_batch : 0, kb0, n_kb);
+                slice_k_blocks<MN>(P, MN ? tile_at<MN, DUAL>(P, tile, tiles_per_slice).slice : 0, kb0, n_kb);
                 for (int kb = 0; kb < n_kb; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
@@ -855,16 +873,16 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
             uint4 mk[8];                                // unused without the backward epilogue
             if (!*abort_flag)
             for (int tile = pair; tile < n_tiles; tile += n_pairs) {
-                const int bt = MN ? tile / tiles_per_batch : 0, tt = tile - bt * tiles_per_batch;
-                const int m0 = bt * P.c_batch_rows + (tt / P.n_tiles_n) * 2 * BLOCK_M + (int)rank * BLOCK_M;
-                const int n0 = (tt % P.n_tiles_n) * 256;
+                const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
+                const int m0 = at.slice * P.c_batch_rows + at.m * 2 * BLOCK_M + (int)rank * BLOCK_M;
+                const int n0 = at.n * 256;
                 if (!mbar_wait(&acc_full[acc], acc_phase, abort_flag)) break;
                 tc_fence_after();
                 const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 256);
 #pragma unroll 1
                 for (int c0 = 0; c0 < 256; c0 += 64) {
                     uint32_t pk[32];
-                    hidden_chunk<false>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, P.bias);
+                    hidden_chunk<false>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, at.second ? P.bias2 : P.bias, nullptr);
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                     __syncwarp();
                     uint8_t *slab = slabs + which * kEpiSlabBytes;
@@ -879,7 +897,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                     __syncwarp();
                     if (lane == 0) {
                         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                     ::"l"(&map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
+                                     ::"l"(at.second ? map_c2 : &map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                     which ^= 1;
@@ -902,15 +920,16 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
             auto issue_mask = [&](uint32_t j) {
                 const int t2 = pair + (int)(j >> 1) * n_pairs;
                 if (t2 >= n_tiles) return;
-                mask_issue(&map_m, ring + (j % kPairRing) * kEpiSlabBytes, &mbar[j % kPairRing],
-                           (t2 % P.n_tiles_n) * 256 + (2 * half + (int)(j & 1u)) * 64,
-                           (t2 / P.n_tiles_n) * 2 * BLOCK_M + (int)rank * BLOCK_M + quad * 32);
+                const TileAt at = tile_at<MN, DUAL>(P, t2, tiles_per_slice);
+                mask_issue(at.second ? map_m2 : &map_m, ring + (j % kPairRing) * kEpiSlabBytes, &mbar[j % kPairRing],
+                           at.n * 256 + (2 * half + (int)(j & 1u)) * 64, at.m * 2 * BLOCK_M + (int)rank * BLOCK_M + quad * 32);
             };
             if (masked && lane == 0 && !*abort_flag) issue_mask(0u);
             if (!*abort_flag)
             for (int tile = pair; tile < n_tiles; tile += n_pairs) {
-                const int m0 = (tile / P.n_tiles_n) * 2 * BLOCK_M + (int)rank * BLOCK_M;
-                const int n0 = (tile % P.n_tiles_n) * 256;
+                const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
+                const int m0 = at.m * 2 * BLOCK_M + (int)rank * BLOCK_M;
+                const int n0 = at.n * 256;
                 // (the column sums shuffle across the whole warp: every lane takes the same decision)
                 if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[acc], acc_phase, abort_flag))) break;
                 tc_fence_after();
@@ -930,7 +949,8 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                         mask_read(slab, lane, mk);
                     } else mask_all_positive(mk);
                     uint32_t pk[32];
-                    hidden_chunk<true>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, P.bias);
+                    hidden_chunk<true>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, at.second ? P.bias2 : P.bias,
+                                       at.second ? P.colsum_partial2 : P.colsum_partial);
                     // each lane overwrites the 128 bytes it read its own mask words from
                     const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
 #pragma unroll
@@ -943,7 +963,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                     __syncwarp();
                     if (lane == 0) {
                         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                     ::"l"(&map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
+                                     ::"l"(at.second ? map_c2 : &map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(m0 + quad * 32) : "memory");
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                     ++ci;
@@ -1036,12 +1056,12 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
     if (warp == 0) {
         dep_wait();                   // nothing before this line touches global memory
         if (lane == 0) {
-            if constexpr (DUAL) producer_role<Plan, BLOCK_N, false, true>(p, &map_a, &map_b, P, n_tiles, &second.a, &second.b);
-            else producer_role<Plan, BLOCK_N>(p, &map_a, &map_b, P, n_tiles);
+            if constexpr (DUAL) producer_role<Plan, BLOCK_N, false, true>(p, &map_a, &map_b, P, n_tiles, net_tiles, &second.a, &second.b);
+            else producer_role<Plan, BLOCK_N>(p, &map_a, &map_b, P, n_tiles, net_tiles);
         }
     } else if (warp == 1) {
         dep_wait();
-        if (lane == 0) mma_role<Plan, BLOCK_N>(p, tmem_base, P, n_tiles);
+        if (lane == 0) mma_role<Plan, BLOCK_N>(p, tmem_base, P, n_tiles, net_tiles);
     } else {
         const int quad = warp & 3;                                  // 32-row band of the tile (TMEM lane quadrant)
         const int group = (warp - 2) >> 2;                          // 16-column groups group, group+4, ...
@@ -1274,86 +1294,44 @@ namespace im {
 
 namespace {
 
-template <int BLOCK_N, bool BWD = false>
-cudaError_t launch_hidden(const TcLayer &L, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
+// L2: the second net's layer of a launch for two (DUAL), else null.
+template <int BLOCK_N, bool MN, bool BWD, bool DUAL>
+cudaError_t launch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
 {
-    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, false, BWD)>;
-    static DeviceOnce once;                      // the attribute is per device
-    {
-        const cudaError_t e = once.run([] { return cudaFuncSetAttribute(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kSmemLimit); });
-        if (e != cudaSuccess) return e;
-    }
-    GemmParams gp = gp_in;
-    gp.stages = Plan::stages_for(Plan::hidden_epi_bytes(BWD));
-    const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes(BWD));
-    const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
-    const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, false, BWD>, dim3(grid), dim3(hidden_threads(BLOCK_N, BWD)), smem, stream, 0,
-                                      L.map_a, L.map_b, L.map_c, L.map_m, gp, NoMaps());
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return le != cudaSuccess ? le : cudaGetLastError();
-}
-
-// 256-wide layers with enough rows to fill the machine run on CTA pairs.
-// The same kernel with both operands stored [contraction rows][M or N columns].
-template <int BLOCK_N>
-cudaError_t launch_hidden_mn(const TcLayer &L, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
-{
-    using Plan = SmemPlan<BLOCK_N>;
-    static DeviceOnce once;                      // the attribute is per device
-    {
-        const cudaError_t e = once.run([] { return cudaFuncSetAttribute(linear_tc_hidden_kernel<BLOCK_N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kSmemLimit); });
-        if (e != cudaSuccess) return e;
-    }
-    GemmParams gp = gp_in;
-    gp.stages = Plan::stages_for(Plan::hidden_epi_bytes());
-    const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes());
-    const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches;
-    const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_kernel<BLOCK_N, true>, dim3(grid), dim3(hidden_threads(BLOCK_N, false)), smem, stream, 0,
-                                      L.map_a, L.map_b, L.map_c, L.map_c, gp, NoMaps());
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return le != cudaSuccess ? le : cudaGetLastError();
-}
-
-template <bool BWD, bool MN = false>
-cudaError_t launch_hidden_pair(const TcLayer &L, const GemmParams &gp, int n_sm, cudaStream_t stream)
-{
-    static DeviceOnce once;                      // the attribute is per device
-    {
-        const cudaError_t e = once.run([] { return cudaFuncSetAttribute(linear_tc_hidden_pair_kernel<BWD, MN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)pair_smem_bytes(BWD)); });
-        if (e != cudaSuccess) return e;
-    }
-    const int tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * (MN ? gp.n_batches : 1);
-    const int pairs = tiles < n_sm / 2 ? tiles : n_sm / 2;
-    const cudaError_t le = launch_pdl(linear_tc_hidden_pair_kernel<BWD, MN>, dim3(2 * pairs), dim3(pair_threads(BWD)), pair_smem_bytes(BWD), stream, 0,
-                                      L.map_a, MN ? L.map_b : L.map_b2, L.map_c, L.map_m, gp);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return le != cudaSuccess ? le : cudaGetLastError();
-}
-
-// The forward products of one layer of two nets (equal widths) in one launch.
-template <int BLOCK_N>
-cudaError_t launch_hidden_dual(const TcLayer &L, const TcLayer &L2, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
-{
-    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, false, false)>;
-    const auto kernel = linear_tc_hidden_kernel<BLOCK_N, false, false, true>;
+    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, MN, BWD)>;
+    const auto kernel = linear_tc_hidden_kernel<BLOCK_N, MN, BWD, DUAL>;
     static DeviceOnce once;                      // the attribute is per device
     const cudaError_t e = once.run([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit); });
     if (e != cudaSuccess) return e;
     GemmParams gp = gp_in;
-    gp.n_batches = 2;
-    gp.stages = Plan::stages_for(Plan::hidden_epi_bytes());
-    const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes());
-    const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * 2;
+    gp.stages = Plan::stages_for(Plan::hidden_epi_bytes(BWD));
+    const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes(BWD));
+    const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches * (DUAL ? 2 : 1);
     const int grid = tiles < n_sm ? tiles : n_sm;
-    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, false)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
-                                      L.map_c, gp, DualMaps{L2.map_a, L2.map_b, L2.map_c});
+    SecondNet<DUAL> second;
+    if constexpr (DUAL) second = {L2->map_a, L2->map_b, L2->map_c, L2->map_m};
+    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, BWD)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
+                                      L.map_m, gp, second);
     g_launches.fetch_add(1, std::memory_order_relaxed);
-    return le;
+    return le != cudaSuccess ? le : cudaGetLastError();
+}
+
+// The same products on CTA pairs (256-column tiles).
+template <bool BWD, bool MN, bool DUAL>
+cudaError_t launch_hidden_pair(const TcLayer &L, const TcLayer *L2, const GemmParams &gp, int n_sm, cudaStream_t stream)
+{
+    const auto kernel = linear_tc_hidden_pair_kernel<BWD, MN, DUAL>;
+    static DeviceOnce once;                      // the attribute is per device
+    const cudaError_t e = once.run([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem_bytes(BWD)); });
+    if (e != cudaSuccess) return e;
+    const int tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * gp.n_batches * (DUAL ? 2 : 1);
+    const int pairs = tiles < n_sm / 2 ? tiles : n_sm / 2;
+    SecondNet<DUAL> second;
+    if constexpr (DUAL) second = {L2->map_a, MN ? L2->map_b : L2->map_b2, L2->map_c, L2->map_m};
+    const cudaError_t le = launch_pdl(kernel, dim3(2 * pairs), dim3(pair_threads(BWD)), pair_smem_bytes(BWD), stream, 0, L.map_a,
+                                      MN ? L.map_b : L.map_b2, L.map_c, L.map_m, gp, second);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return le != cudaSuccess ? le : cudaGetLastError();
 }
 
 template <int BLOCK_N, bool DUAL>
@@ -1367,7 +1345,6 @@ cudaError_t launch_head(const TcLayer &L, const GemmParams &gp_in, int n_sm, con
     GemmParams gp = gp_in;
     const int tiles = (gp.M + BLOCK_M - 1) / BLOCK_M * (DUAL ? 2 : 1);
     gp.bufs = tiles <= n_sm ? 1 : 2;
-    gp.n_batches = DUAL ? 2 : 1;
     const int epi = Plan::head_epi_bytes(gp.N, gp.bufs);
     gp.stages = Plan::stages_for(epi);
     if (gp.stages < 2) return cudaErrorInvalidValue;
@@ -1391,32 +1368,38 @@ cudaError_t dispatch_head(const TcLayer &L, const GemmParams &gp, int n_sm, cons
     }
 }
 
-// Whether a hidden layer's product runs on CTA pairs.  They pay off when the main loop is long enough to amortise the
-// cluster set-up and there are at least two waves of 256 x 256 tiles; otherwise the single-CTA kernel's finer tiles
-// balance the machine better (measured: 16384 x 1024 x 384 is 8 % faster single, 16384 x 1024 x 2048 7 % faster paired).
-// The backward epilogue is the longer part of a tile when K is short, and the pair kernel runs it on eight warps: it
-// takes those products whenever its tiles fill the machine.
-bool takes_pairs(const TcLayer &L, const GemmParams &gp, int n_sm, bool force_pairs)
+// A hidden layer's product, of one net or (DUAL) of two at once.
+template <bool DUAL>
+cudaError_t dispatch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParams &gp, int n_sm, bool force_pairs, cudaStream_t stream)
 {
-    const int pair_tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n;
+    // CTA pairs pay off when the main loop is long enough to amortise the cluster set-up and there
+    // are at least two waves of 256 x 256 tiles; otherwise the single-CTA kernel's finer tiles
+    // balance the machine better (measured: 16384 x 1024 x 384 is 8 % faster single, 16384 x 1024 x 2048
+    // 7 % faster paired).  The tiles of both nets count: actor and critic of 361-1024-512 on 16384 rows take 63.5 us with
+    // the second layer paired, 67.6 with it single; of 577-1024-1024-512 on 11000 rows 60.7 and 71.5 (9001 rows: 48.7, 47.8)
+    const int pair_tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * (DUAL ? 2 : 1);
     const bool bwd = gp.mask || gp.colsum_partial;
-    return L.block_n == 256 && gp.n_batches == 1 &&
-           (force_pairs || (pair_tiles >= n_sm && gp.K_blocks >= 8) || (bwd && pair_tiles >= n_sm / 2));
+    // (the backward epilogue is the longer part of a tile when K is short, and the pair kernel runs it on
+    // eight warps: it takes those products whenever its tiles fill the machine)
+    if (L.block_n == 256 && (force_pairs || (pair_tiles >= n_sm && gp.K_blocks >= 8) || (bwd && pair_tiles >= n_sm / 2)))
+        return bwd ? launch_hidden_pair<true, false, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden_pair<false, false, DUAL>(L, L2, gp, n_sm, stream);
+    switch (L.block_n) {
+    case 256: return bwd ? launch_hidden<256, false, true, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden<256, false, false, DUAL>(L, L2, gp, n_sm, stream);
+    case 128: return bwd ? launch_hidden<128, false, true, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden<128, false, false, DUAL>(L, L2, gp, n_sm, stream);
+    default: return bwd ? launch_hidden<64, false, true, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden<64, false, false, DUAL>(L, L2, gp, n_sm, stream);
+    }
 }
 
-cudaError_t dispatch_tc(const TcLayer &L, const GemmParams &gp, bool last, int n_sm, bool force_pairs, cudaStream_t stream)
+// The same with both operands stored [contraction rows][M or N columns].
+template <bool DUAL>
+cudaError_t dispatch_mn(const TcLayer &L, const TcLayer *L2, const GemmParams &gp, bool pairs, int n_sm, cudaStream_t stream)
 {
-    if (!last) {
-        const bool bwd = gp.mask || gp.colsum_partial;
-        if (takes_pairs(L, gp, n_sm, force_pairs))
-            return bwd ? launch_hidden_pair<true>(L, gp, n_sm, stream) : launch_hidden_pair<false>(L, gp, n_sm, stream);
-        switch (L.block_n) {
-        case 256: return bwd ? launch_hidden<256, true>(L, gp, n_sm, stream) : launch_hidden<256>(L, gp, n_sm, stream);
-        case 128: return bwd ? launch_hidden<128, true>(L, gp, n_sm, stream) : launch_hidden<128>(L, gp, n_sm, stream);
-        default: return bwd ? launch_hidden<64, true>(L, gp, n_sm, stream) : launch_hidden<64>(L, gp, n_sm, stream);
-        }
+    if (pairs) return launch_hidden_pair<false, true, DUAL>(L, L2, gp, n_sm, stream);
+    switch (L.block_n) {
+    case 256: return launch_hidden<256, true, false, DUAL>(L, L2, gp, n_sm, stream);
+    case 128: return launch_hidden<128, true, false, DUAL>(L, L2, gp, n_sm, stream);
+    default: return launch_hidden<64, true, false, DUAL>(L, L2, gp, n_sm, stream);
     }
-    return dispatch_head<false>(L, gp, n_sm, NoMaps(), stream);
 }
 
 }  // namespace
@@ -1581,7 +1564,9 @@ im_status tc_policy_forward(im_policy *p, uint32_t step, int32_t n, const float 
         TcLayer L = cfg.impl == 2 ? tc->layers[l] : with_width(tc->layers[l], (n + BLOCK_M - 1) / BLOCK_M, last, tc->n_sm);
         if (l == 0 && external) L.map_a = src->tc->layers[0].map_a;
         set_layer(gp, L);
-        if (dispatch_tc(L, gp, last, tc->n_sm, cfg.impl == 2, p->stream) != cudaSuccess) return IM_ERR_CUDA;
+        const cudaError_t e = last ? dispatch_head<false>(L, gp, tc->n_sm, NoMaps(), p->stream)
+                                   : dispatch_hidden<false>(L, nullptr, gp, tc->n_sm, cfg.impl == 2, p->stream);
+        if (e != cudaSuccess) return IM_ERR_CUDA;
     }
     return IM_OK;
 }
@@ -1595,12 +1580,11 @@ bool tc_can_pair_nets(const im_policy *a, const im_policy *c, int n)
 }
 
 // Policy and value head on the same observations: the layers of both nets, which have equal widths (tc_can_pair_nets), two by
-// two in one launch.  A layer that runs on CTA pairs fills the machine by itself and keeps a launch per net.  Below some
-// 16,000 rows a layer costs its fixed chain of barriers, loads and stores (about 5 us) rather than its arithmetic, and one
+// two in one launch.  Below some 16,000 rows a layer costs its fixed chain of barriers, loads and stores (about 5 us) rather than its arithmetic, and one
 // net's tiles leave SMs idle: both nets in one launch cost hardly more than one.  Actor (361, 1024, 512, 28) and its
 // critic, us for n = 64 / 1000 / 4096 / 9001 / 16384: one after the other 30.8 / 32.7 / 40.0 / 51.6 / 81.0, together
-// 16.4 / 18.4 / 25.7 / 39.5 / 67.4; (577, 1024, 1024, 512, 69) 33.6 / 36.0 / 44.8 / 61.1 / 94.1 and 18.5 / 20.8 / 30.3 /
-// 47.9 / 90.9.
+// 15.9 / 17.9 / 24.8 / 38.2 / 63.5; (577, 1024, 1024, 512, 69) 33.6 / 36.0 / 44.8 / 61.1 / 94.1 and 17.9 / 20.4 / 29.3 /
+// 48.7 / 77.6.
 im_status tc_policy_value_forward(im_policy *a, im_policy *c, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
                                   float *mean_out, float *action_out, float *logp_out, float *value_out)
 {
@@ -1609,27 +1593,15 @@ im_status tc_policy_value_forward(im_policy *a, im_policy *c, uint32_t step, int
         const im_status s = convert_obs(a, n, obs, ld_obs);
         if (s != IM_OK) return s;
     }
-    GemmParams gp = head_params(a, step, n, mean_out, action_out, logp_out), gc = head_params(c, 0u, n, value_out, nullptr, nullptr);
+    GemmParams gp = head_params(a, step, n, mean_out, action_out, logp_out);
     for (int l = 0; l < a->nl; ++l) {
         const bool last = l == a->nl - 1;
         TcLayer L = with_width(a->tc->layers[l], 2 * rows, last, n_sm), L2 = with_width(c->tc->layers[l], 2 * rows, last, n_sm);
         if (l == 0) L2.map_a = L.map_a;                          // one copy of the observations serves both
         set_layer(gp, L);
-        set_layer(gc, L2);
         gp.bias2 = L2.d_bias; gp.N2 = L2.N; gp.mean2 = value_out;
-        cudaError_t e;
-        if (last) {
-            e = dispatch_head<true>(L, gp, n_sm, DualMaps{L2.map_a, L2.map_b_head(L.block_n), L2.map_a}, a->stream);
-        } else if (takes_pairs(L, gp, n_sm, false)) {
-            e = launch_hidden_pair<false>(L, gp, n_sm, a->stream);
-            if (e == cudaSuccess) e = launch_hidden_pair<false>(L2, gc, n_sm, a->stream);
-        } else {
-            switch (L.block_n) {
-            case 256: e = launch_hidden_dual<256>(L, L2, gp, n_sm, a->stream); break;
-            case 128: e = launch_hidden_dual<128>(L, L2, gp, n_sm, a->stream); break;
-            default: e = launch_hidden_dual<64>(L, L2, gp, n_sm, a->stream); break;
-            }
-        }
+        const cudaError_t e = last ? dispatch_head<true>(L, gp, n_sm, {L2.map_a, L2.map_b_head(L.block_n), L2.map_a, L2.map_a}, a->stream)
+                                   : dispatch_hidden<true>(L, &L2, gp, n_sm, false, a->stream);
         if (e != cudaSuccess) return IM_ERR_CUDA;
     }
     return IM_OK;
@@ -1643,60 +1615,71 @@ cudaError_t tc_set_wait_debug(unsigned long long limit_ns, int skip_loads)
     return e;
 }
 
+namespace {
+
+bool layer_of(TcLayer &L, const GemmOperands &o, int M, int N, int K, int block_n)
+{
+    L.N = N; L.K = K; L.Kpad = K;
+    L.block_n = block_n;
+    L.n_tiles_n = N / block_n;
+    L.d_W = nullptr; L.d_bias = nullptr;
+    if (!make_map(&L.map_a, o.A, (uint64_t)M, (uint64_t)K, (uint64_t)o.lda, BLOCK_M) ||
+        !make_map(&L.map_b, o.B, (uint64_t)N, (uint64_t)K, (uint64_t)o.ldb, (uint32_t)block_n) ||
+        !make_map(&L.map_c, o.C, (uint64_t)M, (uint64_t)N, (uint64_t)o.ldc, 32))
+        return false;
+    if (block_n == 256 && !make_map(&L.map_b2, o.B, (uint64_t)N, (uint64_t)K, (uint64_t)o.ldb, 128)) return false;
+    L.map_m = L.map_c;
+    return !o.mask || make_map(&L.map_m, o.mask, (uint64_t)M, (uint64_t)N, (uint64_t)o.ld_mask, 32);
+}
+
+}  // namespace
+
 // C[M][N] = act(A[M][K] B[N][K]^T + bias) on the hidden-layer kernels, operands anywhere in device
-// memory: the three tensor maps are encoded for this call and travel as kernel parameters.
-im_status tc_gemm(const void *A, int64_t lda, const void *B, int64_t ldb, void *C, int64_t ldc, int M, int N, int K,
-                  const float *bias, bool relu, uint32_t *status, cudaStream_t stream, int batches, const void *mask,
-                  int64_t ld_mask, float *colsum_partial, int ld_partial)
+// memory: the tensor maps are encoded for this call and travel as kernel parameters.  y: a second product of the same
+// sizes in the same launch (both with a mask, or with column sums, or neither), or null.
+im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status,
+                  cudaStream_t stream)
 {
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
-    TcLayer L;
-    L.N = N; L.K = K; L.Kpad = K;
-    L.block_n = pick_block_n((M + BLOCK_M - 1) / BLOCK_M, N, false, n_sm);
-    L.n_tiles_n = N / L.block_n;
-    L.d_W = nullptr; L.d_bias = nullptr;
-    const uint64_t nb = (uint64_t)batches;
-    if (!make_map(&L.map_a, A, nb * (uint64_t)M, (uint64_t)K, (uint64_t)lda, BLOCK_M) ||
-        !make_map(&L.map_b, B, nb * (uint64_t)N, (uint64_t)K, (uint64_t)ldb, (uint32_t)L.block_n) ||
-        !make_map(&L.map_c, C, nb * (uint64_t)M, (uint64_t)N, (uint64_t)ldc, 32))
-        return IM_ERR_CUDA;
-    if (L.block_n == 256 && !make_map(&L.map_b2, B, nb * (uint64_t)N, (uint64_t)K, (uint64_t)ldb, 128)) return IM_ERR_CUDA;
-    L.map_m = L.map_c;
-    if (mask && !make_map(&L.map_m, mask, (uint64_t)M, (uint64_t)N, (uint64_t)ld_mask, 32)) return IM_ERR_CUDA;
+    TcLayer L, L2;
+    const int block_n = pick_block_n((M + BLOCK_M - 1) / BLOCK_M * (y ? 2 : 1), N, false, n_sm);
+    if (!layer_of(L, x, M, N, K, block_n) || (y && !layer_of(L2, *y, M, N, K, block_n))) return IM_ERR_CUDA;
     GemmParams gp;
     std::memset(&gp, 0, sizeof(gp));
-    gp.M = M; gp.N = N; gp.K_blocks = K / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = bias;
+    gp.M = M; gp.N = N; gp.K_blocks = K / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = x.bias;
     gp.act_floor = relu ? 0.0f : -INFINITY;
-    gp.n_batches = batches; gp.a_batch_rows = M; gp.b_batch_rows = N; gp.c_batch_rows = M;
-    if (mask || colsum_partial) gp.bias = nullptr;         // the backward product has no bias: its epilogue skips the add
-    gp.mask = static_cast<const __nv_bfloat16 *>(mask); gp.ld_mask = ld_mask;
-    gp.colsum_partial = colsum_partial; gp.ld_partial = ld_partial;
+    gp.n_batches = 1;
+    if (x.mask || x.colsum_partial) gp.bias = nullptr;     // the backward product has no bias: its epilogue skips the add
+    else if (y) gp.bias2 = y->bias;
+    gp.mask = static_cast<const __nv_bfloat16 *>(x.mask); gp.ld_mask = x.ld_mask;
+    gp.colsum_partial = x.colsum_partial; gp.ld_partial = ld_partial;
+    if (y) gp.colsum_partial2 = y->colsum_partial;
     gp.status = status;
-    return dispatch_tc(L, gp, false, n_sm, false, stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+    const cudaError_t e = y ? dispatch_hidden<true>(L, &L2, gp, n_sm, false, stream) : dispatch_hidden<false>(L, nullptr, gp, n_sm, false, stream);
+    return e == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
-
 
 // CTA pairs (256 x 256 tiles, half of the N operand per SM) when the output splits into whole 256-row tiles, the
 // slices' pitch keeps those tiles apart and there are tiles for most pairs.
-static bool tn_takes_pairs(int Mo, int No, int R, int slices, int c_pitch, int n_sm)
+static bool tn_takes_pairs(int Mo, int No, int R, int slices, int c_pitch, int n_sm, int nets)
 {
-    const int tiles = (Mo / 256) * ((No + 255) / 256) * slices;
+    const int tiles = (Mo / 256) * ((No + 255) / 256) * slices * nets;
     return (No > 256 || No % 256 == 0) && Mo % 256 == 0 && c_pitch % 256 == 0 && tiles >= n_sm / 3 && R / BLOCK_K / slices >= 8;
 }
 
 // Row slices of a transposed product (see tc_gemm_tn) on R rows: the count with the least modelled time.  A wave of
 // tiles takes 0.32 us per k-block (128 x 256 per SM: 5 ns a row, measured at 1024 x 1024 on 262144 rows) plus 4 us to
 // fill, empty and write; every slice writes and the sum over slices reads the output once more in bf16 (1 ps an element).
-int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm)
+int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm, int nets)
 {
     const int kb = R / BLOCK_K, tiles_n = (No + 255) / 256;
     int best = 1;
     double best_cost = -1.0;
     for (int S = 1; S <= max_slices && S <= kb; ++S) {
-        const bool pairs = tn_takes_pairs(Mo, No, R, S, c_pitch, n_sm);
-        const long long tiles = (long long)(pairs ? Mo / 256 : (Mo + 127) / 128) * tiles_n * S, slots = pairs ? n_sm / 2 : n_sm;
-        const double cost = (double)((tiles + slots - 1) / slots) * (0.32e-6 * (double)((kb + S - 1) / S) + 4e-6) + 1e-12 * (double)S * c_pitch * No;
+        const bool pairs = tn_takes_pairs(Mo, No, R, S, c_pitch, n_sm, nets);
+        const long long tiles = (long long)(pairs ? Mo / 256 : (Mo + 127) / 128) * tiles_n * S * nets, slots = pairs ? n_sm / 2 : n_sm;
+        const double cost = (double)((tiles + slots - 1) / slots) * (0.32e-6 * (double)((kb + S - 1) / S) + 4e-6) + 1e-12 * (double)S * nets * c_pitch * No;
         if (best_cost < 0.0 || cost < best_cost * (1.0 - 1e-9)) { best = S; best_cost = cost; }
     }
     return best;
@@ -1706,46 +1689,43 @@ int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm)
 // the transposed product A^T B of two row-major matrices over `slices` row ranges of whole 64-row blocks, the partial
 // results stacked with a pitch of `c_pitch` rows.  Operands are read M/N-major, so no transposed copy
 // of either matrix is needed.
-im_status tc_gemm_tn(const void *A, int64_t lda, const void *B, int64_t ldb, void *C, int64_t ldc, int R, int Mo, int No,
-                     int slices, int c_pitch, uint32_t *status, cudaStream_t stream)
+im_status tc_gemm_tn(const GemmOperands &x, const GemmOperands *y, int R, int Mo, int No, int slices, int c_pitch, uint32_t *status,
+                     cudaStream_t stream)
 {
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
-    TcLayer L;
-    L.N = No; L.K = R; L.Kpad = R;
     // wide outputs take 256-column tiles even when that leaves a ragged last tile (640 columns: three tiles,
     // a sixth of the MMAs wasted, against five 128-column tiles at little more than half the tensor-pipe rate);
     // TMA fills the operand columns past No with zeros and clips the stores
-    L.block_n = No > 256 ? 256 : pick_block_n(1, No, false, 0);
-    L.n_tiles_n = (No + L.block_n - 1) / L.block_n;
-    L.d_W = nullptr; L.d_bias = nullptr;
-    if (!make_map(&L.map_a, A, (uint64_t)R, (uint64_t)Mo, (uint64_t)lda, 64) ||
-        !make_map(&L.map_b, B, (uint64_t)R, (uint64_t)No, (uint64_t)ldb, 64) ||
-        !make_map(&L.map_c, C, (uint64_t)slices * (uint64_t)c_pitch, (uint64_t)No, (uint64_t)ldc, 32))
-        return IM_ERR_CUDA;
+    const int block_n = No > 256 ? 256 : pick_block_n(1, No, false, 0);
+    TcLayer L[2];
+    for (int i = 0; i < (y ? 2 : 1); ++i) {
+        const GemmOperands &o = i ? *y : x;
+        L[i].N = No; L[i].K = R; L[i].Kpad = R;
+        L[i].block_n = block_n;
+        L[i].n_tiles_n = (No + block_n - 1) / block_n;
+        L[i].d_W = nullptr; L[i].d_bias = nullptr;
+        if (!make_map(&L[i].map_a, o.A, (uint64_t)R, (uint64_t)Mo, (uint64_t)o.lda, 64) ||
+            !make_map(&L[i].map_b, o.B, (uint64_t)R, (uint64_t)No, (uint64_t)o.ldb, 64) ||
+            !make_map(&L[i].map_c, o.C, (uint64_t)slices * (uint64_t)c_pitch, (uint64_t)No, (uint64_t)o.ldc, 32))
+            return IM_ERR_CUDA;
+        L[i].map_m = L[i].map_c;
+    }
     GemmParams gp;
     std::memset(&gp, 0, sizeof(gp));
-    gp.M = Mo; gp.N = No; gp.kb_total = R / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = nullptr;    // no bias in this product
+    gp.M = Mo; gp.N = No; gp.kb_total = R / BLOCK_K; gp.n_tiles_n = L[0].n_tiles_n; gp.bias = nullptr;    // no bias in this product
     gp.act_floor = -INFINITY;
     gp.n_batches = slices; gp.c_batch_rows = c_pitch;
     gp.status = status;
-    cudaError_t e;
-    if (tn_takes_pairs(Mo, No, R, slices, c_pitch, n_sm)) {
-        L.map_m = L.map_c;
-        return launch_hidden_pair<false, true>(L, gp, n_sm, stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
-    }
-    switch (L.block_n) {
-    case 256: e = launch_hidden_mn<256>(L, gp, n_sm, stream); break;
-    case 128: e = launch_hidden_mn<128>(L, gp, n_sm, stream); break;
-    default: e = launch_hidden_mn<64>(L, gp, n_sm, stream); break;
-    }
+    const bool pairs = tn_takes_pairs(Mo, No, R, slices, c_pitch, n_sm, y ? 2 : 1);
+    const cudaError_t e = y ? dispatch_mn<true>(L[0], &L[1], gp, pairs, n_sm, stream) : dispatch_mn<false>(L[0], nullptr, gp, pairs, n_sm, stream);
     return e == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
 
-// mean[M][N] (fp32, dense) = A[M][K] B[N][K]^T + bias on the Gaussian-head kernel without sampling.
-// B must hold ceil(N / 16) * 16 rows (rows beyond N zero), bias as many floats.
-im_status tc_gemm_head(const void *A, int64_t lda, const void *B, int64_t ldb, int M, int N, int K, const float *bias,
-                       float *mean_out, uint32_t *status, cudaStream_t stream)
+// mean[M][N] (fp32, dense) = A[M][K] B[N][K]^T + bias on the Gaussian-head kernel without sampling: o.C is the mean.
+// B must hold ceil(N / 16) * 16 rows (rows beyond N zero), bias as many floats.  y: a second product in the same launch,
+// of N2 <= N columns, or null.
+im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int N, int N2, int K, uint32_t *status, cudaStream_t stream)
 {
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
@@ -1754,16 +1734,23 @@ im_status tc_gemm_head(const void *A, int64_t lda, const void *B, int64_t ldb, i
     L.block_n = pick_block_n(1, N, true, n_sm);
     L.n_tiles_n = 1;
     L.d_W = nullptr; L.d_bias = nullptr;
-    if (!make_map(&L.map_a, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BLOCK_M) ||
-        !make_map(&L.map_b, B, (uint64_t)L.block_n, (uint64_t)K, (uint64_t)ldb, (uint32_t)L.block_n))
+    if (!make_map(&L.map_a, x.A, (uint64_t)M, (uint64_t)K, (uint64_t)x.lda, BLOCK_M) ||
+        !make_map(&L.map_b, x.B, (uint64_t)L.block_n, (uint64_t)K, (uint64_t)x.ldb, (uint32_t)L.block_n))
         return IM_ERR_CUDA;
     GemmParams gp;
     std::memset(&gp, 0, sizeof(gp));
-    gp.M = M; gp.N = N; gp.K_blocks = K / BLOCK_K; gp.n_tiles_n = 1; gp.bias = bias;
-    gp.mean = mean_out; gp.sigma = 1.0f;
+    gp.M = M; gp.N = N; gp.K_blocks = K / BLOCK_K; gp.n_tiles_n = 1; gp.bias = x.bias;
+    gp.mean = static_cast<float *>(x.C); gp.sigma = 1.0f;
     gp.n_batches = 1;
     gp.status = status;
-    return dispatch_tc(L, gp, true, n_sm, false, stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+    if (!y) return dispatch_head<false>(L, gp, n_sm, NoMaps(), stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+    DualMaps second;
+    if (!make_map(&second.a, y->A, (uint64_t)M, (uint64_t)K, (uint64_t)y->lda, BLOCK_M) ||
+        !make_map(&second.b, y->B, (uint64_t)((N2 + 15) / 16 * 16), (uint64_t)K, (uint64_t)y->ldb, (uint32_t)L.block_n))
+        return IM_ERR_CUDA;
+    second.c = second.m = second.a;
+    gp.N2 = N2; gp.bias2 = y->bias; gp.mean2 = static_cast<float *>(y->C);
+    return dispatch_head<true>(L, gp, n_sm, second, stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
 
 }  // namespace im

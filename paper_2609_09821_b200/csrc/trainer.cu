@@ -29,7 +29,7 @@ int max_slices(int Np, int Kp, int max_rows, int max_split)
 {
     int most = 1;
     for (int M = 64; M <= max_rows; M += 64) {
-        const int S = im::tc_tn_slices(Np, Kp, pad128(Np), M, max_split, im::device_sm_count());
+        const int S = im::tc_tn_slices(Np, Kp, pad128(Np), M, max_split, im::device_sm_count(), 1);
         most = S > most ? S : most;
         if (most == max_split) break;
     }
@@ -45,6 +45,7 @@ bool adam_ok(const im_adam_config *c)
 
 struct im_trainer {
     int nl, Mb, t, max_split;
+    int s_max[IM_MAX_LAYERS];                              // slices dWs has room for
     int dims[IM_MAX_LAYERS + 1], Kp[IM_MAX_LAYERS], Np[IM_MAX_LAYERS];
     cudaStream_t stream;
     float *W[IM_MAX_LAYERS], *b[IM_MAX_LAYERS], *mW[IM_MAX_LAYERS], *vW[IM_MAX_LAYERS], *mb[IM_MAX_LAYERS], *vb[IM_MAX_LAYERS];
@@ -60,17 +61,42 @@ struct im_trainer {
 
 namespace {
 
-// The net on M input rows x (its own, or those of another trainer of the same input width).
-im_status forward_on(im_trainer *tr, uint16_t *x, int M)
+// One net on its input rows x, or two of equal widths (the last but) whose products of a kind share their launches: a
+// layer's tiles seldom fill the last wave of SMs, and two nets' dW products need half the row slices each.  An update of an
+// actor and a critic (361-1024-512-28 and ...-1) on 16000 rows:
+// 311 -> 258 us (131072 rows of 577-1024-1024-512-69, where every product fills the machine many times over: 2965 -> 2955).
+struct Nets {
+    im_trainer *a, *c;                                     // c: null for one net
+    uint16_t *xa, *xc;                                     // input rows (their own, or those of another trainer)
+};
+bool share_launches(const im_trainer *a, const im_trainer *c)
 {
-    const int L = tr->nl - 1;
-    for (int l = 0; l < L; ++l) {
-        const im_status s = im_gemm_bf16(l == 0 ? x : tr->H[l], tr->Kp[l], tr->Wb[l], tr->Kp[l], tr->H[l + 1], tr->Np[l], M, tr->Np[l],
-                                         tr->Kp[l], tr->b[l], 1, tr->status, tr->stream);
-        if (s != IM_OK) return s;
+    bool same = a->nl == c->nl && a->dims[a->nl] >= c->dims[c->nl];
+    for (int l = 0; same && l < a->nl; ++l) same = a->dims[l] == c->dims[l];
+    return same;
+}
+
+im::GemmOperands operands(const void *A, int lda, const void *B, int ldb, void *C, int ldc, const float *bias = nullptr)
+{
+    return {A, lda, B, ldb, C, ldc, bias, nullptr, 0, nullptr};
+}
+im::GemmOperands forward_operands(im_trainer *tr, uint16_t *x, int l)
+{
+    const bool last = l == tr->nl - 1;
+    return operands(l == 0 ? x : tr->H[l], tr->Kp[l], tr->Wb[l], tr->Kp[l], last ? (void *)tr->out : tr->H[l + 1], last ? tr->dims[tr->nl] : tr->Np[l],
+                    tr->b[l]);
+}
+im_status forward_on(const Nets &n, int M)
+{
+    im_trainer *a = n.a;
+    im_status s = IM_OK;
+    for (int l = 0; l < a->nl && s == IM_OK; ++l) {
+        const im::GemmOperands x = forward_operands(a, n.xa, l), y = n.c ? forward_operands(n.c, n.xc, l) : x;
+        const im::GemmOperands *py = n.c ? &y : nullptr;
+        if (l < a->nl - 1) s = im::tc_gemm(x, py, M, a->Np[l], a->Kp[l], true, 0, a->status, a->stream);
+        else s = im::tc_gemm_head(x, py, M, a->dims[a->nl], n.c ? n.c->dims[n.c->nl] : 0, a->Kp[l], a->status, a->stream);
     }
-    return im_gemm_bf16_f32out(tr->H[L], tr->Kp[L], tr->Wb[L], tr->Kp[L], tr->out, M, tr->dims[tr->nl], tr->Kp[L], tr->b[L],
-                               tr->status, tr->stream);
+    return s;
 }
 
 im::OutGrad out_grad(im_trainer *tr, const float *d_out)
@@ -79,20 +105,38 @@ im::OutGrad out_grad(im_trainer *tr, const float *d_out)
     return {d_out, tr->dZ[L], tr->db_partial[L], tr->dims[tr->nl], tr->Np[L]};
 }
 
-// The tensor-core products of the backward pass.  dW = dZ^T H over slices[l] row slices in one launch (both operands
-// read as they lie, M/N-major tensor-core operands: no transposed copies).  dH = (H > 0) * (dZ W); the product's
-// epilogue applies the ReLU mask and leaves the column sums of every 32-row block, which add up to the bias gradient of
-// the layer below.
-im_status backward_products(im_trainer *tr, uint16_t *x, int M, int *slices)
+// The tensor-core products of the backward pass.  dW = dZ^T H over row slices (slices[net][layer] of them) in one launch
+// (both operands read as they lie, M/N-major tensor-core operands: no transposed copies).  dH = (H > 0) * (dZ W); the
+// product's epilogue applies the ReLU mask and leaves the column sums of every 32-row block, which add up to the bias
+// gradient of the layer below.
+im_status backward_of(im_trainer *tr, uint16_t *x, im_trainer *tr2, uint16_t *x2, int l, int M, int *slices)
+{
+    const int Np = tr->Np[l], Kp = tr->Kp[l], Npb = pad128(Np);
+    const int cap = tr2 && tr2->s_max[l] < tr->s_max[l] ? tr2->s_max[l] : tr->s_max[l];
+    *slices = im::tc_tn_slices(Np, Kp, Npb, M, cap, im::device_sm_count(), tr2 ? 2 : 1);
+    const auto dw = [&](im_trainer *t, uint16_t *in) { return operands(t->dZ[l], Np, l == 0 ? in : t->H[l], Kp, t->dWs[l], Kp); };
+    const auto dh = [&](im_trainer *t) {
+        im::GemmOperands o = operands(t->dZ[l], Np, t->WbT[l], Np, t->dZ[l - 1], Kp);
+        o.mask = t->H[l]; o.ld_mask = Kp; o.colsum_partial = t->db_partial[l - 1];
+        return o;
+    };
+    im::GemmOperands o = tr2 ? dw(tr2, x2) : im::GemmOperands();
+    im_status s = im::tc_gemm_tn(dw(tr, x), tr2 ? &o : nullptr, M, Np, Kp, *slices, Npb, tr->status, tr->stream);
+    if (l == 0 || s != IM_OK) return s;
+    if (tr2) o = dh(tr2);
+    return im::tc_gemm(dh(tr), tr2 ? &o : nullptr, M, Kp, Np, false, Kp, tr->status, tr->stream);
+}
+im_status backward_products(const Nets &n, int M, int (*slices)[IM_MAX_LAYERS])
 {
     im_status s = IM_OK;
-    for (int l = tr->nl - 1; l >= 0 && s == IM_OK; --l) {
-        const int Np = tr->Np[l], Kp = tr->Kp[l], Npb = pad128(Np);
-        slices[l] = im::tc_tn_slices(Np, Kp, Npb, M, tr->max_split, im::device_sm_count());
-        s = im::tc_gemm_tn(tr->dZ[l], Np, l == 0 ? x : tr->H[l], Kp, tr->dWs[l], Kp, M, Np, Kp, slices[l], Npb, tr->status, tr->stream);
-        if (l > 0 && s == IM_OK)
-            s = im_gemm_bf16_dgrad(tr->dZ[l], Np, tr->WbT[l], Np, tr->dZ[l - 1], Kp, M, Kp, Np, tr->H[l], Kp, tr->db_partial[l - 1], Kp,
-                                   tr->status, tr->stream);
+    for (int l = n.a->nl - 1; l >= 0 && s == IM_OK; --l) {
+        if (n.c && n.c->Np[l] == n.a->Np[l]) {
+            s = backward_of(n.a, n.xa, n.c, n.xc, l, M, &slices[0][l]);
+            slices[1][l] = slices[0][l];
+        } else {
+            s = backward_of(n.a, n.xa, nullptr, nullptr, l, M, &slices[0][l]);
+            if (n.c && s == IM_OK) s = backward_of(n.c, n.xc, nullptr, nullptr, l, M, &slices[1][l]);
+        }
     }
     return s;
 }
@@ -140,8 +184,10 @@ static im_status update_on(im_ppo_updater *u, int M, const im_ppo_minibatch *mb,
     if (!adam_ok(&u->cfg.adam) || !(u->cfg.kl_target > 0.0f) || !(u->cfg.lr_min > 0.0f)) return IM_ERR_INVALID_ARG;
     im_trainer *a = u->actor, *c = u->critic;
     cudaStream_t st = a->stream;
-    im_status s = forward_on(a, a->H[0], M);
-    if (s == IM_OK) s = forward_on(c, critic_x, M);
+    const Nets both = {a, c, a->H[0], critic_x}, one_a = {a, nullptr, a->H[0], nullptr}, one_c = {c, nullptr, critic_x, nullptr};
+    const bool shared = share_launches(a, c);
+    im_status s = forward_on(shared ? both : one_a, M);
+    if (s == IM_OK && !shared) s = forward_on(one_c, M);
     if (s != IM_OK) return s;
     const float *mom = nullptr;
     if (u->cfg.normalize_advantage) {
@@ -157,14 +203,14 @@ static im_status update_on(im_ppo_updater *u, int M, const im_ppo_minibatch *mb,
     im::OutGradArgs og = {};
     og.n_nets = 2; og.M = M; og.net[0] = out_grad(a, u->d_mean); og.net[1] = out_grad(c, u->d_value);
     if (im::launch_out_grads(og, st) != cudaSuccess) return IM_ERR_CUDA;
-    int slices_a[IM_MAX_LAYERS], slices_c[IM_MAX_LAYERS];
-    s = backward_products(a, a->H[0], M, slices_a);
-    if (s == IM_OK) s = backward_products(c, critic_x, M, slices_c);
+    int slices[2][IM_MAX_LAYERS];
+    s = backward_products(shared ? both : one_a, M, slices);
+    if (s == IM_OK && !shared) s = backward_products(one_c, M, slices + 1);
     if (s != IM_OK) return s;
     // every gradient tensor of both nets, and the global-norm clip factor over them and the log-std's
     im::GradReduceArgs ga = {};
-    add_weight_grads(ga, a, slices_a);
-    add_weight_grads(ga, c, slices_c);
+    add_weight_grads(ga, a, slices[0]);
+    add_weight_grads(ga, c, slices[1]);
     add_bias_grads(ga, a, M);
     add_bias_grads(ga, c, M);
     ga.extra = u->d_log_std; ga.n_extra = u->A;
@@ -243,8 +289,8 @@ im_status im_trainer_create(int32_t n_layers, const int32_t *dims, const float *
              dev_alloc(&tr->WbT[l], (size_t)Kp * Np, st) && dev_alloc(&tr->H[l], (size_t)max_rows * Kp, st) &&
              dev_alloc(&tr->dZ[l], (size_t)max_rows * Np, st);
         // partial dW products: room for the most slices the model can choose for any number of rows
-        const size_t s_max = (size_t)max_slices(Np, Kp, max_rows, tr->max_split);
-        ok = ok && dev_alloc(&tr->dWs[l], s_max * pad128(Np) * Kp, st, false) &&
+        tr->s_max[l] = max_slices(Np, Kp, max_rows, tr->max_split);
+        ok = ok && dev_alloc(&tr->dWs[l], (size_t)tr->s_max[l] * pad128(Np) * Kp, st, false) &&
              dev_alloc(&tr->db_partial[l], (size_t)(l == n_layers - 1 ? (max_rows + 127) / 128 : max_rows / 32) * Np, st, false);
     }
     ok = ok && dev_alloc(&tr->out, (size_t)max_rows * dims[n_layers], st) && dev_alloc(&tr->status, 1, st);
@@ -304,7 +350,7 @@ im_status im_trainer_set_step_count(im_trainer *tr, int32_t t)
 im_status im_trainer_forward(im_trainer *tr, int32_t M)
 {
     if (!tr || M < 1 || M > tr->Mb) return IM_ERR_INVALID_ARG;
-    return forward_on(tr, tr->H[0], M);
+    return forward_on({tr, nullptr, tr->H[0], nullptr}, M);
 }
 
 im_status im_trainer_backward(im_trainer *tr, const float *d_out, int32_t M)
@@ -313,11 +359,11 @@ im_status im_trainer_backward(im_trainer *tr, const float *d_out, int32_t M)
     im::OutGradArgs og = {};
     og.n_nets = 1; og.M = M; og.net[0] = out_grad(tr, d_out);
     if (im::launch_out_grads(og, tr->stream) != cudaSuccess) return IM_ERR_CUDA;
-    int slices[IM_MAX_LAYERS];
-    const im_status s = backward_products(tr, tr->H[0], M, slices);
+    int slices[1][IM_MAX_LAYERS];
+    const im_status s = backward_products({tr, nullptr, tr->H[0], nullptr}, M, slices);
     if (s != IM_OK) return s;
     im::GradReduceArgs ga = {};
-    add_weight_grads(ga, tr, slices);
+    add_weight_grads(ga, tr, slices[0]);
     add_bias_grads(ga, tr, M);
     return im::launch_grad_reduce(ga, tr->stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
