@@ -11,7 +11,7 @@
 // reads of eight consecutive rows hit distinct banks.  The warps of a CTA share one output tile and split every
 // chunk's k range between them; their partial tiles are added in warp order at the end (bit-reproducible).  Small
 // tiles spread a 64-row layer over the SMs.  Measured (361-1024-512-28, one forward with its noise, CUDA graph):
-// 64 rows 21 us, 300 rows 46 us, 2048 rows 142 us against
+// 64 rows 18 us, 300 rows 41 us, 2048 rows 142 us against
 // 265 us at 64 rows for one 64 x 64 tile per CTA with 16-wide k-steps loaded element by element between barriers
 // and a noise kernel of one thread per row.
 #include <cuda_bf16.h>
@@ -302,13 +302,19 @@ cudaError_t launch_linear_simt(const float *A, int lda, const void *W, bool w_bf
                                int ldc, int M, int N, int K, cudaStream_t stream)
 {
     const LayerArgs L = {A, W, bias, C, lda, ldc, M, N, K};
-    const long long t16 = (long long)((M + 15) / 16) * ((N + 15) / 16), t32 = (long long)((M + 31) / 32) * ((N + 31) / 32);
+    const auto tiles = [&](int bm, int bn) { return (long long)((M + bm - 1) / bm) * ((N + bn - 1) / bn); };
     cudaError_t e;
-    // 16 x 16 tiles while two per SM hold the layer (a forward at 128 rows: 30 us against 39 with 32 x 32; at 300 rows,
-    // 1216 of them, 53 us against 46), 32 x 32 up to four per SM (512 rows: 52 us against 107 with 64 x 64), then
-    // 64 x 64 (2048 rows: 142 us against 156)
-    if (t16 <= 300) e = launch_tile<Tile<512, 16, 16, 256, 1, 1, 3>>(L, w_bf16, stream);
-    else if (t32 <= 600) e = launch_tile<Tile<256, 32, 32, 128, 1, 1, 3>>(L, w_bf16, stream);
+    // The smallest tile whose CTAs, one per SM with sixteen warps, hold the layer in one wave: a wave's time grows with the
+    // tile, a second wave costs more (1024 x 361, us with its head: 64 rows 18.5 as two waves of 16 x 16, 15.0 as one of
+    // 32 x 16; 128 rows 19.2 with 32 x 16, 18.2 with 32 x 32.  512 x 1024: 128 rows 19.0 with 16 x 16, 15.6 with 32 x 16; 200
+    // rows 23.3 with 32 x 16, 21.6 with 32 x 32; 300 rows 29.2 with two 32 x 32 per SM, 23.2 with 24 x 48).  Beyond that two
+    // 32 x 32 CTAs per SM, up to four (512 rows: 52 us against 107 with 64 x 64), then 64 x 64 (2048 rows: 142 us against 156)
+    const int n_sm = 148;
+    if (tiles(16, 16) <= n_sm) e = launch_tile<Tile<512, 16, 16, 256, 1, 1, 3>>(L, w_bf16, stream);
+    else if (tiles(32, 16) <= n_sm) e = launch_tile<Tile<512, 32, 16, 128, 1, 1, 3>>(L, w_bf16, stream);
+    else if (tiles(32, 32) <= n_sm) e = launch_tile<Tile<512, 32, 32, 128, 1, 1, 3>>(L, w_bf16, stream);
+    else if (tiles(24, 48) <= n_sm) e = launch_tile<Tile<512, 24, 48, 256, 1, 1, 3>>(L, w_bf16, stream);
+    else if (tiles(32, 32) <= 4 * n_sm) e = launch_tile<Tile<256, 32, 32, 128, 1, 1, 3>>(L, w_bf16, stream);
     else e = launch_tile<Tile<256, 64, 64, 64, 1, 2, 3>>(L, w_bf16, stream);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return e != cudaSuccess ? e : cudaGetLastError();

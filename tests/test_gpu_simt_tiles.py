@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("n,dims", [
     (1, (5, 3, 2)), (15, (361, 17, 28)), (17, (360, 1024, 512, 28)), (64, (361, 1024, 512, 33)), (65, (259, 130, 69)),
-    (300, (577, 1024, 512, 69)), (1025, (362, 1021, 64, 300)),
+    (300, (577, 1024, 512, 69)), (1025, (362, 1021, 64, 300)), (33, (361, 1023, 530, 28)), (97, (361, 1024, 515, 28)),
+    (127, (364, 1013, 260, 3)), (199, (70, 513, 620, 28)), (289, (361, 520, 517, 30)), (313, (1024, 480, 500, 9)),
 ])
 def test_forward_matches_oracle(n, dims):
     import torch
