@@ -61,7 +61,7 @@ NCU_TRAFFIC = {
     "cfg4_65536_smpl24": dict(
         policy=dict(bytes=645075456, capture="linear_tc_hidden_pair_kernel<0, 0> x 3 + linear_tc_head_kernel<80>, one policy "
                                               "forward at 65536 envs (ncu --set full)"),
-        env=dict(bytes=291532288, capture="env_step_kernel_small<0, 0, 0> writing fp32 and bf16 rows, one launch, "
+        env=dict(bytes=291532288, capture="env_chain_kernel<0, 0> writing fp32 and bf16 rows, one launch, "
                                           "65536 envs (ncu --set full)")),
 }
 
@@ -667,7 +667,7 @@ def main():
                     frac_burst=tf / peaks["bf16_tflops"], frac_sustained=tf / tensor_peak,
                     peak_sustained=tensor_peak, traffic=traffic["policy"]["bytes"], traffic_capture=traffic["policy"]["capture"],
                     peak_source="%s bf16 burst (timed region of milliseconds)" % peaks["source"], seconds_per_launch=t_pol)
-    roofline_env = dict(bound="hbm", kernel="env_step_kernel", achieved=gbs, peak=peaks["hbm_gbs"], unit="GB/s",
+    roofline_env = dict(bound="hbm", kernel="env_chain_kernel / env_role_kernel", achieved=gbs, peak=peaks["hbm_gbs"], unit="GB/s",
                         frac=gbs / peaks["hbm_gbs"], traffic=traffic["env"]["bytes"], traffic_capture=traffic["env"]["capture"],
                         peak_source="%s copy" % peaks["source"],
                         seconds_per_launch=t_env, algorithmic_bytes=env_bytes)

@@ -570,10 +570,11 @@ im_status im_colsum_f32(const float *x, int64_t ld, int64_t rows, int32_t cols, 
  *                        outputs in IM_TRAINER_OUT; every layer's activation is kept for the backward pass.
  *   im_trainer_backward  d_out DEVICE float [M][dims[last]] = dL/d(outputs) of that forward; M a multiple of 64.
  *                        Fills the gradients IM_TRAINER_DW / IM_TRAINER_DB of every layer:
- *                        dW_l = dZ_l^T H_{l-1} (im_gemm_bf16_tn over row slices + im_sum_slices_bf16_to_f32),
- *                        dZ_{l-1} = (H_{l-1} > 0) (dZ_l W_l) and its column sums (im_gemm_bf16_dgrad + im_colsum_f32).
- *   im_trainer_step      one Adam step on every tensor (im_adam_step; lr and grad_scale DEVICE float [1],
- *                        grad_scale may be NULL); the bf16 copies and their transposes follow.
+ *                        dW_l = dZ_l^T H_{l-1} (the product of im_gemm_bf16_tn over slices of whole 64-row blocks),
+ *                        dZ_{l-1} = (H_{l-1} > 0) (dZ_l W_l) and its column sums (the product of im_gemm_bf16_dgrad);
+ *                        one launch adds the slices and the column sums of every layer.
+ *   im_trainer_step      one Adam step on every tensor in one launch (im_adam_step's arithmetic; lr and grad_scale
+ *                        DEVICE float [1], grad_scale may be NULL), the bf16 copies and their transposes with it.
  *   im_trainer_push_to_policy  writes the current weights and biases into a loaded im_policy of the same
  *                        shape and stream, so the next rollout acts with the trained network.
  *   im_trainer_tensor    DEVICE address and shape of one of the trainer's arrays (IM_TRAINER_*; `layer` is
@@ -582,7 +583,8 @@ im_status im_colsum_f32(const float *x, int64_t ld, int64_t rows, int32_t cols, 
  *   im_trainer_set_step_count  sets the Adam step counter (bias correction) -- 0 restarts the optimiser.
  *   im_trainer_dw_slices the number of row slices the dW product of a layer with Np x Kp (padded) weights takes
  *                        on M rows: the power of two that minimises a small time model (waves of output tiles on
- *                        the SMs x rows per slice, plus the pass that adds the partial products).  Host only. */
+ *                        the SMs x rows per slice, plus the pass that adds the partial products), for callers of
+ *                        im_gemm_bf16_tn, whose slices are equal; the trainer's own need not be.  Host only. */
 typedef struct im_trainer im_trainer;
 #define IM_TRAINER_W        0   /* float [dims[l+1]][dims[l]]                      */
 #define IM_TRAINER_B        1   /* float [dims[l+1]] (buffer padded to 64 floats)   */
@@ -616,17 +618,19 @@ int32_t im_trainer_dw_slices(int32_t Np, int32_t Kp, int64_t M, int32_t max_spli
  * log-std, sharing a stream and max_rows.  log_std: HOST float [A], the initial value (also the first
  * "old" log-std).
  *   im_ppo_update  one minibatch update on M rows (a multiple of 64): forward of both nets on their input
- *     rows, advantage moments (if normalize_advantage), im_ppo_loss, both backward passes, im_grad_scale
- *     over every gradient tensor (global-norm clip at max_grad_norm), Adam on every tensor and on the
- *     log-std, im_adaptive_lr from the mean KL.  The minibatch's observations must already sit in both
+ *     rows, advantage moments (if normalize_advantage), im_ppo_loss, both backward passes, the norm over every
+ *     gradient tensor (global-norm clip at max_grad_norm), Adam on every tensor and on the log-std, the
+ *     learning rate from the mean KL (as im_adaptive_lr).  Nets of equal widths but for the last share the
+ *     launches of their products; a wait that runs out there is reported in the actor's status word.  The
+ *     minibatch's observations must already sit in both
  *     trainers' input rows.  mb: DEVICE float arrays -- action, mean_old [M][A]; logp_old, advantage,
  *     value_old (needed with clip_value_loss), returns [M]; log_std_old [A] or NULL for the updater's own copy.
  *   im_ppo_update_rollout  the whole update phase over a collected rollout: `epochs` passes over
  *     `n_minibatches` blocks of the T * N samples (row t * N + e of the time-major arrays of `view`;
  *     T * N / n_minibatches must be a multiple of 64 within max_rows).  perm NULL: contiguous blocks, the
- *     observations converted into both nets' input rows by im_f32_to_bf16_padded, everything else read in
+ *     observations converted into the actor's input rows, which both nets read, everything else read in
  *     place.  perm: DEVICE int32 [epochs][T * N], a permutation of the sample indices per epoch: every array
- *     of a block is gathered by im_gather_rows_f32 (the first shuffled call of a given size allocates the
+ *     of a block is gathered by one launch (a bad index is clamped and sets IM_DEV_BAD_STATE; the first shuffled call of a given size allocates the
  *     gather buffers; make it outside a capture).
  *   im_ppo_updater_tensor  DEVICE address of a state array (IM_PPO_*): the log-std and its Adam moments [A],
  *     the frozen behaviour log-std [A], the learning rate [1], (clip factor, gradient norm) [2], the loss
@@ -677,7 +681,8 @@ im_status im_ppo_updater_set_step_count(im_ppo_updater *u, int32_t t);
  * columns have arrived.  The first call allocates the
  * device staging buffers and the copy streams (so it is not capturable).  Call
  * im_env_reset_all_host first.  sim_host is [13J][N] (pos rows, quat rows,
- * linvel rows, angvel rows); pinned memory gives the copies full speed.
+ * linvel rows, angvel rows); pinned memory gives the copies full speed, and
+ * pinned reward and flag arrays are written by the env kernel itself.
  *   action_host HOST [N][A]   reward_host HOST [N]   flags_host HOST [N] */
 im_status im_env_reset_all_host(im_env *e, uint32_t step);
 im_status im_step_host(im_env *e, im_policy *p, uint32_t step, const float *sim_host,
