@@ -61,7 +61,7 @@ NCU_TRAFFIC = {
     "cfg4_65536_smpl24": dict(
         policy=dict(bytes=645075456, capture="linear_tc_hidden_pair_kernel<0, 0> x 3 + linear_tc_head_kernel<80>, one policy "
                                               "forward at 65536 envs (ncu --set full)"),
-        env=dict(bytes=291532288, capture="env_chain_kernel<0, 0> writing fp32 and bf16 rows, one launch, "
+        env=dict(bytes=291532288, capture="env_step_kernel_small<0, 0, 0> (now env_chain_kernel) writing fp32 and bf16 rows, one launch, "
                                           "65536 envs (ncu --set full)")),
 }
 
