@@ -808,8 +808,10 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
             if (!WIDE) break;
         }
         if (bad) atomicOr(P.status, IM_DEV_BAD_SIM_QUAT);
+        // With write_back the reset states below go where other warps of the tile may still have to load: every warp
+        // reads the root, a scoring warp the parent of its first own body, which another chain owns.
+        if (need_r || P.write_back) __syncthreads();
         if (need_r) {
-            __syncthreads();
             float term[IM_N_TERMS];
             r = reward_of(P, part, C, lane, term);
         }

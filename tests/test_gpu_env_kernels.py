@@ -93,3 +93,48 @@ def test_large_batch_equals_its_shards(name, skeleton):
     if options:
         d = acc - acc_a - acc_b
         assert bool((d[1:] == 0).all()) and abs(int(d[0])) <= 3 * N * 1e-5 * 2 ** 40
+
+
+@pytest.mark.parametrize("records", [False, True])
+@pytest.mark.parametrize("tree", ["humanoid15", "smpl24", 15, 31])
+@pytest.mark.parametrize("n", [33, 2500, 9000])
+def test_writing_reset_states_back_changes_nothing_else(n, tree, records):
+    """The reset states go into the arrays that the same launch scores: flags, rewards, observations and terms are those
+    of a launch that leaves the arrays alone, with a reward that cannot end an episode and with one that could but never
+    does, and the written states are the same in both."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    if isinstance(tree, int):
+        g = np.random.default_rng(tree)
+        skel = dict(parents=np.asarray([-1] + [0] * tree, np.int32), offsets=g.uniform(-0.3, 0.3, (tree + 1, 3)).astype(np.float32), masses=None, J=tree + 1)
+    else:
+        skel = W.make_skeleton(tree, 1)
+    J = skel["J"]
+    lib = W.make_clip_library(J, 4, (20, 40), 30.0, 1)
+    sk = B.Skeleton(skel["parents"], skel["offsets"], skel["masses"])
+    clips = B.Clips(sk, lib["n_frames"], lib["fps"], lib["root_pos"], lib["local_quat"])
+    sims = (torch.randn(8, 13 * J, (n + 3) // 4 * 4, device="cuda", generator=torch.Generator("cuda").manual_seed(n)) * 0.3)[:, :, :n]
+    sims[:, 2] += 0.85
+    out = []
+    for write_back, r_min in ((False, -np.inf), (True, -np.inf), (True, -1.0)):
+        cfg = B.make_env_config(n, 1 / 30, 5, W.REWARD_MULT, 0.8, B.padded_ld(24 * J + 1), r_min=r_min, write_back_reset=write_back)
+        env = B.Env(sk, clips, cfg)
+        obs, rew, fl, terms = env.new_obs(), torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda"), torch.empty(7, n, device="cuda")
+        env.reset_all(obs, 0)
+        got, states = [], []
+        for s in range(sims.shape[0]):
+            if records:
+                st = [sims[s, a * J:b * J].reshape(J, b - a, n).permute(2, 0, 1).contiguous() for a, b in ((0, 3), (3, 7), (7, 10), (10, 13))]
+                env.step_aos(s + 1, *st, obs, rew, fl, terms)
+            else:
+                st = [torch.empty_strided((13 * J, n), sims[s].stride(), device="cuda").copy_(sims[s])]
+                env.step(s + 1, st[0], obs, rew, fl, terms)
+            got += [obs.clone(), rew.clone(), fl.clone(), terms.clone()] + list(env.get_state())
+            states += st
+        assert env.device_status() == 0
+        out.append((got, states))
+    assert bool((out[0][0][2] & 1).any()) and not bool((out[0][0][2] & 1).all())
+    for got, states in out[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got, out[0][0]))
+    assert all(torch.equal(a, b) for a, b in zip(out[1][1], out[2][1]))
+    assert not torch.equal(out[0][1][0], out[1][1][0])
