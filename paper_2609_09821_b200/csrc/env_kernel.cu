@@ -532,6 +532,7 @@ struct EnvState {
     float t;
     ClipMeta cm;
     ClipLoop loop;
+    bool grace;                    // still within its grace steps
     int flags;
     bool reset;
     int clip_new, cyc_new;         // after it (unchanged for an env that is not reset)
@@ -539,12 +540,13 @@ struct EnvState {
     ClipMeta cm_new;
 };
 
-// Flags (step a4) given the reward.
+// Flags (step a4) given the reward; from values loaded before the first warp stores the new state, which would change the
+// decision of a warp that came late.
 template <bool OPT>
-__device__ __forceinline__ int flags_of(const EnvKernelParams &P, int env, float root_z, float r, const EnvState &E)
+__device__ __forceinline__ int flags_of(const EnvKernelParams &P, float root_z, float r, const EnvState &E)
 {
     bool terminated = (root_z < P.reward.h_min) || (r < P.reward.r_min);
-    if (OPT && P.ep_len[env] < P.grace_steps) terminated = false;
+    if (OPT && E.grace) terminated = false;
     const bool truncated = !(OPT && E.loop.on) && __fadd_rn(E.t, P.dt) > E.cm.dur;    // a looped clip has no end
     return (terminated ? 1 : 0) | (truncated ? 2 : 0);
 }
@@ -556,7 +558,7 @@ __device__ __forceinline__ void decide(const EnvKernelParams &P, int env, float 
 {
     E.flags = 0;
     if (!RESET_ALL) {
-        E.flags = flags_of<OPT>(P, env, root_z, r, E);
+        E.flags = flags_of<OPT>(P, root_z, r, E);
         if (OPT && P.n_bins > 0 && (E.flags & 1) && count) {
             // the (clip, phase bin) the episode failed in
             const float span = fmaxf(__fsub_rn(E.cm.dur, P.dt), 0.0f);
@@ -692,6 +694,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     E.clip = 0; E.cyc = 0; E.t = 0.0f;
     E.cm = {2, 1.0f, 1.0f, 0};
     E.loop = {0.0f, 0.0f, 0.0f, 0};
+    E.grace = false;
     Heading H = {0.0f, 0.0f, 1.0f, 0.0f};
     float root_z = 0.0f, r = INFINITY;
     bool bad = false;
@@ -706,6 +709,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
         }
         E.t = __fadd_rn(P.t[envc], P.dt);
         E.cm = P.meta[E.clip];
+        if (OPT) E.grace = P.ep_len[envc] < P.grace_steps;
         if (OPT && P.loops) {
             // a clip played in a loop: the time wraps at the clip's end and the env's cycle count goes up
             E.loop = P.loops[E.clip];
@@ -718,7 +722,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     const ClipLoop loop = E.loop;              // of the clip before a reset
     // whether the reward can end an episode; if not, the root height and the clip end decide, which are known already
     const bool need_r = !RESET_ALL && P.reward.r_min > -INFINITY;
-    const bool known_reset = !RESET_ALL && !need_r && flags_of<OPT>(P, envc, root_z, r, E) != 0;
+    const bool known_reset = !RESET_ALL && !need_r && flags_of<OPT>(P, root_z, r, E) != 0;
 
     if (!RESET_ALL) {
 #pragma unroll 1
@@ -1006,6 +1010,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         for (int i = 15 * J; i < c1; ++i) row1[i] = 0.0f;   // columns between the body blocks and the split
 
     int clip = 0, cyc = 0;
+    bool grace = false;
     float t1 = 0.0f;
     ClipMeta cm = {2, 1.0f, 1.0f, 0};
     ClipLoop loop = {0.0f, 0.0f, 0.0f, 0};
@@ -1023,6 +1028,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         }
         t1 = __fadd_rn(P.t[envc], P.dt);
         cm = P.meta[clip];
+        if (OPT) grace = P.ep_len[envc] < P.grace_steps;
         if (OPT && P.loops) {
             // a clip played in a loop: the time wraps at the clip's end and the env's cycle count goes up
             loop = P.loops[clip];
@@ -1110,7 +1116,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     //      reward only if the reward can terminate an episode (r_min above -inf), else the root height and the
     //      clip end decide alone.  The reset draw is a function of (env, step) and is repeated by every thread.
     EnvState E;
-    E.clip = clip; E.cyc = cyc; E.t = t1; E.cm = cm; E.loop = loop;
+    E.clip = clip; E.cyc = cyc; E.t = t1; E.cm = cm; E.loop = loop; E.grace = grace;
     {
         float term[IM_N_TERMS], r = INFINITY;
         if (c == 0 || P.reward.r_min > -INFINITY) r = reward_of(P, part, C, lane, term);

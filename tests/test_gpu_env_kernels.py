@@ -138,3 +138,34 @@ def test_writing_reset_states_back_changes_nothing_else(n, tree, records):
         assert all(torch.equal(a, b) for a, b in zip(got, out[0][0]))
     assert all(torch.equal(a, b) for a, b in zip(out[1][1], out[2][1]))
     assert not torch.equal(out[0][1][0], out[1][1][0])
+
+
+@pytest.mark.parametrize("skeleton", ["humanoid15", "smpl24"])
+def test_every_warp_decides_alike_at_the_grace_limit(skeleton):
+    """All envs lie below the termination height, half of them have one grace step left: the large batch's flags, state and
+    observation rows (each chain's warp writes its own part of a row) are those of its shards, bit for bit."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    skel, J = W.make_skeleton(skeleton, 1), {"humanoid15": 15, "smpl24": 24}[skeleton]
+    lib = W.make_clip_library(J, 4, (20, 40), 30.0, 1)
+    sk = B.Skeleton(skel["parents"], skel["offsets"], skel["masses"])
+    clips = B.Clips(sk, lib["n_frames"], lib["fps"], lib["root_pos"], lib["local_quat"])
+    sims = torch.randn(12, 13 * J, N, device="cuda", generator=torch.Generator("cuda").manual_seed(3)) * 0.3
+    length = (torch.arange(N, device="cuda", dtype=torch.int32) * 7 % 5)
+
+    def run(base, n):
+        env = B.Env(sk, clips, B.make_env_config(n, 1 / 30, 5, W.REWARD_MULT, 10.0, B.padded_ld(24 * J + 1), env_id_base=base, grace_steps=3))
+        obs, rew, fl = env.new_obs(), torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda")
+        env.reset_all(obs, 0)
+        env.set_state(ep_len=length[base:base + n].contiguous())
+        out, want = [], length[base:base + n].clone()
+        for s in range(sims.shape[0]):
+            env.step(s + 1, sims[s, :, base:base + n].contiguous(), obs, rew, fl)
+            assert torch.equal((fl & 1) != 0, want >= 3)
+            want = torch.where(fl != 0, 0, want + 1)
+            assert torch.equal(env.get_state()[2], want)
+            out += [obs.clone(), rew.clone(), fl.clone()] + list(env.get_state()[:2])
+        return out
+
+    for whole, a, b in zip(run(0, N), run(0, N // 2), run(N // 2, N // 2)):
+        assert torch.equal(whole, torch.cat([a, b]))
