@@ -209,6 +209,7 @@ __global__ void __launch_bounds__(HeadTile::kThreads, HeadTile::kMinBlocks) head
     uint32_t rank, n_ranks;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_ranks));
+    if (n_ranks > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");       // (waited for before the remote store)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int m0 = (int)(blockIdx.x / n_ranks) * T::BM;
@@ -252,13 +253,14 @@ __global__ void __launch_bounds__(HeadTile::kThreads, HeadTile::kMinBlocks) head
             for (int q = 0; q < T::BN / 4; ++q) zz_row += s_zz[threadIdx.x][q];
     }
     if (n_ranks > 1) {
+        asm volatile("barrier.cluster.wait;" ::: "memory");                // every CTA of the cluster has started
         if (threadIdx.x < T::BM) {
             uint32_t dst;
             asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&s_rank_zz[rank][threadIdx.x])), "r"(0));
             asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(zz_row) : "memory");
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         if (rank != 0) return;
         if (threadIdx.x < T::BM) {
             zz_row = 0.0f;

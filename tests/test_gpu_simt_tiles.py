@@ -35,3 +35,23 @@ def test_forward_matches_oracle(n, dims):
     lp = np.asarray(ref["logp"], np.float64)
     assert np.all(np.abs(logp.cpu().numpy() - lp) <= 1e-3 + 1e-5 * np.abs(lp))
     assert torch.equal(mean, m2)
+
+
+@pytest.mark.parametrize("A", [32, 33, 65, 256, 300])
+@pytest.mark.parametrize("n", [1, 16, 17, 4001])
+def test_log_probabilities_across_a_cluster(n, A):
+    """Actions wider than one column tile: the CTAs of a row block send their sums of squares to the first of them, after a
+    contraction of eight steps only, launch after launch."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    w = W.make_policy_weights((4, 8, A), "f32", seed=3)
+    pol = B.Policy((4, 8, A), w["W"], w["b"], "f32", 0.2, 7, n)
+    obs = torch.randn(n, 4, device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    mean, action = torch.empty(n, A, device="cuda"), torch.empty(n, A, device="cuda")
+    logps = torch.full((40, n), 7.0, device="cuda")
+    for i in range(40):
+        pol.forward(5, obs, mean, action, logps[i])
+    ref = O.policy_forward((4, 8, A), w["W"], w["b"], 0.2, 7, 5, obs.cpu().numpy())
+    lp = np.asarray(ref["logp"], np.float64)
+    assert np.all(np.abs(logps[0].cpu().numpy() - lp) <= 1e-3 + 1e-5 * np.abs(lp))      # (as above)
+    assert torch.equal(logps, logps[:1].expand(40, n))
