@@ -762,9 +762,12 @@ static im_status ensure_staging(im_env *e, int A)
     return IM_OK;
 }
 
-// The device address of `bytes` of pinned host memory, or null where the memory is not pinned (asked anew on each call).
-static void *device_view(void *host, size_t bytes)
+// The device address of `bytes` of pinned host memory, or null where the memory is not pinned (asked anew on each call) or
+// does not start on a multiple of `align`, as an array inside a caller's packed record may: a copy takes any address, a
+// kernel's stores do not.
+static void *device_view(void *host, size_t bytes, size_t align)
 {
+    if (reinterpret_cast<uintptr_t>(host) % align) return nullptr;
     cudaPointerAttributes a, z;
     if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&z, static_cast<char *>(host) + bytes - 1) != cudaSuccess) {
         cudaGetLastError();
@@ -806,7 +809,7 @@ im_status im_step_host(im_env *e, im_policy *p, uint32_t step, const float *sim_
     for (int c = 0; c < chunks; ++c) {
         // One range is one contiguous copy: as 13 J rows of 4 KB the step takes 15 us longer at 1000 envs x 15 bodies (at 4096
         // envs the two are alike).  A few KB of pageable memory go faster by rows (64 envs: 82 us a step against 89-107).
-        if (chunks == 1 && (13 * J * n * 4 >= 65536 || device_view(const_cast<float *>(sim_host), 13 * J * n * 4))) IM_CUDA(cudaMemcpyAsync(e->d_sim, sim_host, 13 * J * n * 4, cudaMemcpyHostToDevice, e->h2d_stream));
+        if (chunks == 1 && (13 * J * n * 4 >= 65536 || device_view(const_cast<float *>(sim_host), 13 * J * n * 4, 1))) IM_CUDA(cudaMemcpyAsync(e->d_sim, sim_host, 13 * J * n * 4, cudaMemcpyHostToDevice, e->h2d_stream));
         else IM_CUDA(cudaMemcpy2DAsync(e->d_sim + c * nc, n * 4, sim_host + c * nc, n * 4, nc * 4, 13 * J, cudaMemcpyHostToDevice,
                                        e->h2d_stream));
         IM_CUDA(cudaEventRecord(e->ev_h2d[c], e->h2d_stream));
@@ -823,8 +826,8 @@ im_status im_step_host(im_env *e, im_policy *p, uint32_t step, const float *sim_
     im_body_state sim = {e->d_sim, e->d_sim + 3 * J * n, e->d_sim + 7 * J * n, e->d_sim + 10 * J * n, (int64_t)n};
     // Five bytes per env: where the caller's arrays are pinned the env kernel writes them there itself, which saves two
     // copies after the kernel (a step of 64 envs 55 -> 48 us, of 1000 envs 82 -> 73, of 4096 envs 106 -> 95)
-    float *reward_direct = static_cast<float *>(device_view(reward_host, n * 4));
-    uint8_t *flags_direct = static_cast<uint8_t *>(device_view(flags_host, n));
+    float *reward_direct = static_cast<float *>(device_view(reward_host, n * 4, alignof(float)));
+    uint8_t *flags_direct = static_cast<uint8_t *>(device_view(flags_host, n, 1));
     for (int c = 0; c < chunks; ++c) {
         IM_CUDA(cudaStreamWaitEvent(e->stream, e->ev_h2d[c], 0));
         s = env_step_range(e, step, &sim, e->d_obs, reward_direct ? reward_direct : e->d_reward, flags_direct ? flags_direct : e->d_flags,

@@ -36,3 +36,28 @@ def test_pinned_and_pageable_buffers_agree(n):
     assert any(bool((x != 0).any()) for x in out[0][2::3])
     for other in out[1:]:
         assert all(torch.equal(a, b) for a, b in zip(out[0], other))
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_pinned_rewards_need_no_alignment(shift):
+    """Rewards inside a packed record of the caller's: pinned, but not on a multiple of four bytes."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    n = 70
+    skel, lib = W.make_skeleton("humanoid15", 0), W.make_clip_library(15, 3, (30, 60), 30.0, 0)
+    sk = B.Skeleton(skel["parents"], skel["offsets"], skel["masses"])
+    clips = B.Clips(sk, lib["n_frames"], lib["fps"], lib["root_pos"], lib["local_quat"])
+    w = W.make_policy_weights((361, 128, 28), "bf16", 0)
+    sim = torch.randn(195, n, generator=torch.Generator().manual_seed(2)).pin_memory()
+    out = []
+    for off in (0, shift):
+        env = B.Env(sk, clips, B.make_env_config(n, 1 / 30, 0, W.REWARD_MULT, 0.3, 384))
+        pol = B.Policy((361, 128, 28), w["W_bf16"], w["b"], "bf16", 0.1, 0, n)
+        env.attach_policy(pol)
+        env.reset_all_host(0)
+        raw = torch.full((4 * n + 8,), 9, dtype=torch.uint8).pin_memory()
+        act, fl = torch.zeros(n, 28).pin_memory(), torch.zeros(n, dtype=torch.uint8).pin_memory()
+        B.step_host(env, pol, 1, sim, act, raw[off:], fl)
+        assert bool((raw[:off] == 9).all()) and bool((raw[off + 4 * n:] == 9).all())
+        out.append((raw[off:off + 4 * n].clone(), act, fl))
+    assert bool((out[0][0] != 9).any()) and all(torch.equal(a, b) for a, b in zip(*out))
