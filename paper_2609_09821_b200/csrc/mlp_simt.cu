@@ -26,7 +26,6 @@ namespace im {
 
 namespace {
 
-
 // Tile of a CTA: BM x BN outputs, BK-wide k-chunks.  WM x WN warps cover the tile, KW such groups split
 // the chunk's k range.  A warp's lanes form an 8 x 4 grid over its (BM / WM) x (BN / WN) part, rows and columns
 // interleaved (lane row + 8 i, lane column + 4 j) so that one 16-byte read serves 8 (or 4) distinct rows.
@@ -309,13 +308,15 @@ cudaError_t launch_linear_simt(const float *A, int lda, const void *W, bool w_bf
     // The smallest tile whose CTAs, one per SM with sixteen warps, hold the layer in one wave: a wave's time grows with the
     // tile, a second wave costs more (1024 x 361, us with its head: 64 rows 18.5 as two waves of 16 x 16, 15.0 as one of
     // 32 x 16; 128 rows 19.2 with 32 x 16, 18.2 with 32 x 32.  512 x 1024: 128 rows 19.0 with 16 x 16, 15.6 with 32 x 16; 200
-    // rows 23.3 with 32 x 16, 21.6 with 32 x 32; 300 rows 29.2 with two 32 x 32 per SM, 23.2 with 24 x 48).  Beyond that two
+    // rows 23.3 with 32 x 16, 21.6 with 32 x 32).  32 x 48 is the largest that pays: whole forwards of 361-1024-512-28 on 129 /
+    // 192 / 300 / 416 rows 31.0 / 30.7 / 41.5 / 42.2 us, 34.0 / 33.8 / 46.6 / 47.1 without it (361-2048-1024-28, 192 rows: 59 and 69;
+    // 361-512-256-28, 640 rows: 33.3 and 36.2); 64 x 32 on 300 rows 48.  Beyond that two
     // 32 x 32 CTAs per SM, up to four (512 rows: 52 us against 107 with 64 x 64), then 64 x 64 (2048 rows: 142 us against 156)
-    const int n_sm = 148;
+    const int n_sm = device_sm_count();
     if (tiles(16, 16) <= n_sm) e = launch_tile<Tile<512, 16, 16, 256, 1, 1, 3>>(L, w_bf16, stream);
     else if (tiles(32, 16) <= n_sm) e = launch_tile<Tile<512, 32, 16, 128, 1, 1, 3>>(L, w_bf16, stream);
     else if (tiles(32, 32) <= n_sm) e = launch_tile<Tile<512, 32, 32, 128, 1, 1, 3>>(L, w_bf16, stream);
-    else if (tiles(24, 48) <= n_sm) e = launch_tile<Tile<512, 24, 48, 256, 1, 1, 3>>(L, w_bf16, stream);
+    else if (tiles(32, 48) <= n_sm) e = launch_tile<Tile<512, 32, 48, 128, 1, 1, 3>>(L, w_bf16, stream);
     else if (tiles(32, 32) <= 4 * n_sm) e = launch_tile<Tile<256, 32, 32, 128, 1, 1, 3>>(L, w_bf16, stream);
     else e = launch_tile<Tile<256, 64, 64, 64, 1, 2, 3>>(L, w_bf16, stream);
     g_launches.fetch_add(1, std::memory_order_relaxed);

@@ -55,3 +55,9 @@ def test_log_probabilities_across_a_cluster(n, A):
     lp = np.asarray(ref["logp"], np.float64)
     assert np.all(np.abs(logps[0].cpu().numpy() - lp) <= 1e-3 + 1e-5 * np.abs(lp))      # (as above)
     assert torch.equal(logps, logps[:1].expand(40, n))
+
+
+@pytest.mark.parametrize("n,dims", [(129, (361, 1024, 512, 28)), (192, (70, 1009, 60, 5)), (193, (361, 1024, 96, 28)),
+                                    (385, (577, 512, 530, 9)), (416, (362, 528, 485, 28)), (417, (40, 512, 28)), (832, (361, 240, 12, 3))])
+def test_forward_around_the_largest_one_wave_tile(n, dims):
+    test_forward_matches_oracle(n, dims)
