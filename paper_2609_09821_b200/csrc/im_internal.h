@@ -71,8 +71,10 @@ struct DeviceOnce {
     }
 };
 // Launch with programmatic stream serialization: the kernel's prologue may overlap the tail of the kernel before it in
-// the stream.  The kernel executes griddepcontrol.wait before its first access to global memory.  cluster > 0: blocks per
-// cluster (along x) of a kernel that does not fix them itself.
+// the stream.  The kernel executes griddepcontrol.wait before its first access to global memory.  Its life overlaps that of
+// the kernels before it, so what they may have written is not read-only while it lives: it is read by plain or .cg loads,
+// not by __ldg, nor through const __restrict__ pointers, which the compiler may turn into the same instruction.
+// cluster > 0: blocks per cluster (along x) of a kernel that does not fix them itself.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster, Args &&...args)
 {

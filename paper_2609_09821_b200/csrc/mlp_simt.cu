@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(T::kThreads, T::kMinBlocks) linear_simt_kernel
     for (int i = threadIdx.x; i < T::BM * T::BN; i += T::kThreads) {
         const int m = m0 + i / T::BN, n = n0 + i % T::BN;
         if (m >= L.M || n >= L.N) continue;
-        L.C[(size_t)m * L.ldc + n] = fmaxf(tile_sum<T>(smem, i) + __ldg(L.bias + n), 0.0f);
+        L.C[(size_t)m * L.ldc + n] = fmaxf(tile_sum<T>(smem, i) + L.bias[n], 0.0f);
     }
 }
 
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(HeadTile::kThreads, HeadTile::kMinBlocks) head
         sum_log = (float)L.N * logf(H.sigma);
         if (H.log_std) {
             sum_log = 0.0f;
-            for (int i = 0; i < L.N; ++i) sum_log += __ldg(H.log_std + i);
+            for (int i = 0; i < L.N; ++i) sum_log += H.log_std[i];
         }
     }
     for (int n0 = (int)rank * T::BN; n0 < L.N; n0 += (int)n_ranks * T::BN) {
@@ -236,10 +236,10 @@ __global__ void __launch_bounds__(HeadTile::kThreads, HeadTile::kMinBlocks) head
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (col + i >= L.N) break;
-                    const float mu = tile_sum<T>(smem, r * T::BN + 4 * q + i) + __ldg(L.bias + col + i);
+                    const float mu = tile_sum<T>(smem, r * T::BN + 4 * q + i) + L.bias[col + i];
                     L.C[(size_t)row * L.ldc + col + i] = mu;
                     if (H.action) {
-                        const float sg = H.log_std ? expf(__ldg(H.log_std + col + i)) : H.sigma;
+                        const float sg = H.log_std ? expf(H.log_std[col + i]) : H.sigma;
                         H.action[(size_t)row * L.N + col + i] = mu + sg * z[i];
                         zz += z[i] * z[i];
                     }

@@ -488,7 +488,7 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
         const float4 *b4 = reinterpret_cast<const float4 *>(bias + col0);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const float4 b = __ldg(b4 + i);
+            const float4 b = b4[i];
             v[4 * i] = fmaxf(v[4 * i] + b.x, fl);
             v[4 * i + 1] = fmaxf(v[4 * i + 1] + b.y, fl);
             v[4 * i + 2] = fmaxf(v[4 * i + 2] + b.z, fl);
@@ -1078,9 +1078,9 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
         // the epilogue reads bias and sigma from shared memory as 16-byte words instead of one global load per output
         if ((int)threadIdx.x - 64 < BLOCK_N) {
             const int cidx = (int)threadIdx.x - 64;
-            s_bias[cidx] = __ldg(P.bias + cidx);
-            if (DUAL) s_bias2[cidx] = cidx < P.N2 ? __ldg(P.bias2 + cidx) : 0.0f;
-            s_sigma[cidx] = cidx < A ? (P.log_std ? expf(__ldg(P.log_std + cidx)) : P.sigma) : 0.0f;
+            s_bias[cidx] = P.bias[cidx];
+            if (DUAL) s_bias2[cidx] = cidx < P.N2 ? P.bias2[cidx] : 0.0f;
+            s_sigma[cidx] = cidx < A ? (P.log_std ? expf(P.log_std[cidx]) : P.sigma) : 0.0f;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * kHeadEpiWarps) : "memory");
         float logp_const = 0.0f;
@@ -1088,7 +1088,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
             float sum_log = (float)A * logf(P.sigma);
             if (P.log_std) {                                         // same order in every thread
                 sum_log = 0.0f;
-                for (int i = 0; i < A; ++i) sum_log += __ldg(P.log_std + i);
+                for (int i = 0; i < A; ++i) sum_log += P.log_std[i];
             }
             logp_const = -sum_log - 0.5f * (float)A * 1.8378770664093453f;
         }
@@ -1193,7 +1193,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
 }
 
 // fp32 observations -> bf16 rows of a padded buffer; columns beyond `cols` are written as zero.
-__global__ void obs_to_bf16_kernel(const float *__restrict__ obs, int ld_obs, int cols, __nv_bfloat16 *__restrict__ out,
+__global__ void obs_to_bf16_kernel(const float *obs, int ld_obs, int cols, __nv_bfloat16 *__restrict__ out,
                                    int ld_out, int n, int early)
 {
     if (early) dep_release();
@@ -1204,12 +1204,12 @@ __global__ void obs_to_bf16_kernel(const float *__restrict__ obs, int ld_obs, in
         const int r = (int)(i / chunks), c = (int)(i - (uint32_t)r * chunks) * 8;
         float v[8];
         if (c + 8 <= cols) {
-            const float4 a = *reinterpret_cast<const float4 *>(obs + (size_t)r * ld_obs + c);
-            const float4 b = *reinterpret_cast<const float4 *>(obs + (size_t)r * ld_obs + c + 4);
+            const float4 a = __ldcg(reinterpret_cast<const float4 *>(obs + (size_t)r * ld_obs + c));
+            const float4 b = __ldcg(reinterpret_cast<const float4 *>(obs + (size_t)r * ld_obs + c + 4));
             v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
         } else {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = (c + k < cols) ? obs[(size_t)r * ld_obs + c + k] : 0.0f;
+            for (int k = 0; k < 8; ++k) v[k] = (c + k < cols) ? __ldcg(obs + (size_t)r * ld_obs + c + k) : 0.0f;
         }
         uint32_t pk[4];
 #pragma unroll

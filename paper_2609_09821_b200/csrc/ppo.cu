@@ -110,8 +110,8 @@ __device__ __forceinline__ void setup_lane(const PpoParams &P, int sl, RowConsts
     for (int i = 0; i < NI; ++i) {
         const int k = sl + LPR * i;
         const bool ok = k < P.A;
-        const float ls = ok ? __ldg(P.b.log_std + k) : 0.0f;
-        const float lo = ok ? __ldg(P.b.log_std_old + k) : 0.0f;
+        const float ls = ok ? P.b.log_std[k] : 0.0f;
+        const float lo = ok ? P.b.log_std_old[k] : 0.0f;
         C.inv_sg[i] = expf(-ls);
         // d + (sigma_old^2 / sigma^2 - 1) / 2 with d = ln(sigma / sigma_old): not below zero by more than its own rounding,
         // and zero where the standard deviations are the same
@@ -122,7 +122,7 @@ __device__ __forceinline__ void setup_lane(const PpoParams &P, int sl, RowConsts
     sum_log = group_sum<LPR>(sum_log);
     C.logp_const = -sum_log - 0.5f * (float)P.A * 1.8378770664093453f;
     C.adv_mean = 0.0f; C.adv_rstd = 1.0f;
-    if (P.b.adv_moments) { C.adv_mean = __ldg(P.b.adv_moments); C.adv_rstd = __ldg(P.b.adv_moments + 1); }
+    if (P.b.adv_moments) { C.adv_mean = P.b.adv_moments[0]; C.adv_rstd = P.b.adv_moments[1]; }
     C.eps = P.cfg.clip; C.cv = P.cfg.value_coef; C.inv_M = 1.0f / (float)P.M;
     C.clip_value = P.cfg.clip_value_loss;
     acc.surr = acc.vl = acc.kl = acc.clip = 0.0f;
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(kFinishThreads) ppo_finish_kernel(const PpoPar
             for (int k = 0; k < kFinishBatch; ++k) t += (double)x[k];
         }
         s_grp[threadIdx.x] = t;
-        if (q == groups - 1 && jj < P.A) s_ls[jj] = __ldg(P.b.log_std + jj);
+        if (q == groups - 1 && jj < P.A) s_ls[jj] = P.b.log_std[jj];
     }
     __syncthreads();
     if (q == 0) {
@@ -495,7 +495,7 @@ constexpr int kMomCluster = 8;
 constexpr long long kMomClusterMax = 1 << 17;               // (64 values a thread; more than that wants more SMs)
 
 // This block's sums of x and x^2 over its grid stride, in thread 0.
-__device__ __forceinline__ double2 moments_of_block(const float *__restrict__ x, long long n)
+__device__ __forceinline__ double2 moments_of_block(const float *x, long long n)
 {
     __shared__ double s_sum[kMomThreads], s_sq[kMomThreads];
     double s = 0.0, q = 0.0;
@@ -503,7 +503,7 @@ __device__ __forceinline__ double2 moments_of_block(const float *__restrict__ x,
     for (long long i = (long long)blockIdx.x * kMomThreads + threadIdx.x; i < n; i += 8 * stride) {
         float v[8];                                         // loads in flight together
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = i + k * stride < n ? __ldg(x + i + k * stride) : 0.0f;
+        for (int k = 0; k < 8; ++k) v[k] = i + k * stride < n ? __ldcg(x + i + k * stride) : 0.0f;
 #pragma unroll
         for (int k = 0; k < 8; ++k) { s += (double)v[k]; q = fma((double)v[k], (double)v[k], q); }
     }
@@ -524,14 +524,14 @@ __device__ __forceinline__ void moments_write(double s, double q, long long n, f
     out[0] = (float)mean;
     out[1] = (float)(1.0 / (sqrt(var) + 1e-8));
 }
-__global__ void __launch_bounds__(kMomThreads) moments_partial_kernel(const float *__restrict__ x, long long n,
+__global__ void __launch_bounds__(kMomThreads) moments_partial_kernel(const float *x, long long n,
                                                                       double *__restrict__ partial)
 {
     dep_release_wait();
     const double2 t = moments_of_block(x, n);
     if (threadIdx.x == 0) { partial[2 * blockIdx.x] = t.x; partial[2 * blockIdx.x + 1] = t.y; }
 }
-__global__ void __launch_bounds__(32) moments_finish_kernel(const double *__restrict__ partial, int grid, long long n,
+__global__ void __launch_bounds__(32) moments_finish_kernel(const double *partial, int grid, long long n,
                                                             float *__restrict__ out)
 {
     dep_release_wait();
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(32) moments_finish_kernel(const double *__rest
 // Up to kMomClusterMax values in one launch: the blocks of one cluster, whose first reads the others' sums from their
 // shared memory.  16000 values: 7.7 us in
 // two launches whose last loads of a thread came one by one, 5.5 us.
-__global__ void __cluster_dims__(kMomCluster, 1, 1) __launch_bounds__(kMomThreads) moments_cluster_kernel(const float *__restrict__ x, long long n,
+__global__ void __cluster_dims__(kMomCluster, 1, 1) __launch_bounds__(kMomThreads) moments_cluster_kernel(const float *x, long long n,
                                                                                                           float *__restrict__ out)
 {
     __shared__ double2 s_all[kMomCluster];                  // (the first block's is used)

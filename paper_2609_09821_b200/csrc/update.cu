@@ -61,7 +61,7 @@ __device__ __forceinline__ void adam_update(const im_adam_config &c, const AdamT
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const long long e = on[k] ? i + k * step : 0;
-        p[k] = T.param[e]; g[k] = __ldg(T.grad + e); m[k] = T.m[e]; v[k] = T.v[e];
+        p[k] = T.param[e]; g[k] = T.grad[e]; m[k] = T.m[e]; v[k] = T.v[e];
     }
 #pragma unroll
     for (int k = 0; k < N; ++k) {
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreads) adam_multi_kernel(const __grid_const
     dep_release_wait();
     const AdamTensor T = P.t[owner(P.first_block, P.n_tensors, blockIdx.x)];
     const int blk = (int)blockIdx.x - T.first_block;
-    const float lr = *P.lr, gs = P.grad_scale ? __ldg(P.grad_scale) : 1.0f;
+    const float lr = *P.lr, gs = P.grad_scale ? *P.grad_scale : 1.0f;
     if (!T.wb) {
         const int n = T.rows * T.cols, i0 = blk * kVecElems + threadIdx.x;
         for (int k0 = 0; k0 < kVecElems / kThreads && i0 + k0 * kThreads < n; k0 += kAdamBatch) {
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
         for (int s = 0; s < G.slices; s += kBatch) {
             uint4 w[kBatch];
 #pragma unroll
-            for (int k = 0; k < kBatch; ++k) w[k] = s + k < G.slices ? __ldg(src + (s + k) * stride) : make_uint4(0u, 0u, 0u, 0u);
+            for (int k = 0; k < kBatch; ++k) w[k] = s + k < G.slices ? __ldcg(src + (s + k) * stride) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int k = 0; k < kBatch; ++k) {
                 const uint32_t x[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
                 float4 x[8];                                  // loads in flight together
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-                    x[k] = r + 32 * k < G.n_rows ? __ldg(reinterpret_cast<const float4 *>(G.in + (long long)(r + 32 * k) * G.ld + c))
+                    x[k] = r + 32 * k < G.n_rows ? __ldcg(reinterpret_cast<const float4 *>(G.in + (long long)(r + 32 * k) * G.ld + c))
                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
                 for (int k = 0; k < 8; k += 2) {
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
             }
         }
     } else {
-        for (int i = threadIdx.x; i < P.n_extra; i += kThreads) sq = fma((double)__ldg(P.extra + i), (double)__ldg(P.extra + i), sq);
+        for (int i = threadIdx.x; i < P.n_extra; i += kThreads) sq = fma((double)P.extra[i], (double)P.extra[i], sq);
     }
     if (!P.partial) return;
     sq = block_sum(sq);
@@ -265,6 +265,7 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
 
 // ---------------------------------------------------------------- output gradients
 constexpr int kOutRows = 128;
+constexpr int kOutBatch = 16;
 
 __global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_constant__ OutGradArgs P)
 {
@@ -276,13 +277,22 @@ __global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_consta
     const int r0 = blockIdx.x * kOutRows, r1 = min(r0 + kOutRows, P.M);
     __nv_bfloat16 *dz = reinterpret_cast<__nv_bfloat16 *>(G.dz);
     float s0 = 0.0f, s1 = 0.0f;
-#pragma unroll 16
-    for (int r = r0 + g; r < r1; r += groups) {
-        const float *src = G.d_out + (long long)r * G.cols + c;
-        const float a = c < G.cols ? __ldg(src) : 0.0f, b = c + 1 < G.cols ? __ldg(src + 1) : 0.0f;
-        *reinterpret_cast<__nv_bfloat162 *>(dz + (long long)r * G.ld + c) = __floats2bfloat162_rn(a, b);
-        s0 += a;
-        s1 += b;
+#pragma unroll 1
+    for (int r = r0 + g; r < r1; r += kOutBatch * groups) {
+        float a[kOutBatch], b[kOutBatch];                         // loads in flight together
+#pragma unroll
+        for (int k = 0; k < kOutBatch; ++k) {
+            const bool on = r + k * groups < r1;
+            const float *src = G.d_out + (long long)(r + k * groups) * G.cols + c;
+            a[k] = on && c < G.cols ? __ldcg(src) : 0.0f;
+            b[k] = on && c + 1 < G.cols ? __ldcg(src + 1) : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < kOutBatch; ++k) {
+            if (r + k * groups < r1) *reinterpret_cast<__nv_bfloat162 *>(dz + (long long)(r + k * groups) * G.ld + c) = __floats2bfloat162_rn(a[k], b[k]);
+            s0 += a[k];
+            s1 += b[k];
+        }
     }
     s_sum[g][c] = s0;
     s_sum[g][c + 1] = s1;
@@ -295,6 +305,8 @@ __global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_consta
 }
 
 // ---------------------------------------------------------------- shuffled minibatch
+constexpr int kRowBatch = 4;
+
 // A warp gathers a row; VEC: observation rows start on 16-byte boundaries.
 template <bool VEC>
 __global__ void __launch_bounds__(kThreads) gather_minibatch_kernel(const __grid_constant__ GatherArgs P)
@@ -302,37 +314,55 @@ __global__ void __launch_bounds__(kThreads) gather_minibatch_kernel(const __grid
     dep_release_wait();
     const int lane = threadIdx.x & 31, warps = (gridDim.x * kThreads) >> 5;
     for (int i = (blockIdx.x * kThreads + threadIdx.x) >> 5; i < P.M; i += warps) {
-        long long src = __ldg(P.idx + i);
+        long long src = P.idx[i];
         if (src < 0 || src >= P.n_src) {                          // a bad index is clamped and reported, never followed
             if (lane == 0) atomicOr(P.status, IM_DEV_BAD_STATE);
             src = src < 0 ? 0 : P.n_src - 1;
         }
         const float *row = P.obs + src * P.ld_obs;
         __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(P.h) + (long long)i * P.ld_h;
-#pragma unroll 4
-        for (int c = 4 * lane; c < P.ld_h; c += 128) {
-            float v[4];
-            if (VEC && c + 4 <= P.D) {
-                const float4 x = __ldg(reinterpret_cast<const float4 *>(row + c));
-                v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-            } else {
+#pragma unroll 1
+        for (int c0 = 4 * lane; c0 < P.ld_h; c0 += 128 * kRowBatch) {
+            float v[kRowBatch][4];                                // loads in flight together
 #pragma unroll
-                for (int j = 0; j < 4; ++j) v[j] = c + j < P.D ? __ldg(row + c + j) : 0.0f;
+            for (int q = 0; q < kRowBatch; ++q) {
+                const int c = c0 + 128 * q;
+                if (VEC && c + 4 <= P.D) {
+                    const float4 x = __ldcg(reinterpret_cast<const float4 *>(row + c));
+                    v[q][0] = x.x; v[q][1] = x.y; v[q][2] = x.z; v[q][3] = x.w;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) v[q][j] = c + j < P.D ? __ldcg(row + c + j) : 0.0f;
+                }
             }
-            const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
-            *reinterpret_cast<uint2 *>(h + c) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+#pragma unroll
+            for (int q = 0; q < kRowBatch; ++q) {
+                const int c = c0 + 128 * q;
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(v[q][0], v[q][1]), hi = __floats2bfloat162_rn(v[q][2], v[q][3]);
+                if (c < P.ld_h) *reinterpret_cast<uint2 *>(h + c) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+            }
         }
         const long long o = (long long)i * P.A, s = src * P.A;
-#pragma unroll 4
-        for (int k = lane; k < P.A; k += 32) {
-            P.g_action[o + k] = __ldg(P.action + s + k);
-            P.g_mean[o + k] = __ldg(P.mean + s + k);
+        const float *from = lane == 0 ? P.logp : lane == 1 ? P.advantage : lane == 2 ? P.value : P.returns;
+        float *to = lane == 0 ? P.g_logp : lane == 1 ? P.g_advantage : lane == 2 ? P.g_value : P.g_returns;
+        const float scalar = lane < 4 ? __ldcg(from + src) : 0.0f;
+#pragma unroll 1
+        for (int k0 = lane; k0 < P.A; k0 += 32 * kRowBatch) {
+            float a[kRowBatch], m[kRowBatch];
+#pragma unroll
+            for (int q = 0; q < kRowBatch; ++q) {
+                const bool on = k0 + 32 * q < P.A;
+                a[q] = on ? __ldcg(P.action + s + k0 + 32 * q) : 0.0f;
+                m[q] = on ? __ldcg(P.mean + s + k0 + 32 * q) : 0.0f;
+            }
+#pragma unroll
+            for (int q = 0; q < kRowBatch; ++q) {
+                if (k0 + 32 * q >= P.A) break;
+                P.g_action[o + k0 + 32 * q] = a[q];
+                P.g_mean[o + k0 + 32 * q] = m[q];
+            }
         }
-        if (lane < 4) {
-            const float *from = lane == 0 ? P.logp : lane == 1 ? P.advantage : lane == 2 ? P.value : P.returns;
-            float *to = lane == 0 ? P.g_logp : lane == 1 ? P.g_advantage : lane == 2 ? P.g_value : P.g_returns;
-            to[i] = __ldg(from + src);
-        }
+        if (lane < 4) to[i] = scalar;
     }
 }
 
