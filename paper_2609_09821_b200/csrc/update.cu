@@ -212,11 +212,12 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
             }
         }
     } else if (P.n_vectors > 0 && block < P.n_blocks - (P.n_extra > 0 ? 1 : 0)) {
-        // db: 32 columns, 32 groups of rows in fp32 (two chains each), the groups added in order in fp64
+        // db: 32 columns, 32 groups of rows; eight rows are added in fp32 as a tree, everything beyond in fp64 (a fp32 chain
+        // would grow with the batch; all of it in fp64 costs a conversion a row, 30 -> 42 us for 4096 rows of 64 columns)
         __shared__ double s_col[32][kVecCols + 1];
         const GradVector G = P.v[owner(P.v_first, P.n_vectors, block)];
         const int cg = threadIdx.x & 7, rg = threadIdx.x >> 3, c = (block - G.first_block) * kVecCols + 4 * cg;
-        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
         if (c < G.ld) {
 #pragma unroll 1
             for (int r = rg; r < G.n_rows; r += 8 * 32) {
@@ -226,14 +227,16 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
                     x[k] = r + 32 * k < G.n_rows ? __ldcg(reinterpret_cast<const float4 *>(G.in + (long long)(r + 32 * k) * G.ld + c))
                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-                for (int k = 0; k < 8; k += 2) {
-                    a.x += x[k].x; a.y += x[k].y; a.z += x[k].z; a.w += x[k].w;
-                    b.x += x[k + 1].x; b.y += x[k + 1].y; b.z += x[k + 1].z; b.w += x[k + 1].w;
-                }
+                for (int k = 4; k > 0; k >>= 1)
+#pragma unroll
+                    for (int i = 0; i < k; ++i) {
+                        x[i].x += x[i + k].x; x[i].y += x[i + k].y; x[i].z += x[i + k].z; x[i].w += x[i + k].w;
+                    }
+                a[0] += (double)x[0].x; a[1] += (double)x[0].y; a[2] += (double)x[0].z; a[3] += (double)x[0].w;
             }
         }
-        s_col[rg][4 * cg] = (double)(a.x + b.x); s_col[rg][4 * cg + 1] = (double)(a.y + b.y);
-        s_col[rg][4 * cg + 2] = (double)(a.z + b.z); s_col[rg][4 * cg + 3] = (double)(a.w + b.w);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s_col[rg][4 * cg + j] = a[j];
         __syncthreads();
         if (threadIdx.x < kVecCols) {
             double t = 0.0;

@@ -44,3 +44,18 @@ def test_backward_matches_fp64(M, dims):
             assert float(((got.double() - want).abs() / (want.abs() + rms)).max()) < 2e-2, (l, M)
         if l:
             dz = (q @ Wd[l]) * (H[l] > 0)
+
+
+@pytest.mark.parametrize("M,A", [(64, 28), (64 * 61, 1), (64 * 61, 80), (1 << 20, 28)])
+def test_bias_gradients_are_rounded_once(M, A):
+    """Whole numbers whose sums over 1024 rows fit fp32: the sum over the batch is exact but for its one rounding, however
+    many rows there are."""
+    import torch
+    from paper_2609_09821_b200 import trainer as T
+    w = W.make_policy_weights((64, 64, A), "f32", seed=5)
+    tr = T.MlpTrainer((64, 64, A), w["W"], w["b"], M)
+    d_out = 2 * torch.randint(-2 ** 11, 2 ** 13, (M, A), device="cuda", generator=torch.Generator("cuda").manual_seed(M + A)) + 1
+    tr.input_rows(M).zero_()
+    tr.forward(M)
+    tr.backward(d_out.float(), M)
+    assert torch.equal(tr.db[1], d_out.sum(0).float()) and tr.device_status() == 0
