@@ -628,7 +628,8 @@ int32_t im_trainer_dw_slices(int32_t Np, int32_t Kp, int64_t M, int32_t max_spli
  *   im_ppo_update_rollout  the whole update phase over a collected rollout: `epochs` passes over
  *     `n_minibatches` blocks of the T * N samples (row t * N + e of the time-major arrays of `view`;
  *     T * N / n_minibatches must be a multiple of 64 within max_rows).  perm NULL: contiguous blocks, the
- *     observations converted into the actor's input rows, which both nets read, everything else read in
+ *     observations converted into the actor's input rows, which both nets read (the last minibatch's also into
+ *     the critic's), everything else read in
  *     place.  perm: DEVICE int32 [epochs][T * N], a permutation of the sample indices per epoch: every array
  *     of a block is gathered by one launch (a bad index is clamped and sets IM_DEV_BAD_STATE; the first shuffled call of a given size allocates the
  *     gather buffers; make it outside a capture).

@@ -80,9 +80,9 @@ __global__ void __launch_bounds__(256) transpose_bf16_kernel(const __nv_bfloat16
     }
 }
 
-// out[r][c] = bf16(in[r][c]) for c < cols, 0 for cols <= c < ld_out.
+// out[r][c] = bf16(in[r][c]) for c < cols, 0 for cols <= c < ld_out; out2: a second copy, or null.
 __global__ void __launch_bounds__(256) to_bf16_padded_kernel(const float *__restrict__ in, long long ld_in, int rows, int cols,
-                                                             __nv_bfloat16 *__restrict__ out, int ld_out)
+                                                             __nv_bfloat16 *__restrict__ out, __nv_bfloat16 *__restrict__ out2, int ld_out)
 {
     release_dependents();
     const long long total = (long long)rows * ld_out;
@@ -90,13 +90,14 @@ __global__ void __launch_bounds__(256) to_bf16_padded_kernel(const float *__rest
         const long long r = i / ld_out;
         const int c = (int)(i - r * ld_out);
         out[i] = __float2bfloat16_rn(c < cols ? __ldg(in + r * ld_in + c) : 0.0f);
+        if (out2) out2[i] = out[i];
     }
 }
 
 // The same with 16-byte stores: a thread converts eight consecutive columns of one row (ld_out a multiple of 8,
 // out 16-byte aligned); its eight loads are 32 consecutive bytes, a warp's one contiguous kilobyte of the row.
 __global__ void __launch_bounds__(256) to_bf16_padded_vec_kernel(const float *__restrict__ in, long long ld_in, int rows, int cols,
-                                                                 __nv_bfloat16 *__restrict__ out, int ld_out)
+                                                                 __nv_bfloat16 *__restrict__ out, __nv_bfloat16 *__restrict__ out2, int ld_out)
 {
     release_dependents();
     const int gpr = ld_out >> 3;                                   // 8-column groups per row
@@ -115,6 +116,7 @@ __global__ void __launch_bounds__(256) to_bf16_padded_vec_kernel(const float *__
         h = __floats2bfloat162_rn(v[4], v[5]); o.z = *reinterpret_cast<const uint32_t *>(&h);
         h = __floats2bfloat162_rn(v[6], v[7]); o.w = *reinterpret_cast<const uint32_t *>(&h);
         *reinterpret_cast<uint4 *>(out + r * ld_out + c) = o;
+        if (out2) *reinterpret_cast<uint4 *>(out2 + r * ld_out + c) = o;
     }
 }
 
@@ -288,6 +290,20 @@ im_status colsum(const T *x, int64_t ld, int64_t rows, int32_t cols, float *out,
 
 }  // namespace
 
+im_status f32_to_bf16_padded(const float *in, int64_t ld_in, int rows, int cols, uint16_t *out, uint16_t *out2, int ld_out, cudaStream_t st)
+{
+    if (!in || !out || rows < 1 || cols < 1 || ld_in < cols || ld_out < cols) return IM_ERR_INVALID_ARG;
+    const bool vec = (ld_out & 7) == 0 && al16(out) && al16(out2);
+    const long long total = vec ? (long long)rows * (ld_out >> 3) : (long long)rows * ld_out;
+    const long long g = (total + 255) / 256;
+    const int grid = (int)(g > 148 * 16 ? 148 * 16 : g);
+    __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(out), *o2 = reinterpret_cast<__nv_bfloat16 *>(out2);
+    if (vec) to_bf16_padded_vec_kernel<<<grid, 256, 0, st>>>(in, ld_in, rows, cols, o, o2, ld_out);
+    else to_bf16_padded_kernel<<<grid, 256, 0, st>>>(in, ld_in, rows, cols, o, o2, ld_out);
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+}
+
 }  // namespace im
 
 extern "C" {
@@ -373,20 +389,7 @@ im_status im_transpose_bf16(const uint16_t *in, int64_t ld_in, int32_t rows, int
 im_status im_f32_to_bf16_padded(const float *in, int64_t ld_in, int32_t rows, int32_t cols, uint16_t *out, int32_t ld_out,
                                 void *cuda_stream)
 {
-    using namespace im;
-    if (!in || !out || rows < 1 || cols < 1 || ld_in < cols || ld_out < cols) return IM_ERR_INVALID_ARG;
-    const bool vec = (ld_out & 7) == 0 && al16(out);
-    const long long total = vec ? (long long)rows * (ld_out >> 3) : (long long)rows * ld_out;
-    long long g = (total + 255) / 256;
-    const int grid = (int)(g > 148 * 16 ? 148 * 16 : g);
-    if (vec)
-        to_bf16_padded_vec_kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>(in, ld_in, rows, cols,
-                                                                               reinterpret_cast<__nv_bfloat16 *>(out), ld_out);
-    else
-        to_bf16_padded_kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>(in, ld_in, rows, cols,
-                                                                           reinterpret_cast<__nv_bfloat16 *>(out), ld_out);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+    return im::f32_to_bf16_padded(in, ld_in, rows, cols, out, nullptr, ld_out, (cudaStream_t)cuda_stream);
 }
 
 im_status im_gather_rows_f32(const float *in, int64_t ld_in, const int32_t *idx, int64_t n_src, int32_t rows, int32_t cols,

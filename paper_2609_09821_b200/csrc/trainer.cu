@@ -499,15 +499,17 @@ im_status im_ppo_update_rollout(im_ppo_updater *u, const im_rollout_view *v, int
             const int64_t r0 = (int64_t)k * M;
             im_ppo_minibatch mb;
             im_status s = IM_OK;
-            // (one copy of the observations as bf16 rows, in the actor's input buffer, serves both nets)
+            // one copy of the observations as bf16 rows, in the actor's input buffer, serves both nets; the critic's own holds
+            // the last minibatch afterwards as well
             im_trainer *t = u->actor;
+            uint16_t *critic_rows = ep == epochs - 1 && k == n_minibatches - 1 ? u->critic->H[0] : nullptr;
             if (!perm) {
                 // contiguous block: the observations are converted, the rest is read in place
-                s = im_f32_to_bf16_padded(v->obs + r0 * v->ld_obs, v->ld_obs, M, D, t->H[0], t->Kp[0], st);
+                s = im::f32_to_bf16_padded(v->obs + r0 * v->ld_obs, v->ld_obs, M, D, t->H[0], critic_rows, t->Kp[0], st);
                 mb = {v->action + r0 * A, v->mean + r0 * A, nullptr, v->logp + r0, v->advantage + r0, v->value + r0, v->returns + r0};
             } else {
                 const im::GatherArgs ga = {v->obs, v->action, v->mean, v->logp, v->advantage, v->value, v->returns, perm + (int64_t)ep * total + r0,
-                                           v->ld_obs, total, M, D, A, t->Kp[0], t->H[0], u->g_action, u->g_mean_old, u->g_logp_old,
+                                           v->ld_obs, total, M, D, A, t->Kp[0], t->H[0], critic_rows, u->g_action, u->g_mean_old, u->g_logp_old,
                                            u->g_advantage, u->g_value_old, u->g_returns, t->status};
                 if (im::launch_gather_minibatch(ga, st) != cudaSuccess) s = IM_ERR_CUDA;
                 mb = {u->g_action, u->g_mean_old, nullptr, u->g_logp_old, u->g_advantage, u->g_value_old, u->g_returns};

@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kThreads) gather_minibatch_kernel(const __grid
             src = src < 0 ? 0 : P.n_src - 1;
         }
         const float *row = P.obs + src * P.ld_obs;
-        __nv_bfloat16 *h = reinterpret_cast<__nv_bfloat16 *>(P.h) + (long long)i * P.ld_h;
+        uint16_t *h = P.h + (long long)i * P.ld_h, *h2 = P.h2 ? P.h2 + (long long)i * P.ld_h : nullptr;
 #pragma unroll 1
         for (int c0 = 4 * lane; c0 < P.ld_h; c0 += 128 * kRowBatch) {
             float v[kRowBatch][4];                                // loads in flight together
@@ -342,7 +342,9 @@ __global__ void __launch_bounds__(kThreads) gather_minibatch_kernel(const __grid
             for (int q = 0; q < kRowBatch; ++q) {
                 const int c = c0 + 128 * q;
                 const __nv_bfloat162 lo = __floats2bfloat162_rn(v[q][0], v[q][1]), hi = __floats2bfloat162_rn(v[q][2], v[q][3]);
-                if (c < P.ld_h) *reinterpret_cast<uint2 *>(h + c) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+                const uint2 w = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+                if (c < P.ld_h) *reinterpret_cast<uint2 *>(h + c) = w;
+                if (h2 && c < P.ld_h) *reinterpret_cast<uint2 *>(h2 + c) = w;
             }
         }
         const long long o = (long long)i * P.A, s = src * P.A;

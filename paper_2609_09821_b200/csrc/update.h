@@ -82,10 +82,13 @@ struct GatherArgs {
     const int32_t *idx;
     long long ld_obs, n_src;
     int M, D, A, ld_h;
-    uint16_t *h;
+    uint16_t *h, *h2;                                      // h2: a second copy, or null
     float *g_action, *g_mean, *g_logp, *g_advantage, *g_value, *g_returns;
     uint32_t *status;
 };
 cudaError_t launch_gather_minibatch(const GatherArgs &a, cudaStream_t stream);
+
+// im_f32_to_bf16_padded with an optional second copy.
+im_status f32_to_bf16_padded(const float *in, int64_t ld_in, int rows, int cols, uint16_t *out, uint16_t *out2, int ld_out, cudaStream_t st);
 
 }  // namespace im

@@ -87,3 +87,25 @@ def test_moments_of_any_length(n):
     std = ref.std(ddof=1) if n > 1 else 0.0
     want = np.array([ref.mean(), 1.0 / (std + 1e-8)])
     assert np.all(np.abs(got - want) <= 2e-7 * np.abs(want))         # fp64 sums, one rounding to fp32
+
+
+@pytest.mark.parametrize("shuffled", [False, True])
+@pytest.mark.parametrize("D", [361, 70])
+def test_both_nets_input_rows_hold_the_last_minibatch(shuffled, D):
+    import torch
+    from paper_2609_09821_b200 import rollout as R, trainer as T
+    T_, N, A, ld = 4, 96, 5, (D + 63) // 64 * 64
+    wa, wc = W.make_policy_weights((D, 64, A), "f32", 3), W.make_policy_weights((D, 128, 1), "f32", 4)
+    M = T_ * N // 2
+    a, c = T.MlpTrainer((D, 64, A), wa["W"], wa["b"], M), T.MlpTrainer((D, 128, 1), wc["W"], wc["b"], M)
+    upd = T.PpoUpdater(a, c, torch.full((A,), -1.0), lr=1e-5)
+    st = R.RolloutStorage(T_, N, A, ld)
+    g = torch.Generator("cuda").manual_seed(1)
+    for x in (st.obs, st.action, st.mean, st.logp, st.value, st.advantage, st.returns):
+        x.copy_(torch.randn(x.shape, device="cuda", generator=g))
+    perm = torch.stack([torch.randperm(T_ * N, device="cuda", generator=g) for _ in range(2)]).to(torch.int32) if shuffled else None
+    T.update_from_storage(upd, st, 2, 2, perm)
+    flat = st.obs[:T_].reshape(T_ * N, ld)[:, :D]
+    want = torch.zeros(M, ld, dtype=torch.bfloat16, device="cuda")
+    want[:, :D] = (flat[perm[1, M:].long()] if shuffled else flat[M:]).bfloat16()
+    assert torch.equal(a.input_rows(M), want) and torch.equal(c.input_rows(M), want)
