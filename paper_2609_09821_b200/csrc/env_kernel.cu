@@ -20,6 +20,8 @@
 // that the issue slots count: the chain kernel does both in one warp per chain,
 // which loads every body once, and stages half rows, so that four CTAs share an SM.
 // Figures at launch_env_kernel.
+#include <algorithm>
+
 #include <cuda_bf16.h>
 
 #include "im_internal.h"
@@ -970,7 +972,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
 // the first target floats -- and columns [c1, D) -- the targets.
 // OPT compiles in the optional semantics (grace steps, motion randomisation, adaptive initialisation, extended
 // observation); envs that use none run the instantiation without them.
-template <bool OPT, bool AOS>
+template <bool RESET_ALL, bool OPT, bool AOS>
 __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
     // a successor launched with programmatic stream serialization (the policy's first GEMM) may be scheduled
@@ -1020,7 +1022,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
 
     // ---- pass A: reference at the advanced time, errors against the simulated state,
     //      observation entries of the simulated bodies
-    {
+    if (!RESET_ALL) {
         clip = P.clip_id[envc];
         if (clip < 0 || clip >= P.C) {
             clip = min(max(clip, 0), P.C - 1);
@@ -1109,7 +1111,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
 #pragma unroll
         for (int i = 0; i < kPartials; ++i) part[(i * C + c) * kTile + lane] = acc[i];
     }
-    __syncthreads();
+    if (!RESET_ALL) __syncthreads();
 
     // ---- decision.  Chain 0 adds the chains' partial sums in chain order, forms the reward and writes reward,
     //      flags and the new per-env state.  Every other thread of the env needs the flags as well: it repeats the
@@ -1119,20 +1121,20 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     E.clip = clip; E.cyc = cyc; E.t = t1; E.cm = cm; E.loop = loop; E.grace = grace;
     {
         float term[IM_N_TERMS], r = INFINITY;
-        if (c == 0 || P.reward.r_min > -INFINITY) r = reward_of(P, part, C, lane, term);
-        decide<false, OPT>(P, envc, root_z, r, c == 0 && valid, E);
+        if (!RESET_ALL && (c == 0 || P.reward.r_min > -INFINITY)) r = reward_of(P, part, C, lane, term);
+        decide<RESET_ALL, OPT>(P, envc, root_z, r, c == 0 && valid, E);
         if (c == 0) {
             int ep_done = 0;                    // steps of the episode this step ended (0 where none ended)
-            if (valid) {
+            if (!RESET_ALL && valid) {
                 P.reward_out[env] = r;
                 if (P.terms_out) {
 #pragma unroll
                     for (int k = 0; k < IM_N_TERMS; ++k) P.terms_out[(size_t)k * P.N + env] = term[k];
                 }
                 P.flags_out[env] = (uint8_t)E.flags;
-                ep_done = store_env_state<OPT>(P, env, E);
             }
-            if (OPT && P.summary) add_summary(P, valid, r, E.flags, ep_done, lane);
+            if (valid) ep_done = store_env_state<OPT>(P, env, E);
+            if (OPT && !RESET_ALL && P.summary) add_summary(P, valid, r, E.flags, ep_done, lane);
         }
     }
     const bool reset = E.reset;
@@ -1175,9 +1177,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             if (k == 0) Hn = make_heading(s.q, s.p);
             if ((Lc.flags & LINK_OWN) && reset) {
                 body_obs(Hn, s.q, s.p, s.v, s.w, row1, b);
-                if (P.write_back && valid) {
-                    sv.st_body(b, s.q, s.p, s.v, s.w);
-                }
+                if (!RESET_ALL && P.write_back && valid) sv.st_body(b, s.q, s.p, s.v, s.w);
             }
         }
         if (reset) H = Hn;
@@ -1306,17 +1306,17 @@ __global__ void debug_math_kernel(int op, int n, const float *__restrict__ in, f
 
 // Registers: the chain kernel has 96, so that four CTAs of five chains share an SM (64 for trees with more than eight
 // leaves, whose CTAs have up to 1024 threads); the role kernel 168 where every CTA has an SM of its own, else 96 (two).
-template <bool OPT, bool AOS>
+template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(96) env_chain_kernel(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<OPT, AOS>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS>(P, smem_raw);
 }
-template <bool OPT, bool AOS>
+template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __launch_bounds__(1024, 1) env_chain_kernel_wide(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<OPT, AOS>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS>(P, smem_raw);
 }
 template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(168) env_role_kernel_1(const __grid_constant__ EnvKernelParams P)
@@ -1330,11 +1330,10 @@ __global__ void __maxnreg__(96) env_role_kernel_2(const __grid_constant__ EnvKer
     extern __shared__ __align__(16) float smem_raw[];
     env_role_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
 }
-template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __launch_bounds__(1024, 1) env_role_kernel_wide(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_role_body<RESET_ALL, OPT, AOS, true>(P, smem_raw);
+    env_role_body<false, false, false, true>(P, smem_raw);
 }
 
 template <typename K>
@@ -1347,10 +1346,16 @@ cudaError_t prepare_one()
 {
     cudaError_t e = allow_smem(env_role_kernel_1<RESET_ALL, OPT, AOS>);
     if (e == cudaSuccess) e = allow_smem(env_role_kernel_2<RESET_ALL, OPT, AOS>);
-    if (e == cudaSuccess) e = allow_smem(env_role_kernel_wide<RESET_ALL, OPT, AOS>);
-    if (e == cudaSuccess && !RESET_ALL) e = allow_smem(env_chain_kernel<OPT, AOS>);
-    if (e == cudaSuccess && !RESET_ALL) e = allow_smem(env_chain_kernel_wide<OPT, AOS>);
+    if (e == cudaSuccess) e = allow_smem(env_chain_kernel<RESET_ALL, OPT, AOS>);
+    if (e == cudaSuccess) e = allow_smem(env_chain_kernel_wide<RESET_ALL, OPT, AOS>);
     return e;
+}
+
+// CTAs of `threads` threads that an SM holds, by shared memory, registers and threads.
+int ctas_per_sm(size_t smem, int regs, int threads)
+{
+    const int by_smem = (int)(kMaxSmemFloats * sizeof(float) / (smem + 1024)), by_regs = 65536 / (regs * threads), by_threads = 2048 / threads;
+    return std::max(1, std::min(by_smem, std::min(by_regs, by_threads)));
 }
 
 // (The kernels with options start plainly: started early their CTAs, several to an SM, crowd onto the SMs that drain
@@ -1362,16 +1367,20 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
     const unsigned tiles = (unsigned)((p.N + kTile - 1) / kTile);
     const int extra = (p.n_future - 1) * 9 * __builtin_popcount(p.sk.ee_mask) + p.act_dim;
     const size_t role_smem = role_smem_floats(staged_cols(p.sk.J, C, p.sk.n_links, extra), C, p.sk.n_links) * sizeof(float);
-    const int role_per_sm = C <= 8 && role_smem <= 112 * 1024 && C * 64 * 96 * 2 <= 65536 ? 2 : 1;
-    void (*kernel)(EnvKernelParams);
-    if (RESET_ALL || tiles <= (unsigned)(role_per_sm * n_sm)) {
-        kernel = C > 8 ? env_role_kernel_wide<RESET_ALL, OPT, AOS>
-                 : tiles <= (unsigned)n_sm && C * 64 * 168 <= 65536 ? env_role_kernel_1<RESET_ALL, OPT, AOS> : env_role_kernel_2<RESET_ALL, OPT, AOS>;
+    const unsigned role_fit = (unsigned)n_sm * ctas_per_sm(role_smem, C <= 8 ? 96 : 64, C <= 16 ? 64 * C : 1024);
+    const unsigned chain_fit = (unsigned)n_sm * ctas_per_sm(chain_smem, C <= 8 ? 96 : 64, 32 * C);
+    bool role;
+    if (RESET_ALL) role = C <= 8 && (tiles <= role_fit || (!OPT && tiles > chain_fit));
+    else role = tiles <= std::min(role_fit, 2u * (unsigned)n_sm) && (C <= 8 || (!OPT && !AOS));
+    if (role) {
+        void (*kernel)(EnvKernelParams) = tiles <= (unsigned)n_sm && C * 64 * 168 <= 65536 ? env_role_kernel_1<RESET_ALL, OPT, AOS>
+                                                                                           : env_role_kernel_2<RESET_ALL, OPT, AOS>;
+        if (C > 8) kernel = env_role_kernel_wide;
         const dim3 block(32 * (C <= 16 ? 2 * C : 32));
         if (OPT) kernel<<<tiles, block, role_smem, stream>>>(p);
         else launch_pdl(kernel, dim3(tiles), block, role_smem, stream, 0, p);
-    } else if constexpr (!RESET_ALL) {
-        kernel = C > 8 ? env_chain_kernel_wide<OPT, AOS> : env_chain_kernel<OPT, AOS>;
+    } else {
+        void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS> : env_chain_kernel<RESET_ALL, OPT, AOS>;
         if (OPT) kernel<<<tiles, 32 * C, chain_smem, stream>>>(p);
         else launch_pdl(kernel, dim3(tiles), dim3(32 * C), chain_smem, stream, 0, p);
     }
@@ -1388,7 +1397,8 @@ cudaError_t env_kernel_prepare()
 {
     static DeviceOnce once;
     return once.run([] {
-        cudaError_t e = prepare_one<false, false, false>();
+        cudaError_t e = allow_smem(env_role_kernel_wide);
+        if (e == cudaSuccess) e = prepare_one<false, false, false>();
         if (e == cudaSuccess) e = prepare_one<true, false, false>();
         if (e == cudaSuccess) e = prepare_one<false, true, false>();
         if (e == cudaSuccess) e = prepare_one<true, true, false>();
@@ -1417,8 +1427,14 @@ cudaError_t launch_debug_math(int op, int n, const float *in, float *out, cudaSt
 // Which kernel: the role kernel while its tiles fit the SMs at once, the chain kernel beyond (us per launch in a chain of
 // them, 15 bodies / 24 bodies, role against chain: 64 envs 7.8 / 12.4 against 15.0 / 22.5; 4096 envs 9.7 / 14.1 against
 // 17.6 / 23.6; 9472 envs, two CTAs per SM, 14.2 / 20.9 against 19.4 / 26.2; 12000 envs 24.2 / 34.9 against 23.5 / 32.0;
-// 65536 envs 89.5 / 142 against 88 / 125).  A reset of all envs has no simulated state to load twice: always the role
-// kernel (65536 envs x 24 bodies 77 against 85 us).
+// 65536 envs 89.5 / 142 against 88 / 125).  Trees with more than eight leaves fill an SM with one CTA of either kernel, and
+// only without options and records is the role kernel the faster one (31 leaves, 4096 envs: 25.0 against 25.4 us plain, 41.3
+// against 34.4 with options, 45.0 against 38.0 from records).
+// A reset of all envs: the role kernel while its tiles fit the SMs at once, then the chain kernel while its do (12000 envs, 15 /
+// 24 bodies: 14.2 / 18.4 against 11.8 / 15.1 us), and beyond that, where a plain reset has no simulated state to load twice, the
+// role kernel again (20000 envs 20.5 / 26.9 against 23.3 / 29.1; 65536 envs 47.9 / 64.6 against 51.0 / 65.1), but with options, whose
+// code it spills, the chain kernel (20000 envs x 24 bodies 56.5 against 47.1); trees with more than eight leaves always the chain
+// kernel (12 leaves, 9500 envs: 23.0 against 17.9; with options 46.0 against 28.9).
 cudaError_t launch_env_kernel(const EnvKernelParams &p, bool reset_all, size_t smem, cudaStream_t stream)
 {
     const bool opt = p.grace_steps > 0 || p.reset_noise_std > 0.0f || p.n_bins > 0 || p.n_future > 1 || p.act_dim > 0 ||

@@ -169,3 +169,38 @@ def test_every_warp_decides_alike_at_the_grace_limit(skeleton):
 
     for whole, a, b in zip(run(0, N), run(0, N // 2), run(N // 2, N // 2)):
         assert torch.equal(whole, torch.cat([a, b]))
+
+
+@pytest.mark.parametrize("options", [False, True])
+@pytest.mark.parametrize("tree", ["humanoid15", "smpl24", 1, 9])
+@pytest.mark.parametrize("n", [9472, 9473, 18944, 18945])
+def test_reset_of_all_envs_equals_its_shards(n, tree, options):
+    """Row counts on either side of what fits the SMs at once with two and with four CTAs each; shards of one CTA per SM."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    skel = W.make_skeleton(tree, 1) if isinstance(tree, str) else _tree(tree)
+    J = skel["J"]
+    lib = W.make_clip_library(J, 4, (20, 40), 30.0, 1)
+    sk = B.Skeleton(skel["parents"], skel["offsets"], skel["masses"])
+    clips = B.Clips(sk, lib["n_frames"], lib["fps"], lib["root_pos"], lib["local_quat"])
+    if options:
+        clips.set_cyclic([1, 0, 0, 1])
+    extra = 2 * 9 * sk.n_ee + 7 if options else 0
+
+    def run(base, n):
+        env = B.Env(sk, clips, B.make_env_config(n, 1 / 30, 5, W.REWARD_MULT, 0.3, B.padded_ld(24 * J + 1 + extra), env_id_base=base,
+                                                 **(dict(grace_steps=2, reset_noise_std=0.05) if options else {})))
+        if options:
+            env.set_obs_extension(3, torch.ones(n, 7, device="cuda"))
+            env.set_reset_bins(3, np.arange(12, dtype=np.float32).reshape(4, 3))
+        obs = torch.full((n, env.ld_obs), 7.0, device="cuda")
+        env.reset_all(obs, 3)
+        starts = env.reset_stats()[0] if options else None
+        return [obs] + list(env.get_state()), starts
+
+    whole, starts = run(0, n)
+    parts = [run(b, min(4736, n - b)) for b in range(0, n, 4736)]
+    for i, x in enumerate(whole):
+        assert torch.equal(x, torch.cat([p[0][i] for p in parts]))
+    if options:
+        assert torch.equal(starts, sum(p[1] for p in parts))
