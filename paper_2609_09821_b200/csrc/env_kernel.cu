@@ -975,9 +975,6 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
 template <bool RESET_ALL, bool OPT, bool AOS>
 __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
-    // a successor launched with programmatic stream serialization (the policy's first GEMM) may be scheduled
-    // onto SMs as this grid drains; it waits for this grid's completion before it reads anything
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const SkelDev &sk = P.sk;
     const int J = sk.J;
     const int D = 24 * J + 1;
@@ -1282,6 +1279,11 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     }
     __syncthreads();
     copy_out_any(P, tile, S2, S2 >> 2, c1 >> 2, P.ld_obs >> 2, c, C, lane);
+    // a successor launched with programmatic stream serialization (the policy's first GEMM) may be scheduled onto SMs as this
+    // grid drains; it waits for this grid's completion before it reads anything.  Released last: another env's step right
+    // behind this one would crowd onto the slots that this grid leaves free (12000 envs, 15 / 24 bodies, one step after the
+    // other: released at the start 23.4 / 31.3 us, 25.6 / 49.5 from records; now 20.8 / 28.2 and 21.8 / 39.5)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Diagnostic kernel: the scalar building blocks of the env kernel on caller-given inputs, one thread per item.
