@@ -35,9 +35,10 @@ constexpr int UMMA_K = 16;
 // Epilogue warps of the hidden-layer kernels: two per tensor-memory lane quadrant, which share the tile's 64-column chunks
 // and have one staging slab each (four warps with two slabs against it, in a chain of launches: 8192 x 1024 x 384 10.4 ->
 // 9.1 us, 4096 x 2048 x 384 11.2 -> 9.3, 16384 x 1024 x 384 15.9 -> 14.9).  64-column tiles have one chunk and keep four
-// warps, as does the backward epilogue of the single-CTA kernel.
-constexpr __host__ __device__ int hidden_epi_warps(int block_n, bool bwd) { return bwd || block_n == 64 ? 4 : 8; }
-constexpr __host__ __device__ int hidden_threads(int block_n, bool bwd) { return 64 + 32 * hidden_epi_warps(block_n, bwd); }
+// warps, as do the backward epilogue of the single-CTA kernel and the M/N-major products, which have neither bias nor floor
+// (384 x 2048 over 16 slices of 256 rows: 11.0 us with eight, 10.5 with four).
+constexpr __host__ __device__ int hidden_epi_warps(int block_n, bool mn, bool bwd) { return mn || bwd || block_n == 64 ? 4 : 8; }
+constexpr __host__ __device__ int hidden_threads(int block_n, bool mn, bool bwd) { return 64 + 32 * hidden_epi_warps(block_n, mn, bwd); }
 // Limit of every bounded wait below (2 s unless im_debug_set_wait changed it), and the diagnostic switch that makes the
 // TMA producers issue nothing, so that a test can watch a wait run out with no copy or MMA in flight.
 __device__ unsigned long long g_wait_limit_ns = 2000000000ull;
@@ -266,8 +267,11 @@ template <bool MN>
 __device__ __forceinline__ void slice_k_blocks(const GemmParams &P, int b, int &kb0, int &n_kb)
 {
     if (!MN) { kb0 = 0; n_kb = P.K_blocks; return; }
-    kb0 = (int)((long long)b * P.kb_total / P.n_batches);
-    n_kb = (int)((long long)(b + 1) * P.kb_total / P.n_batches) - kb0;
+    // floor(b kb_total / n) in 32 bits: 64-bit divisions cost a short slice a tenth of its time (there is a remainder only for
+    // the trainer's slices, 64 at most)
+    const uint32_t n = (uint32_t)P.n_batches, q = (uint32_t)P.kb_total / n, r = (uint32_t)P.kb_total % n, u = (uint32_t)b;
+    kb0 = (int)(u * q + (r ? u * r / n : 0u));
+    n_kb = (int)((u + 1u) * q + (r ? (u + 1u) * r / n : 0u)) - kb0;
 }
 
 // Which output tile the number `tile` stands for: net, slice, row and column of tiles.
@@ -545,7 +549,7 @@ template <bool DUAL>
 using SecondNet = std::conditional_t<DUAL, DualMaps, NoMaps>;
 
 template <int BLOCK_N, bool MN = false, bool BWD = false, bool DUAL = false>
-__global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
+__global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, BWD), 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                        const __grid_constant__ CUtensorMap map_b,
                                                                        const __grid_constant__ CUtensorMap map_c,
                                                                        const __grid_constant__ CUtensorMap map_m,
@@ -560,7 +564,7 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
     const int n_tiles = tiles_per_slice * (MN ? P.n_batches : 1) * (DUAL ? 2 : 1);
     const CUtensorMap *map_c2 = &map_c, *map_m2 = &map_m;
     if constexpr (DUAL) { map_c2 = &second.c; map_m2 = &second.m; }
-    pipe_init<Plan>(p, hidden_epi_warps(BLOCK_N, BWD));
+    pipe_init<Plan>(p, hidden_epi_warps(BLOCK_N, MN, BWD));
     const uint32_t tmem_base = *p.tmem_slot;
     dep_release();
     dep_wait();                       // nothing before this line touches global memory
@@ -574,7 +578,7 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, BWD), 1) linear_tc_hid
         if (lane == 0) mma_role<Plan, BLOCK_N, MN, DUAL>(p, tmem_base, P, n_tiles, tiles_per_slice);
     } else {
         const int quad = warp & 3;                    // TMEM lanes 32*quad .. 32*quad+31 belong to this warp
-        constexpr bool kFour = hidden_epi_warps(BLOCK_N, BWD) == 4;
+        constexpr bool kFour = hidden_epi_warps(BLOCK_N, MN, BWD) == 4;
         constexpr int kSlabs = kFour ? 2 : 1, kStep = kFour ? 64 : 128;
         const int half = kFour ? 0 : (warp - 2) >> 2;                            // first chunk of this warp
         uint8_t *slabs = p.epi + (size_t)(warp - 2) * kSlabs * kEpiSlabBytes;  // two are used alternately
@@ -1312,7 +1316,7 @@ cudaError_t launch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParams 
     const int grid = tiles < n_sm ? tiles : n_sm;
     SecondNet<DUAL> second;
     if constexpr (DUAL) second = {L2->map_a, L2->map_b, L2->map_c, L2->map_m};
-    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, BWD)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
+    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, MN, BWD)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
                                       L.map_m, gp, second);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
