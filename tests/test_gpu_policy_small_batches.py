@@ -1,4 +1,4 @@
-"""The policy forward on small batches (narrow tiles, several partial accumulators) against the same layers on CTA pairs:
+"""The policy forward on small batches (narrow tiles) against the same layers on CTA pairs:
 ragged last row blocks, deep and shallow nets, value heads, per-dimension standard deviations, staged input."""
 import pytest
 
@@ -108,3 +108,33 @@ def test_joint_forward_runs_nets_of_other_widths_one_after_the_other():
         critic.value_forward(obs, sep[3])
         actor.forward_with_value(3, critic, obs, *joint)
         assert all(torch.equal(a, b) for a, b in zip(joint, sep))
+
+
+@pytest.mark.parametrize("dims", [(361, 1024, 512, 28), (577, 1024, 1024, 512, 69), (433, 192, 64, 17)])
+@pytest.mark.parametrize("n", [130, 2500, 9001, 20000])
+def test_split_batches_are_the_whole_bit_for_bit(n, dims):
+    """Tile width, CTA pairs and the critic's place in the actor's launches follow the row count; the results do not."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    wa, wc = W.make_policy_weights(dims, "bf16", 1), W.make_policy_weights(dims[:-1] + (1,), "bf16", 2)
+    A = dims[-1]
+    obs = torch.randn(n, B.padded_ld(dims[0]), device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+
+    def run(base, rows, joint):
+        actor = B.Policy(dims, wa["W_bf16"], wa["b"], "bf16", 0.3, 9, rows, env_id_base=base)
+        critic = B.Policy(dims[:-1] + (1,), wc["W_bf16"], wc["b"], "bf16", 0.3, 9, rows)
+        out = [torch.full((rows, k), 7.0, device="cuda") for k in (A, A, 1, 1)]
+        x = obs[base:base + rows]
+        if joint:
+            actor.forward_with_value(3, critic, x, *out)
+        else:
+            actor.forward(3, x, *out[:3])
+            critic.value_forward(x, out[3])
+        torch.cuda.synchronize()
+        assert actor.device_status() == 0 and critic.device_status() == 0
+        return out
+
+    whole, step = run(0, n, False), (n + 6) // 7
+    parts = [run(b, min(step, n - b), b % 2 == 1) for b in range(0, n, step)]
+    for i, (a, b) in enumerate(zip(whole, run(0, n, True))):
+        assert torch.equal(a, b) and torch.equal(a, torch.cat([p[i] for p in parts]))
