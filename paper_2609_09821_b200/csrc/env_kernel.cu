@@ -76,8 +76,8 @@ __host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, 
     return (size_t)kTile * (s1 > s2 ? s1 : s2) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links;
 }
 
-// The role kernel: the staged rows, the chains' partial sums, their link records.  Staged columns: all, or, where an extended observation is too wide for that, the first
-// 24 J (the rest is then written column by column).
+// The role kernel: the staged rows, the chains' partial sums, their link records.  Staged columns: all, or, where an
+// extended observation is too wide for that, the first 24 J (the rest is then written column by column).
 __host__ __device__ inline size_t role_smem_floats(int cols, int n_chains, int n_links)
 {
     return (size_t)kTile * tile_stride(cols) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links;
@@ -662,8 +662,8 @@ __device__ __forceinline__ void st_direct(const EnvKernelParams &P, int env, int
 }
 
 // The role kernel.  OPT compiles in the optional semantics (grace steps, motion randomisation, adaptive initialisation,
-// extended observation, looped clips, summaries); envs that use none run the instantiation without them.  WIDE: more
-// (chain, role) pairs than warps (trees with more than eight leaves).
+// extended observation, looped clips, summaries); envs that use none run the instantiation without them.  WIDE: a
+// warp may have several (chain, role) pairs (trees with more than eight leaves).
 template <bool RESET_ALL, bool OPT, bool AOS, bool WIDE>
 __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *smem_raw)
 {

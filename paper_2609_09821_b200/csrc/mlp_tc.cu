@@ -4,9 +4,10 @@
 //
 //   warp 0      TMA producer: A and W tiles (128B-swizzled, K-major) into a ring of smem stages
 //   warp 1      MMA issuer: tcgen05.mma 128 x BLOCK_N x 16 into one of two TMEM accumulators
-//   warps 2..5  epilogue: tcgen05.ld the finished accumulator, add bias, then either ReLU + bf16
-//               store (hidden layers) or the Gaussian head (last layer: mean, Philox/Box-Muller
-//               noise, action, log-probability), while the MMA warp works on the next tile
+//   warps 2..   epilogue (four or eight warps; sixteen of the last layer): tcgen05.ld the finished
+//               accumulator, add bias, then either ReLU + bf16 store (hidden layers) or the Gaussian
+//               head (last layer: mean, Philox/Box-Muller noise, action, log-probability), while the
+//               MMA warp works on the next tile
 //
 // Hidden activations stay bf16 and L2-resident between layers.  Every wait on
 // an mbarrier is bounded: when the limit runs out the kernel raises
@@ -43,7 +44,6 @@ constexpr __host__ __device__ int hidden_threads(int block_n, bool mn, bool bwd)
 // TMA producers issue nothing, so that a test can watch a wait run out with no copy or MMA in flight.
 __device__ unsigned long long g_wait_limit_ns = 2000000000ull;
 __device__ int g_skip_loads = 0;
-
 
 // ------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -204,7 +204,6 @@ struct GemmParams {
     // forward pass), and the column sums of the masked fp32 values over each 32-row block r / 32 go to
     // colsum_partial[(r / 32) * ld_partial + c] (M a multiple of 32).  Either may be null.
     const __nv_bfloat16 *mask;
-    long long ld_mask;
     float *colsum_partial;
     int ld_partial;
     // Two nets' products of equal sizes in one launch (DUAL instantiations): the first half of the tiles is the first net's,
@@ -455,8 +454,6 @@ __device__ __forceinline__ void reduce_scatter_step(float *v, int lane, int offs
     }
 }
 
-// One epilogue chunk of the hidden-layer kernels: 64 accumulator columns of this thread's row -> bias, floor,
-// (BWD: ReLU mask of the forward activations, column sums over the warp's 32 rows) -> 32 packed bf16 pairs.
 // ReLU mask of the backward epilogue: each epilogue warp keeps two 32-row x 64-column boxes of the forward
 // activations in shared memory (128B-swizzled, like the output slabs), fetched by TMA one chunk ahead.
 __device__ __forceinline__ void mask_issue(const CUtensorMap *map_m, uint8_t *slab, uint64_t *bar, int col0, int row0)
@@ -479,6 +476,8 @@ __device__ __forceinline__ void mask_all_positive(uint4 (&mk)[8])
     for (int c = 0; c < 8; ++c) mk[c] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
 }
 
+// One epilogue chunk of the hidden-layer kernels: 64 accumulator columns of this thread's row -> bias, floor,
+// (BWD: ReLU mask of the forward activations, column sums over the warp's 32 rows) -> 32 packed bf16 pairs.
 template <bool BWD>
 __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_addr, int row, int col0, int lane,
                                              const uint4 (&mk)[8], uint32_t (&pk)[32], const float *bias, float *colsum)
@@ -711,8 +710,6 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// TMA load into this CTA's shared memory whose completion is signalled on a barrier that may live
-// in the peer CTA (cluster address).
 // Tensor memory of a CTA pair: one warp of EACH CTA issues the allocation, both get the same base.
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t *dst_smem, uint32_t ncols)
 {
@@ -723,6 +720,8 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
+// TMA load into this CTA's shared memory whose completion is signalled on a barrier that may live
+// in the peer CTA (cluster address).
 __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *map, uint32_t bar_cluster_addr, int x, int y)
 {
     asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -1202,7 +1201,8 @@ __global__ void obs_to_bf16_kernel(const float *obs, int ld_obs, int cols, __nv_
 {
     if (early) dep_release();
     dep_wait();
-    // (a row's chunks and the rows are below 2^31 together: a batch holds n ld_out bf16 values, 16 bytes a chunk)
+    // (in 32 bits: beside the observations that they come from and the hidden layers' buffers, the device's memory holds fewer
+    // than 2^32 of these 16-byte chunks)
     const uint32_t chunks = (uint32_t)ld_out / 8u, total = (uint32_t)n * chunks;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int r = (int)(i / chunks), c = (int)(i - (uint32_t)r * chunks) * 8;
@@ -1259,8 +1259,8 @@ bool make_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, 
 
 // Columns of a tile: the whole action row for the last layer; else the narrowest of 64, 128, 256 whose tiles still fit
 // the SMs in one wave (a lone tile's time is its operand loads and its epilogue, both shorter when it is narrow:
-// 1024 x 1024 x 384 in a chain of launches 4.96 us with 64 columns, 5.68 with 128, 7.22 with 256; 2048 rows 6.96 / 5.79 /
-// 7.37), and the widest that divides N once there are several waves (8192 rows 17.1 / 12.1 / 10.4).
+// 1024 x 1024 x 384 in a chain of launches 4.62 us with 64 columns, 5.39 with 128, 6.54 with 256; 2048 rows 6.21 / 5.45 /
+// 6.64), and the widest that divides N once there are several waves (4096 rows 9.37 / 7.24 / 6.89, 8192 rows 14.1 / 10.7 / 9.3).
 int pick_block_n(int rows, int N, bool last, int n_sm)       // rows: 128-row tiles
 {
     if (last) return (N + 15) / 16 * 16;
@@ -1381,8 +1381,10 @@ cudaError_t dispatch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParam
     // CTA pairs pay off when the main loop is long enough to amortise the cluster set-up and there
     // are at least two waves of 256 x 256 tiles; otherwise the single-CTA kernel's finer tiles
     // balance the machine better (measured: 16384 x 1024 x 384 is 8 % faster single, 16384 x 1024 x 2048
-    // 7 % faster paired).  The tiles of both nets count: actor and critic of 361-1024-512 on 16384 rows take 63.5 us with
-    // the second layer paired, 67.6 with it single; of 577-1024-1024-512 on 11000 rows 60.7 and 71.5 (9001 rows: 48.7, 47.8)
+    // 7 % faster paired).  The tiles of both nets count.  Actor and critic, conversion included, with and without
+    // pairs: 577-1024-1024-512 on 8000 / 9001 / 10000 / 11000 / 16384 rows 82.8 / 84.2 / 101.0 / 102.8 / 138 us and 82.2 / 84.0 /
+    // 103.4 / 105.7 / 149; 361-2048-1024 on 4800 / 9001 / 16384 rows 65.8 / 93.4 / 163 and 68.2 / 99.6 / 172; 361-1024-512 on 16384 rows
+    // 69.5 and 73.1
     const int pair_tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * (DUAL ? 2 : 1);
     const bool bwd = gp.mask || gp.colsum_partial;
     // (the backward epilogue is the longer part of a tile when K is short, and the pair kernel runs it on
@@ -1541,11 +1543,12 @@ im_status convert_obs(im_policy *p, int n, const float *obs, int ld_obs)
     const long long chunks = (long long)n * (tc->ld_in / 8);
     const int block = 256;
     long long grid = (chunks + block - 1) / block;
-    if (grid > 148 * 16) grid = 148 * 16;
+    const long long most = (long long)tc->n_sm * 16;
+    if (grid > most) grid = most;
     // The first GEMM is let in early while every block of this grid is about to start (64 rows of 361-1024-512-28: 16.8 -> 16.0
     // us a forward, 9001 rows 28.1 -> 27.7); its large CTAs would keep a longer grid's blocks waiting (65536 rows 142 -> 144)
     const dim3 blocks((unsigned)grid), threads(block);
-    if (grid < 148 * 16)
+    if (grid < most)
         launch_pdl(obs_to_bf16_kernel, blocks, threads, 0, p->stream, 0, obs, (int)ld_obs, (int)p->cfg.dims[0], tc->d_in, tc->ld_in, n, 1);
     else obs_to_bf16_kernel<<<blocks, threads, 0, p->stream>>>(obs, ld_obs, p->cfg.dims[0], tc->d_in, tc->ld_in, n, 0);
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -1663,7 +1666,7 @@ im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, in
     gp.n_batches = 1;
     if (x.mask || x.colsum_partial) gp.bias = nullptr;     // the backward product has no bias: its epilogue skips the add
     else if (y) gp.bias2 = y->bias;
-    gp.mask = static_cast<const __nv_bfloat16 *>(x.mask); gp.ld_mask = x.ld_mask;
+    gp.mask = static_cast<const __nv_bfloat16 *>(x.mask);
     gp.colsum_partial = x.colsum_partial; gp.ld_partial = ld_partial;
     if (y) gp.colsum_partial2 = y->colsum_partial;
     gp.status = status;

@@ -2,8 +2,8 @@
 // handle (fp32 master weights, Adam state, bf16 working copies, activation and gradient buffers, the
 // buffer plan and the row-slice choice of the dW products) and a PPO updater handle that sequences one
 // minibatch update of an actor and a critic, or all epochs and minibatches of a collected rollout.
-// Host code only: every arithmetic step is one of the library's kernels, reached through the same entry
-// points a caller could use one by one.
+// Host code only: the products and the loss are the kernels that callers reach one by one, the steps between
+// them those of update.cu.
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -63,8 +63,8 @@ namespace {
 
 // One net on its input rows x, or two of equal widths (the last but) whose products of a kind share their launches: a
 // layer's tiles seldom fill the last wave of SMs, and two nets' dW products need half the row slices each.  An update of an
-// actor and a critic (361-1024-512-28 and ...-1) on 16000 rows:
-// 311 -> 258 us (131072 rows of 577-1024-1024-512-69, where every product fills the machine many times over: 2965 -> 2955).
+// actor and a critic (361-1024-512-28 and ...-1) on 16000 rows, im_ppo_update in a CUDA graph: 279 -> 231 us (131072 rows of
+// 577-1024-1024-512-69, where every product fills the machine many times over: 2904 -> 2886).
 struct Nets {
     im_trainer *a, *c;                                     // c: null for one net
     uint16_t *xa, *xc;                                     // input rows (their own, or those of another trainer)

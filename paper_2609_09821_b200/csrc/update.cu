@@ -1,10 +1,9 @@
 // Multi-tensor kernels of the update phase (see update.h).
 //
-// A small minibatch's update is bound by launches: 16000 rows of 361-1024-512-28 (and ...-1) took 69 of them, two
-// thirds no tensor-core product, 260 us of a 552 us update.  Here each kind of step between the products is one launch
-// over every tensor of both nets: 24 launches, 354 us; 311 us with every thread's loads issued in batches before anything
-// is done with them, 258 us with the two nets' products in common launches (131072 rows of 577-1024-1024-512-69: 3583 ->
-// 3400 -> 3300 -> 3265 us).
+// A small minibatch's update is bound by launches: one of 16000 rows of 361-1024-512-28 (and ...-1) took 62 of them, two
+// thirds no tensor-core product.  Here each kind of step between the products is one launch over every tensor of both nets
+// (22 launches, 14 with the nets' products in common ones), and a thread's loads are issued in batches before anything is
+// done with them.  im_ppo_update in a CUDA graph: 231 us; 131072 rows of 577-1024-1024-512-69 2886 us.
 #include <cmath>
 #include <cuda_bf16.h>
 
@@ -429,7 +428,7 @@ cudaError_t launch_out_grads(const OutGradArgs &a, cudaStream_t stream)
 cudaError_t launch_gather_minibatch(const GatherArgs &a, cudaStream_t stream)
 {
     const bool vec = (reinterpret_cast<uintptr_t>(a.obs) & 15u) == 0 && (a.ld_obs & 3) == 0;
-    const int blocks = (a.M + 7) / 8 < 148 * 16 ? (a.M + 7) / 8 : 148 * 16;
+    const int most = device_sm_count() * 16, blocks = (a.M + 7) / 8 < most ? (a.M + 7) / 8 : most;
     const cudaError_t e = launch_pdl(vec ? gather_minibatch_kernel<true> : gather_minibatch_kernel<false>, dim3((unsigned)blocks), dim3(kThreads), 0,
                                      stream, 0, a);
     g_launches.fetch_add(1, std::memory_order_relaxed);
