@@ -61,8 +61,8 @@ NCU_TRAFFIC = {
     "cfg4_65536_smpl24": dict(
         policy=dict(bytes=645075456, capture="linear_tc_hidden_pair_kernel<0, 0> x 3 + linear_tc_head_kernel<80>, one policy "
                                               "forward at 65536 envs (ncu --set full)"),
-        env=dict(bytes=291532288, capture="env_step_kernel_small<0, 0, 0> (now env_chain_kernel) writing fp32 and bf16 rows, one launch, "
-                                          "65536 envs (ncu --set full)")),
+        env=dict(bytes=289603072, capture="env_chain_kernel<0, 0, 0> writing fp32 and bf16 rows, one launch, 65536 envs "
+                                          "(dram__bytes_read.sum + dram__bytes_write.sum)")),
 }
 
 
@@ -245,7 +245,7 @@ def time_update(B, wl, pol, n, A, D, dev, stream, graph=True, reps=5):
         stream.synchronize()
         up_graph = None
         if graph:
-            # the update's ~100 launches are replayed from one CUDA graph, as a training loop would run them
+            # the update's launches are replayed from one CUDA graph, as a training loop would run them
             up_graph = torch.cuda.CUDAGraph()
             with torch.cuda.graph(up_graph, stream=stream):
                 upd.update(Mu, ub)
