@@ -391,7 +391,8 @@ im_status im_value_forward(im_policy *critic, int32_t n, const float *obs, int32
 im_status im_value_forward_staged(im_policy *critic, im_policy *src, int32_t n, float *value_out);
 /* What a rollout step asks of both nets: im_policy_forward on the actor, then im_value_forward on the critic, on the
  * same observations (obs == NULL: the bf16 rows staged in the actor's buffer, as for the *_staged calls).  Tensor-core
- * nets on one stream with equal widths but for the last run layer by layer in common launches. */
+ * nets on one stream with equal widths but for the last run layer by layer in common launches (a wait that runs out
+ * there is reported in both status words). */
 im_status im_policy_value_forward(im_policy *actor, im_policy *critic, uint32_t step, int32_t n, const float *obs, int32_t ld_obs,
                                   float *mean_out, float *action_out, float *logp_out, float *value_out);
 
@@ -621,9 +622,8 @@ int32_t im_trainer_dw_slices(int32_t Np, int32_t Kp, int64_t M, int32_t max_spli
  *     rows, advantage moments (if normalize_advantage), im_ppo_loss, both backward passes, the norm over every
  *     gradient tensor (global-norm clip at max_grad_norm), Adam on every tensor and on the log-std, the
  *     learning rate from the mean KL (as im_adaptive_lr).  Nets of equal widths but for the last share the
- *     launches of their products; a wait that runs out there is reported in the actor's status word.  The
- *     minibatch's observations must already sit in both
- *     trainers' input rows.  mb: DEVICE float arrays -- action, mean_old [M][A]; logp_old, advantage,
+ *     launches of their products; a wait that runs out there is reported in both status words.  The
+ *     minibatch's observations must already sit in both trainers' input rows.  mb: DEVICE float arrays -- action, mean_old [M][A]; logp_old, advantage,
  *     value_old (needed with clip_value_loss), returns [M]; log_std_old [A] or NULL for the updater's own copy.
  *   im_ppo_update_rollout  the whole update phase over a collected rollout: `epochs` passes over
  *     `n_minibatches` blocks of the T * N samples (row t * N + e of the time-major arrays of `view`;

@@ -52,12 +52,14 @@ struct GemmOperands {
     int64_t ld_mask;
     float *colsum_partial;
 };
-im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status,
+// status2: the second product's status word, or null.
+im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status, uint32_t *status2,
                   cudaStream_t stream);
 int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm, int nets);
 im_status tc_gemm_tn(const GemmOperands &x, const GemmOperands *y, int R, int Mo, int No, int slices, int c_pitch, uint32_t *status,
-                     cudaStream_t stream);
-im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int N, int N2, int K, uint32_t *status, cudaStream_t stream);
+                     uint32_t *status2, cudaStream_t stream);
+im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int N, int N2, int K, uint32_t *status, uint32_t *status2,
+                       cudaStream_t stream);
 // bounded-wait diagnostics of the tensor-core GEMM kernels and of the bulk-copy PPO loss kernel (current device)
 cudaError_t tc_set_wait_debug(unsigned long long limit_ns, int skip_loads);
 cudaError_t ppo_set_wait_debug(unsigned long long limit_ns, int skip_loads);

@@ -218,8 +218,15 @@ struct GemmParams {
     float sigma;
     const float *log_std;   // [N] per-column ln(sigma), or null: the scalar sigma for every column
     uint32_t seed_lo, seed_hi, step, env_id_base;
-    uint32_t *status;
+    uint32_t *status, *status2;      // status2: of the second net, or null
 };
+
+// A wait ran out in this launch: reported to every net that has a part in it.
+__device__ __forceinline__ void report_timeout(const GemmParams &P)
+{
+    atomicOr(P.status, IM_DEV_WAIT_TIMEOUT);
+    if (P.status2) atomicOr(P.status2, IM_DEV_WAIT_TIMEOUT);
+}
 
 constexpr int kEpiSlabBytes = 32 * 128;    // one epilogue warp's 32 rows x 64 bf16 staging slab
 
@@ -334,7 +341,7 @@ __device__ __forceinline__ void pipe_init(const Pipe &p, int epi_arrivals)
 
 // Common exit: everyone meets, the allocating warp frees tensor memory.
 template <class Plan>
-__device__ __forceinline__ void pipe_exit(const Pipe &p, uint32_t tmem_base, uint32_t *status)
+__device__ __forceinline__ void pipe_exit(const Pipe &p, uint32_t tmem_base, const GemmParams &P)
 {
     if (*p.abort_flag && (threadIdx.x & 31) == 0) {
         // a wait ran out: give copies and MMAs that are still in flight time to land (bounded)
@@ -343,7 +350,7 @@ __device__ __forceinline__ void pipe_exit(const Pipe &p, uint32_t tmem_base, uin
     }
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0 && *p.abort_flag) atomicOr(status, IM_DEV_WAIT_TIMEOUT);
+    if (threadIdx.x == 0 && *p.abort_flag) report_timeout(P);
     if ((threadIdx.x >> 5) == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, Plan::kTmemCols);
@@ -653,7 +660,7 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, BWD), 1) linear_tc
         }
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // stores complete before smem goes away
     }
-    pipe_exit<Plan>(p, tmem_base, P.status);
+    pipe_exit<Plan>(p, tmem_base, P);
 }
 
 // ------------------------------------------------------------------ hidden layers, CTA pairs
@@ -990,7 +997,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();
-    if (threadIdx.x == 0 && *abort_flag) atomicOr(P.status, IM_DEV_WAIT_TIMEOUT);
+    if (threadIdx.x == 0 && *abort_flag) report_timeout(P);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem_base, kPairTmemCols);
@@ -1189,7 +1196,7 @@ __global__ void __launch_bounds__(kHeadThreads, 1) linear_tc_head_kernel(const _
         }
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
-    pipe_exit<Plan>(p, tmem_base, P.status);
+    pipe_exit<Plan>(p, tmem_base, P);
     // Released late: the env step usually comes next, several CTAs to an SM, and an earlier start would pack them onto
     // the SMs that this grid leaves idle
     dep_release();
@@ -1613,7 +1620,7 @@ im_status tc_policy_value_forward(im_policy *a, im_policy *c, uint32_t step, int
         TcLayer L = with_width(a->tc->layers[l], 2 * rows, last, n_sm), L2 = with_width(c->tc->layers[l], 2 * rows, last, n_sm);
         if (l == 0) L2.map_a = L.map_a;                          // one copy of the observations serves both
         set_layer(gp, L);
-        gp.bias2 = L2.d_bias; gp.N2 = L2.N; gp.mean2 = value_out;
+        gp.bias2 = L2.d_bias; gp.N2 = L2.N; gp.mean2 = value_out; gp.status2 = c->d_status;
         const cudaError_t e = last ? dispatch_head<true>(L, gp, n_sm, {L2.map_a, L2.map_b_head(L.block_n), L2.map_a, L2.map_a}, a->stream)
                                    : dispatch_hidden<true>(L, &L2, gp, n_sm, false, a->stream);
         if (e != cudaSuccess) return IM_ERR_CUDA;
@@ -1651,7 +1658,7 @@ bool layer_of(TcLayer &L, const GemmOperands &o, int M, int N, int K, int block_
 // C[M][N] = act(A[M][K] B[N][K]^T + bias) on the hidden-layer kernels, operands anywhere in device
 // memory: the tensor maps are encoded for this call and travel as kernel parameters.  y: a second product of the same
 // sizes in the same launch (both with a mask, or with column sums, or neither), or null.
-im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status,
+im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status, uint32_t *status2,
                   cudaStream_t stream)
 {
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
@@ -1669,7 +1676,7 @@ im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, in
     gp.mask = static_cast<const __nv_bfloat16 *>(x.mask);
     gp.colsum_partial = x.colsum_partial; gp.ld_partial = ld_partial;
     if (y) gp.colsum_partial2 = y->colsum_partial;
-    gp.status = status;
+    gp.status = status; gp.status2 = status2;
     const cudaError_t e = y ? dispatch_hidden<true>(L, &L2, gp, n_sm, false, stream) : dispatch_hidden<false>(L, nullptr, gp, n_sm, false, stream);
     return e == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
@@ -1704,7 +1711,7 @@ int tc_tn_slices(int Mo, int No, int c_pitch, int R, int max_slices, int n_sm, i
 // results stacked with a pitch of `c_pitch` rows.  Operands are read M/N-major, so no transposed copy
 // of either matrix is needed.
 im_status tc_gemm_tn(const GemmOperands &x, const GemmOperands *y, int R, int Mo, int No, int slices, int c_pitch, uint32_t *status,
-                     cudaStream_t stream)
+                     uint32_t *status2, cudaStream_t stream)
 {
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
@@ -1730,7 +1737,7 @@ im_status tc_gemm_tn(const GemmOperands &x, const GemmOperands *y, int R, int Mo
     gp.M = Mo; gp.N = No; gp.kb_total = R / BLOCK_K; gp.n_tiles_n = L[0].n_tiles_n; gp.bias = nullptr;    // no bias in this product
     gp.act_floor = -INFINITY;
     gp.n_batches = slices; gp.c_batch_rows = c_pitch;
-    gp.status = status;
+    gp.status = status; gp.status2 = status2;
     const bool pairs = tn_takes_pairs(Mo, No, R, slices, c_pitch, n_sm, y ? 2 : 1);
     const cudaError_t e = y ? dispatch_mn<true>(L[0], &L[1], gp, pairs, n_sm, stream) : dispatch_mn<false>(L[0], nullptr, gp, pairs, n_sm, stream);
     return e == cudaSuccess ? IM_OK : IM_ERR_CUDA;
@@ -1739,7 +1746,8 @@ im_status tc_gemm_tn(const GemmOperands &x, const GemmOperands *y, int R, int Mo
 // mean[M][N] (fp32, dense) = A[M][K] B[N][K]^T + bias on the Gaussian-head kernel without sampling: o.C is the mean.
 // B must hold ceil(N / 16) * 16 rows (rows beyond N zero), bias as many floats.  y: a second product in the same launch,
 // of N2 <= N columns, or null.
-im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int N, int N2, int K, uint32_t *status, cudaStream_t stream)
+im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int N, int N2, int K, uint32_t *status, uint32_t *status2,
+                       cudaStream_t stream)
 {
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
@@ -1756,7 +1764,7 @@ im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int 
     gp.M = M; gp.N = N; gp.K_blocks = K / BLOCK_K; gp.n_tiles_n = 1; gp.bias = x.bias;
     gp.mean = static_cast<float *>(x.C); gp.sigma = 1.0f;
     gp.n_batches = 1;
-    gp.status = status;
+    gp.status = status; gp.status2 = status2;
     if (!y) return dispatch_head<false>(L, gp, n_sm, NoMaps(), stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
     DualMaps second;
     if (!make_map(&second.a, y->A, (uint64_t)M, (uint64_t)K, (uint64_t)y->lda, BLOCK_M) ||

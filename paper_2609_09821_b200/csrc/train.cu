@@ -316,7 +316,7 @@ im_status im_gemm_bf16(const uint16_t *A, int64_t lda, const uint16_t *B, int64_
     if (!A || !B || !C || !bias || !status || M < 1 || N < 64 || K < 64) return IM_ERR_INVALID_ARG;
     if ((N & 63) || (K & 63) || lda < K || ldb < K || ldc < N || (lda & 7) || (ldb & 7) || (ldc & 7)) return IM_ERR_INVALID_ARG;
     if (!al16(A) || !al16(B) || !al16(C) || !al16(bias)) return IM_ERR_INVALID_ARG;
-    return tc_gemm({A, lda, B, ldb, C, ldc, bias, nullptr, 0, nullptr}, nullptr, M, N, K, relu != 0, 0, status, (cudaStream_t)cuda_stream);
+    return tc_gemm({A, lda, B, ldb, C, ldc, bias, nullptr, 0, nullptr}, nullptr, M, N, K, relu != 0, 0, status, nullptr, (cudaStream_t)cuda_stream);
 }
 
 im_status im_gemm_bf16_dgrad(const uint16_t *dZ, int64_t ld_dz, const uint16_t *Wt, int64_t ld_wt, uint16_t *dH, int64_t ld_dh,
@@ -329,7 +329,7 @@ im_status im_gemm_bf16_dgrad(const uint16_t *dZ, int64_t ld_dz, const uint16_t *
     if (!al16(dZ) || !al16(Wt) || !al16(dH)) return IM_ERR_INVALID_ARG;
     if (H && (ld_h < N || (ld_h & 7) || !al16(H))) return IM_ERR_INVALID_ARG;
     if (colsum_partial && (ld_partial < N || (ld_partial & 1) || (reinterpret_cast<uintptr_t>(colsum_partial) & 7u))) return IM_ERR_INVALID_ARG;
-    return tc_gemm({dZ, ld_dz, Wt, ld_wt, dH, ld_dh, nullptr, H, ld_h, colsum_partial}, nullptr, M, N, K, false, ld_partial, status,
+    return tc_gemm({dZ, ld_dz, Wt, ld_wt, dH, ld_dh, nullptr, H, ld_h, colsum_partial}, nullptr, M, N, K, false, ld_partial, status, nullptr,
                    (cudaStream_t)cuda_stream);
 }
 
@@ -343,7 +343,7 @@ im_status im_gemm_bf16_tn(const uint16_t *A, int64_t lda, const uint16_t *B, int
         return IM_ERR_INVALID_ARG;
     if (c_pitch < Mo || (c_pitch & 127)) return IM_ERR_INVALID_ARG;
     if (!al16(A) || !al16(B) || !al16(C)) return IM_ERR_INVALID_ARG;
-    return tc_gemm_tn({A, lda, B, ldb, C, ldc, nullptr, nullptr, 0, nullptr}, nullptr, R, Mo, No, slices, c_pitch, status, (cudaStream_t)cuda_stream);
+    return tc_gemm_tn({A, lda, B, ldb, C, ldc, nullptr, nullptr, 0, nullptr}, nullptr, R, Mo, No, slices, c_pitch, status, nullptr, (cudaStream_t)cuda_stream);
 }
 
 im_status im_sum_slices_bf16_to_f32(const uint16_t *in, int64_t slice_stride, int64_t ld_in, int32_t slices, int32_t rows,
@@ -367,7 +367,7 @@ im_status im_gemm_bf16_f32out(const uint16_t *A, int64_t lda, const uint16_t *B,
     if (!A || !B || !C || !bias || !status || M < 1 || N < 1 || N > 80 || K < 64) return IM_ERR_INVALID_ARG;
     if ((K & 63) || lda < K || ldb < K || (lda & 7) || (ldb & 7)) return IM_ERR_INVALID_ARG;
     if (!al16(A) || !al16(B) || !al16(C)) return IM_ERR_INVALID_ARG;
-    return tc_gemm_head({A, lda, B, ldb, C, N, bias, nullptr, 0, nullptr}, nullptr, M, N, 0, K, status, (cudaStream_t)cuda_stream);
+    return tc_gemm_head({A, lda, B, ldb, C, N, bias, nullptr, 0, nullptr}, nullptr, M, N, 0, K, status, nullptr, (cudaStream_t)cuda_stream);
 }
 
 im_status im_transpose_bf16(const uint16_t *in, int64_t ld_in, int32_t rows, int32_t cols, uint16_t *out, int64_t ld_out,

@@ -89,12 +89,13 @@ im::GemmOperands forward_operands(im_trainer *tr, uint16_t *x, int l)
 im_status forward_on(const Nets &n, int M)
 {
     im_trainer *a = n.a;
+    uint32_t *status2 = n.c ? n.c->status : nullptr;
     im_status s = IM_OK;
     for (int l = 0; l < a->nl && s == IM_OK; ++l) {
         const im::GemmOperands x = forward_operands(a, n.xa, l), y = n.c ? forward_operands(n.c, n.xc, l) : x;
         const im::GemmOperands *py = n.c ? &y : nullptr;
-        if (l < a->nl - 1) s = im::tc_gemm(x, py, M, a->Np[l], a->Kp[l], true, 0, a->status, a->stream);
-        else s = im::tc_gemm_head(x, py, M, a->dims[a->nl], n.c ? n.c->dims[n.c->nl] : 0, a->Kp[l], a->status, a->stream);
+        if (l < a->nl - 1) s = im::tc_gemm(x, py, M, a->Np[l], a->Kp[l], true, 0, a->status, status2, a->stream);
+        else s = im::tc_gemm_head(x, py, M, a->dims[a->nl], n.c ? n.c->dims[n.c->nl] : 0, a->Kp[l], a->status, status2, a->stream);
     }
     return s;
 }
@@ -121,10 +122,11 @@ im_status backward_of(im_trainer *tr, uint16_t *x, im_trainer *tr2, uint16_t *x2
         return o;
     };
     im::GemmOperands o = tr2 ? dw(tr2, x2) : im::GemmOperands();
-    im_status s = im::tc_gemm_tn(dw(tr, x), tr2 ? &o : nullptr, M, Np, Kp, *slices, Npb, tr->status, tr->stream);
+    uint32_t *status2 = tr2 ? tr2->status : nullptr;
+    im_status s = im::tc_gemm_tn(dw(tr, x), tr2 ? &o : nullptr, M, Np, Kp, *slices, Npb, tr->status, status2, tr->stream);
     if (l == 0 || s != IM_OK) return s;
     if (tr2) o = dh(tr2);
-    return im::tc_gemm(dh(tr), tr2 ? &o : nullptr, M, Kp, Np, false, Kp, tr->status, tr->stream);
+    return im::tc_gemm(dh(tr), tr2 ? &o : nullptr, M, Kp, Np, false, Kp, tr->status, status2, tr->stream);
 }
 im_status backward_products(const Nets &n, int M, int (*slices)[IM_MAX_LAYERS])
 {

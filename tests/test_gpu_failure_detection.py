@@ -72,3 +72,21 @@ def test_ppo_loss_wait_runs_out_and_the_next_launch_is_correct(short_wait_withou
     want = O.ppo_loss(pb_np, 0.2, 2.0, 2.5e-4, True)
     np.testing.assert_allclose(outs[3].cpu().numpy()[:4], want["summary"][:4], rtol=2e-4, atol=2e-5)
     assert torch.isfinite(outs[0]).all()
+
+
+def test_a_wait_in_a_common_launch_is_reported_to_both_nets(short_wait_without_loads):
+    """Actor and critic of equal widths run in common launches, in a forward and in an update; either handle's status word
+    tells of a wait that ran out there, as it does where the launches are the nets' own."""
+    from paper_2609_09821_b200 import trainer as T
+    M, dims, cdims = 64, (64, 64, 4), (64, 64, 1)
+    for c in (cdims, (64, 128, 1)):
+        wa, wc = W.make_policy_weights(dims, "bf16", 1), W.make_policy_weights(c, "bf16", 2)
+        actor, critic = B.Policy(dims, wa["W_bf16"], wa["b"], "bf16", 0.3, 9, M), B.Policy(c, wc["W_bf16"], wc["b"], "bf16", 0.3, 9, M)
+        out = [torch.zeros(M, k, device="cuda") for k in (4, 4, 1, 1)]
+        actor.forward_with_value(1, critic, torch.zeros(M, 64, device="cuda"), *out)
+        assert actor.device_status() & IM_DEV_WAIT_TIMEOUT and critic.device_status() & IM_DEV_WAIT_TIMEOUT
+        a, v = T.MlpTrainer(dims, wa["W"], wa["b"], M), T.MlpTrainer(c, wc["W"], wc["b"], M)
+        upd = T.PpoUpdater(a, v, torch.full((4,), -1.0), lr=1e-5)
+        z = lambda *s: torch.zeros(*s, device="cuda")
+        upd.update(M, dict(action=z(M, 4), mean_old=z(M, 4), logp_old=z(M), advantage=z(M), value_old=z(M), returns=z(M)))
+        assert a.device_status() & IM_DEV_WAIT_TIMEOUT and v.device_status() & IM_DEV_WAIT_TIMEOUT
