@@ -39,6 +39,7 @@ __device__ __forceinline__ uint2 pack_bf16x4(float4 v)
 }
 
 constexpr int kTile = 32;          // envs per CTA
+constexpr int kRing = 13;          // words per env of a staged body: rotation, position, linear and angular velocity
 constexpr int kPartials = 9;       // pose, vel, ee_pos, ee_rot, body_pos, body_vel, weighted com difference (3)
 
 // The bounds-checked build (-DIM_DEBUG, a second library next to the regular one): every index the kernel forms
@@ -68,12 +69,18 @@ __host__ __device__ inline int tile_stride(int D)
 // up to a multiple of four columns so that both halves start on a 16-byte boundary.
 __host__ __device__ inline int split_col(int J) { return (15 * J + 3) / 4 * 4; }
 
-// Shared memory, in floats: the staged half rows, the chains' partial sums, the chains' link records.
+// Shared memory of the chain kernel, in floats: the first half rows and behind them a staged body per chain (whose place the
+// chain's partial sums take later), or the second half rows, which are assembled when both are done with; then the chains'
+// link records.  (The second half's limit counts the partial sums: it decides which extended observations are accepted.)
+__host__ __device__ inline int chain_floats(int c1, int D_ext, int n_chains)
+{
+    const int s1 = tile_stride(c1), s2 = tile_stride(D_ext - c1);
+    const int first = kTile * s1 + kRing * n_chains * kTile, both = kTile * (s1 > s2 ? s1 : s2) + kPartials * n_chains * kTile;
+    return first > both ? first : both;
+}
 __host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, int extra_cols)
 {
-    const int D = 24 * J + 1 + extra_cols, c1 = split_col(J);
-    const int s1 = tile_stride(c1), s2 = tile_stride(D - c1);
-    return (size_t)kTile * (s1 > s2 ? s1 : s2) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links;
+    return (size_t)chain_floats(split_col(J), 24 * J + 1 + extra_cols, n_chains) + (size_t)8 * n_links;
 }
 
 // The role kernel: the staged rows, the chains' partial sums, their link records.  Staged columns: all, or, where an
@@ -424,6 +431,25 @@ __device__ __forceinline__ Quat sanitize(Quat q, uint32_t *status)
     return q;
 }
 
+// Four bytes from global to shared memory, behind the thread's back.  The policy as for the streaming loads below.
+__device__ __forceinline__ void cp_async_word(uint32_t dst, const float *src, uint64_t policy)
+{
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "l"(policy) : "memory");
+}
+__device__ __forceinline__ float lds32(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+// A body staged by stage_body, once its copies have landed.
+__device__ __forceinline__ SimBody lds_body(uint32_t a)
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return {{lds32(a), lds32(a + 128), lds32(a + 256), lds32(a + 384)}, {lds32(a + 512), lds32(a + 640), lds32(a + 768)},
+            {lds32(a + 896), lds32(a + 1024), lds32(a + 1152)}, {lds32(a + 1280), lds32(a + 1408), lds32(a + 1536)}};
+}
+
 // Body-state access of one thread (one env).  Two layouts:
 //   component rows (AOS = false): element (row, env) of an array lies at row * stride + env, rows 3 b + c (4 b + c for
 //     the quaternions); a warp load is one full line.  Offsets are 32-bit (the launcher checks the array sizes).
@@ -463,6 +489,30 @@ struct SimView {
         if (AOS) { const float *p = base + (long long)b * bs; return {p[0], p[1], p[2]}; }
         const uint32_t o = 3 * (uint32_t)b * st + e;
         return {__ldcs(base + o), __ldcs(base + o + st), __ldcs(base + o + 2 * st)};
+    }
+    // This env's state of body b to shared memory, asynchronously: component i (rotation, position, velocities) to the
+    // word at dst + 128 i bytes.  Every lane copies and later reads its own words.  The chain kernel, whose warps are bound by
+    // the latency of what they load (20 of them on an SM), so asks for a body while it walks the one before, at the price of no
+    // registers: us per step with the loads in the walk itself / staged a body ahead, 15 bodies x 16384 envs 23.9 / 22.5, x 65536
+    // 88.2 / 83.7; 24 bodies x 16384 32.6 / 30.7, x 65536 125.0 / 121.1; from records 24 bodies x 12000 43.6 / 42.1 (15: 28.5 /
+    // 28.7); spilled bytes 48 / 0.
+    __device__ __forceinline__ void stage_body(int b, uint32_t dst, uint64_t policy) const
+    {
+        if (AOS) {
+            const float *q = quat + (long long)b * bs_quat, *v[3] = {pos + (long long)b * bs_pos, lin + (long long)b * bs_lin, ang + (long long)b * bs_ang};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp_async_word(dst + 128 * i, q + i, policy);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) cp_async_word(dst + 128 * (4 + i), v[i / 3] + i % 3, policy);
+        } else {
+            const uint32_t o = 4 * (uint32_t)b * st + e, o3 = 3 * (uint32_t)b * st + e;
+            const float *v[3] = {pos, lin, ang};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp_async_word(dst + 128 * i, quat + (o + i * st), policy);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) cp_async_word(dst + 128 * (4 + i), v[i / 3] + (o3 + (i % 3) * st), policy);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
     __device__ __forceinline__ SimBody ld_body(int b) const { return {ld_quat(b), ld_pos(b), ld_lin(b), ld_ang(b)}; }
     __device__ __forceinline__ Vec3 ld_pos(int b) const { return ld_vec(pos, bs_pos, b); }
@@ -598,13 +648,14 @@ __device__ __forceinline__ void decide(const EnvKernelParams &P, int env, float 
 }
 
 // The seven error terms of an env from the chains' partial sums, added in chain order, and the reward.
+template <int PER_CHAIN>
 __device__ __forceinline__ float reward_of(const EnvKernelParams &P, const float *part, int C, int lane, float (&term)[IM_N_TERMS])
 {
     float e[kPartials];
 #pragma unroll
     for (int i = 0; i < kPartials; ++i) {
         float a = 0.0f;
-        for (int cc = 0; cc < C; ++cc) a += part[(i * C + cc) * kTile + lane];
+        for (int cc = 0; cc < C; ++cc) a += part[(cc * PER_CHAIN + i) * kTile + lane];
         e[i] = a;
     }
     // term order of the configuration: pose, vel, ee_pos, ee_rot, com, body_pos, body_vel
@@ -798,7 +849,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
                     }
                 }
 #pragma unroll
-                for (int i = 0; i < kPartials; ++i) part[(i * C + c) * kTile + lane] = acc[i];
+                for (int i = 0; i < kPartials; ++i) part[(c * kPartials + i) * kTile + lane] = acc[i];
             } else {
                 // ---- observation entries of the simulated bodies (an env known to be reset gets the reference's instead)
                 bool ignore = false;
@@ -819,7 +870,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
         if (need_r || P.write_back) __syncthreads();
         if (need_r) {
             float term[IM_N_TERMS];
-            r = reward_of(P, part, C, lane, term);
+            r = reward_of<kPartials>(P, part, C, lane, term);
         }
     }
     decide<RESET_ALL, OPT>(P, envc, root_z, r, warp == 0 && valid, E);
@@ -953,7 +1004,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     int ep_done = 0;                            // steps of the episode this step ended (0 where none ended)
     if (!RESET_ALL) {
         float term[IM_N_TERMS];
-        r = reward_of(P, part, C, lane, term);
+        r = reward_of<kPartials>(P, part, C, lane, term);
         if (valid) {
             P.reward_out[env] = r;
             P.flags_out[env] = (uint8_t)E.flags;
@@ -991,7 +1042,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     const bool valid = env < P.N;
     const int envc = valid ? env : P.N - 1;
     float *tile = smem_raw;
-    float *part = smem_raw + (size_t)kTile * (S1 > S2 ? S1 : S2);
+    float *part = smem_raw + kTile * S1;
     float *row1 = tile + (size_t)lane * S1;
     float *row2 = tile + (size_t)lane * S2;
     const int len = sk.chain_len[c];
@@ -999,7 +1050,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     const int RS = 2 + 2 * J;
 
     // this chain's link records: global -> shared, private to the warp
-    float4 *links = reinterpret_cast<float4 *>(part + (size_t)kPartials * C * kTile) + 2 * sk.link_start[c];
+    float4 *links = reinterpret_cast<float4 *>(smem_raw + chain_floats(c1, D_ext, C)) + 2 * sk.link_start[c];
     for (int i = lane; i < 2 * len; i += 32) links[i] = __ldg(P.links + 2 * sk.link_start[c] + i);
     __syncwarp();
     // this kernel is launched the same way: everything above reads only what the env's creation left in memory
@@ -1038,6 +1089,10 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         float alpha;
         lookup(cm, t1, frame, alpha);
         const float4 *r0 = P.frames + (size_t)IM_CHECKED(frame, P.n_rows) * RS;
+        uint64_t stream_policy;
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_policy));
+        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(part + c * kRing * kTile + lane);
+        sv.stage_body(ld_link(links, first_own).b, ring, stream_policy);
         LinkRec L = ld_link(links, 0);
         KeyPair keys = ld_keys(r0, L.b);
 
@@ -1061,14 +1116,6 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             const LinkRec Lc = L;
             const int b = Lc.b;
             const bool own = Lc.flags & LINK_OWN;
-            SimBody sim;
-            if (own) {                                // issue the loads before the interpolation math
-                if (!AOS) (void)IM_CHECKED((4 * (uint32_t)b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
-                sim.q = sv.ld_quat(b);
-                sim.p = sv.ld_pos(b);
-                sim.v = sv.ld_lin(b);
-                sim.w = sv.ld_ang(b);
-            }
             const KeyPair cur = keys;
             if (k + 1 < len) {                        // next joint's link and keyframe words in flight
                 L = ld_link(links, k + 1);
@@ -1079,6 +1126,11 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             joint_step<true>(r0, cur, alpha, cm.fps, Lc, k, s, ql, wl);
             if (OPT && k == 0) s.p = s.p + loop_shift(loop, cyc);    // completed cycles of a looped clip move the root
             if (own) {
+                SimBody sim = lds_body(ring);
+                if (k + 1 < len) {                    // the next body of the chain is an own one too
+                    if (!AOS) (void)IM_CHECKED((4 * (uint32_t)L.b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
+                    sv.stage_body(L.b, ring, stream_policy);
+                }
                 sim.q = sanitize(sim.q, P.status);
                 // the root's "parent" is the identity: qa = (1, 0, 0, 0), wa = 0 on the chain that owns it
                 const Quat ql_sim = qmul_conj(qa, sim.q);
@@ -1106,7 +1158,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             }
         }
 #pragma unroll
-        for (int i = 0; i < kPartials; ++i) part[(i * C + c) * kTile + lane] = acc[i];
+        for (int i = 0; i < kPartials; ++i) part[(c * kRing + i) * kTile + lane] = acc[i];
     }
     if (!RESET_ALL) __syncthreads();
 
@@ -1118,7 +1170,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     E.clip = clip; E.cyc = cyc; E.t = t1; E.cm = cm; E.loop = loop; E.grace = grace;
     {
         float term[IM_N_TERMS], r = INFINITY;
-        if (!RESET_ALL && (c == 0 || P.reward.r_min > -INFINITY)) r = reward_of(P, part, C, lane, term);
+        if (!RESET_ALL && (c == 0 || P.reward.r_min > -INFINITY)) r = reward_of<kRing>(P, part, C, lane, term);
         decide<RESET_ALL, OPT>(P, envc, root_z, r, c == 0 && valid, E);
         if (c == 0) {
             int ep_done = 0;                    // steps of the episode this step ended (0 where none ended)
