@@ -78,6 +78,8 @@ __host__ __device__ inline int chain_floats(int c1, int D_ext, int n_chains)
     const int first = kTile * s1 + kRing * n_chains * kTile, both = kTile * (s1 > s2 ? s1 : s2) + kPartials * n_chains * kTile;
     return first > both ? first : both;
 }
+// With whole rows staged.
+__host__ __device__ inline int whole_floats(int D_ext, int n_chains) { return kTile * (tile_stride(D_ext) + kRing * n_chains); }
 __host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, int extra_cols)
 {
     return (size_t)chain_floats(split_col(J), 24 * J + 1 + extra_cols, n_chains) + (size_t)8 * n_links;
@@ -1023,9 +1025,16 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
 // the first target floats -- and columns [c1, D) -- the targets.
 // OPT compiles in the optional semantics (grace steps, motion randomisation, adaptive initialisation, extended
 // observation); envs that use none run the instantiation without them.
-template <bool RESET_ALL, bool OPT, bool AOS>
+// WHOLE: the whole row is staged at once (both halves side by side), where that leaves as many CTAs on an SM.
+template <bool RESET_ALL, bool OPT, bool AOS, bool WHOLE>
 __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
+    // EARLY: the decision is taken before the reward is known, where it can be, and the first warp forms the reward while the
+    // others send rows out.  Not from records: warps of a tile that walk apart lose the lines that the records of their bodies
+    // share in L1 (15 bodies x 30000 envs 67.3 us, 71.0 with it).  us per step with two halves and the decision after the reward
+    // / EARLY / and WHOLE: 24 bodies x 65536 envs 121.0 / 116.6, x 30000 61.4 / 60.2; 15 bodies x 12000 19.6 / - / 17.8, x 16384
+    // 22.5 / - / 21.1, x 65536 83.6 / - / 76.6.
+    constexpr bool EARLY = !OPT && !AOS;
     const SkelDev &sk = P.sk;
     const int J = sk.J;
     const int D = 24 * J + 1;
@@ -1034,7 +1043,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     const int n_ee = OPT ? __popc(sk.ee_mask) : 0;
     const int ext_future = (OPT && P.n_future > 1) ? (P.n_future - 1) * 9 * n_ee : 0;
     const int D_ext = D + ext_future + (OPT ? P.act_dim : 0);
-    const int S1 = tile_stride(c1), S2 = tile_stride(D_ext - c1);
+    const int S1 = tile_stride(WHOLE ? D_ext : c1), S2 = WHOLE ? S1 : tile_stride(D_ext - c1);
     const int C = sk.n_chains;
     const int lane = threadIdx.x & 31;
     const int c = threadIdx.x >> 5;                 // this thread's chain
@@ -1044,13 +1053,13 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     float *tile = smem_raw;
     float *part = smem_raw + kTile * S1;
     float *row1 = tile + (size_t)lane * S1;
-    float *row2 = tile + (size_t)lane * S2;
+    float *row2 = tile + (size_t)lane * S2 + (WHOLE ? c1 : 0);
     const int len = sk.chain_len[c];
     const int first_own = sk.chain_first_own[c];
     const int RS = 2 + 2 * J;
 
     // this chain's link records: global -> shared, private to the warp
-    float4 *links = reinterpret_cast<float4 *>(smem_raw + chain_floats(c1, D_ext, C)) + 2 * sk.link_start[c];
+    float4 *links = reinterpret_cast<float4 *>(smem_raw + (WHOLE ? whole_floats(D_ext, C) : chain_floats(c1, D_ext, C))) + 2 * sk.link_start[c];
     for (int i = lane; i < 2 * len; i += 32) links[i] = __ldg(P.links + 2 * sk.link_start[c] + i);
     __syncwarp();
     // this kernel is launched the same way: everything above reads only what the env's creation left in memory
@@ -1160,32 +1169,32 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
 #pragma unroll
         for (int i = 0; i < kPartials; ++i) part[(c * kRing + i) * kTile + lane] = acc[i];
     }
-    if (!RESET_ALL) __syncthreads();
-
-    // ---- decision.  Chain 0 adds the chains' partial sums in chain order, forms the reward and writes reward,
-    //      flags and the new per-env state.  Every other thread of the env needs the flags as well: it repeats the
-    //      reward only if the reward can terminate an episode (r_min above -inf), else the root height and the
-    //      clip end decide alone.  The reset draw is a function of (env, step) and is repeated by every thread.
+    // ---- decision, by every thread of the env, which waits for the reward only where that can end an episode (r_min above
+    //      -inf); else the root height and the clip end decide alone, and with EARLY the warps do not meet before their rows are
+    //      whole.  The reset draw is a function of (env, step).  With write_back the reset states below go where other warps may
+    //      still have to load: every warp reads the root, and its chain's parent of the first own body, which another chain owns.
+    const bool need_r = !RESET_ALL && P.reward.r_min > -INFINITY;
+    if (!RESET_ALL && (!EARLY || need_r || P.write_back)) __syncthreads();
     EnvState E;
     E.clip = clip; E.cyc = cyc; E.t = t1; E.cm = cm; E.loop = loop; E.grace = grace;
-    {
-        float term[IM_N_TERMS], r = INFINITY;
-        if (!RESET_ALL && (c == 0 || P.reward.r_min > -INFINITY)) r = reward_of<kRing>(P, part, C, lane, term);
-        decide<RESET_ALL, OPT>(P, envc, root_z, r, c == 0 && valid, E);
-        if (c == 0) {
-            int ep_done = 0;                    // steps of the episode this step ended (0 where none ended)
-            if (!RESET_ALL && valid) {
-                P.reward_out[env] = r;
-                if (P.terms_out) {
+    float term[IM_N_TERMS], r = INFINITY;
+    if (need_r || (!RESET_ALL && !EARLY && c == 0)) r = reward_of<kRing>(P, part, C, lane, term);
+    decide<RESET_ALL, OPT>(P, envc, root_z, r, c == 0 && valid, E);
+    // The first warp writes reward, flags and the new per-env state.
+    const auto store_results = [&] {
+        int ep_done = 0;                        // steps of the episode this step ended (0 where none ended)
+        if (!RESET_ALL && valid) {
+            P.reward_out[env] = r;
+            if (P.terms_out) {
 #pragma unroll
-                    for (int k = 0; k < IM_N_TERMS; ++k) P.terms_out[(size_t)k * P.N + env] = term[k];
-                }
-                P.flags_out[env] = (uint8_t)E.flags;
+                for (int k = 0; k < IM_N_TERMS; ++k) P.terms_out[(size_t)k * P.N + env] = term[k];
             }
-            if (valid) ep_done = store_env_state<OPT>(P, env, E);
-            if (OPT && !RESET_ALL && P.summary) add_summary(P, valid, r, E.flags, ep_done, lane);
+            P.flags_out[env] = (uint8_t)E.flags;
         }
-    }
+        if (valid) ep_done = store_env_state<OPT>(P, env, E);
+        if (OPT && !RESET_ALL && P.summary) add_summary(P, valid, r, E.flags, ep_done, lane);
+    };
+    if (!EARLY && c == 0) store_results();
     const bool reset = E.reset;
     const float t_cur = E.t_new;
     const ClipMeta cmc = E.cm_new;
@@ -1253,17 +1262,26 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             if (15 * J + 2 < c1) row1[15 * J + 2] = tp.y;
         }
     }
-    __syncthreads();
-
-    // ---- first half of the rows to global memory
-    copy_out_any(P, tile, S1, c1 >> 2, 0, c1 >> 2, c, C, lane);
-    __syncthreads();
+    // Rows leave by all warps, or (EARLY) by all but the first, which forms the reward meanwhile
+    const bool apart = EARLY && C > 1;
+    const int copier = apart ? c - 1 : c, n_copiers = apart ? C - 1 : C;
+    const auto finish = [&] {
+        if (!RESET_ALL) r = reward_of<kRing>(P, part, C, lane, term);
+        store_results();
+    };
+    if (!WHOLE) {
+        __syncthreads();
+        // ---- first half of the rows to global memory
+        if (EARLY && c == 0) finish();
+        if (copier >= 0) copy_out_any(P, tile, S1, c1 >> 2, 0, c1 >> 2, copier, n_copiers, lane);
+        __syncthreads();
+    }
 
     // ---- pass B: reference pose one control interval ahead, seen from the same heading frame,
     //      into the second half (which reuses the shared memory of the first)
     {
         if (c == 0) {
-            for (int i = D_ext - c1; i < S2; ++i) row2[i] = 0.0f;
+            for (int i = D_ext - c1; i < (WHOLE ? S2 - c1 : S2); ++i) row2[i] = 0.0f;
             if (15 * J >= c1) row2[15 * J - c1] = phase;
         }
         LinkRec L = ld_link(links, 0);
@@ -1330,7 +1348,12 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         }
     }
     __syncthreads();
-    copy_out_any(P, tile, S2, S2 >> 2, c1 >> 2, P.ld_obs >> 2, c, C, lane);
+    if (WHOLE) {
+        if (c == 0) finish();
+        if (copier >= 0) copy_out_any(P, tile, S1, S1 >> 2, 0, P.ld_obs >> 2, copier, n_copiers, lane);
+    } else {
+        copy_out_any(P, tile, S2, S2 >> 2, c1 >> 2, P.ld_obs >> 2, c, C, lane);
+    }
     // a successor launched with programmatic stream serialization (the policy's first GEMM) may be scheduled onto SMs as this
     // grid drains; it waits for this grid's completion before it reads anything.  Released last: another env's step right
     // behind this one would crowd onto the slots that this grid leaves free (12000 envs, 15 / 24 bodies, one step after the
@@ -1364,13 +1387,18 @@ template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(96) env_chain_kernel(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<RESET_ALL, OPT, AOS>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
+}
+__global__ void __maxnreg__(96) env_chain_kernel_whole(const __grid_constant__ EnvKernelParams P)
+{
+    extern __shared__ __align__(16) float smem_raw[];
+    env_chain_body<false, false, false, true>(P, smem_raw);
 }
 template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __launch_bounds__(1024, 1) env_chain_kernel_wide(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<RESET_ALL, OPT, AOS>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
 }
 template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(168) env_role_kernel_1(const __grid_constant__ EnvKernelParams P)
@@ -1435,8 +1463,16 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         else launch_pdl(kernel, dim3(tiles), block, role_smem, stream, 0, p);
     } else {
         void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS> : env_chain_kernel<RESET_ALL, OPT, AOS>;
-        if (OPT) kernel<<<tiles, 32 * C, chain_smem, stream>>>(p);
-        else launch_pdl(kernel, dim3(tiles), dim3(32 * C), chain_smem, stream, 0, p);
+        // (a reset of all envs keeps the halves: its warps have little to wait for, and 12000 envs x 15 bodies took 14.4 us with whole
+        // rows, 12.7 without)
+        const size_t whole = ((size_t)whole_floats(24 * p.sk.J + 1, C) + 8 * p.sk.n_links) * sizeof(float);
+        size_t smem = chain_smem;
+        if (!RESET_ALL && !OPT && !AOS && C <= 8 && ctas_per_sm(whole, 96, 32 * C) >= ctas_per_sm(chain_smem, 96, 32 * C)) {
+            kernel = env_chain_kernel_whole;
+            smem = whole;
+        }
+        if (OPT) kernel<<<tiles, 32 * C, smem, stream>>>(p);
+        else launch_pdl(kernel, dim3(tiles), dim3(32 * C), smem, stream, 0, p);
     }
 }
 
@@ -1452,6 +1488,7 @@ cudaError_t env_kernel_prepare()
     static DeviceOnce once;
     return once.run([] {
         cudaError_t e = allow_smem(env_role_kernel_wide);
+        if (e == cudaSuccess) e = allow_smem(env_chain_kernel_whole);
         if (e == cudaSuccess) e = prepare_one<false, false, false>();
         if (e == cudaSuccess) e = prepare_one<true, false, false>();
         if (e == cudaSuccess) e = prepare_one<false, true, false>();

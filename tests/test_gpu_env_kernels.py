@@ -27,6 +27,8 @@ CASES = {
     "wide_extension": dict(options=True, n_future=8, act_dim=900),
     "many_leaves": dict(leaves=12, options=True, h_min=0.8),
     "too_many_leaves_for_a_warp_each": dict(leaves=15, h_min=0.8),
+    "one_chain": dict(leaves=1, h_min=0.8),
+    "one_chain_reward": dict(leaves=1, reward=W.REWARD_FIG5, r_min=0.3, write_back=True),
 }
 
 
