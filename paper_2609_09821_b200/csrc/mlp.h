@@ -51,6 +51,9 @@ struct GemmOperands {
     const void *mask;
     int64_t ld_mask;
     float *colsum_partial;
+    uint2 *bits_out;          // forward: one bit per output, whether it is positive ([N / 64][ld_bits] words), or null
+    const uint2 *bits_in;     // backward: those bits in the place of `mask`
+    int ld_bits;              // (of both nets)
 };
 // status2: the second product's status word, or null.
 im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status, uint32_t *status2,

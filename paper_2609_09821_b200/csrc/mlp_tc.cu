@@ -33,13 +33,21 @@ namespace {
 constexpr int BLOCK_M = 128;
 constexpr int BLOCK_K = 64;               // 64 bf16 = 128 bytes = one swizzle row
 constexpr int UMMA_K = 16;
+// Epilogues of the hidden-layer kernels: bias and floor; the same and the outputs' signs as bits; backward with the ReLU mask as
+// boxes of the forward activations; backward with the mask as bits.  A box costs as much L2 traffic as the output, which these
+// products are bound by: a minibatch update with boxes / bits, actor and critic, 16000 rows of 361-1024-512-28 258 / 250 us,
+// 131072 rows of 577-1024-1024-512-69 3435 / 3315.  (The bits are an epilogue of their own: tested for at run time they cost the
+// policy's products 1 %.)
+constexpr int kFwd = 0, kFwdBits = 1, kBwdBoxes = 2, kBwdBits = 3;
+constexpr __host__ __device__ bool is_bwd(int epi) { return epi >= kBwdBoxes; }
+
 // Epilogue warps of the hidden-layer kernels: two per tensor-memory lane quadrant, which share the tile's 64-column chunks
 // and have one staging slab each (four warps with two slabs against it, in a chain of launches: 8192 x 1024 x 384 10.4 ->
 // 9.1 us, 4096 x 2048 x 384 11.2 -> 9.3, 16384 x 1024 x 384 15.9 -> 14.9).  64-column tiles have one chunk and keep four
 // warps, as do the backward epilogue of the single-CTA kernel and the M/N-major products, which have neither bias nor floor
 // (384 x 2048 over 16 slices of 256 rows: 11.0 us with eight, 10.5 with four).
-constexpr __host__ __device__ int hidden_epi_warps(int block_n, bool mn, bool bwd) { return mn || bwd || block_n == 64 ? 4 : 8; }
-constexpr __host__ __device__ int hidden_threads(int block_n, bool mn, bool bwd) { return 64 + 32 * hidden_epi_warps(block_n, mn, bwd); }
+constexpr __host__ __device__ int hidden_epi_warps(int block_n, bool mn, int epi) { return mn || is_bwd(epi) || block_n == 64 ? 4 : 8; }
+constexpr __host__ __device__ int hidden_threads(int block_n, bool mn, int epi) { return 64 + 32 * hidden_epi_warps(block_n, mn, epi); }
 // Limit of every bounded wait below (2 s unless im_debug_set_wait changed it), and the diagnostic switch that makes the
 // TMA producers issue nothing, so that a test can watch a wait run out with no copy or MMA in flight.
 __device__ unsigned long long g_wait_limit_ns = 2000000000ull;
@@ -200,12 +208,17 @@ struct GemmParams {
     // M/N-major products: the contraction's kb_total k-blocks are shared out over the batches ("slices") as evenly as
     // whole k-blocks allow, slice b taking [b kb_total / n_batches, (b + 1) kb_total / n_batches)
     int kb_total;
-    // Backward-pass epilogue (BWD instantiations): output (r, c) is zeroed where mask[r][c] <= 0 (the ReLU of the
+    // Backward-pass epilogue (kBwdBoxes, kBwdBits): output (r, c) is zeroed where mask[r][c] <= 0 (the ReLU of the
     // forward pass), and the column sums of the masked fp32 values over each 32-row block r / 32 go to
     // colsum_partial[(r / 32) * ld_partial + c] (M a multiple of 32).  Either may be null.
     const __nv_bfloat16 *mask;
     float *colsum_partial;
     int ld_partial;
+    // The same mask as one bit per output (sign_bits): the epilogue kFwdBits of the forward product leaves it, kBwdBits of the
+    // backward product reads it.  The words of row r and columns 64 c .. 64 c + 63 lie at c * ld_bits + r.
+    uint2 *bits_out, *bits_out2;
+    const uint2 *bits_in, *bits_in2;
+    int ld_bits;
     // Two nets' products of equal sizes in one launch (DUAL instantiations): the first half of the tiles is the first net's,
     // the second half the second's, which has operand, output and mask maps of its own; its head is a value head (no
     // sampling) and may have fewer columns.
@@ -250,7 +263,7 @@ struct SmemPlan {
     static constexpr int kMaxStages = 8;
     // hidden layers: eight staging slabs for the TMA stores, shared out over the epilogue warps
     // (backward epilogue: two per warp and two more for the ReLU mask boxes)
-    static constexpr __host__ __device__ int hidden_epi_bytes(bool bwd = false) { return (bwd ? 4 * 4 : 8) * kEpiSlabBytes; }
+    static constexpr __host__ __device__ int hidden_epi_bytes(int epi = kFwd) { return (epi == kBwdBoxes ? 4 * 4 : 8) * kEpiSlabBytes; }
     // head: [2 accumulators][mean, action][128 rows][A] floats laid out as in global memory,
     // partial sums of z^2 [2][4][128], band counters [2][4]
     // (+ bias, per-column sigma and the second net's bias of the tile's columns, 3 x 128 floats)
@@ -483,11 +496,34 @@ __device__ __forceinline__ void mask_all_positive(uint4 (&mk)[8])
     for (int c = 0; c < 8; ++c) mk[c] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
 }
 
+// Which of 64 packed outputs are positive: columns 2 i and 2 i + 1 in bits i and 16 + i, of x for i < 16, of y for the rest.
+// The outputs have passed a ReLU, so that none has its sign bit set and a bf16 is positive when it is not zero.
+__device__ __forceinline__ uint2 sign_bits(const uint32_t (&pk)[32])
+{
+    uint2 r = make_uint2(0u, 0u);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        r.x |= ((pk[i] + 0x7fff7fffu) >> (15 - i)) & (0x00010001u << i);
+        r.y |= ((pk[i + 16] + 0x7fff7fffu) >> (15 - i)) & (0x00010001u << i);
+    }
+    return r;
+}
+// ... of row `row` and the 64 columns from col0, for the backward epilogue (past the last row: none).
+__device__ __forceinline__ uint2 load_bits(const GemmParams &P, bool second, int row, int col0)
+{
+    return row < P.M ? __ldcg((second ? P.bits_in2 : P.bits_in) + (size_t)(col0 >> 6) * P.ld_bits + row) : make_uint2(0u, 0u);
+}
+__device__ __forceinline__ void store_bits(const GemmParams &P, bool second, int row, int col0, const uint32_t (&pk)[32])
+{
+    const uint2 b = sign_bits(pk);
+    if (row < P.M) (second ? P.bits_out2 : P.bits_out)[(size_t)(col0 >> 6) * P.ld_bits + row] = b;
+}
+
 // One epilogue chunk of the hidden-layer kernels: 64 accumulator columns of this thread's row -> bias, floor,
-// (BWD: ReLU mask of the forward activations, column sums over the warp's 32 rows) -> 32 packed bf16 pairs.
-template <bool BWD>
+// (backward: ReLU mask of the forward activations, column sums over the warp's 32 rows) -> 32 packed bf16 pairs.
+template <int EPI>
 __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_addr, int row, int col0, int lane,
-                                             const uint4 (&mk)[8], uint32_t (&pk)[32], const float *bias, float *colsum)
+                                             const uint4 (&mk)[8], uint2 bits, uint32_t (&pk)[32], const float *bias, float *colsum)
 {
     float v[64];
     tmem_ld32_issue(t_addr, v);
@@ -508,7 +544,15 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
 #pragma unroll
         for (int i = 0; i < 64; ++i) v[i] = fmaxf(v[i], fl);
     }
-    if (BWD) {
+    if (EPI == kBwdBits) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const uint32_t w = i < 16 ? bits.x : bits.y;
+            if (!(w & (1u << (i & 15)))) v[2 * i] = 0.0f;
+            if (!(w & (0x10000u << (i & 15)))) v[2 * i + 1] = 0.0f;
+        }
+    }
+    if (EPI == kBwdBoxes) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const uint32_t w[4] = {mk[c].x, mk[c].y, mk[c].z, mk[c].w};
@@ -525,7 +569,7 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
         const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
         pk[i] = *reinterpret_cast<const uint32_t *>(&h);
     }
-    if (BWD) {
+    if (is_bwd(EPI)) {
         if (colsum) {
             reduce_scatter_step<32>(v, lane, 16);
             reduce_scatter_step<16>(v, lane, 8);
@@ -544,7 +588,7 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
 // C = relu(A W^T + b) as bf16.  Each epilogue warp owns 32 rows of the tile: it
 // reads 64 accumulator columns at a time, applies bias and ReLU, packs to bf16
 // into a 128B-swizzled slab in shared memory and hands the slab to a TMA store.
-constexpr __host__ __device__ int hidden_depth(int block_n, bool mn, bool bwd) { return block_n < 256 && !mn && !bwd ? 2 : 1; }
+constexpr __host__ __device__ int hidden_depth(int block_n, bool mn, int epi) { return block_n < 256 && !mn && !is_bwd(epi) ? 2 : 1; }
 
 // Kernel parameters of the second net of a DUAL launch (m: mask, as map_m).
 struct NoMaps {};
@@ -554,23 +598,23 @@ struct DualMaps {
 template <bool DUAL>
 using SecondNet = std::conditional_t<DUAL, DualMaps, NoMaps>;
 
-template <int BLOCK_N, bool MN = false, bool BWD = false, bool DUAL = false>
-__global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, BWD), 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
+template <int BLOCK_N, bool MN = false, int EPI = kFwd, bool DUAL = false>
+__global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, EPI), 1) linear_tc_hidden_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                        const __grid_constant__ CUtensorMap map_b,
                                                                        const __grid_constant__ CUtensorMap map_c,
                                                                        const __grid_constant__ CUtensorMap map_m,
                                                                        const GemmParams P,
                                                                        const __grid_constant__ SecondNet<DUAL> second)
 {
-    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, MN, BWD)>;
+    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, MN, EPI)>;
     extern __shared__ uint8_t smem_raw[];
-    const Pipe p = carve_pipe<Plan>(smem_raw, P.stages, Plan::hidden_epi_bytes(BWD));
+    const Pipe p = carve_pipe<Plan>(smem_raw, P.stages, Plan::hidden_epi_bytes(EPI));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_per_slice = ((P.M + BLOCK_M - 1) / BLOCK_M) * P.n_tiles_n;
     const int n_tiles = tiles_per_slice * (MN ? P.n_batches : 1) * (DUAL ? 2 : 1);
     const CUtensorMap *map_c2 = &map_c, *map_m2 = &map_m;
     if constexpr (DUAL) { map_c2 = &second.c; map_m2 = &second.m; }
-    pipe_init<Plan>(p, hidden_epi_warps(BLOCK_N, MN, BWD));
+    pipe_init<Plan>(p, hidden_epi_warps(BLOCK_N, MN, EPI));
     const uint32_t tmem_base = *p.tmem_slot;
     dep_release();
     dep_wait();                       // nothing before this line touches global memory
@@ -584,16 +628,16 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, BWD), 1) linear_tc
         if (lane == 0) mma_role<Plan, BLOCK_N, MN, DUAL>(p, tmem_base, P, n_tiles, tiles_per_slice);
     } else {
         const int quad = warp & 3;                    // TMEM lanes 32*quad .. 32*quad+31 belong to this warp
-        constexpr bool kFour = hidden_epi_warps(BLOCK_N, MN, BWD) == 4;
+        constexpr bool kFour = hidden_epi_warps(BLOCK_N, MN, EPI) == 4;
         constexpr int kSlabs = kFour ? 2 : 1, kStep = kFour ? 64 : 128;
         const int half = kFour ? 0 : (warp - 2) >> 2;                            // first chunk of this warp
         uint8_t *slabs = p.epi + (size_t)(warp - 2) * kSlabs * kEpiSlabBytes;  // two are used alternately
         int which = 0;
         int acc = 0;
         uint32_t acc_phase = 0;
-        // BWD: the mask box of a chunk is fetched one chunk ahead (across tile boundaries), so its latency
+        // kBwdBoxes: the mask box of a chunk is fetched one chunk ahead (across tile boundaries), so its latency
         // hides behind the previous chunk and the wait for the accumulator
-        const bool masked = BWD && P.mask != nullptr;
+        const bool masked = EPI == kBwdBoxes && P.mask != nullptr;
         uint8_t *mslabs = p.epi + (size_t)(4 + warp - 2) * 2 * kEpiSlabBytes;
         uint64_t *mbar = p.mask_bar + (warp - 2) * 2;
         uint32_t ci = 0;                               // chunks consumed by this warp
@@ -606,15 +650,21 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, BWD), 1) linear_tc
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
             const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
             const int m0 = at.slice * P.c_batch_rows + at.m * BLOCK_M, n0 = at.n * BLOCK_N;
+            uint2 bits = make_uint2(0u, 0u), bits_next = bits;           // (this chunk's and the next one's)
+            if (EPI == kBwdBits) bits_next = load_bits(P, at.second, m0 + quad * 32 + lane, n0);
             bool ready = mbar_wait(&p.acc_full[acc], acc_phase, p.abort_flag);
-            if (BWD) ready = __all_sync(0xffffffffu, ready);           // the column sums shuffle across the whole warp
+            if (is_bwd(EPI)) ready = __all_sync(0xffffffffu, ready);           // the column sums shuffle across the whole warp
             if (!ready) break;
             tc_fence_after();
             const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * Plan::kAccStride);
 #pragma unroll 1
             for (int c0 = 64 * half; c0 < BLOCK_N; c0 += kStep) {
                 uint32_t pk[32];
-                if (BWD) {
+                if (EPI == kBwdBits) {
+                    bits = bits_next;
+                    if (c0 + 64 < BLOCK_N) bits_next = load_bits(P, at.second, m0 + quad * 32 + lane, n0 + c0 + 64);
+                }
+                if (EPI == kBwdBoxes) {
                     if (masked) {
                         if (lane == 0) {
                             uint8_t *nslab = mslabs + ((ci + 1u) & 1u) * kEpiSlabBytes;
@@ -630,8 +680,9 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, BWD), 1) linear_tc
                         ++ci;
                     } else mask_all_positive(mk);
                 }
-                hidden_chunk<BWD>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, at.second ? P.bias2 : P.bias,
+                hidden_chunk<EPI>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, bits, pk, at.second ? P.bias2 : P.bias,
                                   at.second ? P.colsum_partial2 : P.colsum_partial);
+                if (EPI == kFwdBits) store_bits(P, at.second, m0 + quad * 32 + lane, n0 + c0, pk);
                 // the last store from this slab must have finished reading shared memory
                 if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSlabs - 1) : "memory");
                 __syncwarp();
@@ -682,17 +733,18 @@ constexpr int kPairTmemCols = 512;                                     // two 25
 // tensor-memory lane quadrant, each owning one half of the tile's columns; every warp cycles through a ring of
 // three 4 KB slabs, each of which first receives a chunk's mask box and is then overwritten with the chunk's
 // output for the TMA store.  The ring takes the room of two operand stages.
+// With the mask as bits the slabs only hold output, one per warp.
 constexpr int kPairEpiWarpsBwd = 8;
 constexpr int kPairRing = 3;
-constexpr __host__ __device__ int pair_epi_warps(bool bwd) { return bwd ? kPairEpiWarpsBwd : 4; }
-constexpr __host__ __device__ int pair_threads(bool bwd) { return 64 + 32 * pair_epi_warps(bwd); }
-constexpr __host__ __device__ int pair_stages(bool bwd) { return bwd ? kPairStages - 2 : kPairStages; }
-constexpr __host__ __device__ int pair_epi_bytes(bool bwd)
+constexpr __host__ __device__ int pair_epi_warps(int epi) { return is_bwd(epi) ? kPairEpiWarpsBwd : 4; }
+constexpr __host__ __device__ int pair_threads(int bwd) { return 64 + 32 * pair_epi_warps(bwd); }
+constexpr __host__ __device__ int pair_stages(int bwd) { return bwd == kBwdBoxes ? kPairStages - 2 : kPairStages; }
+constexpr __host__ __device__ int pair_epi_bytes(int bwd)
 {
-    return bwd ? kPairEpiWarpsBwd * kPairRing * kEpiSlabBytes : 4 * 2 * kEpiSlabBytes;
+    return bwd == kBwdBoxes ? kPairEpiWarpsBwd * kPairRing * kEpiSlabBytes : 8 * kEpiSlabBytes;
 }
-constexpr size_t pair_smem_bytes(bool bwd) { return 1024 + (size_t)pair_stages(bwd) * kPairStageBytes + pair_epi_bytes(bwd) + 512; }
-static_assert(pair_smem_bytes(true) <= kSmemLimit && pair_smem_bytes(false) <= kSmemLimit, "shared memory plan of the pair kernel");
+constexpr size_t pair_smem_bytes(int bwd) { return 1024 + (size_t)pair_stages(bwd) * kPairStageBytes + pair_epi_bytes(bwd) + 512; }
+static_assert(pair_smem_bytes(kBwdBoxes) <= kSmemLimit && pair_smem_bytes(kFwd) <= kSmemLimit, "shared memory plan of the pair kernel");
 static_assert((2 * kPairStages + 5 + kPairEpiWarpsBwd * kPairRing) * 8 <= 512, "barrier area of the pair kernel");
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -750,18 +802,18 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t *bar)
 
 // MN: both operands are stored [contraction rows][M or N columns] (the transposed product of two row-major
 // matrices, as in the single-CTA kernel's MN instantiation), possibly over several row slices ("batches").
-template <bool BWD = false, bool MN = false, bool DUAL = false>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads(BWD), 1)
+template <int EPI = kFwd, bool MN = false, bool DUAL = false>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads(EPI), 1)
 linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                              const __grid_constant__ CUtensorMap map_c, const __grid_constant__ CUtensorMap map_m,
                              const GemmParams P, const __grid_constant__ SecondNet<DUAL> second)
 {
-    constexpr int kStages = pair_stages(BWD);
-    constexpr int kEpi = pair_epi_warps(BWD);
+    constexpr int kStages = pair_stages(EPI);
+    constexpr int kEpi = pair_epi_warps(EPI);
     extern __shared__ uint8_t smem_raw[];
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *epi = tiles + (size_t)kStages * kPairStageBytes;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(epi + pair_epi_bytes(BWD));
+    uint64_t *bars = reinterpret_cast<uint64_t *>(epi + pair_epi_bytes(EPI));
     uint64_t *mask_bar = bars + 2 * kPairStages + 5;
     uint64_t *full = bars, *empty = bars + kPairStages, *acc_full = bars + 2 * kPairStages,
              *acc_empty = bars + 2 * kPairStages + 2;
@@ -779,7 +831,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-        if (BWD)
+        if (EPI == kBwdBoxes)
             for (int i = 0; i < kPairEpiWarpsBwd * kPairRing; ++i) mbar_init(&mask_bar[i], 1);
         for (int a = 0; a < 2; ++a) { mbar_init(&acc_full[a], 1); mbar_init(&acc_empty[a], 2 * kEpi); }
         *abort_flag = 0;
@@ -877,7 +929,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
         const int quad = warp & 3;                     // tensor-memory lanes 32 quad .. 32 quad + 31
         int acc = 0;
         uint32_t acc_phase = 0;
-        if constexpr (!BWD) {
+        if constexpr (!is_bwd(EPI)) {
             uint8_t *slabs = epi + (size_t)(warp - 2) * 2 * kEpiSlabBytes;
             int which = 0;
             uint4 mk[8];                                // unused without the backward epilogue
@@ -892,7 +944,9 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
 #pragma unroll 1
                 for (int c0 = 0; c0 < 256; c0 += 64) {
                     uint32_t pk[32];
-                    hidden_chunk<false>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, at.second ? P.bias2 : P.bias, nullptr);
+                    hidden_chunk<kFwd>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, make_uint2(0u, 0u), pk,
+                                       at.second ? P.bias2 : P.bias, nullptr);
+                    if (EPI == kFwdBits) store_bits(P, at.second, m0 + quad * 32 + lane, n0 + c0, pk);
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                     __syncwarp();
                     uint8_t *slab = slabs + which * kEpiSlabBytes;
@@ -911,6 +965,50 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                     which ^= 1;
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_u32(&acc_empty[acc]), 0));   // the leader's barrier
+                if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+            }
+        } else if constexpr (EPI == kBwdBits) {
+            // warp 2 + e: quadrant (2 + e) & 3, column chunks 2 (e / 4) and 2 (e / 4) + 1 of every tile, through one slab; the
+            // mask's words are asked for before the accumulator is waited for
+            const int ew = warp - 2, half = ew >> 2;
+            uint8_t *slab = epi + (size_t)ew * kEpiSlabBytes;
+            const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
+            const uint4 mk[8] = {};                     // (unused)
+            if (!*abort_flag)
+            for (int tile = pair; tile < n_tiles; tile += n_pairs) {
+                const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
+                const int row = at.m * 2 * BLOCK_M + (int)rank * BLOCK_M + quad * 32 + lane, n0 = at.n * 256 + 128 * half;
+                uint2 bits = load_bits(P, at.second, row, n0);
+                const uint2 bits1 = load_bits(P, at.second, row, n0 + 64);
+                // (the column sums shuffle across the whole warp: every lane takes the same decision)
+                if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[acc], acc_phase, abort_flag))) break;
+                tc_fence_after();
+                const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 256 + 128 * half);
+#pragma unroll 1
+                for (int c0 = 0; c0 < 128; c0 += 64) {
+                    uint32_t pk[32];
+                    hidden_chunk<kBwdBits>(P, t_row + (uint32_t)c0, row, n0 + c0, lane, mk, bits, pk, at.second ? P.bias2 : P.bias,
+                                           at.second ? P.colsum_partial2 : P.colsum_partial);
+                    bits = bits1;
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const uint32_t dst = slab_row + (uint32_t)((c ^ (lane & 7)) << 4);      // 128B swizzle
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pk[4 * c]), "r"(pk[4 * c + 1]),
+                                     "r"(pk[4 * c + 2]), "r"(pk[4 * c + 3]) : "memory");
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+                                     ::"l"(at.second ? map_c2 : &map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(row) : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -959,8 +1057,8 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                         mask_read(slab, lane, mk);
                     } else mask_all_positive(mk);
                     uint32_t pk[32];
-                    hidden_chunk<true>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, at.second ? P.bias2 : P.bias,
-                                       at.second ? P.colsum_partial2 : P.colsum_partial);
+                    hidden_chunk<kBwdBoxes>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, make_uint2(0u, 0u), pk,
+                                            at.second ? P.bias2 : P.bias, at.second ? P.colsum_partial2 : P.colsum_partial);
                     // each lane overwrites the 128 bytes it read its own mask words from
                     const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
 #pragma unroll
@@ -1308,40 +1406,40 @@ namespace im {
 namespace {
 
 // L2: the second net's layer of a launch for two (DUAL), else null.
-template <int BLOCK_N, bool MN, bool BWD, bool DUAL>
+template <int BLOCK_N, bool MN, int EPI, bool DUAL>
 cudaError_t launch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParams &gp_in, int n_sm, cudaStream_t stream)
 {
-    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, MN, BWD)>;
-    const auto kernel = linear_tc_hidden_kernel<BLOCK_N, MN, BWD, DUAL>;
+    using Plan = SmemPlan<BLOCK_N, hidden_depth(BLOCK_N, MN, EPI)>;
+    const auto kernel = linear_tc_hidden_kernel<BLOCK_N, MN, EPI, DUAL>;
     static DeviceOnce once;                      // the attribute is per device
     const cudaError_t e = once.run([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit); });
     if (e != cudaSuccess) return e;
     GemmParams gp = gp_in;
-    gp.stages = Plan::stages_for(Plan::hidden_epi_bytes(BWD));
-    const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes(BWD));
+    gp.stages = Plan::stages_for(Plan::hidden_epi_bytes(EPI));
+    const size_t smem = Plan::bytes(gp.stages, Plan::hidden_epi_bytes(EPI));
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches * (DUAL ? 2 : 1);
     const int grid = tiles < n_sm ? tiles : n_sm;
     SecondNet<DUAL> second;
     if constexpr (DUAL) second = {L2->map_a, L2->map_b, L2->map_c, L2->map_m};
-    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, MN, BWD)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
+    const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, MN, EPI)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
                                       L.map_m, gp, second);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
 }
 
 // The same products on CTA pairs (256-column tiles).
-template <bool BWD, bool MN, bool DUAL>
+template <int EPI, bool MN, bool DUAL>
 cudaError_t launch_hidden_pair(const TcLayer &L, const TcLayer *L2, const GemmParams &gp, int n_sm, cudaStream_t stream)
 {
-    const auto kernel = linear_tc_hidden_pair_kernel<BWD, MN, DUAL>;
+    const auto kernel = linear_tc_hidden_pair_kernel<EPI, MN, DUAL>;
     static DeviceOnce once;                      // the attribute is per device
-    const cudaError_t e = once.run([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem_bytes(BWD)); });
+    const cudaError_t e = once.run([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pair_smem_bytes(EPI)); });
     if (e != cudaSuccess) return e;
     const int tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * gp.n_batches * (DUAL ? 2 : 1);
     const int pairs = tiles < n_sm / 2 ? tiles : n_sm / 2;
     SecondNet<DUAL> second;
     if constexpr (DUAL) second = {L2->map_a, MN ? L2->map_b : L2->map_b2, L2->map_c, L2->map_m};
-    const cudaError_t le = launch_pdl(kernel, dim3(2 * pairs), dim3(pair_threads(BWD)), pair_smem_bytes(BWD), stream, 0, L.map_a,
+    const cudaError_t le = launch_pdl(kernel, dim3(2 * pairs), dim3(pair_threads(EPI)), pair_smem_bytes(EPI), stream, 0, L.map_a,
                                       MN ? L.map_b : L.map_b2, L.map_c, L.map_m, gp, second);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -1381,6 +1479,17 @@ cudaError_t dispatch_head(const TcLayer &L, const GemmParams &gp, int n_sm, cons
     }
 }
 
+template <int EPI, bool DUAL>
+cudaError_t dispatch_width(const TcLayer &L, const TcLayer *L2, const GemmParams &gp, int n_sm, bool pairs, cudaStream_t stream)
+{
+    if (pairs) return launch_hidden_pair<EPI, false, DUAL>(L, L2, gp, n_sm, stream);
+    switch (L.block_n) {
+    case 256: return launch_hidden<256, false, EPI, DUAL>(L, L2, gp, n_sm, stream);
+    case 128: return launch_hidden<128, false, EPI, DUAL>(L, L2, gp, n_sm, stream);
+    default: return launch_hidden<64, false, EPI, DUAL>(L, L2, gp, n_sm, stream);
+    }
+}
+
 // A hidden layer's product, of one net or (DUAL) of two at once.
 template <bool DUAL>
 cudaError_t dispatch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParams &gp, int n_sm, bool force_pairs, cudaStream_t stream)
@@ -1393,27 +1502,26 @@ cudaError_t dispatch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParam
     // 103.4 / 105.7 / 149; 361-2048-1024 on 4800 / 9001 / 16384 rows 65.8 / 93.4 / 163 and 68.2 / 99.6 / 172; 361-1024-512 on 16384 rows
     // 69.5 and 73.1
     const int pair_tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * (DUAL ? 2 : 1);
-    const bool bwd = gp.mask || gp.colsum_partial;
+    const bool bwd = gp.mask || gp.colsum_partial || gp.bits_in;
     // (the backward epilogue is the longer part of a tile when K is short, and the pair kernel runs it on
     // eight warps: it takes those products whenever its tiles fill the machine)
-    if (L.block_n == 256 && (force_pairs || (pair_tiles >= n_sm && gp.K_blocks >= 8) || (bwd && pair_tiles >= n_sm / 2)))
-        return bwd ? launch_hidden_pair<true, false, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden_pair<false, false, DUAL>(L, L2, gp, n_sm, stream);
-    switch (L.block_n) {
-    case 256: return bwd ? launch_hidden<256, false, true, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden<256, false, false, DUAL>(L, L2, gp, n_sm, stream);
-    case 128: return bwd ? launch_hidden<128, false, true, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden<128, false, false, DUAL>(L, L2, gp, n_sm, stream);
-    default: return bwd ? launch_hidden<64, false, true, DUAL>(L, L2, gp, n_sm, stream) : launch_hidden<64, false, false, DUAL>(L, L2, gp, n_sm, stream);
-    }
+    const bool pairs = L.block_n == 256 && (force_pairs || (pair_tiles >= n_sm && gp.K_blocks >= 8) || (bwd && pair_tiles >= n_sm / 2));
+    if (!bwd) return gp.bits_out ? dispatch_width<kFwdBits, DUAL>(L, L2, gp, n_sm, pairs, stream) : dispatch_width<kFwd, DUAL>(L, L2, gp, n_sm, pairs, stream);
+    if (gp.bits_in) return dispatch_width<kBwdBits, DUAL>(L, L2, gp, n_sm, pairs, stream);
+    // (a common launch for two nets has its masks as bits)
+    if constexpr (DUAL) return cudaErrorInvalidValue;
+    else return dispatch_width<kBwdBoxes, false>(L, L2, gp, n_sm, pairs, stream);
 }
 
 // The same with both operands stored [contraction rows][M or N columns].
 template <bool DUAL>
 cudaError_t dispatch_mn(const TcLayer &L, const TcLayer *L2, const GemmParams &gp, bool pairs, int n_sm, cudaStream_t stream)
 {
-    if (pairs) return launch_hidden_pair<false, true, DUAL>(L, L2, gp, n_sm, stream);
+    if (pairs) return launch_hidden_pair<kFwd, true, DUAL>(L, L2, gp, n_sm, stream);
     switch (L.block_n) {
-    case 256: return launch_hidden<256, true, false, DUAL>(L, L2, gp, n_sm, stream);
-    case 128: return launch_hidden<128, true, false, DUAL>(L, L2, gp, n_sm, stream);
-    default: return launch_hidden<64, true, false, DUAL>(L, L2, gp, n_sm, stream);
+    case 256: return launch_hidden<256, true, kFwd, DUAL>(L, L2, gp, n_sm, stream);
+    case 128: return launch_hidden<128, true, kFwd, DUAL>(L, L2, gp, n_sm, stream);
+    default: return launch_hidden<64, true, kFwd, DUAL>(L, L2, gp, n_sm, stream);
     }
 }
 
@@ -1671,11 +1779,12 @@ im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, in
     gp.M = M; gp.N = N; gp.K_blocks = K / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = x.bias;
     gp.act_floor = relu ? 0.0f : -INFINITY;
     gp.n_batches = 1;
-    if (x.mask || x.colsum_partial) gp.bias = nullptr;     // the backward product has no bias: its epilogue skips the add
+    if (x.mask || x.colsum_partial || x.bits_in) gp.bias = nullptr;     // the backward product has no bias: its epilogue skips the add
     else if (y) gp.bias2 = y->bias;
     gp.mask = static_cast<const __nv_bfloat16 *>(x.mask);
     gp.colsum_partial = x.colsum_partial; gp.ld_partial = ld_partial;
-    if (y) gp.colsum_partial2 = y->colsum_partial;
+    gp.bits_out = x.bits_out; gp.bits_in = x.bits_in; gp.ld_bits = x.ld_bits;
+    if (y) { gp.colsum_partial2 = y->colsum_partial; gp.bits_out2 = y->bits_out; gp.bits_in2 = y->bits_in; }
     gp.status = status; gp.status2 = status2;
     const cudaError_t e = y ? dispatch_hidden<true>(L, &L2, gp, n_sm, false, stream) : dispatch_hidden<false>(L, nullptr, gp, n_sm, false, stream);
     return e == cudaSuccess ? IM_OK : IM_ERR_CUDA;

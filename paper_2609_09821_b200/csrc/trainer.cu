@@ -52,6 +52,7 @@ struct im_trainer {
     float *dW[IM_MAX_LAYERS], *db[IM_MAX_LAYERS];
     uint16_t *Wb[IM_MAX_LAYERS], *WbT[IM_MAX_LAYERS];      // bf16 [Np][Kp] and its transpose [Kp][Np]
     uint16_t *H[IM_MAX_LAYERS];                            // H[0]: input rows [Mb][Kp0]; H[l]: activations [Mb][Np[l-1]]
+    uint2 *bits[IM_MAX_LAYERS];                            // which of H[l] are positive, a bit each [Kp[l] / 64][Mb]; the update's ReLU mask
     uint16_t *dZ[IM_MAX_LAYERS];                           // gradient at layer l's pre-activation [Mb][Np[l]]
     float *out;                                            // [Mb][dims[nl]]
     uint16_t *dWs[IM_MAX_LAYERS];                          // partial dW products, all row slices
@@ -68,6 +69,9 @@ namespace {
 struct Nets {
     im_trainer *a, *c;                                     // c: null for one net
     uint16_t *xa, *xc;                                     // input rows (their own, or those of another trainer)
+    // The forward pass leaves every hidden activation's sign as a bit, which the backward pass takes for the ReLU mask.  Only
+    // within one update: between the calls of a forward and a backward pass the activations are the caller's to change.
+    bool bits;
 };
 bool share_launches(const im_trainer *a, const im_trainer *c)
 {
@@ -92,7 +96,8 @@ im_status forward_on(const Nets &n, int M)
     uint32_t *status2 = n.c ? n.c->status : nullptr;
     im_status s = IM_OK;
     for (int l = 0; l < a->nl && s == IM_OK; ++l) {
-        const im::GemmOperands x = forward_operands(a, n.xa, l), y = n.c ? forward_operands(n.c, n.xc, l) : x;
+        im::GemmOperands x = forward_operands(a, n.xa, l), y = n.c ? forward_operands(n.c, n.xc, l) : x;
+        if (n.bits && l < a->nl - 1) { x.bits_out = a->bits[l + 1]; y.bits_out = n.c ? n.c->bits[l + 1] : nullptr; x.ld_bits = a->Mb; }
         const im::GemmOperands *py = n.c ? &y : nullptr;
         if (l < a->nl - 1) s = im::tc_gemm(x, py, M, a->Np[l], a->Kp[l], true, 0, a->status, status2, a->stream);
         else s = im::tc_gemm_head(x, py, M, a->dims[a->nl], n.c ? n.c->dims[n.c->nl] : 0, a->Kp[l], a->status, status2, a->stream);
@@ -110,7 +115,7 @@ im::OutGrad out_grad(im_trainer *tr, const float *d_out)
 // (both operands read as they lie, M/N-major tensor-core operands: no transposed copies).  dH = (H > 0) * (dZ W); the
 // product's epilogue applies the ReLU mask and leaves the column sums of every 32-row block, which add up to the bias
 // gradient of the layer below.
-im_status backward_of(im_trainer *tr, uint16_t *x, im_trainer *tr2, uint16_t *x2, int l, int M, int *slices)
+im_status backward_of(im_trainer *tr, uint16_t *x, im_trainer *tr2, uint16_t *x2, bool bits, int l, int M, int *slices)
 {
     const int Np = tr->Np[l], Kp = tr->Kp[l], Npb = pad128(Np);
     const int cap = tr2 && tr2->s_max[l] < tr->s_max[l] ? tr2->s_max[l] : tr->s_max[l];
@@ -118,7 +123,9 @@ im_status backward_of(im_trainer *tr, uint16_t *x, im_trainer *tr2, uint16_t *x2
     const auto dw = [&](im_trainer *t, uint16_t *in) { return operands(t->dZ[l], Np, l == 0 ? in : t->H[l], Kp, t->dWs[l], Kp); };
     const auto dh = [&](im_trainer *t) {
         im::GemmOperands o = operands(t->dZ[l], Np, t->WbT[l], Np, t->dZ[l - 1], Kp);
-        o.mask = t->H[l]; o.ld_mask = Kp; o.colsum_partial = t->db_partial[l - 1];
+        if (bits) { o.bits_in = t->bits[l]; o.ld_bits = t->Mb; }
+        else { o.mask = t->H[l]; o.ld_mask = Kp; }
+        o.colsum_partial = t->db_partial[l - 1];
         return o;
     };
     im::GemmOperands o = tr2 ? dw(tr2, x2) : im::GemmOperands();
@@ -133,11 +140,11 @@ im_status backward_products(const Nets &n, int M, int (*slices)[IM_MAX_LAYERS])
     im_status s = IM_OK;
     for (int l = n.a->nl - 1; l >= 0 && s == IM_OK; --l) {
         if (n.c && n.c->Np[l] == n.a->Np[l]) {
-            s = backward_of(n.a, n.xa, n.c, n.xc, l, M, &slices[0][l]);
+            s = backward_of(n.a, n.xa, n.c, n.xc, n.bits, l, M, &slices[0][l]);
             slices[1][l] = slices[0][l];
         } else {
-            s = backward_of(n.a, n.xa, nullptr, nullptr, l, M, &slices[0][l]);
-            if (n.c && s == IM_OK) s = backward_of(n.c, n.xc, nullptr, nullptr, l, M, &slices[1][l]);
+            s = backward_of(n.a, n.xa, nullptr, nullptr, n.bits, l, M, &slices[0][l]);
+            if (n.c && s == IM_OK) s = backward_of(n.c, n.xc, nullptr, nullptr, n.bits, l, M, &slices[1][l]);
         }
     }
     return s;
@@ -186,7 +193,7 @@ static im_status update_on(im_ppo_updater *u, int M, const im_ppo_minibatch *mb,
     if (!adam_ok(&u->cfg.adam) || !(u->cfg.kl_target > 0.0f) || !(u->cfg.lr_min > 0.0f)) return IM_ERR_INVALID_ARG;
     im_trainer *a = u->actor, *c = u->critic;
     cudaStream_t st = a->stream;
-    const Nets both = {a, c, a->H[0], critic_x}, one_a = {a, nullptr, a->H[0], nullptr}, one_c = {c, nullptr, critic_x, nullptr};
+    const Nets both = {a, c, a->H[0], critic_x, true}, one_a = {a, nullptr, a->H[0], nullptr, true}, one_c = {c, nullptr, critic_x, nullptr, true};
     const bool shared = share_launches(a, c);
     im_status s = forward_on(shared ? both : one_a, M);
     if (s == IM_OK && !shared) s = forward_on(one_c, M);
@@ -254,7 +261,7 @@ void im_trainer_destroy(im_trainer *tr)
     if (!tr) return;
     for (int l = 0; l < IM_MAX_LAYERS; ++l) {
         cudaFree(tr->W[l]); cudaFree(tr->b[l]); cudaFree(tr->mW[l]); cudaFree(tr->vW[l]); cudaFree(tr->mb[l]); cudaFree(tr->vb[l]);
-        cudaFree(tr->dW[l]); cudaFree(tr->db[l]); cudaFree(tr->Wb[l]); cudaFree(tr->WbT[l]); cudaFree(tr->H[l]); cudaFree(tr->dZ[l]);
+        cudaFree(tr->dW[l]); cudaFree(tr->db[l]); cudaFree(tr->Wb[l]); cudaFree(tr->WbT[l]); cudaFree(tr->H[l]); cudaFree(tr->bits[l]); cudaFree(tr->dZ[l]);
         cudaFree(tr->dWs[l]); cudaFree(tr->db_partial[l]);
     }
     cudaFree(tr->out); cudaFree(tr->status);
@@ -289,7 +296,7 @@ im_status im_trainer_create(int32_t n_layers, const int32_t *dims, const float *
              dev_alloc(&tr->vW[l], wn, st) && dev_alloc(&tr->mb[l], (size_t)N, st) && dev_alloc(&tr->vb[l], (size_t)N, st) &&
              dev_alloc(&tr->dW[l], wn, st) && dev_alloc(&tr->db[l], (size_t)N, st) && dev_alloc(&tr->Wb[l], (size_t)Np * Kp, st) &&
              dev_alloc(&tr->WbT[l], (size_t)Kp * Np, st) && dev_alloc(&tr->H[l], (size_t)max_rows * Kp, st) &&
-             dev_alloc(&tr->dZ[l], (size_t)max_rows * Np, st);
+             (l == 0 || dev_alloc(&tr->bits[l], (size_t)max_rows * (Kp / 64), st, false)) && dev_alloc(&tr->dZ[l], (size_t)max_rows * Np, st);
         // partial dW products: room for the most slices the model can choose for any number of rows
         tr->s_max[l] = max_slices(Np, Kp, max_rows, tr->max_split);
         ok = ok && dev_alloc(&tr->dWs[l], (size_t)tr->s_max[l] * pad128(Np) * Kp, st, false) &&
@@ -352,7 +359,7 @@ im_status im_trainer_set_step_count(im_trainer *tr, int32_t t)
 im_status im_trainer_forward(im_trainer *tr, int32_t M)
 {
     if (!tr || M < 1 || M > tr->Mb) return IM_ERR_INVALID_ARG;
-    return forward_on({tr, nullptr, tr->H[0], nullptr}, M);
+    return forward_on({tr, nullptr, tr->H[0], nullptr, false}, M);
 }
 
 im_status im_trainer_backward(im_trainer *tr, const float *d_out, int32_t M)
@@ -362,7 +369,7 @@ im_status im_trainer_backward(im_trainer *tr, const float *d_out, int32_t M)
     og.n_nets = 1; og.M = M; og.net[0] = out_grad(tr, d_out);
     if (im::launch_out_grads(og, tr->stream) != cudaSuccess) return IM_ERR_CUDA;
     int slices[1][IM_MAX_LAYERS];
-    const im_status s = backward_products({tr, nullptr, tr->H[0], nullptr}, M, slices);
+    const im_status s = backward_products({tr, nullptr, tr->H[0], nullptr, false}, M, slices);
     if (s != IM_OK) return s;
     im::GradReduceArgs ga = {};
     add_weight_grads(ga, tr, slices[0]);
