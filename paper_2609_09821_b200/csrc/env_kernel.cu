@@ -78,6 +78,13 @@ __host__ __device__ inline int chain_floats(int c1, int D_ext, int n_chains)
     const int first = kTile * s1 + kRing * n_chains * kTile, both = kTile * (s1 > s2 ? s1 : s2) + kPartials * n_chains * kTile;
     return first > both ? first : both;
 }
+// With the bodies of records staged all at once, an odd number of words from one component to the next.
+__host__ __device__ inline int records_floats(int J, int D_ext)
+{
+    const int s1 = tile_stride(split_col(J)), s2 = tile_stride(D_ext - split_col(J));
+    const int first = kTile * s1 + (J * kRing * (kTile + 1) + 3) / 4 * 4, second = kTile * s2;
+    return first > second ? first : second;
+}
 // With whole rows staged.
 __host__ __device__ inline int whole_floats(int D_ext, int n_chains) { return kTile * (tile_stride(D_ext) + kRing * n_chains); }
 __host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, int extra_cols)
@@ -85,17 +92,17 @@ __host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, 
     return (size_t)chain_floats(split_col(J), 24 * J + 1 + extra_cols, n_chains) + (size_t)8 * n_links;
 }
 
-// The role kernel: the staged rows, the chains' partial sums, their link records.  Staged columns: all, or, where an
+// The role kernel: the staged rows, the chains' partial sums, their link records, staged body states.  Staged columns: all, or, where an
 // extended observation is too wide for that, the first 24 J (the rest is then written column by column).
-__host__ __device__ inline size_t role_smem_floats(int cols, int n_chains, int n_links)
+__host__ __device__ inline size_t role_smem_floats(int cols, int n_chains, int n_links, int staged_bodies)
 {
-    return (size_t)kTile * tile_stride(cols) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links;
+    return (size_t)kTile * tile_stride(cols) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links + (size_t)staged_bodies * kRing * (kTile + 1);
 }
 constexpr size_t kMaxSmemFloats = 232448 / 4;       // opt-in shared memory per block on this architecture (227 KB)
-__host__ __device__ inline int staged_cols(int J, int n_chains, int n_links, int extra_cols)
+__host__ __device__ inline int staged_cols(int J, int n_chains, int n_links, int extra_cols, bool staged_bodies)
 {
     const int cols = 24 * J + 1 + extra_cols;
-    return extra_cols == 0 || role_smem_floats(cols, n_chains, n_links) <= kMaxSmemFloats ? cols : 24 * J;
+    return extra_cols == 0 || role_smem_floats(cols, n_chains, n_links, staged_bodies ? J : 0) <= kMaxSmemFloats ? cols : 24 * J;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -267,6 +274,12 @@ __device__ __forceinline__ LinkRec ld_link_checked(const float4 *links, int k, i
     return L;
 }
 #endif
+
+// The body at the end of chain c, from the link records of all chains.
+__device__ __forceinline__ int ld_leaf(const float4 *all_links, const SkelDev &sk, int c)
+{
+    return reinterpret_cast<const int4 *>(all_links + 2 * (sk.link_start[c] + sk.chain_len[c] - 1) + 1)->x;
+}
 
 // Compose the interpolated joint onto the running transform.  k == 0 is the root, whose position is the
 // lerp of the row's root position along its displacement.
@@ -444,12 +457,13 @@ __device__ __forceinline__ float lds32(uint32_t addr)
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
     return v;
 }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // A body staged by stage_body, once its copies have landed.
+template <int PITCH = kTile>
 __device__ __forceinline__ SimBody lds_body(uint32_t a)
 {
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    return {{lds32(a), lds32(a + 128), lds32(a + 256), lds32(a + 384)}, {lds32(a + 512), lds32(a + 640), lds32(a + 768)},
-            {lds32(a + 896), lds32(a + 1024), lds32(a + 1152)}, {lds32(a + 1280), lds32(a + 1408), lds32(a + 1536)}};
+    const auto w = [a](int i) { return lds32(a + (uint32_t)(4 * PITCH * i)); };
+    return {{w(0), w(1), w(2), w(3)}, {w(4), w(5), w(6)}, {w(7), w(8), w(9)}, {w(10), w(11), w(12)}};
 }
 
 // Body-state access of one thread (one env).  Two layouts:
@@ -513,6 +527,25 @@ struct SimView {
             for (int i = 0; i < 4; ++i) cp_async_word(dst + 128 * i, quat + (o + i * st), policy);
 #pragma unroll
             for (int i = 0; i < 9; ++i) cp_async_word(dst + 128 * (4 + i), v[i / 3] + (o3 + (i % 3) * st), policy);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    // Records: the whole state of env `src` of the batch to column `col` of the staged bodies (component i of body b: the word
+    // (13 b + i) * pitch + col), by the lanes of a warp, which walk along the record: a request takes the few lines that its
+    // words lie in, where a lane to every env takes 32.  An odd pitch keeps the words of a request in different banks.
+    static __device__ __forceinline__ void stage_record(const EnvKernelParams &P, int src, int J, uint32_t dst, uint32_t pitch, int col, int lane,
+                                                        uint64_t policy)
+    {
+        const float *a[4] = {P.quat + (long long)src * P.aos_env_stride[1], P.pos + (long long)src * P.aos_env_stride[0],
+                             P.lin + (long long)src * P.aos_env_stride[2], P.ang + (long long)src * P.aos_env_stride[3]};
+        const int bs[4] = {P.aos_body_stride[1], P.aos_body_stride[0], P.aos_body_stride[2], P.aos_body_stride[3]};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int n = k == 0 ? 4 : 3, off = k == 0 ? 0 : 1 + 3 * k;
+            for (int i = lane; i < n * J; i += 32) {
+                const int b = i / n, c = i - n * b;
+                cp_async_word(dst + 4u * ((uint32_t)(kRing * b + off + c) * pitch + (uint32_t)col), a[k] + (long long)b * bs[k] + c, policy);
+            }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
@@ -650,14 +683,15 @@ __device__ __forceinline__ void decide(const EnvKernelParams &P, int env, float 
 }
 
 // The seven error terms of an env from the chains' partial sums, added in chain order, and the reward.
-template <int PER_CHAIN>
-__device__ __forceinline__ float reward_of(const EnvKernelParams &P, const float *part, int C, int lane, float (&term)[IM_N_TERMS])
+// Sum i of chain cc lies at part_of(cc)[i * PITCH].
+template <int PITCH = kTile, typename F>
+__device__ __forceinline__ float reward_of(const EnvKernelParams &P, F part_of, int C, float (&term)[IM_N_TERMS])
 {
     float e[kPartials];
 #pragma unroll
     for (int i = 0; i < kPartials; ++i) {
         float a = 0.0f;
-        for (int cc = 0; cc < C; ++cc) a += part[(cc * PER_CHAIN + i) * kTile + lane];
+        for (int cc = 0; cc < C; ++cc) a += part_of(cc)[i * PITCH];
         e[i] = a;
     }
     // term order of the configuration: pose, vel, ee_pos, ee_rot, com, body_pos, body_vel
@@ -717,7 +751,8 @@ __device__ __forceinline__ void st_direct(const EnvKernelParams &P, int env, int
 // The role kernel.  OPT compiles in the optional semantics (grace steps, motion randomisation, adaptive initialisation,
 // extended observation, looped clips, summaries); envs that use none run the instantiation without them.  WIDE: a
 // warp may have several (chain, role) pairs (trees with more than eight leaves).
-template <bool RESET_ALL, bool OPT, bool AOS, bool WIDE>
+// STAGED: the bodies of a simulator's records are staged all at once before the walk (see staged_records).
+template <bool RESET_ALL, bool OPT, bool AOS, bool WIDE, bool STAGED>
 __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *smem_raw)
 {
     // a successor launched with programmatic stream serialization (the policy's first GEMM) may be scheduled
@@ -729,7 +764,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     const int n_ee = OPT ? __popc(sk.ee_mask) : 0;
     const int ext_future = (OPT && P.n_future > 1) ? (P.n_future - 1) * 9 * n_ee : 0;
     const int D_ext = D + ext_future + (OPT ? P.act_dim : 0);
-    const int cols = OPT ? staged_cols(J, C, sk.n_links, D_ext - D) : D;
+    const int cols = OPT ? staged_cols(J, C, sk.n_links, D_ext - D, STAGED) : D;
     const bool direct = OPT && cols < D;
     const int S = tile_stride(cols);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
@@ -739,6 +774,8 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     float *row = smem_raw + (size_t)lane * S;
     float *part = smem_raw + (size_t)kTile * S;
     float4 *all_links = reinterpret_cast<float4 *>(part + (size_t)kPartials * C * kTile);
+    const auto part_of = [&](int cc) { return part + cc * kPartials * kTile + lane; };
+    const uint32_t bodies = (uint32_t)__cvta_generic_to_shared(all_links + 2 * sk.n_links) + 4u * lane;    // [J][13][32]
 
     for (int i = threadIdx.x; i < 2 * sk.n_links; i += blockDim.x) all_links[i] = __ldg(P.links + i);
     __syncthreads();
@@ -754,9 +791,20 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     float root_z = 0.0f, r = INFINITY;
     bool bad = false;
     const SimView<AOS> sv(P, envc);
+    constexpr int kPitch = kTile + 1;
+    const auto body = [&](int b) { return STAGED ? lds_body<kPitch>(bodies + (uint32_t)b * (kRing * kPitch * 4)) : sv.ld_body(b); };
     if (!RESET_ALL) {
-        const Quat q_root = sv.ld_quat(0);
-        const Vec3 p_root = sv.ld_pos(0);
+        Quat q_root = {1.0f, 0.0f, 0.0f, 0.0f};
+        Vec3 p_root = {0.0f, 0.0f, 0.0f};
+        if (STAGED) {
+            uint64_t policy;
+            asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+            const int e0 = blockIdx.x * kTile;
+            for (int i = warp; i < kTile; i += n_warps) sv.stage_record(P, min(e0 + i, P.N - 1), J, bodies - 4u * lane, kPitch, i, lane, policy);
+        } else {
+            q_root = sv.ld_quat(0);
+            p_root = sv.ld_pos(0);
+        }
         E.clip = P.clip_id[envc];
         if (E.clip < 0 || E.clip >= P.C) {
             E.clip = min(max(E.clip, 0), P.C - 1);
@@ -771,14 +819,23 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
             E.cyc = P.cycle[envc];
             if (E.loop.on && E.t >= E.cm.dur) { E.t = __fsub_rn(E.t, E.cm.dur); ++E.cyc; }
         }
-        H = make_heading(sanitize(q_root, bad), p_root);
-        root_z = p_root.z;
+        if (!STAGED) {
+            H = make_heading(sanitize(q_root, bad), p_root);
+            root_z = p_root.z;
+        }
     }
     const ClipLoop loop = E.loop;              // of the clip before a reset
+    // Every warp of the tile comes by here once, before it reads a staged body
+    const auto take_staged = [&] {
+        if (!STAGED) return;
+        cp_async_wait();
+        asm volatile("bar.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+        const SimBody root = body(0);
+        H = make_heading(sanitize(root.q, bad), root.p);
+        root_z = root.p.z;
+    };
     // whether the reward can end an episode; if not, the root height and the clip end decide, which are known already
     const bool need_r = !RESET_ALL && P.reward.r_min > -INFINITY;
-    const bool known_reset = !RESET_ALL && !need_r && flags_of<OPT>(P, root_z, r, E) != 0;
-
     if (!RESET_ALL) {
 #pragma unroll 1
         for (int task = warp; task < 2 * C; task += n_warps) {
@@ -793,6 +850,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
                 const float4 *r0 = P.frames + (size_t)IM_CHECKED(frame, P.n_rows) * RS;
                 LinkRec L = ld_link(links, 0);
                 KeyPair keys = ld_keys(r0, L.b);
+                take_staged();
                 float acc[kPartials];
 #pragma unroll
                 for (int i = 0; i < kPartials; ++i) acc[i] = 0.0f;
@@ -801,15 +859,22 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
                 Vec3 wa = {0, 0, 0};
                 if (first_own > 0) {
                     const int a = ld_link(links, first_own - 1).b;
-                    qa = sanitize(sv.ld_quat(a), bad);
-                    wa = sv.ld_ang(a);
+                    if (STAGED) {
+                        const SimBody parent = body(a);
+                        qa = sanitize(parent.q, bad);
+                        wa = parent.w;
+                    } else {
+                        qa = sanitize(sv.ld_quat(a), bad);
+                        wa = sv.ld_ang(a);
+                    }
                 }
                 for (int k = 0; k < len; ++k) {
                     const LinkRec Lc = L;
                     const int b = Lc.b;
                     const bool own = Lc.flags & LINK_OWN;
                     SimBody sim;
-                    if (own) {                                // issue the loads before the interpolation math
+                    if (own && STAGED) sim = body(b);
+                    if (own && !STAGED) {                     // issue the loads before the interpolation math
                         if (!AOS) (void)IM_CHECKED((4 * (uint32_t)b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
                         sim.q = sv.ld_quat(b);
                         sim.p = sv.ld_pos(b);
@@ -851,15 +916,17 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
                     }
                 }
 #pragma unroll
-                for (int i = 0; i < kPartials; ++i) part[(c * kPartials + i) * kTile + lane] = acc[i];
+                for (int i = 0; i < kPartials; ++i) part_of(c)[i * kTile] = acc[i];
             } else {
                 // ---- observation entries of the simulated bodies (an env known to be reset gets the reference's instead)
                 bool ignore = false;
-                SimBody next = sv.ld_body(ld_link(links, first_own).b);
+                take_staged();
+                const bool known_reset = !need_r && flags_of<OPT>(P, root_z, r, E) != 0;
+                SimBody next = body(ld_link(links, first_own).b);
                 for (int k = first_own; k < len; ++k) {
                     const int b = ld_link(links, k).b;
                     const SimBody sim = next;
-                    if (k + 1 < len) next = sv.ld_body(ld_link(links, k + 1).b);
+                    if (k + 1 < len) next = body(ld_link(links, k + 1).b);
                     (void)IM_CHECKED(15 * b + 14, S);
                     if (!known_reset) body_obs(H, sanitize(sim.q, ignore), sim.p, sim.v, sim.w, row, b);
                 }
@@ -872,7 +939,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
         if (need_r || P.write_back) __syncthreads();
         if (need_r) {
             float term[IM_N_TERMS];
-            r = reward_of<kPartials>(P, part, C, lane, term);
+            r = reward_of(P, part_of, C, term);
         }
     }
     decide<RESET_ALL, OPT>(P, envc, root_z, r, warp == 0 && valid, E);
@@ -1006,7 +1073,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     int ep_done = 0;                            // steps of the episode this step ended (0 where none ended)
     if (!RESET_ALL) {
         float term[IM_N_TERMS];
-        r = reward_of<kPartials>(P, part, C, lane, term);
+        r = reward_of(P, part_of, C, term);
         if (valid) {
             P.reward_out[env] = r;
             P.flags_out[env] = (uint8_t)E.flags;
@@ -1026,15 +1093,17 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
 // OPT compiles in the optional semantics (grace steps, motion randomisation, adaptive initialisation, extended
 // observation); envs that use none run the instantiation without them.
 // WHOLE: the whole row is staged at once (both halves side by side), where that leaves as many CTAs on an SM.
-template <bool RESET_ALL, bool OPT, bool AOS, bool WHOLE>
+// RECORDS: the bodies of a simulator's records are staged all at once before the walk, where that leaves as many CTAs on an SM.
+template <bool RESET_ALL, bool OPT, bool AOS, bool WHOLE, bool RECORDS>
 __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
     // EARLY: the decision is taken before the reward is known, where it can be, and the first warp forms the reward while the
-    // others send rows out.  Not from records: warps of a tile that walk apart lose the lines that the records of their bodies
+    // others send rows out.  Not from records in place: warps of a tile that walk apart lose the lines that the records of their bodies
     // share in L1 (15 bodies x 30000 envs 67.3 us, 71.0 with it).  us per step with two halves and the decision after the reward
     // / EARLY / and WHOLE: 24 bodies x 65536 envs 121.0 / 116.6, x 30000 61.4 / 60.2; 15 bodies x 12000 19.6 / - / 17.8, x 16384
     // 22.5 / - / 21.1, x 65536 83.6 / - / 76.6.
-    constexpr bool EARLY = !OPT && !AOS;
+    constexpr bool EARLY = !OPT && (!AOS || RECORDS);
+    constexpr int kPitch = RECORDS ? kTile + 1 : kTile;
     const SkelDev &sk = P.sk;
     const int J = sk.J;
     const int D = 24 * J + 1;
@@ -1059,9 +1128,14 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     const int RS = 2 + 2 * J;
 
     // this chain's link records: global -> shared, private to the warp
-    float4 *links = reinterpret_cast<float4 *>(smem_raw + (WHOLE ? whole_floats(D_ext, C) : chain_floats(c1, D_ext, C))) + 2 * sk.link_start[c];
+    float4 *links = reinterpret_cast<float4 *>(smem_raw + (WHOLE ? whole_floats(D_ext, C) : RECORDS ? records_floats(J, D_ext) : chain_floats(c1, D_ext, C))) + 2 * sk.link_start[c];
     for (int i = lane; i < 2 * len; i += 32) links[i] = __ldg(P.links + 2 * sk.link_start[c] + i);
     __syncwarp();
+    // A chain's partial sums take the place of the body staged for it, or, of bodies staged all at once, that of its last one, a
+    // leaf, whose state no other chain reads.
+    const auto part_of = [&](int cc) {
+        return part + (RECORDS ? kRing * kPitch * ld_leaf(reinterpret_cast<const float4 *>(smem_raw + records_floats(J, D_ext)), sk, cc) : cc * kRing * kTile) + lane;
+    };
     // this kernel is launched the same way: everything above reads only what the env's creation left in memory
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -1080,6 +1154,14 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     // ---- pass A: reference at the advanced time, errors against the simulated state,
     //      observation entries of the simulated bodies
     if (!RESET_ALL) {
+        uint64_t stream_policy;
+        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_policy));
+        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(part + (RECORDS ? 0 : c * kRing * kTile) + lane);
+        const auto body = [&](int b) { return lds_body<kPitch>(ring + (uint32_t)b * (kRing * kPitch * 4)); };       // (RECORDS)
+        if (RECORDS) {
+            const int e0 = blockIdx.x * kTile;
+            for (int i = c; i < kTile; i += C) sv.stage_record(P, min(e0 + i, P.N - 1), J, ring - 4u * lane, kPitch, i, lane, stream_policy);
+        }
         clip = P.clip_id[envc];
         if (clip < 0 || clip >= P.C) {
             clip = min(max(clip, 0), P.C - 1);
@@ -1098,17 +1180,19 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         float alpha;
         lookup(cm, t1, frame, alpha);
         const float4 *r0 = P.frames + (size_t)IM_CHECKED(frame, P.n_rows) * RS;
-        uint64_t stream_policy;
-        asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_policy));
-        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(part + c * kRing * kTile + lane);
-        sv.stage_body(ld_link(links, first_own).b, ring, stream_policy);
+        if (!RECORDS) sv.stage_body(ld_link(links, first_own).b, ring, stream_policy);
         LinkRec L = ld_link(links, 0);
         KeyPair keys = ld_keys(r0, L.b);
 
-        const Quat q_root = sanitize(sv.ld_quat(0), P.status);
-        const Vec3 p_root = sv.ld_pos(0);
-        H = make_heading(q_root, p_root);
-        root_z = p_root.z;
+        if (RECORDS) {
+            cp_async_wait();
+            __syncthreads();
+        }
+        SimBody root;
+        if (RECORDS) root = body(0);
+        else { root.q = sv.ld_quat(0); root.p = sv.ld_pos(0); }
+        H = make_heading(sanitize(root.q, P.status), root.p);
+        root_z = root.p.z;
 
         float acc[kPartials];
 #pragma unroll
@@ -1118,8 +1202,11 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         Vec3 wa = {0, 0, 0};
         if (first_own > 0) {
             const int a = ld_link(links, first_own - 1).b;
-            qa = sanitize(sv.ld_quat(a), P.status);
-            wa = sv.ld_ang(a);
+            SimBody parent;
+            if (RECORDS) parent = body(a);
+            else { parent.q = sv.ld_quat(a); parent.w = sv.ld_ang(a); }
+            qa = sanitize(parent.q, P.status);
+            wa = parent.w;
         }
         for (int k = 0; k < len; ++k) {
             const LinkRec Lc = L;
@@ -1135,8 +1222,10 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             joint_step<true>(r0, cur, alpha, cm.fps, Lc, k, s, ql, wl);
             if (OPT && k == 0) s.p = s.p + loop_shift(loop, cyc);    // completed cycles of a looped clip move the root
             if (own) {
-                SimBody sim = lds_body(ring);
-                if (k + 1 < len) {                    // the next body of the chain is an own one too
+                SimBody sim;
+                if (RECORDS) sim = body(b);
+                else { cp_async_wait(); sim = lds_body(ring); }
+                if (!RECORDS && k + 1 < len) {                    // the next body of the chain is an own one too
                     if (!AOS) (void)IM_CHECKED((4 * (uint32_t)L.b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
                     sv.stage_body(L.b, ring, stream_policy);
                 }
@@ -1166,8 +1255,9 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
                 wa = sim.w;
             }
         }
+        float *mine = part_of(c);
 #pragma unroll
-        for (int i = 0; i < kPartials; ++i) part[(c * kRing + i) * kTile + lane] = acc[i];
+        for (int i = 0; i < kPartials; ++i) mine[i * kPitch] = acc[i];
     }
     // ---- decision, by every thread of the env, which waits for the reward only where that can end an episode (r_min above
     //      -inf); else the root height and the clip end decide alone, and with EARLY the warps do not meet before their rows are
@@ -1178,7 +1268,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     EnvState E;
     E.clip = clip; E.cyc = cyc; E.t = t1; E.cm = cm; E.loop = loop; E.grace = grace;
     float term[IM_N_TERMS], r = INFINITY;
-    if (need_r || (!RESET_ALL && !EARLY && c == 0)) r = reward_of<kRing>(P, part, C, lane, term);
+    if (need_r || (!RESET_ALL && !EARLY && c == 0)) r = reward_of<kPitch>(P, part_of, C, term);
     decide<RESET_ALL, OPT>(P, envc, root_z, r, c == 0 && valid, E);
     // The first warp writes reward, flags and the new per-env state.
     const auto store_results = [&] {
@@ -1266,7 +1356,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     const bool apart = EARLY && C > 1;
     const int copier = apart ? c - 1 : c, n_copiers = apart ? C - 1 : C;
     const auto finish = [&] {
-        if (!RESET_ALL) r = reward_of<kRing>(P, part, C, lane, term);
+        if (!RESET_ALL) r = reward_of<kPitch>(P, part_of, C, term);
         store_results();
     };
     if (!WHOLE) {
@@ -1387,35 +1477,53 @@ template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(96) env_chain_kernel(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS, false, false>(P, smem_raw);
 }
 __global__ void __maxnreg__(96) env_chain_kernel_whole(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<false, false, false, true>(P, smem_raw);
+    env_chain_body<false, false, false, true, false>(P, smem_raw);
+}
+template <bool OPT>
+__global__ void __maxnreg__(96) env_chain_kernel_records(const __grid_constant__ EnvKernelParams P)
+{
+    extern __shared__ __align__(16) float smem_raw[];
+    env_chain_body<false, OPT, true, false, true>(P, smem_raw);
 }
 template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __launch_bounds__(1024, 1) env_chain_kernel_wide(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS, false, false>(P, smem_raw);
 }
 template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(168) env_role_kernel_1(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_role_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
+    env_role_body<RESET_ALL, OPT, AOS, false, false>(P, smem_raw);
 }
 template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(96) env_role_kernel_2(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_role_body<RESET_ALL, OPT, AOS, false>(P, smem_raw);
+    env_role_body<RESET_ALL, OPT, AOS, false, false>(P, smem_raw);
+}
+template <bool OPT>
+__global__ void __maxnreg__(168) env_role_kernel_records_1(const __grid_constant__ EnvKernelParams P)
+{
+    extern __shared__ __align__(16) float smem_raw[];
+    env_role_body<false, OPT, true, false, true>(P, smem_raw);
+}
+template <bool OPT>
+__global__ void __maxnreg__(96) env_role_kernel_records_2(const __grid_constant__ EnvKernelParams P)
+{
+    extern __shared__ __align__(16) float smem_raw[];
+    env_role_body<false, OPT, true, false, true>(P, smem_raw);
 }
 __global__ void __launch_bounds__(1024, 1) env_role_kernel_wide(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_role_body<false, false, false, true>(P, smem_raw);
+    env_role_body<false, false, false, true, false>(P, smem_raw);
 }
 
 template <typename K>
@@ -1433,11 +1541,31 @@ cudaError_t prepare_one()
     return e;
 }
 
+template <bool OPT>
+cudaError_t prepare_records()
+{
+    cudaError_t e = allow_smem(env_role_kernel_records_1<OPT>);
+    if (e == cudaSuccess) e = allow_smem(env_role_kernel_records_2<OPT>);
+    if (e == cudaSuccess) e = allow_smem(env_chain_kernel_records<OPT>);
+    return e;
+}
+
 // CTAs of `threads` threads that an SM holds, by shared memory, registers and threads.
 int ctas_per_sm(size_t smem, int regs, int threads)
 {
     const int by_smem = (int)(kMaxSmemFloats * sizeof(float) / (smem + 1024)), by_regs = 65536 / (regs * threads), by_threads = 2048 / threads;
     return std::max(1, std::min(by_smem, std::min(by_regs, by_threads)));
+}
+
+// Whether records are staged all at once: where the envs of an array lie a multiple of 256 bytes apart, so that the words that a
+// lane to every env asks for at a time crowd into few sets of the L1 cache.  us per step in place / staged: 16 records an env of 3, 4
+// and 6 words (256 and 384 bytes apart), 15 of them bodies, 4096 envs 15.0 / 12.0, 12000 28.7 / 25.0, 30000 67.3 / 53.7; 25 records
+// (300, 400 and 600 bytes apart), 4096 envs 15.2 / 15.7.
+bool staged_records(const EnvKernelParams &p)
+{
+    bool crowded = false;
+    for (long long stride : p.aos_env_stride) crowded = crowded || stride % 64 == 0;
+    return crowded;
 }
 
 // (The kernels with options start plainly: started early their CTAs, several to an SM, crowd onto the SMs that drain
@@ -1448,19 +1576,27 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
     const int C = p.sk.n_chains, n_sm = device_sm_count();
     const unsigned tiles = (unsigned)((p.N + kTile - 1) / kTile);
     const int extra = (p.n_future - 1) * 9 * __builtin_popcount(p.sk.ee_mask) + p.act_dim;
-    const size_t role_smem = role_smem_floats(staged_cols(p.sk.J, C, p.sk.n_links, extra), C, p.sk.n_links) * sizeof(float);
+    const auto role_bytes = [&](bool staged) {
+        return role_smem_floats(staged_cols(p.sk.J, C, p.sk.n_links, extra, staged), C, p.sk.n_links, staged ? p.sk.J : 0) * sizeof(float);
+    };
+    const size_t role_smem = role_bytes(false);
     const unsigned role_fit = (unsigned)n_sm * ctas_per_sm(role_smem, C <= 8 ? 96 : 64, C <= 16 ? 64 * C : 1024);
     const unsigned chain_fit = (unsigned)n_sm * ctas_per_sm(chain_smem, C <= 8 ? 96 : 64, 32 * C);
     bool role;
     if (RESET_ALL) role = C <= 8 && (tiles <= role_fit || (!OPT && tiles > chain_fit));
     else role = tiles <= std::min(role_fit, 2u * (unsigned)n_sm) && (C <= 8 || (!OPT && !AOS));
     if (role) {
-        void (*kernel)(EnvKernelParams) = tiles <= (unsigned)n_sm && C * 64 * 168 <= 65536 ? env_role_kernel_1<RESET_ALL, OPT, AOS>
-                                                                                           : env_role_kernel_2<RESET_ALL, OPT, AOS>;
+        const bool alone = tiles <= (unsigned)n_sm && C * 64 * 168 <= 65536;
+        void (*kernel)(EnvKernelParams) = alone ? env_role_kernel_1<RESET_ALL, OPT, AOS> : env_role_kernel_2<RESET_ALL, OPT, AOS>;
         if (C > 8) kernel = env_role_kernel_wide;
+        size_t smem = role_smem;
+        if (AOS && C <= 8 && staged_records(p) && (alone || tiles <= (unsigned)n_sm * ctas_per_sm(role_bytes(true), 96, 64 * C))) {
+            kernel = alone ? env_role_kernel_records_1<OPT> : env_role_kernel_records_2<OPT>;
+            smem = role_bytes(true);
+        }
         const dim3 block(32 * (C <= 16 ? 2 * C : 32));
-        if (OPT) kernel<<<tiles, block, role_smem, stream>>>(p);
-        else launch_pdl(kernel, dim3(tiles), block, role_smem, stream, 0, p);
+        if (OPT) kernel<<<tiles, block, smem, stream>>>(p);
+        else launch_pdl(kernel, dim3(tiles), block, smem, stream, 0, p);
     } else {
         void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS> : env_chain_kernel<RESET_ALL, OPT, AOS>;
         // (a reset of all envs keeps the halves: its warps have little to wait for, and 12000 envs x 15 bodies took 14.4 us with whole
@@ -1470,6 +1606,11 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         if (!RESET_ALL && !OPT && !AOS && C <= 8 && ctas_per_sm(whole, 96, 32 * C) >= ctas_per_sm(chain_smem, 96, 32 * C)) {
             kernel = env_chain_kernel_whole;
             smem = whole;
+        }
+        const size_t records = ((size_t)records_floats(p.sk.J, 24 * p.sk.J + 1 + extra) + 8 * p.sk.n_links) * sizeof(float);
+        if (AOS && C <= 8 && staged_records(p) && ctas_per_sm(records, 96, 32 * C) >= ctas_per_sm(chain_smem, 96, 32 * C)) {
+            kernel = env_chain_kernel_records<OPT>;
+            smem = records;
         }
         if (OPT) kernel<<<tiles, 32 * C, smem, stream>>>(p);
         else launch_pdl(kernel, dim3(tiles), dim3(32 * C), smem, stream, 0, p);
@@ -1489,6 +1630,8 @@ cudaError_t env_kernel_prepare()
     return once.run([] {
         cudaError_t e = allow_smem(env_role_kernel_wide);
         if (e == cudaSuccess) e = allow_smem(env_chain_kernel_whole);
+        if (e == cudaSuccess) e = prepare_records<false>();
+        if (e == cudaSuccess) e = prepare_records<true>();
         if (e == cudaSuccess) e = prepare_one<false, false, false>();
         if (e == cudaSuccess) e = prepare_one<true, false, false>();
         if (e == cudaSuccess) e = prepare_one<false, true, false>();

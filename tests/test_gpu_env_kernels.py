@@ -234,3 +234,49 @@ def test_records_equal_rows(n, skeleton, staged):
         out.append(got)
     assert bool((out[0][2] & 1).any())
     assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("options", [False, True])
+@pytest.mark.parametrize("skeleton", ["humanoid15", "smpl24", 1])
+@pytest.mark.parametrize("n", [41, 4801, N - 95])
+def test_records_a_power_of_two_apart_equal_rows(n, skeleton, options):
+    """Records whose envs lie a multiple of 256 bytes apart are staged before the walk; ragged last tiles, one and several tiles
+    per SM, a single chain."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    skel = _tree(skeleton) if skeleton == 1 else W.make_skeleton(skeleton, 1)
+    J, extra = skel["J"], 0
+    lib = W.make_clip_library(J, 4, (20, 40), 30.0, 1)
+    sk = B.Skeleton(skel["parents"], skel["offsets"], skel["masses"])
+    clips = B.Clips(sk, lib["n_frames"], lib["fps"], lib["root_pos"], lib["local_quat"])
+    if options:
+        extra = 2 * 9 * sk.n_ee
+    sims = (torch.randn(3, 13 * J, (n + 3) // 4 * 4, device="cuda", generator=torch.Generator("cuda").manual_seed(n)) * 0.3)[:, :, :n]
+    sims[:, 2] += 0.9
+    out = []
+    for records in (False, True):
+        env = B.Env(sk, clips, B.make_env_config(n, 1 / 30, 5, W.REWARD_MULT, 0.8, B.padded_ld(24 * J + 1 + extra), write_back_reset=True,
+                                                 **(dict(grace_steps=2, reset_noise_std=0.05) if options else {})))
+        if options:
+            env.set_obs_extension(3)
+        obs, rew, fl, terms = env.new_obs(), torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda"), torch.empty(7, n, device="cuda")
+        env.reset_all(obs, 0)
+        got = []
+        for s in range(sims.shape[0]):
+            if records:
+                rec = []
+                for a, b in ((0, 3), (3, 7), (7, 10), (10, 13)):
+                    w = b - a
+                    wide = torch.zeros(n, (w * J + 63) // 64 * 64, device="cuda")
+                    view = wide[:, :w * J].unflatten(1, (J, w))
+                    view.copy_(sims[s, a * J:b * J].reshape(J, w, n).permute(2, 0, 1))
+                    rec.append(view)
+                env.step_aos(s + 1, *rec, obs, rew, fl, terms)
+                sim = torch.cat([r.permute(1, 2, 0).reshape(-1, n) for r in rec])
+            else:
+                sim = torch.empty_strided((13 * J, n), sims[s].stride(), device="cuda").copy_(sims[s])
+                env.step(s + 1, sim, obs, rew, fl, terms)
+            got += [obs.clone(), rew.clone(), fl.clone(), terms.clone(), sim] + list(env.get_state())
+        out.append(got)
+    assert any(bool((fl & 1).any()) for fl in out[0][2::8])        # (in some step: with options the first two are grace steps)
+    assert all(torch.equal(a, b) for a, b in zip(*out))
