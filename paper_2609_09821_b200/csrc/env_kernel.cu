@@ -951,6 +951,11 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     const float4 *rn0 = P.frames + (size_t)IM_CHECKED(frame_n, P.n_rows) * RS;
     const bool any_reset = __any_sync(0xffffffffu, E.reset);
     const bool noisy = OPT && P.reset_noise_std > 0.0f;
+    // The reference's frames 1 .. n_future ahead, a walk each: the observing warps take the first `near` of them, the scoring
+    // warps, which may have the reset envs' walk before them (about two walks of a frame) or come late from the first pass (one),
+    // the rest, so that both are done at about the same time.
+    const int n_frames = OPT ? P.n_future : 1;
+    const int near = OPT ? min(n_frames, (n_frames + 1 + (any_reset ? 2 : 0) + (need_r || P.write_back ? 0 : 1)) / 2) : 1;
 #pragma unroll 1
     for (int task = warp; task < 2 * C; task += n_warps) {
         const int c = task < C ? task : task - C;
@@ -991,7 +996,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
                 }
             }
         }
-        if (any_reset && (OPT || task >= C)) {
+        if (any_reset && (task >= C || near < n_frames)) {
             // heading of the observed root where it is a reset env's new one
             Quat ql;
             Vec3 wl;
@@ -1004,9 +1009,8 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
             if (E.reset) H = Hn;
         }
         // the reference one control interval ahead (frame 1), seen from the observed root's heading frame; frames
-        // f = 2 .. n_future of an extended observation, t + f dt (two fp32 operations, clamped to the clip's end), go to the
-        // warps of the other role, which are the less loaded ones
-        const int f0 = task < C ? 2 : 1, f1 = task < C ? (OPT ? P.n_future : 1) : 1;
+        // f = 2 .. n_future of an extended observation lie at t + f dt (two fp32 operations, clamped to the clip's end)
+        const int f0 = task < C ? near + 1 : 1, f1 = task < C ? n_frames : near;
         for (int f = f0; f <= f1; ++f) {
             int cyc_f = E.cyc_new, frame_f;
             float alpha_f;
