@@ -158,6 +158,20 @@ __device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, float *v)
                    "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                  : "r"(taddr));
 }
+// 64 columns of 16 lanes, issue only: thread t gets columns 8 j + 2 (t % 4) + {0, 1} of lane t / 4 in v[4 j], v[4 j + 1] and of lane
+// t / 4 + 8 in v[4 j + 2], v[4 j + 3].
+__device__ __forceinline__ void tmem_ld_16x64_issue(uint32_t taddr, float *v)
+{
+    uint32_t *r = reinterpret_cast<uint32_t *>(v);
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor: K-major tile of 128-byte rows, 128B swizzle,
@@ -508,10 +522,17 @@ __device__ __forceinline__ uint2 sign_bits(const uint32_t (&pk)[32])
     }
     return r;
 }
-// ... of row `row` and the 64 columns from col0, for the backward epilogue (past the last row: none).
-__device__ __forceinline__ uint2 load_bits(const GemmParams &P, bool second, int row, int col0)
+// ... of this thread's rows of the band from row0, in the layout of bits_chunk, and the 64 columns from col0 (past the last row: none).
+struct BandBits {
+    uint2 w[4];
+};
+__device__ __forceinline__ BandBits load_bits(const GemmParams &P, bool second, int row0, int col0, int lane)
 {
-    return row < P.M ? __ldcg((second ? P.bits_in2 : P.bits_in) + (size_t)(col0 >> 6) * P.ld_bits + row) : make_uint2(0u, 0u);
+    const uint2 *src = (second ? P.bits_in2 : P.bits_in) + (size_t)(col0 >> 6) * P.ld_bits + row0 + (lane >> 2);
+    BandBits b;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) b.w[i] = row0 + (lane >> 2) + 8 * i < P.M ? __ldcg(src + 8 * i) : make_uint2(0u, 0u);
+    return b;
 }
 __device__ __forceinline__ void store_bits(const GemmParams &P, bool second, int row, int col0, const uint32_t (&pk)[32])
 {
@@ -523,7 +544,7 @@ __device__ __forceinline__ void store_bits(const GemmParams &P, bool second, int
 // (backward: ReLU mask of the forward activations, column sums over the warp's 32 rows) -> 32 packed bf16 pairs.
 template <int EPI>
 __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_addr, int row, int col0, int lane,
-                                             const uint4 (&mk)[8], uint2 bits, uint32_t (&pk)[32], const float *bias, float *colsum)
+                                             const uint4 (&mk)[8], uint32_t (&pk)[32], const float *bias, float *colsum)
 {
     float v[64];
     tmem_ld32_issue(t_addr, v);
@@ -543,14 +564,6 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
     } else if (fl > -INFINITY) {
 #pragma unroll
         for (int i = 0; i < 64; ++i) v[i] = fmaxf(v[i], fl);
-    }
-    if (EPI == kBwdBits) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const uint32_t w = i < 16 ? bits.x : bits.y;
-            if (!(w & (1u << (i & 15)))) v[2 * i] = 0.0f;
-            if (!(w & (0x10000u << (i & 15)))) v[2 * i + 1] = 0.0f;
-        }
     }
     if (EPI == kBwdBoxes) {
 #pragma unroll
@@ -580,6 +593,64 @@ __device__ __forceinline__ void hidden_chunk(const GemmParams &P, uint32_t t_add
             if (row0 < P.M)
                 *reinterpret_cast<float2 *>(colsum + (long long)(row0 >> 5) * P.ld_partial + col0 + 2 * lane) =
                     make_float2(v[0], v[1]);
+        }
+    }
+}
+
+// The chunk of the kBwdBits epilogue, from tensor memory to the slab.  A thread has columns 8 j + 2 q + {0, 1} (q = lane % 4) of the
+// rows g, g + 8, g + 16, g + 24 (g = lane / 4) of the 32-row band, so that a column's sum needs three exchanges between lanes
+// instead of five, and the packed pairs are the fragments that stmatrix takes.  The sums are added in the same order as above: rows
+// 16, then 8, 4, 2, 1 apart.  `free` makes sure that the slab may be written.  This epilogue is the longer part of a product with a
+// short contraction, and its instructions what bounds it (a row to a thread, as in hidden_chunk: 250 of 430 were the column sums).
+// Updates with a row to a thread / this: 8 minibatches of 16000 rows (361-1024-512-28 and -1) 2015 / 1978 us, 131072 rows
+// (577-1024-1024-512-69 and -1) 3296 / 3259.
+template <typename Free>
+__device__ __forceinline__ void bits_chunk(const GemmParams &P, uint32_t t_addr, int row0, int col0, int lane, const BandBits &bits, uint8_t *slab,
+                                           float *colsum, Free free)
+{
+    float v[64];
+    tmem_ld_16x64_issue(t_addr, v);
+    tmem_ld_16x64_issue(t_addr + (16u << 16), v + 32);
+    tmem_ld_wait();
+    const int q = lane & 3;
+    uint32_t w[4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { w[i][0] = bits.w[i].x >> q; w[i][1] = bits.w[i].y >> q; }
+#pragma unroll
+    for (int k = 0; k < 64; ++k) {                       // k = 32 h + 4 j + 2 s + c: row 16 h + 8 s + g
+        const int j = (k >> 2) & 7, i = 2 * (k >> 5) + ((k >> 1) & 1), c = k & 1;
+        if (!(w[i][j >> 2] & (1u << (4 * (j & 3) + 16 * c)))) v[k] = 0.0f;
+    }
+    uint32_t pk[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+        pk[k] = *reinterpret_cast<const uint32_t *>(&h);
+    }
+    if (colsum) {
+        float sum[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int o = 4 * (k >> 1) + (k & 1);
+            sum[k] = (v[o] + v[o + 32]) + (v[o + 2] + v[o + 34]);
+        }
+        reduce_scatter_step<8>(sum, lane, 16);
+        reduce_scatter_step<4>(sum, lane, 8);
+        reduce_scatter_step<2>(sum, lane, 4);
+        const int j = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+        if (row0 < P.M)
+            *reinterpret_cast<float2 *>(colsum + (long long)(row0 >> 5) * P.ld_partial + col0 + 8 * j + 2 * q) = make_float2(sum[0], sum[1]);
+    }
+    free();
+    // 8 x 8 matrices: lane L gives the address of row L % 8 of matrix L / 8 (128B-swizzled rows of 128 bytes)
+    const uint32_t at = smem_u32(slab) + (uint32_t)(lane & 7) * 128u + (uint32_t)(((lane >> 3) ^ (lane & 7)) << 4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {                        // rows 8 i ..
+#pragma unroll
+        for (int jj = 0; jj < 2; ++jj) {
+            const uint32_t *f = pk + 16 * (i >> 1) + 8 * jj + (i & 1);
+            asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"((at ^ (64u * jj)) + 1024u * i), "r"(f[0]),
+                         "r"(f[2]), "r"(f[4]), "r"(f[6]) : "memory");
         }
     }
 }
@@ -650,8 +721,8 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, EPI), 1) linear_tc
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
             const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
             const int m0 = at.slice * P.c_batch_rows + at.m * BLOCK_M, n0 = at.n * BLOCK_N;
-            uint2 bits = make_uint2(0u, 0u), bits_next = bits;           // (this chunk's and the next one's)
-            if (EPI == kBwdBits) bits_next = load_bits(P, at.second, m0 + quad * 32 + lane, n0);
+            BandBits bits_next = {};                                       // (the next chunk's)
+            if (EPI == kBwdBits) bits_next = load_bits(P, at.second, m0 + quad * 32, n0, lane);
             bool ready = mbar_wait(&p.acc_full[acc], acc_phase, p.abort_flag);
             if (is_bwd(EPI)) ready = __all_sync(0xffffffffu, ready);           // the column sums shuffle across the whole warp
             if (!ready) break;
@@ -659,40 +730,45 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, EPI), 1) linear_tc
             const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * Plan::kAccStride);
 #pragma unroll 1
             for (int c0 = 64 * half; c0 < BLOCK_N; c0 += kStep) {
-                uint32_t pk[32];
-                if (EPI == kBwdBits) {
-                    bits = bits_next;
-                    if (c0 + 64 < BLOCK_N) bits_next = load_bits(P, at.second, m0 + quad * 32 + lane, n0 + c0 + 64);
-                }
-                if (EPI == kBwdBoxes) {
-                    if (masked) {
-                        if (lane == 0) {
-                            uint8_t *nslab = mslabs + ((ci + 1u) & 1u) * kEpiSlabBytes;
-                            if (c0 + 64 < BLOCK_N) mask_issue(at.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], n0 + c0 + 64, m0 + quad * 32);
-                            else if (tile + (int)gridDim.x < n_tiles) {
-                                const TileAt next = tile_at<MN, DUAL>(P, tile + (int)gridDim.x, tiles_per_slice);
-                                mask_issue(next.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], next.n * BLOCK_N,
-                                           next.m * BLOCK_M + quad * 32);
-                            }
-                        }
-                        if (!__all_sync(0xffffffffu, mbar_wait(&mbar[ci & 1u], (ci >> 1) & 1u, p.abort_flag))) { bail = true; break; }
-                        mask_read(mslabs + (ci & 1u) * kEpiSlabBytes, lane, mk);
-                        ++ci;
-                    } else mask_all_positive(mk);
-                }
-                hidden_chunk<EPI>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, bits, pk, at.second ? P.bias2 : P.bias,
-                                  at.second ? P.colsum_partial2 : P.colsum_partial);
-                if (EPI == kFwdBits) store_bits(P, at.second, m0 + quad * 32 + lane, n0 + c0, pk);
-                // the last store from this slab must have finished reading shared memory
-                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSlabs - 1) : "memory");
-                __syncwarp();
                 uint8_t *slab = slabs + which * kEpiSlabBytes;
-                const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
+                // the last store from this slab must have finished reading shared memory
+                const auto slab_free = [&] {
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSlabs - 1) : "memory");
+                    __syncwarp();
+                };
+                if constexpr (EPI == kBwdBits) {
+                    const BandBits bits = bits_next;
+                    if (c0 + 64 < BLOCK_N) bits_next = load_bits(P, at.second, m0 + quad * 32, n0 + c0 + 64, lane);
+                    bits_chunk(P, t_row + (uint32_t)c0, m0 + quad * 32, n0 + c0, lane, bits, slab, at.second ? P.colsum_partial2 : P.colsum_partial, slab_free);
+                } else {
+                    uint32_t pk[32];
+                    if (EPI == kBwdBoxes) {
+                        if (masked) {
+                            if (lane == 0) {
+                                uint8_t *nslab = mslabs + ((ci + 1u) & 1u) * kEpiSlabBytes;
+                                if (c0 + 64 < BLOCK_N) mask_issue(at.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], n0 + c0 + 64, m0 + quad * 32);
+                                else if (tile + (int)gridDim.x < n_tiles) {
+                                    const TileAt next = tile_at<MN, DUAL>(P, tile + (int)gridDim.x, tiles_per_slice);
+                                    mask_issue(next.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], next.n * BLOCK_N,
+                                               next.m * BLOCK_M + quad * 32);
+                                }
+                            }
+                            if (!__all_sync(0xffffffffu, mbar_wait(&mbar[ci & 1u], (ci >> 1) & 1u, p.abort_flag))) { bail = true; break; }
+                            mask_read(mslabs + (ci & 1u) * kEpiSlabBytes, lane, mk);
+                            ++ci;
+                        } else mask_all_positive(mk);
+                    }
+                    hidden_chunk<EPI>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk, at.second ? P.bias2 : P.bias,
+                                      at.second ? P.colsum_partial2 : P.colsum_partial);
+                    if (EPI == kFwdBits) store_bits(P, at.second, m0 + quad * 32 + lane, n0 + c0, pk);
+                    slab_free();
+                    const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint32_t dst = slab_row + (uint32_t)((c ^ (lane & 7)) << 4);      // 128B swizzle
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pk[4 * c]), "r"(pk[4 * c + 1]),
-                                 "r"(pk[4 * c + 2]), "r"(pk[4 * c + 3]) : "memory");
+                    for (int c = 0; c < 8; ++c) {
+                        const uint32_t dst = slab_row + (uint32_t)((c ^ (lane & 7)) << 4);      // 128B swizzle
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pk[4 * c]), "r"(pk[4 * c + 1]),
+                                     "r"(pk[4 * c + 2]), "r"(pk[4 * c + 3]) : "memory");
+                    }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -944,7 +1020,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
 #pragma unroll 1
                 for (int c0 = 0; c0 < 256; c0 += 64) {
                     uint32_t pk[32];
-                    hidden_chunk<kFwd>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, make_uint2(0u, 0u), pk,
+                    hidden_chunk<kFwd>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk,
                                        at.second ? P.bias2 : P.bias, nullptr);
                     if (EPI == kFwdBits) store_bits(P, at.second, m0 + quad * 32 + lane, n0 + c0, pk);
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
@@ -976,37 +1052,28 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
             // mask's words are asked for before the accumulator is waited for
             const int ew = warp - 2, half = ew >> 2;
             uint8_t *slab = epi + (size_t)ew * kEpiSlabBytes;
-            const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
-            const uint4 mk[8] = {};                     // (unused)
             if (!*abort_flag)
             for (int tile = pair; tile < n_tiles; tile += n_pairs) {
                 const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
-                const int row = at.m * 2 * BLOCK_M + (int)rank * BLOCK_M + quad * 32 + lane, n0 = at.n * 256 + 128 * half;
-                uint2 bits = load_bits(P, at.second, row, n0);
-                const uint2 bits1 = load_bits(P, at.second, row, n0 + 64);
+                const int row0 = at.m * 2 * BLOCK_M + (int)rank * BLOCK_M + quad * 32, n0 = at.n * 256 + 128 * half;
+                BandBits bits = load_bits(P, at.second, row0, n0, lane);
+                const BandBits bits1 = load_bits(P, at.second, row0, n0 + 64, lane);
                 // (the column sums shuffle across the whole warp: every lane takes the same decision)
                 if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[acc], acc_phase, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * 256 + 128 * half);
 #pragma unroll 1
                 for (int c0 = 0; c0 < 128; c0 += 64) {
-                    uint32_t pk[32];
-                    hidden_chunk<kBwdBits>(P, t_row + (uint32_t)c0, row, n0 + c0, lane, mk, bits, pk, at.second ? P.bias2 : P.bias,
-                                           at.second ? P.colsum_partial2 : P.colsum_partial);
+                    bits_chunk(P, t_row + (uint32_t)c0, row0, n0 + c0, lane, bits, slab, at.second ? P.colsum_partial2 : P.colsum_partial, [&] {
+                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        __syncwarp();
+                    });
                     bits = bits1;
-                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                    __syncwarp();
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const uint32_t dst = slab_row + (uint32_t)((c ^ (lane & 7)) << 4);      // 128B swizzle
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(pk[4 * c]), "r"(pk[4 * c + 1]),
-                                     "r"(pk[4 * c + 2]), "r"(pk[4 * c + 3]) : "memory");
-                    }
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) {
                         asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                                     ::"l"(at.second ? map_c2 : &map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(row) : "memory");
+                                     ::"l"(at.second ? map_c2 : &map_c), "r"(smem_u32(slab)), "r"(n0 + c0), "r"(row0) : "memory");
                         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
                     }
                 }
@@ -1057,7 +1124,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                         mask_read(slab, lane, mk);
                     } else mask_all_positive(mk);
                     uint32_t pk[32];
-                    hidden_chunk<kBwdBoxes>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, make_uint2(0u, 0u), pk,
+                    hidden_chunk<kBwdBoxes>(P, t_row + (uint32_t)c0, m0 + quad * 32 + lane, n0 + c0, lane, mk, pk,
                                             at.second ? P.bias2 : P.bias, at.second ? P.colsum_partial2 : P.colsum_partial);
                     // each lane overwrites the 128 bytes it read its own mask words from
                     const uint32_t slab_row = smem_u32(slab) + (uint32_t)lane * 128u;
