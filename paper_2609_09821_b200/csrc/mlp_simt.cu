@@ -11,7 +11,7 @@
 // reads of eight consecutive rows hit distinct banks.  The warps of a CTA share one output tile and split every
 // chunk's k range between them; their partial tiles are added in warp order at the end (bit-reproducible).  Small
 // tiles spread a 64-row layer over the SMs.  Measured (361-1024-512-28, one forward with its noise, CUDA graph):
-// 64 rows 18 us, 300 rows 41 us, 2048 rows 142 us against
+// 64 rows 17 us, 300 rows 37 us, 2048 rows 128 us against
 // 265 us at 64 rows for one 64 x 64 tile per CTA with 16-wide k-steps loaded element by element between barriers
 // and a noise kernel of one thread per row.
 #include <cuda_bf16.h>
@@ -38,7 +38,11 @@ struct Tile {
     static constexpr int kMinBlocks = kThreads == 512 ? 1 : 2;          // (two 16 x 16 CTAs per SM need 64 registers: 23.6 us against 21.0 at 64 rows)
     static constexpr int LD = BK + 4;                                   // floats between two rows of a chunk
     static constexpr int kStageFloats = (BM + BN) * LD;
-    static constexpr int kRedFloats = KW * BM * BN;                     // partial tiles (reuse the stages' space)
+    // Partial tiles (reuse the stages' space), their rows four floats longer than the tile's: a warp's 8 x 4 lanes then write to 32
+    // banks.  Unpadded rows put its eight rows into the same four banks, or into eight (forwards of 361-1024-512-28 on 64 / 300 /
+    // 2048 rows 18.0 / 41.4 / 141 us; padded 17.2 / 37.4 / 128)
+    static constexpr int kRedLd = BN + 4;
+    static constexpr int kRedFloats = KW * BM * kRedLd;
     static constexpr size_t kSmem = sizeof(float) * (kStages * kStageFloats > kRedFloats ? kStages * kStageFloats : kRedFloats);
     static_assert(BK % (4 * KW) == 0 && TM >= 1 && TN >= 1, "k range of a warp is whole 16-byte words");
 };
@@ -104,7 +108,7 @@ struct LayerArgs {
     int lda, ldc, M, N, K;
 };
 
-// One BM x BN tile at (m0, n0): leaves its sums in shared memory as KW partial tiles [KW][BM][BN] and meets.
+// One BM x BN tile at (m0, n0): leaves its sums in shared memory as KW partial tiles [KW][BM][kRedLd] and meets.
 template <class T, Source SA, Source SW>
 __device__ __forceinline__ void tile_product(const LayerArgs &L, int m0, int n0, float *smem)
 {
@@ -153,20 +157,21 @@ __device__ __forceinline__ void tile_product(const LayerArgs &L, int m0, int n0,
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    float *red = smem + kw * (T::BM * T::BN);
+    float *red = smem + kw * (T::BM * T::kRedLd);
 #pragma unroll
     for (int i = 0; i < T::TM; ++i)
 #pragma unroll
         for (int j = 0; j < T::TN; ++j)
-            red[(wm * (T::BM / T::WM) + lm + 8 * i) * T::BN + wn * (T::BN / T::WN) + ln + 4 * j] = acc[i][j];
+            red[(wm * (T::BM / T::WM) + lm + 8 * i) * T::kRedLd + wn * (T::BN / T::WN) + ln + 4 * j] = acc[i][j];
     __syncthreads();
 }
 template <class T>
 __device__ __forceinline__ float tile_sum(const float *smem, int i)
 {
-    float s = smem[i];
+    const float *p = smem + i / T::BN * T::kRedLd + i % T::BN;
+    float s = p[0];
 #pragma unroll
-    for (int q = 1; q < T::KW; ++q) s += smem[q * (T::BM * T::BN) + i];
+    for (int q = 1; q < T::KW; ++q) s += p[q * (T::BM * T::kRedLd)];
     return s;
 }
 
