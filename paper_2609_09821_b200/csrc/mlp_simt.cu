@@ -11,7 +11,7 @@
 // reads of eight consecutive rows hit distinct banks.  The warps of a CTA share one output tile and split every
 // chunk's k range between them; their partial tiles are added in warp order at the end (bit-reproducible).  Small
 // tiles spread a 64-row layer over the SMs.  Measured (361-1024-512-28, one forward with its noise, CUDA graph):
-// 64 rows 17 us, 300 rows 37 us, 2048 rows 128 us against
+// 64 rows 17 us, 300 rows 35 us, 2048 rows 128 us against
 // 265 us at 64 rows for one 64 x 64 tile per CTA with 16-wide k-steps loaded element by element between barriers
 // and a noise kernel of one thread per row.
 #include <cuda_bf16.h>
@@ -313,15 +313,18 @@ cudaError_t launch_linear_simt(const float *A, int lda, const void *W, bool w_bf
     // The smallest tile whose CTAs, one per SM with sixteen warps, hold the layer in one wave: a wave's time grows with the
     // tile, a second wave costs more (1024 x 361, us with its head: 64 rows 18.5 as two waves of 16 x 16, 15.0 as one of
     // 32 x 16; 128 rows 19.2 with 32 x 16, 18.2 with 32 x 32.  512 x 1024: 128 rows 19.0 with 16 x 16, 15.6 with 32 x 16; 200
-    // rows 23.3 with 32 x 16, 21.6 with 32 x 32).  32 x 48 is the largest that pays: whole forwards of 361-1024-512-28 on 129 /
-    // 192 / 300 / 416 rows 31.0 / 30.7 / 41.5 / 42.2 us, 34.0 / 33.8 / 46.6 / 47.1 without it (361-2048-1024-28, 192 rows: 59 and 69;
-    // 361-512-256-28, 640 rows: 33.3 and 36.2); 64 x 32 on 300 rows 48.  Beyond that two
-    // 32 x 32 CTAs per SM, up to four (512 rows: 52 us against 107 with 64 x 64), then 64 x 64 (2048 rows: 142 us against 156)
+    // rows 23.3 with 32 x 16, 21.6 with 32 x 32).  Whole forwards of 361-1024-512-28 on 129 / 192 / 300 / 416 rows with 32 x 48
+    // 31.0 / 30.7 / 41.5 / 42.2 us, 34.0 / 33.8 / 46.6 / 47.1 without it (361-2048-1024-28, 192 rows: 59 and 69; 361-512-256-28, 640
+    // rows: 33.3 and 36.2; all of these before the partial tiles were padded).  Beyond that two 32 x 32 CTAs per SM while they are
+    // one wave; then 64 x 48 while that is (300 / 700 rows: 37.4 / 65.5 us without, 34.8 / 62.9 with; where one wave of 32 x 32
+    // does, at 200 rows, 30.0 and 32.4), 32 x 32 up to four per SM (512 rows: 52 us against 107 with 64 x 64; one wave of 64 x 64
+    // with sixteen warps 51 against 45.6), and 64 x 64 (2048 rows: 142 us against 156)
     const int n_sm = device_sm_count();
     if (tiles(16, 16) <= n_sm) e = launch_tile<Tile<512, 16, 16, 256, 1, 1, 3>>(L, w_bf16, stream);
     else if (tiles(32, 16) <= n_sm) e = launch_tile<Tile<512, 32, 16, 128, 1, 1, 3>>(L, w_bf16, stream);
     else if (tiles(32, 32) <= n_sm) e = launch_tile<Tile<512, 32, 32, 128, 1, 1, 3>>(L, w_bf16, stream);
     else if (tiles(32, 48) <= n_sm) e = launch_tile<Tile<512, 32, 48, 128, 1, 1, 3>>(L, w_bf16, stream);
+    else if (tiles(32, 32) > 2 * n_sm && tiles(64, 48) <= n_sm) e = launch_tile<Tile<512, 64, 48, 128, 1, 2, 3>>(L, w_bf16, stream);
     else if (tiles(32, 32) <= 4 * n_sm) e = launch_tile<Tile<256, 32, 32, 128, 1, 1, 3>>(L, w_bf16, stream);
     else e = launch_tile<Tile<256, 64, 64, 64, 1, 2, 3>>(L, w_bf16, stream);
     g_launches.fetch_add(1, std::memory_order_relaxed);

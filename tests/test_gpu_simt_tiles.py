@@ -61,3 +61,9 @@ def test_log_probabilities_across_a_cluster(n, A):
                                     (385, (577, 512, 530, 9)), (416, (362, 528, 485, 28)), (417, (40, 512, 28)), (832, (361, 240, 12, 3))])
 def test_forward_around_the_largest_one_wave_tile(n, dims):
     test_forward_matches_oracle(n, dims)
+
+
+@pytest.mark.parametrize("n,dims", [(300, (361, 1024, 512, 28)), (321, (362, 1021, 70, 5)), (384, (577, 1008, 33, 9)), (385, (40, 1000, 64)),
+                                    (641, (70, 529, 260, 3)), (833, (5, 432, 40, 3)), (832, (1024, 490, 40, 3))])
+def test_forward_on_64_by_48_tiles(n, dims):
+    test_forward_matches_oracle(n, dims)
