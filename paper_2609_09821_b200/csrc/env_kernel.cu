@@ -18,7 +18,7 @@
 // and about equally long -- one scores the simulated bodies against the reference,
 // the other builds the observation -- and stages whole rows.  With more tiles than
 // that the issue slots count: the chain kernel does both in one warp per chain,
-// which loads every body once, and stages half rows, so that four CTAs share an SM.
+// which loads every body once, and stages half rows (whole ones of small trees), so that four CTAs share an SM.
 // Figures at launch_env_kernel.
 #include <algorithm>
 
@@ -1665,7 +1665,8 @@ cudaError_t launch_debug_math(int op, int n, const float *in, float *out, cudaSt
 // Which kernel: the role kernel while its tiles fit the SMs at once, the chain kernel beyond (us per launch in a chain of
 // them, 15 bodies / 24 bodies, role against chain: 64 envs 7.8 / 12.4 against 15.0 / 22.5; 4096 envs 9.7 / 14.1 against
 // 17.6 / 23.6; 9472 envs, two CTAs per SM, 14.2 / 20.9 against 19.4 / 26.2; 12000 envs 24.2 / 34.9 against 23.5 / 32.0;
-// 65536 envs 89.5 / 142 against 88 / 125).  Trees with more than eight leaves fill an SM with one CTA of either kernel, and
+// 65536 envs 89.5 / 142 against 88 / 125; since its body states are staged and the decision is early the chain kernel takes 17.5 / 25.7
+// at 12000 and 76.7 / 117 at 65536).  Trees with more than eight leaves fill an SM with one CTA of either kernel, and
 // only without options and records is the role kernel the faster one (31 leaves, 4096 envs: 25.0 against 25.4 us plain, 41.3
 // against 34.4 with options, 45.0 against 38.0 from records).
 // A reset of all envs: the role kernel while its tiles fit the SMs at once, then the chain kernel while its do (12000 envs, 15 /
