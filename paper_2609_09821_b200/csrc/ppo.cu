@@ -20,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include "im_internal.h"
+#include "ppo_finish.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -37,11 +38,8 @@ __device__ __forceinline__ void dep_release_wait()
 }
 
 constexpr int kFinishThreads = 1024;
-constexpr int kFinishGroups = 32;
-constexpr int kFinishBatch = 16;            // partial rows of a group whose loads are in flight together
-constexpr int kMaxA = 128;
-constexpr int kScalars = 4;               // surrogate, value loss, kl, clip count
-constexpr int kPartial = kMaxA + kScalars;
+constexpr int kMaxA = kPpoMaxA;
+constexpr int kPartial = kPpoPartial;
 
 struct PpoParams {
     im_ppo_config cfg;
@@ -438,55 +436,10 @@ __global__ void __launch_bounds__(32 * bulk_warps(LPR)) ppo_loss_bulk_kernel(con
     fold_and_write<LPR, NI, kBulkWarps>(acc, s_acc, P.partial + (size_t)(P.partial_begin + blockIdx.x) * kPartial);
 }
 
-// Sums the CTAs' partial rows (fp64: as many interleaved groups of rows as the block has threads for the A + kScalars
-// columns in use, each in order, then the groups in order) and writes d_log_std and the summary.  One block's time is its
-// chain of loads: 500 rows of A = 28 took 9 to 12 us in four groups
-// of one load at a time, 4.8 us now.
-__global__ void __launch_bounds__(kFinishThreads) ppo_finish_kernel(const PpoParams P, int grid)
+__global__ void __launch_bounds__(kFinishThreads) ppo_finish_kernel(const PpoFinish F)
 {
-    __shared__ double s_grp[kFinishThreads];               // [groups][columns]
-    __shared__ double s_tot[kPartial];
-    __shared__ double s_H;
-    __shared__ float s_ls[kMaxA];
-    const int cols = P.A + kScalars, groups = min(kFinishThreads / cols, kFinishGroups);
-    const int jj = (int)threadIdx.x % cols, q = (int)threadIdx.x / cols, j = jj < P.A ? jj : kMaxA + jj - P.A;
     dep_release_wait();
-    if (q < groups) {
-        const float *col = P.partial + j;
-        double t = 0.0;
-        for (int g = q; g < grid; g += kFinishBatch * groups) {
-            float x[kFinishBatch];                          // loads in flight together, added in order
-#pragma unroll
-            for (int k = 0; k < kFinishBatch; ++k) x[k] = g + k * groups < grid ? __ldcg(col + (size_t)(g + k * groups) * kPartial) : 0.0f;
-#pragma unroll
-            for (int k = 0; k < kFinishBatch; ++k) t += (double)x[k];
-        }
-        s_grp[threadIdx.x] = t;
-        if (q == groups - 1 && jj < P.A) s_ls[jj] = P.b.log_std[jj];
-    }
-    __syncthreads();
-    if (q == 0) {
-        double t = 0.0;
-        for (int k = 0; k < groups; ++k) t += s_grp[k * cols + jj];
-        s_tot[j] = t;
-        if (jj < P.A) P.d_log_std[jj] = (float)(t - (double)P.cfg.entropy_coef);   // the row terms already carry 1/M
-    } else if (threadIdx.x == kFinishThreads - 1) {
-        double H = 0.0;
-        for (int k = 0; k < P.A; ++k) H += (double)s_ls[k] + 0.5 * 2.8378770664093453;   // 1/2 ln(2 pi e)
-        s_H = H;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const double M = (double)P.M;
-        const double H = s_H;
-        const double surr = s_tot[kMaxA + 0] / M, vl = s_tot[kMaxA + 1] / M;
-        P.summary[0] = (float)(surr + (double)P.cfg.value_coef * vl - (double)P.cfg.entropy_coef * H);
-        P.summary[1] = (float)surr;
-        P.summary[2] = (float)vl;
-        P.summary[3] = (float)H;
-        P.summary[4] = (float)(s_tot[kMaxA + 2] / M);
-        P.summary[5] = (float)(s_tot[kMaxA + 3] / M);
-    }
+    ppo_finish<kFinishThreads>(F);
 }
 
 // ---- moments: mean and 1 / (std + 1e-8), n - 1 divisor
@@ -573,36 +526,9 @@ cudaError_t ppo_set_wait_debug(unsigned long long limit_ns, int skip_loads)
     return e;
 }
 
-}  // namespace im
-
-extern "C" {
-
-size_t im_ppo_workspace_bytes(void) { return (size_t)(2 * im::kMaxGrid) * im::kPartial * sizeof(float); }
-
-im_status im_moments(const float *x, int64_t n, float *out2, void *workspace, void *cuda_stream)
+im_status ppo_loss_rows(const im_ppo_config *cfg, int64_t M, int32_t A, const im_ppo_batch *batch, float *d_mean, float *d_log_std,
+                        float *d_value, float *summary, void *workspace, void *cuda_stream, PpoFinish *fin)
 {
-    using namespace im;
-    if (!x || !out2 || !workspace || n < 1) return IM_ERR_INVALID_ARG;
-    if (reinterpret_cast<uintptr_t>(workspace) & 7u) return IM_ERR_INVALID_ARG;
-    long long g = (n + kMomThreads * 8 - 1) / (kMomThreads * 8);
-    const int grid = (int)(g < 1 ? 1 : (g > kMaxGrid ? kMaxGrid : g));
-    cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (n <= kMomClusterMax) {
-        if (launch_pdl(moments_cluster_kernel, dim3(kMomCluster), dim3(kMomThreads), 0, st, 0, x, (long long)n, out2) != cudaSuccess) return IM_ERR_CUDA;
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
-    }
-    if (launch_pdl(moments_partial_kernel, dim3(grid), dim3(kMomThreads), 0, st, 0, x, (long long)n, static_cast<double *>(workspace)) != cudaSuccess ||
-        launch_pdl(moments_finish_kernel, dim3(1), dim3(32), 0, st, 0, static_cast<const double *>(workspace), grid, (long long)n, out2) != cudaSuccess)
-        return IM_ERR_CUDA;
-    g_launches.fetch_add(2, std::memory_order_relaxed);
-    return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
-}
-
-im_status im_ppo_loss(const im_ppo_config *cfg, int64_t M, int32_t A, const im_ppo_batch *batch, float *d_mean,
-                      float *d_log_std, float *d_value, float *summary, void *workspace, void *cuda_stream)
-{
-    using namespace im;
     if (!cfg || !batch || !d_mean || !d_log_std || !d_value || !summary || !workspace) return IM_ERR_INVALID_ARG;
     if (M < 1 || A < 1 || A > kMaxA) return IM_ERR_INVALID_ARG;
     if (!batch->mean || !batch->log_std || !batch->action || !batch->logp_old || !batch->mean_old ||
@@ -692,9 +618,44 @@ im_status im_ppo_loss(const im_ppo_config *cfg, int64_t M, int32_t A, const im_p
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
 #undef IM_PPO_DISPATCH
-    grid += grid_bulk;
-    if (launch_pdl(ppo_finish_kernel, dim3(1), dim3(kFinishThreads), 0, st, 0, p, grid) != cudaSuccess) return IM_ERR_CUDA;
-    g_launches.fetch_add(1, std::memory_order_relaxed);
+    *fin = {p.partial, grid + grid_bulk, A, M, batch->log_std, cfg->value_coef, cfg->entropy_coef, d_log_std, summary};
+    return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+}
+
+}  // namespace im
+
+extern "C" {
+
+size_t im_ppo_workspace_bytes(void) { return (size_t)(2 * im::kMaxGrid) * im::kPartial * sizeof(float); }
+
+im_status im_moments(const float *x, int64_t n, float *out2, void *workspace, void *cuda_stream)
+{
+    using namespace im;
+    if (!x || !out2 || !workspace || n < 1) return IM_ERR_INVALID_ARG;
+    if (reinterpret_cast<uintptr_t>(workspace) & 7u) return IM_ERR_INVALID_ARG;
+    long long g = (n + kMomThreads * 8 - 1) / (kMomThreads * 8);
+    const int grid = (int)(g < 1 ? 1 : (g > kMaxGrid ? kMaxGrid : g));
+    cudaStream_t st = (cudaStream_t)cuda_stream;
+    if (n <= kMomClusterMax) {
+        if (launch_pdl(moments_cluster_kernel, dim3(kMomCluster), dim3(kMomThreads), 0, st, 0, x, (long long)n, out2) != cudaSuccess) return IM_ERR_CUDA;
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+    }
+    if (launch_pdl(moments_partial_kernel, dim3(grid), dim3(kMomThreads), 0, st, 0, x, (long long)n, static_cast<double *>(workspace)) != cudaSuccess ||
+        launch_pdl(moments_finish_kernel, dim3(1), dim3(32), 0, st, 0, static_cast<const double *>(workspace), grid, (long long)n, out2) != cudaSuccess)
+        return IM_ERR_CUDA;
+    g_launches.fetch_add(2, std::memory_order_relaxed);
+    return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
+}
+
+im_status im_ppo_loss(const im_ppo_config *cfg, int64_t M, int32_t A, const im_ppo_batch *batch, float *d_mean,
+                      float *d_log_std, float *d_value, float *summary, void *workspace, void *cuda_stream)
+{
+    im::PpoFinish fin;
+    const im_status s = im::ppo_loss_rows(cfg, M, A, batch, d_mean, d_log_std, d_value, summary, workspace, cuda_stream, &fin);
+    if (s != IM_OK) return s;
+    if (im::launch_pdl(im::ppo_finish_kernel, dim3(1), dim3(im::kFinishThreads), 0, (cudaStream_t)cuda_stream, 0, fin) != cudaSuccess) return IM_ERR_CUDA;
+    im::g_launches.fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
 

@@ -207,9 +207,9 @@ static im_status update_on(im_ppo_updater *u, int M, const im_ppo_minibatch *mb,
     const im_ppo_config pc = {u->cfg.clip, u->cfg.value_coef, u->cfg.entropy_coef, u->cfg.clip_value_loss};
     const im_ppo_batch pb = {a->out, u->log_std, mb->action, mb->logp_old, mb->mean_old,
                              mb->log_std_old ? mb->log_std_old : u->log_std_old, mb->advantage, mom, c->out, mb->value_old, mb->returns};
-    s = im_ppo_loss(&pc, M, u->A, &pb, u->d_mean, u->d_log_std, u->d_value, u->summary, u->ws, st);
-    if (s != IM_OK) return s;
     im::OutGradArgs og = {};
+    s = im::ppo_loss_rows(&pc, M, u->A, &pb, u->d_mean, u->d_log_std, u->d_value, u->summary, u->ws, st, &og.fin);
+    if (s != IM_OK) return s;
     og.n_nets = 2; og.M = M; og.net[0] = out_grad(a, u->d_mean); og.net[1] = out_grad(c, u->d_value);
     if (im::launch_out_grads(og, st) != cudaSuccess) return IM_ERR_CUDA;
     int slices[2][IM_MAX_LAYERS];

@@ -269,14 +269,18 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
 constexpr int kOutRows = 128;
 constexpr int kOutBatch = 16;
 
+// 128 rows of a net to a block; the first block has the loss's sums, which nothing waits for before the gradient reduction (as a
+// launch of their own they took 5 us between the loss and this one).
 __global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_constant__ OutGradArgs P)
 {
     __shared__ float s_sum[8][128];
     dep_release_wait();
-    const OutGrad &G = P.net[blockIdx.y];
+    if (P.fin.partial && blockIdx.x == 0) { ppo_finish<kThreads>(P.fin); return; }
+    const int block = (int)blockIdx.x - (P.fin.partial ? 1 : 0), row_block = block / P.n_nets;
+    const OutGrad &G = P.net[block - row_block * P.n_nets];
     const int lanes = G.ld >> 1, groups = kThreads / lanes;       // a thread owns two columns of every `groups`-th row
     const int c = 2 * ((int)threadIdx.x % lanes), g = (int)threadIdx.x / lanes;
-    const int r0 = blockIdx.x * kOutRows, r1 = min(r0 + kOutRows, P.M);
+    const int r0 = row_block * kOutRows, r1 = min(r0 + kOutRows, P.M);
     __nv_bfloat16 *dz = reinterpret_cast<__nv_bfloat16 *>(G.dz);
     float s0 = 0.0f, s1 = 0.0f;
 #pragma unroll 1
@@ -302,7 +306,7 @@ __global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_consta
     if ((int)threadIdx.x < G.ld) {
         float t = 0.0f;
         for (int k = 0; k < groups; ++k) t += s_sum[k][threadIdx.x];
-        G.partial[(long long)blockIdx.x * G.ld + threadIdx.x] = t;
+        G.partial[(long long)row_block * G.ld + threadIdx.x] = t;
     }
 }
 
@@ -419,7 +423,7 @@ cudaError_t launch_grad_reduce(GradReduceArgs &a, cudaStream_t stream)
 
 cudaError_t launch_out_grads(const OutGradArgs &a, cudaStream_t stream)
 {
-    const cudaError_t e = launch_pdl(out_grads_kernel, dim3((unsigned)((a.M + kOutRows - 1) / kOutRows), (unsigned)a.n_nets), dim3(kThreads), 0,
+    const cudaError_t e = launch_pdl(out_grads_kernel, dim3((unsigned)((a.M + kOutRows - 1) / kOutRows * a.n_nets + (a.fin.partial ? 1 : 0))), dim3(kThreads), 0,
                                      stream, 0, a);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return e;

@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include "../../include/im.h"
+#include "ppo_finish.cuh"
 
 namespace im {
 
@@ -73,6 +74,7 @@ struct OutGrad {
 struct OutGradArgs {
     OutGrad net[2];
     int n_nets, M;
+    PpoFinish fin;                                         // the loss's sums, by a block of the same launch (fin.partial null: none)
 };
 cudaError_t launch_out_grads(const OutGradArgs &a, cudaStream_t stream);
 

@@ -40,6 +40,8 @@ def test_mask_bits_give_the_gradients_of_the_activations(M, dims, cdims):
                                       torch.empty(6, device="cuda"))
     B.ppo_loss(dict(batch, mean=mean, value=value[:, 0].contiguous(), log_std=log_std, log_std_old=log_std), d_mean, d_ls, d_value, summary,
                B.ppo_workspace(), 0.2, 2.0, 0.0, True)
+    # the loss's sums, by another number of threads: added in fp64 in another order, one rounding to fp32 each
+    assert torch.allclose(upd.summary, summary, rtol=2.5e-7, atol=1e-9 * float(summary.abs().max()))
     ref[0].backward(d_mean, M)
     ref[1].backward(d_value.view(M, 1), M)
     torch.cuda.synchronize()
