@@ -1102,11 +1102,11 @@ template <bool RESET_ALL, bool OPT, bool AOS, bool WHOLE, bool RECORDS>
 __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
     // EARLY: the decision is taken before the reward is known, where it can be, and the first warp forms the reward while the
-    // others send rows out.  Not from records in place: warps of a tile that walk apart lose the lines that the records of their bodies
+    // others send rows out.  Not in a reset of all envs, which has no reward to form; not from records in place: warps of a tile that walk apart lose the lines that the records of their bodies
     // share in L1 (15 bodies x 30000 envs 67.3 us, 71.0 with it).  us per step with two halves and the decision after the reward
     // / EARLY / and WHOLE: 24 bodies x 65536 envs 121.0 / 116.6, x 30000 61.4 / 60.2; 15 bodies x 12000 19.6 / - / 17.8, x 16384
     // 22.5 / - / 21.1, x 65536 83.6 / - / 76.6.
-    constexpr bool EARLY = !OPT && (!AOS || RECORDS);
+    constexpr bool EARLY = !RESET_ALL && !OPT && (!AOS || RECORDS);
     constexpr int kPitch = RECORDS ? kTile + 1 : kTile;
     const SkelDev &sk = P.sk;
     const int J = sk.J;
@@ -1360,7 +1360,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     const bool apart = EARLY && C > 1;
     const int copier = apart ? c - 1 : c, n_copiers = apart ? C - 1 : C;
     const auto finish = [&] {
-        if (!RESET_ALL) r = reward_of<kPitch>(P, part_of, C, term);
+        r = reward_of<kPitch>(P, part_of, C, term);
         store_results();
     };
     if (!WHOLE) {
