@@ -39,7 +39,8 @@ __device__ __forceinline__ uint2 pack_bf16x4(float4 v)
 }
 
 constexpr int kTile = 32;          // envs per CTA
-constexpr int kRing = 13;          // words per env of a staged body: rotation, position, linear and angular velocity
+constexpr int kVectors = 9;        // words per env of a staged body: position, linear and angular velocity ..
+constexpr int kBody = 13;          // .. and rotation
 constexpr int kPartials = 9;       // pose, vel, ee_pos, ee_rot, body_pos, body_vel, weighted com difference (3)
 
 // The bounds-checked build (-DIM_DEBUG, a second library next to the regular one): every index the kernel forms
@@ -69,34 +70,35 @@ __host__ __device__ inline int tile_stride(int D)
 // up to a multiple of four columns so that both halves start on a 16-byte boundary.
 __host__ __device__ inline int split_col(int J) { return (15 * J + 3) / 4 * 4; }
 
-// Shared memory of the chain kernel, in floats: the first half rows and behind them a staged body per chain (whose place the
-// chain's partial sums take later), or the second half rows, which are assembled when both are done with; then the chains'
-// link records.  (The second half's limit counts the partial sums: it decides which extended observations are accepted.)
-__host__ __device__ inline int chain_floats(int c1, int D_ext, int n_chains)
+// Shared memory of the chain kernel, in floats: the first half rows and behind them, per chain, `slot` words per env of the body
+// that is staged ahead, whose place the chain's partial sums take later; or the second half rows, which are assembled when both
+// are done with; then the chains' link records.  (The second half's limit counts the partial sums: it decides which extended
+// observations are accepted.)
+__host__ __device__ inline int chain_floats(int c1, int D_ext, int n_chains, int slot)
 {
     const int s1 = tile_stride(c1), s2 = tile_stride(D_ext - c1);
-    const int first = kTile * s1 + kRing * n_chains * kTile, both = kTile * (s1 > s2 ? s1 : s2) + kPartials * n_chains * kTile;
+    const int first = kTile * s1 + slot * n_chains * kTile, both = kTile * (s1 > s2 ? s1 : s2) + kPartials * n_chains * kTile;
     return first > both ? first : both;
 }
 // With the bodies of records staged all at once, an odd number of words from one component to the next.
 __host__ __device__ inline int records_floats(int J, int D_ext)
 {
     const int s1 = tile_stride(split_col(J)), s2 = tile_stride(D_ext - split_col(J));
-    const int first = kTile * s1 + (J * kRing * (kTile + 1) + 3) / 4 * 4, second = kTile * s2;
+    const int first = kTile * s1 + (J * kBody * (kTile + 1) + 3) / 4 * 4, second = kTile * s2;
     return first > second ? first : second;
 }
 // With whole rows staged.
-__host__ __device__ inline int whole_floats(int D_ext, int n_chains) { return kTile * (tile_stride(D_ext) + kRing * n_chains); }
-__host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, int extra_cols)
+__host__ __device__ inline int whole_floats(int D_ext, int n_chains) { return kTile * (tile_stride(D_ext) + kBody * n_chains); }
+__host__ __device__ inline size_t smem_floats(int J, int n_chains, int n_links, int extra_cols, int slot)
 {
-    return (size_t)chain_floats(split_col(J), 24 * J + 1 + extra_cols, n_chains) + (size_t)8 * n_links;
+    return (size_t)chain_floats(split_col(J), 24 * J + 1 + extra_cols, n_chains, slot) + (size_t)8 * n_links;
 }
 
 // The role kernel: the staged rows, the chains' partial sums, their link records, staged body states.  Staged columns: all, or, where an
 // extended observation is too wide for that, the first 24 J (the rest is then written column by column).
 __host__ __device__ inline size_t role_smem_floats(int cols, int n_chains, int n_links, int staged_bodies)
 {
-    return (size_t)kTile * tile_stride(cols) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links + (size_t)staged_bodies * kRing * (kTile + 1);
+    return (size_t)kTile * tile_stride(cols) + (size_t)kPartials * n_chains * kTile + (size_t)8 * n_links + (size_t)staged_bodies * kBody * (kTile + 1);
 }
 constexpr size_t kMaxSmemFloats = 232448 / 4;       // opt-in shared memory per block on this architecture (227 KB)
 __host__ __device__ inline int staged_cols(int J, int n_chains, int n_links, int extra_cols, bool staged_bodies)
@@ -458,12 +460,17 @@ __device__ __forceinline__ float lds32(uint32_t addr)
     return v;
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-// A body staged by stage_body, once its copies have landed.
-template <int PITCH = kTile>
+// A staged body, once its copies have landed; of one that is staged without its rotation the vectors.
+template <int PITCH = kTile, int WORDS = kBody>
 __device__ __forceinline__ SimBody lds_body(uint32_t a)
 {
     const auto w = [a](int i) { return lds32(a + (uint32_t)(4 * PITCH * i)); };
-    return {{w(0), w(1), w(2), w(3)}, {w(4), w(5), w(6)}, {w(7), w(8), w(9)}, {w(10), w(11), w(12)}};
+    SimBody s;
+    if constexpr (WORDS == kBody) s.q = {w(9), w(10), w(11), w(12)};
+    s.p = {w(0), w(1), w(2)};
+    s.v = {w(3), w(4), w(5)};
+    s.w = {w(6), w(7), w(8)};
+    return s;
 }
 
 // Body-state access of one thread (one env).  Two layouts:
@@ -506,27 +513,27 @@ struct SimView {
         const uint32_t o = 3 * (uint32_t)b * st + e;
         return {__ldcs(base + o), __ldcs(base + o + st), __ldcs(base + o + 2 * st)};
     }
-    // This env's state of body b to shared memory, asynchronously: component i (rotation, position, velocities) to the
-    // word at dst + 128 i bytes.  Every lane copies and later reads its own words.  The chain kernel, whose warps are bound by
-    // the latency of what they load (20 of them on an SM), so asks for a body while it walks the one before, at the price of no
-    // registers: us per step with the loads in the walk itself / staged a body ahead, 15 bodies x 16384 envs 23.9 / 22.5, x 65536
-    // 88.2 / 83.7; 24 bodies x 16384 32.6 / 30.7, x 65536 125.0 / 121.1; from records 24 bodies x 12000 43.6 / 42.1 (15: 28.5 /
-    // 28.7); spilled bytes 48 / 0.
+    // This env's state of body b, or its vectors alone, to shared memory, asynchronously: component i (position, velocities,
+    // rotation) to the word at dst + 128 i bytes.  Every lane copies and later reads its own words.  The chain kernel, whose
+    // warps are bound by the latency of what they load (20 of them on an SM), so asks for a body while it walks the one before, at
+    // the price of no registers: us per step with the loads in the walk itself / staged a body ahead, 15 bodies x 16384 envs 20.6 /
+    // 18.8, x 65536 76.2 / 66.5; 24 bodies x 16384 28.7 / 27.6, x 65536 102.0 / 96.1; spilled bytes 48 / 0.
+    template <int WORDS>
     __device__ __forceinline__ void stage_body(int b, uint32_t dst, uint64_t policy) const
     {
         if (AOS) {
-            const float *q = quat + (long long)b * bs_quat, *v[3] = {pos + (long long)b * bs_pos, lin + (long long)b * bs_lin, ang + (long long)b * bs_ang};
+            const float *v[3] = {pos + (long long)b * bs_pos, lin + (long long)b * bs_lin, ang + (long long)b * bs_ang}, *q = quat + (long long)b * bs_quat;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) cp_async_word(dst + 128 * i, q + i, policy);
+            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * i, v[i / 3] + i % 3, policy);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) cp_async_word(dst + 128 * (4 + i), v[i / 3] + i % 3, policy);
+            for (int i = kVectors; i < WORDS; ++i) cp_async_word(dst + 128 * i, q + (i - kVectors), policy);
         } else {
             const uint32_t o = 4 * (uint32_t)b * st + e, o3 = 3 * (uint32_t)b * st + e;
             const float *v[3] = {pos, lin, ang};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) cp_async_word(dst + 128 * i, quat + (o + i * st), policy);
+            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * i, v[i / 3] + (o3 + (i % 3) * st), policy);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) cp_async_word(dst + 128 * (4 + i), v[i / 3] + (o3 + (i % 3) * st), policy);
+            for (int i = kVectors; i < WORDS; ++i) cp_async_word(dst + 128 * i, quat + (o + (i - kVectors) * st), policy);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
@@ -541,10 +548,10 @@ struct SimView {
         const int bs[4] = {P.aos_body_stride[1], P.aos_body_stride[0], P.aos_body_stride[2], P.aos_body_stride[3]};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int n = k == 0 ? 4 : 3, off = k == 0 ? 0 : 1 + 3 * k;
+            const int n = k == 0 ? 4 : 3, off = k == 0 ? kVectors : 3 * k - 3;
             for (int i = lane; i < n * J; i += 32) {
                 const int b = i / n, c = i - n * b;
-                cp_async_word(dst + 4u * ((uint32_t)(kRing * b + off + c) * pitch + (uint32_t)col), a[k] + (long long)b * bs[k] + c, policy);
+                cp_async_word(dst + 4u * ((uint32_t)(kBody * b + off + c) * pitch + (uint32_t)col), a[k] + (long long)b * bs[k] + c, policy);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -792,7 +799,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     bool bad = false;
     const SimView<AOS> sv(P, envc);
     constexpr int kPitch = kTile + 1;
-    const auto body = [&](int b) { return STAGED ? lds_body<kPitch>(bodies + (uint32_t)b * (kRing * kPitch * 4)) : sv.ld_body(b); };
+    const auto body = [&](int b) { return STAGED ? lds_body<kPitch>(bodies + (uint32_t)b * (kBody * kPitch * 4)) : sv.ld_body(b); };
     if (!RESET_ALL) {
         Quat q_root = {1.0f, 0.0f, 0.0f, 0.0f};
         Vec3 p_root = {0.0f, 0.0f, 0.0f};
@@ -1098,7 +1105,8 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
 // observation); envs that use none run the instantiation without them.
 // WHOLE: the whole row is staged at once (both halves side by side), where that leaves as many CTAs on an SM.
 // RECORDS: the bodies of a simulator's records are staged all at once before the walk, where that leaves as many CTAs on an SM.
-template <bool RESET_ALL, bool OPT, bool AOS, bool WHOLE, bool RECORDS>
+// AHEAD: words per env that are staged of a body, one body ahead of the walk (kVectors: the rotation is loaded in the walk).
+template <bool RESET_ALL, bool OPT, bool AOS, bool WHOLE, bool RECORDS, int AHEAD>
 __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
     // EARLY: the decision is taken before the reward is known, where it can be, and the first warp forms the reward while the
@@ -1108,6 +1116,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     // 22.5 / - / 21.1, x 65536 83.6 / - / 76.6.
     constexpr bool EARLY = !RESET_ALL && !OPT && (!AOS || RECORDS);
     constexpr int kPitch = RECORDS ? kTile + 1 : kTile;
+    constexpr int kSlot = AHEAD > kPartials ? AHEAD : kPartials;         // words per env of a chain behind the rows
     const SkelDev &sk = P.sk;
     const int J = sk.J;
     const int D = 24 * J + 1;
@@ -1132,13 +1141,13 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     const int RS = 2 + 2 * J;
 
     // this chain's link records: global -> shared, private to the warp
-    float4 *links = reinterpret_cast<float4 *>(smem_raw + (WHOLE ? whole_floats(D_ext, C) : RECORDS ? records_floats(J, D_ext) : chain_floats(c1, D_ext, C))) + 2 * sk.link_start[c];
+    float4 *links = reinterpret_cast<float4 *>(smem_raw + (WHOLE ? whole_floats(D_ext, C) : RECORDS ? records_floats(J, D_ext) : chain_floats(c1, D_ext, C, kSlot))) + 2 * sk.link_start[c];
     for (int i = lane; i < 2 * len; i += 32) links[i] = __ldg(P.links + 2 * sk.link_start[c] + i);
     __syncwarp();
     // A chain's partial sums take the place of the body staged for it, or, of bodies staged all at once, that of its last one, a
     // leaf, whose state no other chain reads.
     const auto part_of = [&](int cc) {
-        return part + (RECORDS ? kRing * kPitch * ld_leaf(reinterpret_cast<const float4 *>(smem_raw + records_floats(J, D_ext)), sk, cc) : cc * kRing * kTile) + lane;
+        return part + (RECORDS ? kBody * kPitch * ld_leaf(reinterpret_cast<const float4 *>(smem_raw + records_floats(J, D_ext)), sk, cc) : cc * kSlot * kTile) + lane;
     };
     // this kernel is launched the same way: everything above reads only what the env's creation left in memory
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1160,8 +1169,8 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     if (!RESET_ALL) {
         uint64_t stream_policy;
         asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_policy));
-        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(part + (RECORDS ? 0 : c * kRing * kTile) + lane);
-        const auto body = [&](int b) { return lds_body<kPitch>(ring + (uint32_t)b * (kRing * kPitch * 4)); };       // (RECORDS)
+        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(part + (RECORDS ? 0 : c * kSlot * kTile) + lane);
+        const auto body = [&](int b) { return lds_body<kPitch>(ring + (uint32_t)b * (kBody * kPitch * 4)); };       // (RECORDS)
         if (RECORDS) {
             const int e0 = blockIdx.x * kTile;
             for (int i = c; i < kTile; i += C) sv.stage_record(P, min(e0 + i, P.N - 1), J, ring - 4u * lane, kPitch, i, lane, stream_policy);
@@ -1184,7 +1193,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         float alpha;
         lookup(cm, t1, frame, alpha);
         const float4 *r0 = P.frames + (size_t)IM_CHECKED(frame, P.n_rows) * RS;
-        if (!RECORDS) sv.stage_body(ld_link(links, first_own).b, ring, stream_policy);
+        if constexpr (AHEAD > 0) sv.template stage_body<AHEAD>(ld_link(links, first_own).b, ring, stream_policy);
         LinkRec L = ld_link(links, 0);
         KeyPair keys = ld_keys(r0, L.b);
 
@@ -1216,6 +1225,8 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             const LinkRec Lc = L;
             const int b = Lc.b;
             const bool own = Lc.flags & LINK_OWN;
+            SimBody sim;
+            if (own && AHEAD == kVectors) sim.q = sv.ld_quat(b);      // asked for before the interpolation math
             const KeyPair cur = keys;
             if (k + 1 < len) {                        // next joint's link and keyframe words in flight
                 L = ld_link(links, k + 1);
@@ -1226,12 +1237,16 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             joint_step<true>(r0, cur, alpha, cm.fps, Lc, k, s, ql, wl);
             if (OPT && k == 0) s.p = s.p + loop_shift(loop, cyc);    // completed cycles of a looped clip move the root
             if (own) {
-                SimBody sim;
                 if (RECORDS) sim = body(b);
-                else { cp_async_wait(); sim = lds_body(ring); }
-                if (!RECORDS && k + 1 < len) {                    // the next body of the chain is an own one too
-                    if (!AOS) (void)IM_CHECKED((4 * (uint32_t)L.b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
-                    sv.stage_body(L.b, ring, stream_policy);
+                if constexpr (AHEAD > 0) {
+                    cp_async_wait();
+                    SimBody staged = lds_body<kTile, AHEAD>(ring);
+                    if (AHEAD == kVectors) staged.q = sim.q;
+                    sim = staged;
+                    if (k + 1 < len) {                // the next body of the chain is an own one too
+                        if (!AOS) (void)IM_CHECKED((4 * (uint32_t)L.b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
+                        sv.template stage_body<AHEAD>(L.b, ring, stream_policy);
+                    }
                 }
                 sim.q = sanitize(sim.q, P.status);
                 // the root's "parent" is the identity: qa = (1, 0, 0, 0), wa = 0 on the chain that owns it
@@ -1477,28 +1492,28 @@ __global__ void debug_math_kernel(int op, int n, const float *__restrict__ in, f
 
 // Registers: the chain kernel has 96, so that four CTAs of five chains share an SM (64 for trees with more than eight
 // leaves, whose CTAs have up to 1024 threads); the role kernel 168 where every CTA has an SM of its own, else 96 (two).
-template <bool RESET_ALL, bool OPT, bool AOS>
+template <bool RESET_ALL, bool OPT, bool AOS, int AHEAD>
 __global__ void __maxnreg__(96) env_chain_kernel(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<RESET_ALL, OPT, AOS, false, false>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS, false, false, AHEAD>(P, smem_raw);
 }
 __global__ void __maxnreg__(96) env_chain_kernel_whole(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<false, false, false, true, false>(P, smem_raw);
+    env_chain_body<false, false, false, true, false, kBody>(P, smem_raw);
 }
 template <bool OPT>
 __global__ void __maxnreg__(96) env_chain_kernel_records(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<false, OPT, true, false, true>(P, smem_raw);
+    env_chain_body<false, OPT, true, false, true, 0>(P, smem_raw);
 }
-template <bool RESET_ALL, bool OPT, bool AOS>
+template <bool RESET_ALL, bool OPT, bool AOS, int AHEAD>
 __global__ void __launch_bounds__(1024, 1) env_chain_kernel_wide(const __grid_constant__ EnvKernelParams P)
 {
     extern __shared__ __align__(16) float smem_raw[];
-    env_chain_body<RESET_ALL, OPT, AOS, false, false>(P, smem_raw);
+    env_chain_body<RESET_ALL, OPT, AOS, false, false, AHEAD>(P, smem_raw);
 }
 template <bool RESET_ALL, bool OPT, bool AOS>
 __global__ void __maxnreg__(168) env_role_kernel_1(const __grid_constant__ EnvKernelParams P)
@@ -1540,8 +1555,13 @@ cudaError_t prepare_one()
 {
     cudaError_t e = allow_smem(env_role_kernel_1<RESET_ALL, OPT, AOS>);
     if (e == cudaSuccess) e = allow_smem(env_role_kernel_2<RESET_ALL, OPT, AOS>);
-    if (e == cudaSuccess) e = allow_smem(env_chain_kernel<RESET_ALL, OPT, AOS>);
-    if (e == cudaSuccess) e = allow_smem(env_chain_kernel_wide<RESET_ALL, OPT, AOS>);
+    constexpr int ahead = RESET_ALL ? 0 : kBody;
+    if (e == cudaSuccess) e = allow_smem(env_chain_kernel<RESET_ALL, OPT, AOS, ahead>);
+    if (e == cudaSuccess) e = allow_smem(env_chain_kernel_wide<RESET_ALL, OPT, AOS, ahead>);
+    if constexpr (!RESET_ALL && !AOS) {
+        if (e == cudaSuccess) e = allow_smem(env_chain_kernel<false, OPT, false, kVectors>);
+        if (e == cudaSuccess) e = allow_smem(env_chain_kernel_wide<false, OPT, false, kVectors>);
+    }
     return e;
 }
 
@@ -1602,19 +1622,36 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         if (OPT) kernel<<<tiles, block, smem, stream>>>(p);
         else launch_pdl(kernel, dim3(tiles), block, smem, stream, 0, p);
     } else {
-        void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS> : env_chain_kernel<RESET_ALL, OPT, AOS>;
+        // Shared memory for whole staged bodies costs trees of some sizes a CTA per SM.  Where that makes the tiles take more waves,
+        // the rotations stay out: us per step with whole bodies / their vectors alone, 26 bodies in 4 chains x 16384 envs (two waves /
+        // one) 44.0 / 30.5, x 30000 (3 / 2) 64.7 / 58.1, x 45000 (4 / 3) 85.4 / 84.5, x 65536 (5 / 4) 106.6 / 110.0; 31 in 10, where
+        // 64 registers spill more, x 20000 (3 / 2) 61.7 / 60.0, x 30000 (4 / 3) 85.7 / 91.2.  A reset stages nothing and, while that makes
+        // no further wave, asks for that memory all the same (31 in 10 x 16384, two waves with three CTAs per SM or two: 31.7 and 26.8;
+        // x 12000, one wave or two: 20.0 and 26.2).
+        constexpr int ahead = RESET_ALL ? 0 : kBody;
+        void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS, ahead> : env_chain_kernel<RESET_ALL, OPT, AOS, ahead>;
+        const size_t body_smem = smem_floats(p.sk.J, C, p.sk.n_links, extra, kBody) * sizeof(float);
+        size_t smem = body_smem;
+        const auto ctas = [&](size_t bytes) { return (unsigned)ctas_per_sm(bytes, C <= 8 ? 96 : 64, 32 * C); };
+        const auto waves = [&](size_t bytes) { const unsigned fit = n_sm * ctas(bytes); return (tiles + fit - 1) / fit; };
+        const unsigned few = waves(chain_smem), many = waves(body_smem);
         // (a reset of all envs keeps the halves: its warps have little to wait for, and 12000 envs x 15 bodies took 14.4 us with whole
         // rows, 12.7 without)
         const size_t whole = ((size_t)whole_floats(24 * p.sk.J + 1, C) + 8 * p.sk.n_links) * sizeof(float);
-        size_t smem = chain_smem;
-        if (!RESET_ALL && !OPT && !AOS && C <= 8 && ctas_per_sm(whole, 96, 32 * C) >= ctas_per_sm(chain_smem, 96, 32 * C)) {
+        if constexpr (RESET_ALL) {
+            if (few < many) smem = chain_smem;
+        } else if constexpr (AOS) {
+            const size_t records = ((size_t)records_floats(p.sk.J, 24 * p.sk.J + 1 + extra) + 8 * p.sk.n_links) * sizeof(float);
+            if (C <= 8 && staged_records(p) && ctas(records) >= ctas(body_smem)) {
+                kernel = env_chain_kernel_records<OPT>;
+                smem = records;
+            }
+        } else if (C <= 8 ? 4 * few <= 3 * many : 3 * few <= 2 * many) {
+            kernel = C > 8 ? env_chain_kernel_wide<false, OPT, false, kVectors> : env_chain_kernel<false, OPT, false, kVectors>;
+            smem = chain_smem;
+        } else if (!OPT && C <= 8 && ctas(whole) >= ctas(body_smem)) {
             kernel = env_chain_kernel_whole;
             smem = whole;
-        }
-        const size_t records = ((size_t)records_floats(p.sk.J, 24 * p.sk.J + 1 + extra) + 8 * p.sk.n_links) * sizeof(float);
-        if (AOS && C <= 8 && staged_records(p) && ctas_per_sm(records, 96, 32 * C) >= ctas_per_sm(chain_smem, 96, 32 * C)) {
-            kernel = env_chain_kernel_records<OPT>;
-            smem = records;
         }
         if (OPT) kernel<<<tiles, 32 * C, smem, stream>>>(p);
         else launch_pdl(kernel, dim3(tiles), dim3(32 * C), smem, stream, 0, p);
@@ -1625,7 +1662,7 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
 
 size_t env_kernel_smem_bytes(int J, int n_chains, int n_links, int extra_cols)
 {
-    return smem_floats(J, n_chains, n_links, extra_cols) * sizeof(float);
+    return smem_floats(J, n_chains, n_links, extra_cols, kPartials) * sizeof(float);
 }
 
 cudaError_t env_kernel_prepare()

@@ -280,3 +280,20 @@ def test_records_a_power_of_two_apart_equal_rows(n, skeleton, options):
         out.append(got)
     assert any(bool((fl & 1).any()) for fl in out[0][2::8])        # (in some step: with options the first two are grace steps)
     assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("leaves,bodies,n,case", [
+    (4, 26, 16384, dict(h_min=0.8)),
+    (3, 21, 20000, dict(reward=W.REWARD_FIG5, r_min=0.3, write_back=True)),
+    (5, 25, 16384, dict(options=True, h_min=0.8)),
+    (10, 31, 12000, dict(h_min=0.8)),
+    (10, 31, 12000, dict(options=True, r_min=0.1, reward=W.REWARD_ADD4)),
+])
+def test_trees_whose_rotations_are_not_staged(leaves, bodies, n, case, monkeypatch):
+    """Trees of which an SM holds a CTA more without them, at sizes where that saves a wave; half of the envs fit one wave."""
+    parents = np.asarray([-1] + [max(j - leaves, 0) for j in range(1, bodies)], np.int32)
+    offsets = np.random.default_rng(leaves).uniform(-0.3, 0.3, (bodies, 3)).astype(np.float32)
+    monkeypatch.setitem(globals(), "_tree", lambda _: dict(parents=parents, offsets=offsets, masses=None, J=bodies))
+    monkeypatch.setitem(globals(), "N", n)
+    monkeypatch.setitem(CASES, "tree", dict(case, leaves=leaves))
+    test_large_batch_equals_its_shards("tree", "humanoid15")
