@@ -39,8 +39,8 @@ __device__ __forceinline__ uint2 pack_bf16x4(float4 v)
 }
 
 constexpr int kTile = 32;          // envs per CTA
-constexpr int kVectors = 9;        // words per env of a staged body: position, linear and angular velocity ..
-constexpr int kBody = 13;          // .. and rotation
+constexpr int kBody = 13;          // words per env of a staged body: rotation, position, linear and angular velocity
+constexpr int kVectors = 9;        // without the rotation
 constexpr int kPartials = 9;       // pose, vel, ee_pos, ee_rot, body_pos, body_vel, weighted com difference (3)
 
 // The bounds-checked build (-DIM_DEBUG, a second library next to the regular one): every index the kernel forms
@@ -466,10 +466,11 @@ __device__ __forceinline__ SimBody lds_body(uint32_t a)
 {
     const auto w = [a](int i) { return lds32(a + (uint32_t)(4 * PITCH * i)); };
     SimBody s;
-    if constexpr (WORDS == kBody) s.q = {w(9), w(10), w(11), w(12)};
-    s.p = {w(0), w(1), w(2)};
-    s.v = {w(3), w(4), w(5)};
-    s.w = {w(6), w(7), w(8)};
+    constexpr int o = WORDS - kVectors;
+    if constexpr (WORDS == kBody) s.q = {w(0), w(1), w(2), w(3)};
+    s.p = {w(o), w(o + 1), w(o + 2)};
+    s.v = {w(o + 3), w(o + 4), w(o + 5)};
+    s.w = {w(o + 6), w(o + 7), w(o + 8)};
     return s;
 }
 
@@ -513,27 +514,28 @@ struct SimView {
         const uint32_t o = 3 * (uint32_t)b * st + e;
         return {__ldcs(base + o), __ldcs(base + o + st), __ldcs(base + o + 2 * st)};
     }
-    // This env's state of body b, or its vectors alone, to shared memory, asynchronously: component i (position, velocities,
-    // rotation) to the word at dst + 128 i bytes.  Every lane copies and later reads its own words.  The chain kernel, whose
+    // This env's state of body b, or its vectors alone, to shared memory, asynchronously: component i (rotation, position,
+    // velocities) to the word at dst + 128 i bytes.  Every lane copies and later reads its own words.  The chain kernel, whose
     // warps are bound by the latency of what they load (20 of them on an SM), so asks for a body while it walks the one before, at
     // the price of no registers: us per step with the loads in the walk itself / staged a body ahead, 15 bodies x 16384 envs 20.6 /
     // 18.8, x 65536 76.2 / 66.5; 24 bodies x 16384 28.7 / 27.6, x 65536 102.0 / 96.1; spilled bytes 48 / 0.
     template <int WORDS>
     __device__ __forceinline__ void stage_body(int b, uint32_t dst, uint64_t policy) const
     {
+        constexpr int kRot = WORDS - kVectors;           // words of the rotation
         if (AOS) {
             const float *v[3] = {pos + (long long)b * bs_pos, lin + (long long)b * bs_lin, ang + (long long)b * bs_ang}, *q = quat + (long long)b * bs_quat;
 #pragma unroll
-            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * i, v[i / 3] + i % 3, policy);
+            for (int i = 0; i < kRot; ++i) cp_async_word(dst + 128 * i, q + i, policy);
 #pragma unroll
-            for (int i = kVectors; i < WORDS; ++i) cp_async_word(dst + 128 * i, q + (i - kVectors), policy);
+            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * (kRot + i), v[i / 3] + i % 3, policy);
         } else {
             const uint32_t o = 4 * (uint32_t)b * st + e, o3 = 3 * (uint32_t)b * st + e;
             const float *v[3] = {pos, lin, ang};
 #pragma unroll
-            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * i, v[i / 3] + (o3 + (i % 3) * st), policy);
+            for (int i = 0; i < kRot; ++i) cp_async_word(dst + 128 * i, quat + (o + i * st), policy);
 #pragma unroll
-            for (int i = kVectors; i < WORDS; ++i) cp_async_word(dst + 128 * i, quat + (o + (i - kVectors) * st), policy);
+            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * (kRot + i), v[i / 3] + (o3 + (i % 3) * st), policy);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
@@ -548,7 +550,7 @@ struct SimView {
         const int bs[4] = {P.aos_body_stride[1], P.aos_body_stride[0], P.aos_body_stride[2], P.aos_body_stride[3]};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int n = k == 0 ? 4 : 3, off = k == 0 ? kVectors : 3 * k - 3;
+            const int n = k == 0 ? 4 : 3, off = k == 0 ? 0 : 1 + 3 * k;
             for (int i = lane; i < n * J; i += 32) {
                 const int b = i / n, c = i - n * b;
                 cp_async_word(dst + 4u * ((uint32_t)(kBody * b + off + c) * pitch + (uint32_t)col), a[k] + (long long)b * bs[k] + c, policy);
@@ -1625,8 +1627,8 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         // Shared memory for whole staged bodies costs trees of some sizes a CTA per SM.  Where that makes the tiles take more waves,
         // the rotations stay out: us per step with whole bodies / their vectors alone, 26 bodies in 4 chains x 16384 envs (two waves /
         // one) 44.0 / 30.5, x 30000 (3 / 2) 64.7 / 58.1, x 45000 (4 / 3) 85.4 / 84.5, x 65536 (5 / 4) 106.6 / 110.0; 31 in 10, where
-        // 64 registers spill more, x 20000 (3 / 2) 61.7 / 60.0, x 30000 (4 / 3) 85.7 / 91.2.  A reset stages nothing and, while that makes
-        // no further wave, asks for that memory all the same (31 in 10 x 16384, two waves with three CTAs per SM or two: 31.7 and 26.8;
+        // 64 registers spill more, x 20000 (3 / 2) 61.7 / 60.0, x 30000 (4 / 3) 85.7 / 91.2.  A reset stages nothing, but where fewer
+        // CTAs make no further wave it asks for that memory all the same (31 in 10 x 16384, two waves with three CTAs per SM or two: 31.7 and 26.8;
         // x 12000, one wave or two: 20.0 and 26.2).
         constexpr int ahead = RESET_ALL ? 0 : kBody;
         void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS, ahead> : env_chain_kernel<RESET_ALL, OPT, AOS, ahead>;
@@ -1639,7 +1641,7 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         // rows, 12.7 without)
         const size_t whole = ((size_t)whole_floats(24 * p.sk.J + 1, C) + 8 * p.sk.n_links) * sizeof(float);
         if constexpr (RESET_ALL) {
-            if (few < many) smem = chain_smem;
+            if (few < many || ctas(chain_smem) == ctas(body_smem)) smem = chain_smem;
         } else if constexpr (AOS) {
             const size_t records = ((size_t)records_floats(p.sk.J, 24 * p.sk.J + 1 + extra) + 8 * p.sk.n_links) * sizeof(float);
             if (C <= 8 && staged_records(p) && ctas(records) >= ctas(body_smem)) {
