@@ -514,29 +514,23 @@ struct SimView {
         const uint32_t o = 3 * (uint32_t)b * st + e;
         return {__ldcs(base + o), __ldcs(base + o + st), __ldcs(base + o + 2 * st)};
     }
-    // This env's state of body b, or its vectors alone, to shared memory, asynchronously: component i (rotation, position,
+    // Rows: this env's state of body b, or its vectors alone, to shared memory, asynchronously: component i (rotation, position,
     // velocities) to the word at dst + 128 i bytes.  Every lane copies and later reads its own words.  The chain kernel, whose
     // warps are bound by the latency of what they load (20 of them on an SM), so asks for a body while it walks the one before, at
     // the price of no registers: us per step with the loads in the walk itself / staged a body ahead, 15 bodies x 16384 envs 20.6 /
-    // 18.8, x 65536 76.2 / 66.5; 24 bodies x 16384 28.7 / 27.6, x 65536 102.0 / 96.1; spilled bytes 48 / 0.
+    // 18.8, x 65536 76.2 / 66.5; 24 bodies x 16384 28.7 / 27.6, x 65536 102.0 / 96.1; spilled bytes 48 / 0.  Records
+    // are read in the walk itself: the words of a body lie together, and the first load of them brings the others into L1 (24 bodies x
+    // 12000 envs, 25 records of 13 words 30.2 us, staged ahead 35.4; of 3, 4 and 6 words 36.8 / 40.7).
     template <int WORDS>
     __device__ __forceinline__ void stage_body(int b, uint32_t dst, uint64_t policy) const
     {
         constexpr int kRot = WORDS - kVectors;           // words of the rotation
-        if (AOS) {
-            const float *v[3] = {pos + (long long)b * bs_pos, lin + (long long)b * bs_lin, ang + (long long)b * bs_ang}, *q = quat + (long long)b * bs_quat;
+        const uint32_t o = 4 * (uint32_t)b * st + e, o3 = 3 * (uint32_t)b * st + e;
+        const float *v[3] = {pos, lin, ang};
 #pragma unroll
-            for (int i = 0; i < kRot; ++i) cp_async_word(dst + 128 * i, q + i, policy);
+        for (int i = 0; i < kRot; ++i) cp_async_word(dst + 128 * i, quat + (o + i * st), policy);
 #pragma unroll
-            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * (kRot + i), v[i / 3] + i % 3, policy);
-        } else {
-            const uint32_t o = 4 * (uint32_t)b * st + e, o3 = 3 * (uint32_t)b * st + e;
-            const float *v[3] = {pos, lin, ang};
-#pragma unroll
-            for (int i = 0; i < kRot; ++i) cp_async_word(dst + 128 * i, quat + (o + i * st), policy);
-#pragma unroll
-            for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * (kRot + i), v[i / 3] + (o3 + (i % 3) * st), policy);
-        }
+        for (int i = 0; i < kVectors; ++i) cp_async_word(dst + 128 * (kRot + i), v[i / 3] + (o3 + (i % 3) * st), policy);
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     // Records: the whole state of env `src` of the batch to column `col` of the staged bodies (component i of body b: the word
@@ -1107,7 +1101,8 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
 // observation); envs that use none run the instantiation without them.
 // WHOLE: the whole row is staged at once (both halves side by side), where that leaves as many CTAs on an SM.
 // RECORDS: the bodies of a simulator's records are staged all at once before the walk, where that leaves as many CTAs on an SM.
-// AHEAD: words per env that are staged of a body, one body ahead of the walk (kVectors: the rotation is loaded in the walk).
+// AHEAD: words per env that are staged of a body, one body ahead of the walk (kVectors: the rotation is loaded in the walk; 0, from
+// records in place: all of it).
 template <bool RESET_ALL, bool OPT, bool AOS, bool WHOLE, bool RECORDS, int AHEAD>
 __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *smem_raw)
 {
@@ -1228,7 +1223,10 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             const int b = Lc.b;
             const bool own = Lc.flags & LINK_OWN;
             SimBody sim;
-            if (own && AHEAD == kVectors) sim.q = sv.ld_quat(b);      // asked for before the interpolation math
+            if (own && !RECORDS && AHEAD < kBody) {   // asked for before the interpolation math
+                if (AHEAD == 0) sim = sv.ld_body(b);
+                else sim.q = sv.ld_quat(b);
+            }
             const KeyPair cur = keys;
             if (k + 1 < len) {                        // next joint's link and keyframe words in flight
                 L = ld_link(links, k + 1);
@@ -1246,7 +1244,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
                     if (AHEAD == kVectors) staged.q = sim.q;
                     sim = staged;
                     if (k + 1 < len) {                // the next body of the chain is an own one too
-                        if (!AOS) (void)IM_CHECKED((4 * (uint32_t)L.b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
+                        (void)IM_CHECKED((4 * (uint32_t)L.b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
                         sv.template stage_body<AHEAD>(L.b, ring, stream_policy);
                     }
                 }
@@ -1557,7 +1555,7 @@ cudaError_t prepare_one()
 {
     cudaError_t e = allow_smem(env_role_kernel_1<RESET_ALL, OPT, AOS>);
     if (e == cudaSuccess) e = allow_smem(env_role_kernel_2<RESET_ALL, OPT, AOS>);
-    constexpr int ahead = RESET_ALL ? 0 : kBody;
+    constexpr int ahead = RESET_ALL || AOS ? 0 : kBody;
     if (e == cudaSuccess) e = allow_smem(env_chain_kernel<RESET_ALL, OPT, AOS, ahead>);
     if (e == cudaSuccess) e = allow_smem(env_chain_kernel_wide<RESET_ALL, OPT, AOS, ahead>);
     if constexpr (!RESET_ALL && !AOS) {
@@ -1627,10 +1625,11 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         // Shared memory for whole staged bodies costs trees of some sizes a CTA per SM.  Where that makes the tiles take more waves,
         // the rotations stay out: us per step with whole bodies / their vectors alone, 26 bodies in 4 chains x 16384 envs (two waves /
         // one) 44.0 / 30.5, x 30000 (3 / 2) 64.7 / 58.1, x 45000 (4 / 3) 85.4 / 84.5, x 65536 (5 / 4) 106.6 / 110.0; 31 in 10, where
-        // 64 registers spill more, x 20000 (3 / 2) 61.7 / 60.0, x 30000 (4 / 3) 85.7 / 91.2.  A reset stages nothing, but where fewer
-        // CTAs make no further wave it asks for that memory all the same (31 in 10 x 16384, two waves with three CTAs per SM or two: 31.7 and 26.8;
-        // x 12000, one wave or two: 20.0 and 26.2).
-        constexpr int ahead = RESET_ALL ? 0 : kBody;
+        // 64 registers spill more, x 20000 (3 / 2) 61.7 / 60.0, x 30000 (4 / 3) 85.7 / 91.2.  What stages nothing asks for
+        // that memory all the same where fewer CTAs make no further wave: a reset of 31 in 10 x 16384, two waves with three CTAs per SM or
+        // two 31.7 and 26.8 (x 12000, one wave or two: 20.0 and 26.2); 32 records of 3, 4 and 6 words, 20 bodies in 4 chains x 30000, two
+        // waves with five or four 89.4 and 76.5.
+        constexpr int ahead = RESET_ALL || AOS ? 0 : kBody;
         void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS, ahead> : env_chain_kernel<RESET_ALL, OPT, AOS, ahead>;
         const size_t body_smem = smem_floats(p.sk.J, C, p.sk.n_links, extra, kBody) * sizeof(float);
         size_t smem = body_smem;
@@ -1640,8 +1639,8 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         // (a reset of all envs keeps the halves: its warps have little to wait for, and 12000 envs x 15 bodies took 14.4 us with whole
         // rows, 12.7 without)
         const size_t whole = ((size_t)whole_floats(24 * p.sk.J + 1, C) + 8 * p.sk.n_links) * sizeof(float);
+        if (ahead == 0 && (few < many || ctas(chain_smem) == ctas(body_smem))) smem = chain_smem;
         if constexpr (RESET_ALL) {
-            if (few < many || ctas(chain_smem) == ctas(body_smem)) smem = chain_smem;
         } else if constexpr (AOS) {
             const size_t records = ((size_t)records_floats(p.sk.J, 24 * p.sk.J + 1 + extra) + 8 * p.sk.n_links) * sizeof(float);
             if (C <= 8 && staged_records(p) && ctas(records) >= ctas(body_smem)) {
