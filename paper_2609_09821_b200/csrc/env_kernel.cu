@@ -1371,8 +1371,9 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
             if (15 * J + 2 < c1) row1[15 * J + 2] = tp.y;
         }
     }
-    // Rows leave by all warps, or (EARLY) by all but the first, which forms the reward meanwhile
-    const bool apart = EARLY && C > 1;
+    // Rows leave by all warps, or (EARLY) by all but the first, which forms the reward meanwhile: not with two chains, where one warp
+    // would be left for the rows (24 bodies x 65536 envs 124.5 us, 120.0 by both)
+    const bool apart = EARLY && C > 2;
     const int copier = apart ? c - 1 : c, n_copiers = apart ? C - 1 : C;
     const auto finish = [&] {
         r = reward_of<kPitch>(P, part_of, C, term);

@@ -297,3 +297,9 @@ def test_trees_whose_rotations_are_not_staged(leaves, bodies, n, case, monkeypat
     monkeypatch.setitem(globals(), "N", n)
     monkeypatch.setitem(CASES, "tree", dict(case, leaves=leaves))
     test_large_batch_equals_its_shards("tree", "humanoid15")
+
+
+@pytest.mark.parametrize("case", [dict(h_min=0.8), dict(reward=W.REWARD_FIG5, r_min=0.3, write_back=True), dict(aos=True, h_min=0.8)])
+def test_trees_with_two_chains(case, monkeypatch):
+    monkeypatch.setitem(CASES, "two_chains", dict(case, leaves=2))
+    test_large_batch_equals_its_shards("two_chains", "humanoid15")
