@@ -303,3 +303,50 @@ def test_trees_whose_rotations_are_not_staged(leaves, bodies, n, case, monkeypat
 def test_trees_with_two_chains(case, monkeypatch):
     monkeypatch.setitem(CASES, "two_chains", dict(case, leaves=2))
     test_large_batch_equals_its_shards("two_chains", "humanoid15")
+
+
+@pytest.mark.parametrize("form", ["plain", "reward", "extension", "rotations_only", "positions_only"])
+@pytest.mark.parametrize("skeleton", ["humanoid15", "smpl24"])
+@pytest.mark.parametrize("n", [41, 4700, 4801, N - 95])
+def test_staged_records_equal_rows_in_every_form(n, skeleton, form):
+    """Staged records of a step that leaves the states alone (no barrier before the decision), of one whose reward ends episodes, with
+    an extension too wide to stage, and where the envs of one of the arrays alone lie a multiple of 256 bytes apart."""
+    import torch
+    from paper_2609_09821_b200 import binding as B
+    skel = W.make_skeleton(skeleton, 1)
+    J = skel["J"]
+    lib = W.make_clip_library(J, 4, (20, 40), 30.0, 1)
+    sk = B.Skeleton(skel["parents"], skel["offsets"], skel["masses"])
+    clips = B.Clips(sk, lib["n_frames"], lib["fps"], lib["root_pos"], lib["local_quat"])
+    reward, extension = form == "reward", form == "extension"
+    extra = 7 * 9 * sk.n_ee + 900 if extension else 0
+    g = torch.Generator("cuda").manual_seed(n)
+    sims = (torch.randn(3, 13 * J, (n + 3) // 4 * 4, device="cuda", generator=g) * 0.3)[:, :, :n]
+    sims[:, 2] += 0.9
+    prev = torch.randn(n, 900, device="cuda", generator=g)
+    out = []
+    for records in (False, True):
+        env = B.Env(sk, clips, B.make_env_config(n, 1 / 30, 5, W.REWARD_FIG5 if reward else W.REWARD_MULT, 0.3 if reward else 0.8,
+                                                 B.padded_ld(24 * J + 1 + extra), r_min=0.3 if reward else -np.inf))
+        if extension:
+            env.set_obs_extension(8, prev)
+        obs, rew, fl, terms = env.new_obs(), torch.empty(n, device="cuda"), torch.empty(n, dtype=torch.uint8, device="cuda"), torch.empty(7, n, device="cuda")
+        env.reset_all(obs, 0)
+        got = []
+        for s in range(sims.shape[0]):
+            if records:
+                rec = []
+                for i, (a, b) in enumerate(((0, 3), (3, 7), (7, 10), (10, 13))):
+                    w, crowded = b - a, i == dict(positions_only=0, rotations_only=1).get(form, i)
+                    wide = torch.zeros(n, (w * J + 63) // 64 * 64 + (0 if crowded else 4), device="cuda")
+                    view = wide[:, :w * J].unflatten(1, (J, w))
+                    view.copy_(sims[s, a * J:b * J].reshape(J, w, n).permute(2, 0, 1))
+                    rec.append(view)
+                env.step_aos(s + 1, *rec, obs, rew, fl, terms)
+            else:
+                env.step(s + 1, torch.empty_strided((13 * J, n), sims[s].stride(), device="cuda").copy_(sims[s]), obs, rew, fl, terms)
+            got += [obs.clone(), rew.clone(), fl.clone(), terms.clone()] + list(env.get_state())
+        assert env.device_status() == 0
+        out.append(got)
+    assert any(bool((fl & 1).any()) for fl in out[0][2::7])
+    assert all(torch.equal(a, b) for a, b in zip(*out))
