@@ -539,6 +539,7 @@ struct SimView {
     static __device__ __forceinline__ void stage_record(const EnvKernelParams &P, int src, int J, uint32_t dst, uint32_t pitch, int col, int lane,
                                                         uint64_t policy)
     {
+        (void)IM_CHECKED(src, P.N);
         const float *a[4] = {P.quat + (long long)src * P.aos_env_stride[1], P.pos + (long long)src * P.aos_env_stride[0],
                              P.lin + (long long)src * P.aos_env_stride[2], P.ang + (long long)src * P.aos_env_stride[3]};
         const int bs[4] = {P.aos_body_stride[1], P.aos_body_stride[0], P.aos_body_stride[2], P.aos_body_stride[3]};
@@ -547,7 +548,8 @@ struct SimView {
             const int n = k == 0 ? 4 : 3, off = k == 0 ? 0 : 1 + 3 * k;
             for (int i = lane; i < n * J; i += 32) {
                 const int b = i / n, c = i - n * b;
-                cp_async_word(dst + 4u * ((uint32_t)(kBody * b + off + c) * pitch + (uint32_t)col), a[k] + (long long)b * bs[k] + c, policy);
+                const uint32_t word = (uint32_t)(kBody * IM_CHECKED(b, J) + off + c) * pitch + (uint32_t)col;
+                cp_async_word(dst + 4u * IM_CHECKED(word, (uint32_t)(J * kBody) * pitch), a[k] + (long long)b * bs[k] + c, policy);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -1144,7 +1146,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
     // A chain's partial sums take the place of the body staged for it, or, of bodies staged all at once, that of its last one, a
     // leaf, whose state no other chain reads.
     const auto part_of = [&](int cc) {
-        return part + (RECORDS ? kBody * kPitch * ld_leaf(reinterpret_cast<const float4 *>(smem_raw + records_floats(J, D_ext)), sk, cc) : cc * kSlot * kTile) + lane;
+        return part + (RECORDS ? kBody * kPitch * (int)IM_CHECKED(ld_leaf(reinterpret_cast<const float4 *>(smem_raw + records_floats(J, D_ext)), sk, cc), J) : cc * kSlot * kTile) + lane;
     };
     // this kernel is launched the same way: everything above reads only what the env's creation left in memory
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1190,7 +1192,11 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
         float alpha;
         lookup(cm, t1, frame, alpha);
         const float4 *r0 = P.frames + (size_t)IM_CHECKED(frame, P.n_rows) * RS;
-        if constexpr (AHEAD > 0) sv.template stage_body<AHEAD>(ld_link(links, first_own).b, ring, stream_policy);
+        const auto stage = [&](int b) {
+            (void)IM_CHECKED((4 * (uint32_t)b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
+            if constexpr (AHEAD > 0) sv.template stage_body<AHEAD>(b, ring, stream_policy);
+        };
+        if (AHEAD > 0) stage(ld_link(links, first_own).b);
         LinkRec L = ld_link(links, 0);
         KeyPair keys = ld_keys(r0, L.b);
 
@@ -1243,10 +1249,7 @@ __device__ __forceinline__ void env_chain_body(const EnvKernelParams &P, float *
                     SimBody staged = lds_body<kTile, AHEAD>(ring);
                     if (AHEAD == kVectors) staged.q = sim.q;
                     sim = staged;
-                    if (k + 1 < len) {                // the next body of the chain is an own one too
-                        (void)IM_CHECKED((4 * (uint32_t)L.b + 3) * sv.st + sv.e, 4u * (uint32_t)J * sv.st);
-                        sv.template stage_body<AHEAD>(L.b, ring, stream_policy);
-                    }
+                    if (k + 1 < len) stage(L.b);      // the next body of the chain is an own one too
                 }
                 sim.q = sanitize(sim.q, P.status);
                 // the root's "parent" is the identity: qa = (1, 0, 0, 0), wa = 0 on the chain that owns it

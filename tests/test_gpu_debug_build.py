@@ -22,6 +22,10 @@ CASES = [
     "tests/test_gpu_edge_cases.py::test_skeletons_with_more_than_eight_leaves",
     "tests/test_gpu_edge_cases.py::test_two_keyframe_clips_reset_every_step",
     "tests/test_gpu_edge_cases.py::test_training_summaries_accumulate_on_the_device",
+    # batches large enough for the chain kernel, with whole bodies and with vectors staged ahead, and staged records
+    "tests/test_gpu_env_kernels.py::test_large_batch_equals_its_shards",
+    "tests/test_gpu_env_kernels.py::test_trees_whose_rotations_are_not_staged",
+    "tests/test_gpu_env_kernels.py::test_staged_records_equal_rows_in_every_form",
 ]
 
 
