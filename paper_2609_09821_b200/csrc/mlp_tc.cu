@@ -275,8 +275,8 @@ struct SmemPlan {
     static constexpr int kTmemCols = 2 * kAccStride;
     static constexpr int kBarBytes = 256;
     static constexpr int kMaxStages = 8;
-    // hidden layers: eight staging slabs for the TMA stores, shared out over the epilogue warps
-    // (backward epilogue: two per warp and two more for the ReLU mask boxes)
+    // hidden layers: eight staging slabs for the TMA stores, shared out over the epilogue warps (kBwdBoxes: two per warp and two
+    // more for the ReLU mask boxes)
     static constexpr __host__ __device__ int hidden_epi_bytes(int epi = kFwd) { return (epi == kBwdBoxes ? 4 * 4 : 8) * kEpiSlabBytes; }
     // head: [2 accumulators][mean, action][128 rows][A] floats laid out as in global memory,
     // partial sums of z^2 [2][4][128], band counters [2][4]
@@ -661,10 +661,10 @@ __device__ __forceinline__ void bits_chunk(const GemmParams &P, uint32_t t_addr,
 // into a 128B-swizzled slab in shared memory and hands the slab to a TMA store.
 constexpr __host__ __device__ int hidden_depth(int block_n, bool mn, int epi) { return block_n < 256 && !mn && !is_bwd(epi) ? 2 : 1; }
 
-// Kernel parameters of the second net of a DUAL launch (m: mask, as map_m).
+// Kernel parameters of the second net of a DUAL launch (its ReLU mask comes as bits only).
 struct NoMaps {};
 struct DualMaps {
-    CUtensorMap a, b, c, m;
+    CUtensorMap a, b, c;
 };
 template <bool DUAL>
 using SecondNet = std::conditional_t<DUAL, DualMaps, NoMaps>;
@@ -683,8 +683,8 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, EPI), 1) linear_tc
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_per_slice = ((P.M + BLOCK_M - 1) / BLOCK_M) * P.n_tiles_n;
     const int n_tiles = tiles_per_slice * (MN ? P.n_batches : 1) * (DUAL ? 2 : 1);
-    const CUtensorMap *map_c2 = &map_c, *map_m2 = &map_m;
-    if constexpr (DUAL) { map_c2 = &second.c; map_m2 = &second.m; }
+    const CUtensorMap *map_c2 = &map_c;
+    if constexpr (DUAL) map_c2 = &second.c;
     pipe_init<Plan>(p, hidden_epi_warps(BLOCK_N, MN, EPI));
     const uint32_t tmem_base = *p.tmem_slot;
     dep_release();
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, EPI), 1) linear_tc
         uint4 mk[8];
         if (masked && (int)blockIdx.x < n_tiles && lane == 0) {
             const TileAt at = tile_at<MN, DUAL>(P, blockIdx.x, tiles_per_slice);
-            mask_issue(at.second ? map_m2 : &map_m, mslabs, &mbar[0], at.n * BLOCK_N, at.m * BLOCK_M + quad * 32);
+            mask_issue(&map_m, mslabs, &mbar[0], at.n * BLOCK_N, at.m * BLOCK_M + quad * 32);
         }
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
             const TileAt at = tile_at<MN, DUAL>(P, tile, tiles_per_slice);
@@ -746,10 +746,10 @@ __global__ void __launch_bounds__(hidden_threads(BLOCK_N, MN, EPI), 1) linear_tc
                         if (masked) {
                             if (lane == 0) {
                                 uint8_t *nslab = mslabs + ((ci + 1u) & 1u) * kEpiSlabBytes;
-                                if (c0 + 64 < BLOCK_N) mask_issue(at.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], n0 + c0 + 64, m0 + quad * 32);
+                                if (c0 + 64 < BLOCK_N) mask_issue(&map_m, nslab, &mbar[(ci + 1u) & 1u], n0 + c0 + 64, m0 + quad * 32);
                                 else if (tile + (int)gridDim.x < n_tiles) {
                                     const TileAt next = tile_at<MN, DUAL>(P, tile + (int)gridDim.x, tiles_per_slice);
-                                    mask_issue(next.second ? map_m2 : &map_m, nslab, &mbar[(ci + 1u) & 1u], next.n * BLOCK_N,
+                                    mask_issue(&map_m, nslab, &mbar[(ci + 1u) & 1u], next.n * BLOCK_N,
                                                next.m * BLOCK_M + quad * 32);
                                 }
                             }
@@ -902,8 +902,8 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
     const int tiles_m = (P.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M);
     const int tiles_per_slice = tiles_m * P.n_tiles_n;               // 256 x 256 tiles
     const int n_tiles = tiles_per_slice * (MN ? P.n_batches : 1) * (DUAL ? 2 : 1);
-    const CUtensorMap *map_a2 = &map_a, *map_b2 = &map_b, *map_c2 = &map_c, *map_m2 = &map_m;
-    if constexpr (DUAL) { map_a2 = &second.a; map_b2 = &second.b; map_c2 = &second.c; map_m2 = &second.m; }
+    const CUtensorMap *map_a2 = &map_a, *map_b2 = &map_b, *map_c2 = &map_c;
+    if constexpr (DUAL) { map_a2 = &second.a; map_b2 = &second.b; map_c2 = &second.c; }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -1096,7 +1096,7 @@ linear_tc_hidden_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __
                 const int t2 = pair + (int)(j >> 1) * n_pairs;
                 if (t2 >= n_tiles) return;
                 const TileAt at = tile_at<MN, DUAL>(P, t2, tiles_per_slice);
-                mask_issue(at.second ? map_m2 : &map_m, ring + (j % kPairRing) * kEpiSlabBytes, &mbar[j % kPairRing],
+                mask_issue(&map_m, ring + (j % kPairRing) * kEpiSlabBytes, &mbar[j % kPairRing],
                            at.n * 256 + (2 * half + (int)(j & 1u)) * 64, at.m * 2 * BLOCK_M + (int)rank * BLOCK_M + quad * 32);
             };
             if (masked && lane == 0 && !*abort_flag) issue_mask(0u);
@@ -1487,7 +1487,7 @@ cudaError_t launch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParams 
     const int tiles = ((gp.M + BLOCK_M - 1) / BLOCK_M) * gp.n_tiles_n * gp.n_batches * (DUAL ? 2 : 1);
     const int grid = tiles < n_sm ? tiles : n_sm;
     SecondNet<DUAL> second;
-    if constexpr (DUAL) second = {L2->map_a, L2->map_b, L2->map_c, L2->map_m};
+    if constexpr (DUAL) second = {L2->map_a, L2->map_b, L2->map_c};
     const cudaError_t le = launch_pdl(kernel, dim3(grid), dim3(hidden_threads(BLOCK_N, MN, EPI)), smem, stream, 0, L.map_a, L.map_b, L.map_c,
                                       L.map_m, gp, second);
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -1505,7 +1505,7 @@ cudaError_t launch_hidden_pair(const TcLayer &L, const TcLayer *L2, const GemmPa
     const int tiles = ((gp.M + 2 * BLOCK_M - 1) / (2 * BLOCK_M)) * gp.n_tiles_n * gp.n_batches * (DUAL ? 2 : 1);
     const int pairs = tiles < n_sm / 2 ? tiles : n_sm / 2;
     SecondNet<DUAL> second;
-    if constexpr (DUAL) second = {L2->map_a, MN ? L2->map_b : L2->map_b2, L2->map_c, L2->map_m};
+    if constexpr (DUAL) second = {L2->map_a, MN ? L2->map_b : L2->map_b2, L2->map_c};
     const cudaError_t le = launch_pdl(kernel, dim3(2 * pairs), dim3(pair_threads(EPI)), pair_smem_bytes(EPI), stream, 0, L.map_a,
                                       MN ? L.map_b : L.map_b2, L.map_c, L.map_m, gp, second);
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -1575,8 +1575,7 @@ cudaError_t dispatch_hidden(const TcLayer &L, const TcLayer *L2, const GemmParam
     const bool pairs = L.block_n == 256 && (force_pairs || (pair_tiles >= n_sm && gp.K_blocks >= 8) || (bwd && pair_tiles >= n_sm / 2));
     if (!bwd) return gp.bits_out ? dispatch_width<kFwdBits, DUAL>(L, L2, gp, n_sm, pairs, stream) : dispatch_width<kFwd, DUAL>(L, L2, gp, n_sm, pairs, stream);
     if (gp.bits_in) return dispatch_width<kBwdBits, DUAL>(L, L2, gp, n_sm, pairs, stream);
-    // (a common launch for two nets has its masks as bits)
-    if constexpr (DUAL) return cudaErrorInvalidValue;
+    if constexpr (DUAL) return cudaErrorInvalidValue;              // (refused by tc_gemm)
     else return dispatch_width<kBwdBoxes, false>(L, L2, gp, n_sm, pairs, stream);
 }
 
@@ -1796,7 +1795,7 @@ im_status tc_policy_value_forward(im_policy *a, im_policy *c, uint32_t step, int
         if (l == 0) L2.map_a = L.map_a;                          // one copy of the observations serves both
         set_layer(gp, L);
         gp.bias2 = L2.d_bias; gp.N2 = L2.N; gp.mean2 = value_out; gp.status2 = c->d_status;
-        const cudaError_t e = last ? dispatch_head<true>(L, gp, n_sm, {L2.map_a, L2.map_b_head(L.block_n), L2.map_a, L2.map_a}, a->stream)
+        const cudaError_t e = last ? dispatch_head<true>(L, gp, n_sm, {L2.map_a, L2.map_b_head(L.block_n), L2.map_a}, a->stream)
                                    : dispatch_hidden<true>(L, &L2, gp, n_sm, false, a->stream);
         if (e != cudaSuccess) return IM_ERR_CUDA;
     }
@@ -1832,12 +1831,16 @@ bool layer_of(TcLayer &L, const GemmOperands &o, int M, int N, int K, int block_
 
 // C[M][N] = act(A[M][K] B[N][K]^T + bias) on the hidden-layer kernels, operands anywhere in device
 // memory: the tensor maps are encoded for this call and travel as kernel parameters.  y: a second product of the same
-// sizes in the same launch (both with a mask, or with column sums, or neither), or null.
+// sizes in the same launch, or null: two forward products (both with bits_out or neither), or two backward products with
+// their masks as bits (both with column sums or neither).
 im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, int K, bool relu, int ld_partial, uint32_t *status, uint32_t *status2,
                   cudaStream_t stream)
 {
     const int n_sm = device_sm_count();          // 0 unless the current device is an sm_100 part
     if (n_sm <= 0 || !encode_tiled_fn()) return IM_ERR_UNSUPPORTED;
+    const bool bwd = x.mask || x.colsum_partial || x.bits_in;
+    if (y && ((bwd && !x.bits_in) || y->mask || !x.bits_in != !y->bits_in || !x.bits_out != !y->bits_out || !x.colsum_partial != !y->colsum_partial))
+        return IM_ERR_INVALID_ARG;
     TcLayer L, L2;
     const int block_n = pick_block_n((M + BLOCK_M - 1) / BLOCK_M * (y ? 2 : 1), N, false, n_sm);
     if (!layer_of(L, x, M, N, K, block_n) || (y && !layer_of(L2, *y, M, N, K, block_n))) return IM_ERR_CUDA;
@@ -1846,7 +1849,7 @@ im_status tc_gemm(const GemmOperands &x, const GemmOperands *y, int M, int N, in
     gp.M = M; gp.N = N; gp.K_blocks = K / BLOCK_K; gp.n_tiles_n = L.n_tiles_n; gp.bias = x.bias;
     gp.act_floor = relu ? 0.0f : -INFINITY;
     gp.n_batches = 1;
-    if (x.mask || x.colsum_partial || x.bits_in) gp.bias = nullptr;     // the backward product has no bias: its epilogue skips the add
+    if (bwd) gp.bias = nullptr;     // the backward product has no bias: its epilogue skips the add
     else if (y) gp.bias2 = y->bias;
     gp.mask = static_cast<const __nv_bfloat16 *>(x.mask);
     gp.colsum_partial = x.colsum_partial; gp.ld_partial = ld_partial;
@@ -1946,7 +1949,7 @@ im_status tc_gemm_head(const GemmOperands &x, const GemmOperands *y, int M, int 
     if (!make_map(&second.a, y->A, (uint64_t)M, (uint64_t)K, (uint64_t)y->lda, BLOCK_M) ||
         !make_map(&second.b, y->B, (uint64_t)((N2 + 15) / 16 * 16), (uint64_t)K, (uint64_t)y->ldb, (uint32_t)L.block_n))
         return IM_ERR_CUDA;
-    second.c = second.m = second.a;
+    second.c = second.a;
     gp.N2 = N2; gp.bias2 = y->bias; gp.mean2 = static_cast<float *>(y->C);
     return dispatch_head<true>(L, gp, n_sm, second, stream) == cudaSuccess ? IM_OK : IM_ERR_CUDA;
 }
