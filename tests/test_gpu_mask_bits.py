@@ -51,3 +51,12 @@ def test_mask_bits_give_the_gradients_of_the_activations(M, dims, cdims):
             assert torch.equal(got.db[l], want.db[l]), (l, M)
             if not shared:
                 assert torch.equal(got.dW[l], want.dW[l]), (l, M)
+
+
+def test_fewer_rows_than_the_trainer_has_room_for(monkeypatch):
+    """The mask words' columns lie max_rows apart, not as many as the minibatch has rows."""
+    from paper_2609_09821_b200 import trainer as T
+    make = T.MlpTrainer
+    monkeypatch.setattr(T, "MlpTrainer", lambda dims, W, b, rows: make(dims, W, b, rows + 192))
+    for dims, cdims in (((361, 1024, 512, 28), (361, 512, 256, 1)), ((361, 1024, 512, 28), (361, 1024, 512, 1))):
+        test_mask_bits_give_the_gradients_of_the_activations(64 * 61, dims, cdims)
