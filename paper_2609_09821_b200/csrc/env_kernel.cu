@@ -535,7 +535,8 @@ struct SimView {
     }
     // Records: the whole state of env `src` of the batch to column `col` of the staged bodies (component i of body b: the word
     // (13 b + i) * pitch + col), by the lanes of a warp, which walk along the record: a request takes the few lines that its
-    // words lie in, where a lane to every env takes 32.  An odd pitch keeps the words of a request in different banks.
+    // words lie in, where a lane to every env takes 32.  With an odd pitch the 32 words of a request meet two to a bank (rotations) or
+    // three (vectors), 13 words from body to body; with one of 32 they would all meet in one.
     static __device__ __forceinline__ void stage_record(const EnvKernelParams &P, int src, int J, uint32_t dst, uint32_t pitch, int col, int lane,
                                                         uint64_t policy)
     {
@@ -780,7 +781,7 @@ __device__ __forceinline__ void env_role_body(const EnvKernelParams &P, float *s
     float *part = smem_raw + (size_t)kTile * S;
     float4 *all_links = reinterpret_cast<float4 *>(part + (size_t)kPartials * C * kTile);
     const auto part_of = [&](int cc) { return part + cc * kPartials * kTile + lane; };
-    const uint32_t bodies = (uint32_t)__cvta_generic_to_shared(all_links + 2 * sk.n_links) + 4u * lane;    // [J][13][32]
+    const uint32_t bodies = (uint32_t)__cvta_generic_to_shared(all_links + 2 * sk.n_links) + 4u * lane;    // [J][13][kPitch]
 
     for (int i = threadIdx.x; i < 2 * sk.n_links; i += blockDim.x) all_links[i] = __ldg(P.links + i);
     __syncthreads();
@@ -1585,10 +1586,12 @@ int ctas_per_sm(size_t smem, int regs, int threads)
     return std::max(1, std::min(by_smem, std::min(by_regs, by_threads)));
 }
 
-// Whether records are staged all at once: where the envs of an array lie a multiple of 256 bytes apart, so that the words that a
-// lane to every env asks for at a time crowd into few sets of the L1 cache.  us per step in place / staged: 16 records an env of 3, 4
-// and 6 words (256 and 384 bytes apart), 15 of them bodies, 4096 envs 15.0 / 12.0, 12000 28.7 / 25.0, 30000 67.3 / 53.7; 25 records
-// (300, 400 and 600 bytes apart), 4096 envs 15.2 / 15.7.
+// Whether records are staged all at once: where the envs of one of the arrays lie a multiple of 256 bytes apart, so that the words
+// that a lane to every env asks for at a time crowd into few sets of the L1 cache.  us per step of 4096 envs in place / staged, records
+// of 3, 4 and 6 words: 15 bodies of 16 records an env (only the rotations 256 bytes apart) 14.7 / 11.8, of 32 15.8 / 11.8, but of 17 9.7 in
+// place; 24 bodies of 32 22.2 / 15.0, of 48 20.8 / 15.0, but of 25 (400 bytes) 14.5 in
+// place.  12000 and 30000 envs, 16 records:
+// 27.5 / 24.3 and 64.3 / 51.4.
 bool staged_records(const EnvKernelParams &p)
 {
     bool crowded = false;
@@ -1640,8 +1643,7 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         const auto ctas = [&](size_t bytes) { return (unsigned)ctas_per_sm(bytes, C <= 8 ? 96 : 64, 32 * C); };
         const auto waves = [&](size_t bytes) { const unsigned fit = n_sm * ctas(bytes); return (tiles + fit - 1) / fit; };
         const unsigned few = waves(chain_smem), many = waves(body_smem);
-        // (a reset of all envs keeps the halves: its warps have little to wait for, and 12000 envs x 15 bodies took 14.4 us with whole
-        // rows, 12.7 without)
+        // (a reset of all envs keeps the halves: its warps have little to wait for, and whole rows made 12000 envs x 15 bodies 13 % slower)
         const size_t whole = ((size_t)whole_floats(24 * p.sk.J + 1, C) + 8 * p.sk.n_links) * sizeof(float);
         if (ahead == 0 && (few < many || ctas(chain_smem) == ctas(body_smem))) smem = chain_smem;
         if constexpr (RESET_ALL) {

@@ -318,7 +318,7 @@ cudaError_t launch_linear_simt(const float *A, int lda, const void *W, bool w_bf
     // rows: 33.3 and 36.2; all of these before the partial tiles were padded).  Beyond that two 32 x 32 CTAs per SM while they are
     // one wave; then 64 x 48 while that is (300 / 700 rows: 37.4 / 65.5 us without, 34.8 / 62.9 with; where one wave of 32 x 32
     // does, at 200 rows, 30.0 and 32.4), 32 x 32 up to four per SM (512 rows: 52 us against 107 with 64 x 64; one wave of 64 x 64
-    // with sixteen warps 51 against 45.6), and 64 x 64 (2048 rows: 142 us against 156)
+    // with sixteen warps 51 against 45.6), and 64 x 64 (2048 rows, before the padding too: 142 us against 156)
     const int n_sm = device_sm_count();
     if (tiles(16, 16) <= n_sm) e = launch_tile<Tile<512, 16, 16, 256, 1, 1, 3>>(L, w_bf16, stream);
     else if (tiles(32, 16) <= n_sm) e = launch_tile<Tile<512, 32, 16, 128, 1, 1, 3>>(L, w_bf16, stream);

@@ -269,8 +269,10 @@ __global__ void __launch_bounds__(kThreads) grad_reduce_kernel(const __grid_cons
 constexpr int kOutRows = 128;
 constexpr int kOutBatch = 16;
 
-// 128 rows of a net to a block; the first block has the loss's sums, which nothing waits for before the gradient reduction (as a
-// launch of their own they took 5 us between the loss and this one).
+// 128 rows of a net to a block; the first block has the loss's sums, which the gradient reduction reads.  The products in between wait
+// for this grid, sums and all, so that what is saved is a launch (us per update with one of its own, of 1024 threads / here, 256: 4096
+// rows of 361-1024-512-28 and -1 111.8 / 109.0, 131072 1310 / 1303; 131072 rows, 888 partial sums, of 577-1024-512-69 1538 / 1529, -80
+// 1551 / 1545).
 __global__ void __launch_bounds__(kThreads) out_grads_kernel(const __grid_constant__ OutGradArgs P)
 {
     __shared__ float s_sum[8][128];
