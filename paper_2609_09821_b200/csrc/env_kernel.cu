@@ -1635,7 +1635,7 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         // 64 registers spill more, x 20000 (3 / 2) 61.7 / 60.0, x 30000 (4 / 3) 85.7 / 91.2.  What stages nothing asks for
         // that memory all the same where fewer CTAs make no further wave: a reset of 31 in 10 x 16384, two waves with three CTAs per SM or
         // two 31.7 and 26.8 (x 12000, one wave or two: 20.0 and 26.2); 32 records of 3, 4 and 6 words, 20 bodies in 4 chains x 30000, two
-        // waves with five or four 89.4 and 76.5.
+        // waves with five or four 89.4 and 73.1.
         constexpr int ahead = RESET_ALL || AOS ? 0 : kBody;
         void (*kernel)(EnvKernelParams) = C > 8 ? env_chain_kernel_wide<RESET_ALL, OPT, AOS, ahead> : env_chain_kernel<RESET_ALL, OPT, AOS, ahead>;
         const size_t body_smem = smem_floats(p.sk.J, C, p.sk.n_links, extra, kBody) * sizeof(float);
@@ -1643,10 +1643,10 @@ void launch_one(const EnvKernelParams &p, size_t chain_smem, cudaStream_t stream
         const auto ctas = [&](size_t bytes) { return (unsigned)ctas_per_sm(bytes, C <= 8 ? 96 : 64, 32 * C); };
         const auto waves = [&](size_t bytes) { const unsigned fit = n_sm * ctas(bytes); return (tiles + fit - 1) / fit; };
         const unsigned few = waves(chain_smem), many = waves(body_smem);
-        // (a reset of all envs keeps the halves: its warps have little to wait for, and whole rows made 12000 envs x 15 bodies 13 % slower)
         const size_t whole = ((size_t)whole_floats(24 * p.sk.J + 1, C) + 8 * p.sk.n_links) * sizeof(float);
         if (ahead == 0 && (few < many || ctas(chain_smem) == ctas(body_smem))) smem = chain_smem;
         if constexpr (RESET_ALL) {
+            // (the halves: a reset's warps have little to wait for, and whole rows made 12000 envs x 15 bodies 13 % slower)
         } else if constexpr (AOS) {
             const size_t records = ((size_t)records_floats(p.sk.J, 24 * p.sk.J + 1 + extra) + 8 * p.sk.n_links) * sizeof(float);
             if (C <= 8 && staged_records(p) && ctas(records) >= ctas(body_smem)) {

@@ -36,9 +36,8 @@ constexpr int UMMA_K = 16;
 // Epilogues of the hidden-layer kernels: bias and floor; the same and the outputs' signs as bits; backward with the ReLU mask as
 // boxes of the forward activations; backward with the mask as bits.  A box costs as much L2 traffic as the output, which these
 // products are bound by: a minibatch update with boxes / bits, actor and critic, 16000 rows of 361-1024-512-28 258 / 250 us,
-// 131072 rows of 577-1024-1024-512-69 3435 / 3315; on 64-column tiles, whose forward epilogue is the longer part, the two are even
-// (361-320-192-33, 16000 rows 133.3 / 131.1, 131072 rows 652 / 658).  (The bits are an epilogue of their own: tested for at run time they cost the
-// policy's products 1 %.)
+// 131072 rows of 577-1024-1024-512-69 3435 / 3315; on 64-column tiles the two are even (361-320-192-33, 16000 rows 133.3 / 131.1,
+// 131072 rows 652 / 658).  (The bits are an epilogue of their own: tested for at run time they cost the policy's products 1 %.)
 constexpr int kFwd = 0, kFwdBits = 1, kBwdBoxes = 2, kBwdBits = 3;
 constexpr __host__ __device__ bool is_bwd(int epi) { return epi >= kBwdBoxes; }
 
